@@ -201,7 +201,8 @@ int lts_transfer_bytes(lts_t* h, int64_t* h2d, int64_t* d2h);
  * error per product). LTS_CONTRACT_SPARSE (the default): FP32 CUDA cores with
  * the products of K_c, of the face matrices F~_i and of their transposes generated at build
  * time from the nonzero entries only (Sec. IV-A "all sparsity"), in the predict kernel and
- * in a neighbour kernel that forms X F-_{j,h} as (X F~_j) R_h (R_h the face-basis map of the
+ * in a neighbour kernel that reads the traces X F~_j which the predict kernel stores as its LTS
+ * buffers and forms X F-_{j,h} as (X F~_j) R_h (R_h the face-basis map of the
  * orientation); with fused simulations it runs (element, simulation) slots, and a
  * partitioned run keeps the other engines' neighbour kernel. The adjoint's reverse predict
  * pass (lts_misfit_gradient) uses the same generated products (their transposed forms);
@@ -213,8 +214,8 @@ enum { LTS_CONTRACT_FP32 = 0, LTS_CONTRACT_TF32X3 = 1, LTS_CONTRACT_TF32 = 2, LT
 int lts_set_contraction(lts_t* h, int mode);
 
 /* Tile variant of the sparse engine's neighbour kernel (Sec. III-A neighbour surface
- * kernel): 0 = 8 elements per CTA (two CTAs per SM), 1 = 4 elements per CTA (four CTAs per
- * SM; the default). The arithmetic per element is the same, so the results are bitwise
+ * kernel): 0 = 10 elements per CTA (fused simulations: 8 slots), 1 = 5 elements (4 slots; the
+ * default). The arithmetic per element is the same, so the results are bitwise
  * identical; only the grouping of elements into CTAs changes. Set by lts_autotune; ignored
  * by the other engines. Errors: LTS_ERR_ARG for another value. */
 int lts_set_tile(lts_t* h, int tile);
@@ -341,7 +342,7 @@ int lts_set_wait_limit(lts_t* h, int64_t cycles, int suppress_commit);
 /* Autotuner over launch configurations: contraction engine (FP32 CUDA cores, sparse
  * products, split-tf32 tensor cores, and plain tf32 only if allow_tf32) x resident CTAs per
  * SM the predict and neighbour grids are sized for (the occupancy maximum and one fewer) x
- * tile variant (sparse engine: the neighbour kernel's 8 or 4 elements per CTA; other
+ * tile variant (sparse engine: the neighbour kernel's 10 or 5 elements per CTA; other
  * engines: 0). Each candidate advances one macro step from a device-side snapshot of the
  * state, timed with CUDA events on `cuda_stream` after one untimed warm-up step; the state
  * (DOFs, LTS buffers, time, receiver samples) is restored exactly after every trial, so the

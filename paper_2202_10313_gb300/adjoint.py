@@ -117,7 +117,7 @@ def main():
     ap.add_argument("--receivers", type=int, default=32)
     ap.add_argument("--fd", type=int, default=3, help="elements checked by central differences")
     ap.add_argument("--tile", type=int, default=None,
-                    help="tile variant of the sparse engine's neighbour kernel (0: 8 elements per CTA, 1: 4)")
+                    help="tile variant of the sparse engine's neighbour kernel (0: 10 elements per CTA, 1: 5)")
     ap.add_argument("--fused", type=int, default=1,
                     help="F > 1: F sources in one fused run (gradient of the summed misfit), timed "
                          "against one single-source gradient")

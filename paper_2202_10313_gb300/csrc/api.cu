@@ -238,7 +238,7 @@ void face_orientation_maps(const lts::RefOps& ops, std::vector<float>& out) {
 }
 
 struct Layout {
-  size_t Q, B1, B2, B3, edata, ndata, nbr, ncode, meta, emat, partial, err, K, Ft, Fh, Fb, Rh, rphi, sphi, cut, msg,
+  size_t Q, B1, B2, B3, edata, ndata, sdata, sndata, nbr, ncode, meta, emat, partial, err, K, Ft, Fh, Fb, Rh, rphi, sphi, cut, msg,
       total;
 };
 
@@ -260,11 +260,18 @@ Layout layout_of(const lts_solver* h, int64_t K) {
   const Launchers& X = h->L;
   const size_t qs = (size_t)q_stride(h), bs = (size_t)buf_stride(h);
   L.Q = take(sizeof(float) * K * qs);
+  // the LTS buffers: as modes (B1, B2, B3), or as the sparse engine's face traces (T1, T2) in the
+  // same memory; every buffer is rewritten within a macro step, so an engine change between
+  // macro steps needs nothing
   L.B1 = take(sizeof(float) * K * bs);
   L.B2 = take(sizeof(float) * K * bs);
   L.B3 = take(sizeof(float) * K * bs);
+  const size_t traces = sizeof(float) * 2 * K * (size_t)X.TS * h->nsim;
+  if (off < L.B1 + traces) take(L.B1 + traces - off);
   L.edata = take(sizeof(float) * K * ltsdev::ED);
   L.ndata = take(sizeof(float) * K * ltsdev::ND);
+  L.sdata = take(sizeof(float) * K * ltsdev::EDS);
+  L.sndata = take(sizeof(float) * K * ltsdev::NDS);
   L.nbr = take(sizeof(int) * K * 4);
   L.ncode = take(sizeof(int) * K * 4);
   L.meta = take(sizeof(int) * K);
@@ -347,7 +354,8 @@ void setup_device(lts_solver* h) {
   for (int64_t i = 0; i < K; ++i) h->cbeg[h->cluster[i] + 1]++;
   for (int l = 0; l < h->nc; ++l) h->cbeg[l + 1] += h->cbeg[l];
   // ---- host tables in internal order
-  std::vector<float> edata(K * ltsdev::ED, 0.f), ndata(K * ltsdev::ND, 0.f);
+  std::vector<float> edata(K * ltsdev::ED, 0.f), ndata(K * ltsdev::ND, 0.f), sdata(K * ltsdev::EDS, 0.f),
+      sndata(K * ltsdev::NDS, 0.f);
   std::vector<int> nbr(4 * K, -1), ncode(4 * K, 0), meta(K, 0);
   std::vector<double> emat(4 * K);
   const lts::Mesh& M = h->mesh;
@@ -367,6 +375,14 @@ void setup_device(lts_solver* h) {
     nd[0] = ed[9];
     nd[1] = ed[10];
     nd[2] = ed[11];
+    float* sd = &sdata[nk * ltsdev::EDS];
+    std::copy(ed, ed + 9, sd);
+    for (int d = 0; d < 3; ++d)
+      sd[9 + d] = (float)-(M.Jinv[9 * k + d] + M.Jinv[9 * k + 3 + d] + M.Jinv[9 * k + 6 + d]);
+    std::copy(ed + 9, ed + 12 + 2 * m, sd + 12);
+    float* sn = &sndata[nk * ltsdev::NDS];
+    std::copy(sd, sd + 15, sn);
+    int rels = 0;
     emat[4 * nk + 0] = h->lam[k];
     emat[4 * nk + 1] = h->mu[k];
     emat[4 * nk + 2] = rho;
@@ -392,16 +408,31 @@ void setup_device(lts_solver* h) {
         lf[3 + q] = (float)cl[q];
         nf[3 + q] = (float)cn[q];
       }
+      // the sparse engine's interface states take the traction scaled by s = scale and return
+      // v* unscaled and s t* (interface_state)
+      float* sf = sd + 24 + 12 * f;
+      const double factor[4] = {1.0 / scale, 1.0 / (scale * scale), 1.0 / scale, 1.0};
+      for (int d = 0; d < 3; ++d) sf[d] = lf[d];
+      for (int q = 0; q < 8; ++q) sf[3 + q] = (float)(cl[q] * factor[q % 4]);
+      // the neighbour's trace carries its traction scaled by its own s and its own normal
+      float* snf = sn + 16 + 12 * f;
+      const double sn_ = nb >= 0 ? -2.0 * M.area[4 * nb + M.nbr_face[4 * k + f]] / M.detJ[nb] : scale;
+      const double nfactor[4] = {1.0 / scale, -1.0 / (scale * sn_), -1.0 / sn_, 1.0};
+      for (int d = 0; d < 3; ++d) snf[d] = lf[d];
+      for (int q = 0; q < 8; ++q) snf[3 + q] = (float)(cn[q] * nfactor[q % 4]);
       if (nb >= 0) {
         nbr[4 * nk + f] = (int)h->iperm[nb];
         const int dc = h->cluster[nb] - h->cluster[k];
         const int rel = dc == 0 ? 0 : (dc < 0 ? 1 : 2);
         ncode[4 * nk + f] = (M.nbr_face[4 * k + f] * 3 + M.nbr_orient[4 * k + f]) | (rel << 8);
+        rels |= (dc == 0 ? 1 : (dc < 0 ? 2 : 3)) << (2 * f);
         if (dc < 0) flags |= ltsdev::FLAG_FINER;
         if (dc > 0) flags |= ltsdev::FLAG_COARSER;
       }
     }
     meta[nk] = flags;
+    std::memcpy(sd + 23, &flags, sizeof(int));
+    std::memcpy(sd + 21, &rels, sizeof(int));
   }
   // ---- operators (float)
   const int B = X.B, F = X.F;
@@ -472,6 +503,10 @@ void setup_device(lts_solver* h) {
   h->dst.B3 = reinterpret_cast<float*>(base + Lo.B3);
   h->dst.edata = reinterpret_cast<float*>(base + Lo.edata);
   h->dst.ndata = reinterpret_cast<float*>(base + Lo.ndata);
+  h->dst.sdata = reinterpret_cast<float*>(base + Lo.sdata);
+  h->dst.sndata = reinterpret_cast<float*>(base + Lo.sndata);
+  h->dst.T1 = h->dst.B1;
+  h->dst.T2 = h->dst.T1 + K * (int64_t)X.TS * h->nsim;
   h->dst.nbr = reinterpret_cast<int*>(base + Lo.nbr);
   h->dst.ncode = reinterpret_cast<int*>(base + Lo.ncode);
   h->dst.meta = reinterpret_cast<int*>(base + Lo.meta);
@@ -495,12 +530,12 @@ void setup_device(lts_solver* h) {
   h->dst.bs = buf_stride(h);
   h->dst.nsim = h->nsim;
   ck(cudaMemset(h->dst.Q, 0, sizeof(float) * K * h->dst.qs), "memset Q");
-  ck(cudaMemset(h->dst.B1, 0, sizeof(float) * K * h->dst.bs), "memset B1");
-  ck(cudaMemset(h->dst.B2, 0, sizeof(float) * K * h->dst.bs), "memset B2");
-  ck(cudaMemset(h->dst.B3, 0, sizeof(float) * K * h->dst.bs), "memset B3");
+  ck(cudaMemset(h->dst.B1, 0, Lo.edata - Lo.B1), "memset LTS buffers");
   ck(cudaMemset(h->d_err, 0, sizeof(int)), "memset error word");
   up(h->dst.edata, edata.data(), sizeof(float) * edata.size());
   up(h->dst.ndata, ndata.data(), sizeof(float) * ndata.size());
+  up(h->dst.sdata, sdata.data(), sizeof(float) * sdata.size());
+  up(h->dst.sndata, sndata.data(), sizeof(float) * sndata.size());
   up(h->dst.nbr, nbr.data(), sizeof(int) * nbr.size());
   up(h->dst.ncode, ncode.data(), sizeof(int) * ncode.size());
   up(h->dst.meta, meta.data(), sizeof(int) * meta.size());
@@ -698,7 +733,10 @@ PhaseArgs phase_args(const lts_solver* h, const Phase& ph) {
 // Enqueues the launches of one phase on `stream` (work items at the start of the item
 // buffers); returns the number of kernels launched. Receivers are skipped when
 // with_receivers is false (state-only replays).
-int enqueue_phase(lts_solver* h, const Phase& ph, cudaStream_t stream, bool with_receivers = true) {
+// adjoint (replays whose buffers the reverse sweep reads): the LTS buffers also as modes, the face
+// traces in the memory given.
+int enqueue_phase(lts_solver* h, const Phase& ph, cudaStream_t stream, bool with_receivers = true,
+                  float* adjoint_traces = nullptr) {
   const Launchers& X = h->L;
   const bool use_sp = h->contraction == LTS_CONTRACT_SPARSE;
   const bool use_tc = h->contraction == LTS_CONTRACT_TF32X3 || h->contraction == LTS_CONTRACT_TF32;
@@ -711,7 +749,13 @@ int enqueue_phase(lts_solver* h, const Phase& ph, cudaStream_t stream, bool with
   const int maxn = std::max(1, use_nsp ? X.blocks_neighbour_sp[tv] : X.blocks_neighbour);
   const int grid_cap_p = h->num_sms * (h->ctas_predict > 0 ? std::min(h->ctas_predict, maxp) : maxp);
   const int grid_cap_n = h->num_sms * (h->ctas_neighbour > 0 ? std::min(h->ctas_neighbour, maxn) : maxn);
-  const PhaseArgs pa = phase_args(h, ph);
+  PhaseArgs pa = phase_args(h, ph);
+  pa.bufs = !use_nsp ? ltsdev::BUFS_MODAL : (adjoint_traces ? ltsdev::BUFS_MODAL | ltsdev::BUFS_TRACES : ltsdev::BUFS_TRACES);
+  DevState dst = h->dst;
+  if (adjoint_traces) {
+    dst.T1 = adjoint_traces;
+    dst.T2 = adjoint_traces + h->mesh.K * (int64_t)X.TS * h->nsim;
+  }
   const int nelem = pa.end - pa.begin;
   if (nelem <= 0) return 0;
   int launches = 0;
@@ -747,14 +791,14 @@ int enqueue_phase(lts_solver* h, const Phase& ph, cudaStream_t stream, bool with
   }
   if (h->profiling) ck(cudaEventRecord(next_event(h), stream), "event record");
   if (ph.kind == 0 && use_nsp)
-    X.neighbour_sp[tv](h->dops, h->dst, pa, std::min(nb, grid_cap_n), stream);
+    X.neighbour_sp[tv](h->dops, dst, pa, std::min(nb, grid_cap_n), stream);
   else if (ph.kind == 0)
     X.neighbour(h->dops, h->dst, pa, std::min(nb, grid_cap_n), stream);
   else if (use_tc)
     X.predict_tc(h->dops, h->dst, pa, std::min(nb, grid_cap_p), passes, h->d_err, h->wait_cycles, h->suppress_commit,
                  stream);
   else if (use_sp)
-    X.predict_sp(h->dops, h->dst, pa, std::min(nb, grid_cap_p), stream);
+    X.predict_sp(h->dops, dst, pa, std::min(nb, grid_cap_p), stream);
   else
     X.predict(h->dops, h->dst, pa, std::min(nb, grid_cap_p), stream);
   ++launches;
@@ -1113,7 +1157,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   const int64_t ns = (int64_t)nsim * nrec * 3;   // sample values per sample time
   // the reverse sweep's state (adjoints, correlations, checkpoints) only when it runs
   const bool reverse = grad || dq0;
-  DevBuf d_syn, d_res, d_lq, d_lb, d_w, d_cp, d_mac, d_qn;
+  DevBuf d_syn, d_res, d_lq, d_lb, d_w, d_cp, d_mac, d_qn, d_tr;
   d_syn.alloc(sizeof(float) * (n_macro + 1) * ns);
   if (reverse) {
     d_res.alloc(sizeof(float) * (n_macro + 1) * ns);
@@ -1122,6 +1166,10 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
     d_w.alloc(sizeof(double) * K * ltsdev::AM_SIZE);
     d_cp.alloc(sizeof(float) * ncp * K * qs);
     d_qn.alloc(sizeof(float) * K * qs);
+    // the replays write the LTS buffers as modes for the reverse sweep; the sparse engine's face
+    // traces, which usually share their memory, get their own
+    if (h->contraction == LTS_CONTRACT_SPARSE && h->n_parts <= 1)
+      d_tr.alloc(sizeof(float) * 2 * K * (size_t)X.TS * nsim);
   }
   // moment-tensor gradient: [source][6] and one pass's source items with their scales
   const int nsrc = (int)h->sources.size();
@@ -1297,7 +1345,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
         dcopy(dst + one, h->dst.B2, one);
         dcopy(dst + 2 * one, h->dst.B3, one);
       }
-      enqueue_phase(h, ph, stream, false);
+      enqueue_phase(h, ph, stream, false, d_tr.get<float>());
     }
     for (int r = 0; r < nrec; ++r) {
       h->receivers[r].t.resize(nrec_t[r]);

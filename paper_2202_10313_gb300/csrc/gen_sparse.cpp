@@ -26,6 +26,20 @@
 //       the four faces' interface states, F^_i = F~_i^T in the orthonormal face basis).
 //   sp_ntrace_o{O}(j, x, y): G_j[f] = sum_k x[k] F~_j[k][f] of one row of a neighbour's
 //       buffer on the face j that each thread asks for (neighbour kernel).
+// The forward kernels' products come in row form (sg_*): a thread holds one row of a set,
+// contiguous in memory, and reads and writes it four modes at a time. Set c (0, 1, 2: reference
+// direction xi_c; 3: the direction of the fourth barycentric coordinate) has six rows: the
+// velocities v_j and the direction's stress rows tau_c = sum_d dxi_c/dx_d sigma_d. One reference
+// derivative is all a row of set c needs, so the products of a set use K_c alone:
+//   sg_time_o{O}(variant, part, x, dx, y): y[c DY + b] = sum_k x[c dx + k] K_c[b][k], c < 3
+//   sg_vol_o{O}(part, x, dx, y, g): y[c DY + b] = sum_k x[c dx + k] K_c[k][b] (c < 3) and the
+//       trace of set c on its face f(c), g[f DG + m] = sum_k x[c dx + k] F~_f[k][m]
+//   sg_proj_o{O}(part, g, y, p): F^_f of the face states g[f DG + m], added to y[c(f) DY + b]
+//       for c < 3, written to p[b] for face 3
+//   sg_nproj_o{O}(face, g, y): y[face DY + b] = F^_face of g[face DG + m] (neighbour kernel)
+// (x, y: the row of set 0; dx: the distance between a thread's rows of consecutive sets, 0 for
+// the velocities, which all sets share; DY, DG template parameters). Outputs are split into parts
+// of equal multiply-add count.
 // and for the reverse predict pass of the discrete adjoint (k_adj_pred_sp):
 //   sp_trace_o{O}(part, x, g): G_i[f] = sum_k x[k] F~_i[k][f] alone (the traces of sp_vol).
 //   sp_tproj_o{O}(part, x, y): y[b] = sum_i sum_f x[i F + f] F~_i[b][f] (the transposed face
@@ -40,6 +54,9 @@
 //
 // Usage: gen_sparse <out.cuh>      writes the header
 //        gen_sparse --list <order> lists every product term, one line each:
+//        gen_sparse --list-rows <order> lists the terms of the row-form products likewise:
+//        kind T (output c B + b, input c B + k), V (volume, the same), G (trace, output f F + m,
+//        input k) or P (output f B + b, input f F + m);
 //        "<kind> <part> <output> <input> <value>", kind t (time kernel, output c B + b, full
 //        variant), v (volume, output c B + b), g (face trace, output i F + f), p (face
 //        projection, output i B + b, input i F + f), n (neighbour face trace, output j F + f),
@@ -66,6 +83,34 @@ struct Out {
 };
 
 using Parts = std::vector<std::vector<int>>;
+
+// One output of a row-form product: set (or face) it belongs to, output row id, inputs.
+struct RowOut {
+  char kind;                             // T, V, G, P
+  int set;                               // set of the input row (P: face)
+  int idx, count;                        // output mode and the outputs of its row (stores in fours)
+  std::vector<std::pair<int, float>> t;  // (input mode, value), ascending
+};
+
+// The face opposite barycentric coordinate c: xi_c = 0 for c < 3 (faces 2, 1, 0), face 3 for c = 3.
+int face_of_set(int c) { return c < 3 ? 2 - c : 3; }
+
+// Consecutive runs of the outputs with multiply-add shares as the weights ask.
+Parts partition_weighted(const std::vector<RowOut>& outs, const std::vector<double>& weights) {
+  double total = 0.0, wsum = 0.0;
+  for (const RowOut& u : outs) total += u.t.size();
+  for (double w : weights) wsum += w;
+  Parts parts(weights.size());
+  size_t p = 0;
+  double acc = 0.0, upto = weights[0] / wsum * total;
+  for (size_t o = 0; o < outs.size(); ++o) {
+    const double w = (double)outs[o].t.size();
+    while (p + 1 < parts.size() && acc + 0.5 * w > upto) upto += weights[++p] / wsum * total;
+    parts[p].push_back((int)o);
+    acc += w;
+  }
+  return parts;
+}
 
 // Parts of nearly equal multiply-add count (a store counts as one), each a contiguous run
 // of the outputs in the given order.
@@ -104,6 +149,55 @@ struct Products {
   std::vector<std::vector<Out>> kvol;    // reverse time kernel, per level
   std::vector<Parts> kvol_parts;
   size_t time_terms = 0, vol_terms = 0, face_terms = 0;
+  // row-form products: outputs of set c (or face f), see RowOut
+  std::vector<std::vector<RowOut>> rtime;   // per variant
+  std::vector<Parts> rtime_parts;
+  std::vector<RowOut> rvol, rproj;
+  Parts rvol_parts, rproj_parts;
+
+  template <typename NzK, typename NzF>
+  void build_rows(const lts::RefOps& ops, const NzK& nzk, const NzF& nzf) {
+    const std::vector<double> wt(O == 5 ? 4 : (O == 4 ? 3 : 1), 1.0), wv = wt, wp = wt;
+    for (int v = 0; v <= O - 2; ++v) {
+      const int kend = nb(O - v), bend = nb(O - 1 - v);
+      std::vector<RowOut> outs;
+      for (int c = 0; c < 3; ++c)
+        for (int b = 0; b < bend; ++b) {
+          RowOut u{'T', c, b, bend, {}};
+          for (int k = 0; k < kend; ++k)
+            if (nzk(ops.K[c][b * B + k])) u.t.push_back({k, (float)ops.K[c][b * B + k]});
+          outs.push_back(u);
+        }
+      rtime_parts.push_back(partition_weighted(outs, wt));
+      rtime.push_back(outs);
+    }
+    for (int q = 0; q < 4; ++q) {
+      const int c = (q + 3) % 4;   // set 3 has a trace only
+      if (c < 3)
+        for (int b = 0; b < B; ++b) {
+          RowOut u{'V', c, b, B, {}};
+          for (int k = 0; k < B; ++k)
+            if (nzk(ops.K[c][k * B + b])) u.t.push_back({k, (float)ops.K[c][k * B + b]});
+          rvol.push_back(u);
+        }
+      for (int m = 0; m < F; ++m) {
+        RowOut u{'G', c, m, F, {}};
+        const int f = face_of_set(c);
+        for (int k = 0; k < B; ++k)
+          if (nzf(ops.Ft[f][k * F + m])) u.t.push_back({k, (float)ops.Ft[f][k * F + m]});
+        rvol.push_back(u);
+      }
+    }
+    rvol_parts = partition_weighted(rvol, wv);
+    for (int f = 0; f < 4; ++f)
+      for (int b = 0; b < B; ++b) {
+        RowOut u{'P', f, b, B, {}};
+        for (int m = 0; m < F; ++m)
+          if (nzf(ops.Ft[f][b * F + m])) u.t.push_back({m, (float)ops.Ft[f][b * F + m]});
+        rproj.push_back(u);
+      }
+    rproj_parts = partition_weighted(rproj, wp);
+  }
 
   void build(int order, int np) {
     O = order;
@@ -189,6 +283,7 @@ struct Products {
       }
       ntrace.push_back(outs);
     }
+    build_rows(ops, nzk, nzf);
     // adjoint products: the face traces alone (as in vol, by face mode then face)
     ord.clear();
     for (const Out& u : vol)
@@ -282,38 +377,122 @@ void emit_dispatch(FILE* f, const char* name, const char* args, const char* call
   std::fprintf(f, "}\n");
 }
 
-// sp_ntrace_o{O}(j, x, y): G_j[f] = sum_k x[k] F~_j[k][f] for the face j the thread asks for
-// (j < 0: none). A warp computes the faces that any of its lanes asks for (warp-uniform
-// branches; every lane of the warp must call it) and each lane stores its own face's F
-// outputs y[f * XP].
-void emit_ntrace(FILE* f, int O, const Products& P) {
-  std::fprintf(f, "template <int XP>\n__device__ __forceinline__ void sp_ntrace_o%d(int j, const float* __restrict__ x, "
-               "float* __restrict__ y) {\n", O);
-  std::vector<int> need;
-  for (auto& outs : P.ntrace)
-    for (auto& u : outs)
-      for (auto& t : u.t) need.push_back(t.first);
-  std::sort(need.begin(), need.end());
-  need.erase(std::unique(need.begin(), need.end()), need.end());
-  for (int k : need) std::fprintf(f, "  const float x%d = x[%d * XP];\n", k, k);
-  for (int j = 0; j < 4; ++j) {
-    std::fprintf(f, "  if (__any_sync(0xffffffffu, j == %d)) {\n", j);
-    const auto& outs = P.ntrace[j];
-    for (size_t m = 0; m < outs.size(); ++m) {
-      const Out& u = outs[m];
-      if (u.t.empty()) {
-        std::fprintf(f, "    const float a%zu = 0.f;\n", m);
-        continue;
-      }
-      std::fprintf(f, "    float a%zu = x%d * %s;\n", m, u.t[0].first, flt(u.t[0].second).c_str());
-      for (size_t i = 1; i < u.t.size(); ++i)
-        std::fprintf(f, "    a%zu = fmaf(x%d, %s, a%zu);\n", m, u.t[i].first, flt(u.t[i].second).c_str(), m);
+// Straight-line body of one part of a row-form product: per set, the input row four modes at a
+// time, one fma chain per output, stores of four outputs where the part holds all four (padding
+// modes are stored as zeros).
+// apart: projections are written per face instead of added to their direction's row.
+void emit_row_part(FILE* f, const std::vector<RowOut>& outs, const std::vector<int>& part, bool apart) {
+  size_t i = 0;
+  while (i < part.size()) {
+    const int set = outs[part[i]].set;
+    size_t e = i;
+    std::vector<int> need;
+    while (e < part.size() && outs[part[e]].set == set) {
+      for (auto& t : outs[part[e]].t) need.push_back(t.first / 4);
+      ++e;
     }
-    std::fprintf(f, "    if (j == %d) {\n", j);
-    for (size_t m = 0; m < outs.size(); ++m) std::fprintf(f, "      %s = a%zu;\n", outs[m].dst.c_str(), m);
-    std::fprintf(f, "    }\n  }\n");
+    std::sort(need.begin(), need.end());
+    need.erase(std::unique(need.begin(), need.end()), need.end());
+    const bool proj = outs[part[i]].kind == 'P';
+    std::fprintf(f, "    {\n");
+    if (proj)
+      std::fprintf(f, "      const float* xs = g + %d * DG;\n", set);
+    else
+      std::fprintf(f, "      const float* xs = x + %d * dx;\n", set);
+    for (int g : need)
+      std::fprintf(f, "      const float4 q%d = *reinterpret_cast<const float4*>(xs + %d);\n", g, 4 * g);
+    while (i < e) {
+      // the outputs of this group of four that the part holds
+      const RowOut& u0 = outs[part[i]];
+      const int grp = u0.idx / 4;
+      size_t j = i;
+      while (j < e && outs[part[j]].kind == u0.kind && outs[part[j]].idx / 4 == grp) ++j;
+      const int have = (int)(j - i), want = std::min(4, u0.count - 4 * grp);
+      char dst[64];
+      if (u0.kind == 'G')
+        std::snprintf(dst, sizeof dst, "g + %d * DG", face_of_set(set));
+      else if (proj && apart)
+        std::snprintf(dst, sizeof dst, "y + %d * DY", set);
+      else if (proj && set == 3)
+        std::snprintf(dst, sizeof dst, "p");
+      else
+        std::snprintf(dst, sizeof dst, "y + %d * DY", proj ? 2 - set : set);
+      const bool add = proj && set < 3 && !apart;
+      std::fprintf(f, "      {\n        float* d = %s + %d;\n", dst, 4 * grp);
+      const bool whole = have == want;
+      static const char* comp = "xyzw";
+      if (whole && add) std::fprintf(f, "        const float4 s = *reinterpret_cast<const float4*>(d);\n");
+      for (size_t o = i; o < j; ++o) {
+        const RowOut& u = outs[part[o]];
+        const int l = u.idx % 4;
+        if (add && whole)
+          std::fprintf(f, "        float a%d = s.%c;\n", l, comp[l]);
+        else if (add)
+          std::fprintf(f, "        float a%d = d[%d];\n", l, l);
+        else if (u.t.empty())
+          std::fprintf(f, "        float a%d = 0.f;\n", l);
+        for (size_t k = 0; k < u.t.size(); ++k) {
+          const int g = u.t[k].first / 4;
+          const char cc = comp[u.t[k].first % 4];
+          if (k == 0 && !add)
+            std::fprintf(f, "        float a%d = q%d.%c * %s;\n", l, g, cc, flt(u.t[k].second).c_str());
+          else
+            std::fprintf(f, "        a%d = fmaf(q%d.%c, %s, a%d);\n", l, g, cc, flt(u.t[k].second).c_str(), l);
+        }
+      }
+      if (whole) {
+        std::fprintf(f, "        *reinterpret_cast<float4*>(d) = make_float4(");
+        for (int l = 0; l < 4; ++l) std::fprintf(f, l < want ? "%sa%d" : "%s0.f", l ? ", " : "", l);
+        std::fprintf(f, ");\n");
+      } else {
+        for (size_t o = i; o < j; ++o) std::fprintf(f, "        d[%d] = a%d;\n", outs[part[o]].idx % 4, outs[part[o]].idx % 4);
+      }
+      std::fprintf(f, "      }\n");
+      i = j;
+    }
+    std::fprintf(f, "    }\n");
+  }
+}
+
+void emit_row_dispatch(FILE* f, const char* name, const char* tmpl, const char* targs, const char* args,
+                       const char* call, const std::vector<Parts>& parts, const std::vector<std::vector<RowOut>>& outs,
+                       bool apart = false) {
+  for (size_t v = 0; v < parts.size(); ++v)
+    for (size_t p = 0; p < parts[v].size(); ++p) {
+      std::fprintf(f, "template <%s>\n__device__ __forceinline__ void %s_v%zu_p%zu(%s) {\n", tmpl, name, v, p, args);
+      emit_row_part(f, outs[v], parts[v][p], apart);
+      std::fprintf(f, "}\n");
+    }
+  std::fprintf(f, "template <%s>\n__device__ __forceinline__ void %s(int variant, int part, %s) {\n", tmpl, name, args);
+  for (size_t v = 0; v < parts.size(); ++v) {
+    if (parts.size() > 1) std::fprintf(f, "  if (variant == %zu) {\n", v);
+    std::fprintf(f, "  switch (part) {\n");
+    for (size_t p = 0; p < parts[v].size(); ++p)
+      std::fprintf(f, "    case %zu: %s_v%zu_p%zu<%s>(%s); break;\n", p, name, v, p, targs, call);
+    std::fprintf(f, "    default: break;\n  }\n");
+    if (parts.size() > 1) std::fprintf(f, "  return;\n  }\n");
   }
   std::fprintf(f, "}\n");
+}
+
+void emit_rows(FILE* f, int O, const Products& P) {
+  char nm[64];
+  std::snprintf(nm, sizeof nm, "sg_time_o%d", O);
+  emit_row_dispatch(f, nm, "int DY", "DY", "const float* __restrict__ x, int dx, float* __restrict__ y", "x, dx, y",
+                    P.rtime_parts, P.rtime);
+  std::snprintf(nm, sizeof nm, "sg_vol_o%d", O);
+  emit_row_dispatch(f, nm, "int DY, int DG", "DY, DG",
+                    "const float* __restrict__ x, int dx, float* __restrict__ y, float* __restrict__ g", "x, dx, y, g",
+                    {P.rvol_parts}, {P.rvol});
+  std::snprintf(nm, sizeof nm, "sg_proj_o%d", O);
+  emit_row_dispatch(f, nm, "int DY, int DG", "DY, DG",
+                    "const float* __restrict__ g, float* __restrict__ y, float* __restrict__ p", "g, y, p",
+                    {P.rproj_parts}, {P.rproj});
+  std::snprintf(nm, sizeof nm, "sg_nproj_o%d", O);
+  Parts faces(4);
+  for (size_t o = 0; o < P.rproj.size(); ++o) faces[P.rproj[o].set].push_back((int)o);
+  emit_row_dispatch(f, nm, "int DY, int DG", "DY, DG", "const float* __restrict__ g, float* __restrict__ y", "g, y",
+                    {faces}, {P.rproj}, true);
 }
 
 void emit_order(FILE* f, int O, int nparts) {
@@ -327,12 +506,6 @@ void emit_order(FILE* f, int O, int nparts) {
   char nm[64];
   std::snprintf(nm, sizeof nm, "sp_time_o%d", O);
   emit_dispatch(f, nm, "const float* __restrict__ x, float* __restrict__ y", "x, y", P.time_parts, P.time, true);
-  std::snprintf(nm, sizeof nm, "sp_vol_o%d", O);
-  emit_dispatch(f, nm, "const float* __restrict__ x, float* __restrict__ y, float* __restrict__ g", "x, y, g",
-                {P.vol_parts}, {P.vol}, false);
-  std::snprintf(nm, sizeof nm, "sp_proj_o%d", O);
-  emit_dispatch(f, nm, "const float* __restrict__ x, float* __restrict__ y", "x, y", {P.proj_parts}, {P.proj}, false);
-  emit_ntrace(f, O, P);
   std::snprintf(nm, sizeof nm, "sp_trace_o%d", O);
   emit_dispatch(f, nm, "const float* __restrict__ x, float* __restrict__ g", "x, g", {P.trace_parts}, {P.trace},
                 false);
@@ -341,6 +514,7 @@ void emit_order(FILE* f, int O, int nparts) {
                 false);
   std::snprintf(nm, sizeof nm, "sp_kvol_o%d", O);
   emit_dispatch(f, nm, "const float* __restrict__ x, float* __restrict__ y", "x, y", P.kvol_parts, P.kvol, true);
+  emit_rows(f, O, P);
 }
 
 int parts_of(int O) { return O == 5 ? 4 : (O == 4 ? 2 : 1); }
@@ -367,6 +541,26 @@ int list_terms(int O) {
   return 0;
 }
 
+int list_rows(int O) {
+  Products P;
+  P.build(O, parts_of(O));
+  auto list = [&](const std::vector<RowOut>& outs, const Parts& parts) {
+    for (size_t p = 0; p < parts.size(); ++p)
+      for (int o : parts[p]) {
+        const RowOut& u = outs[o];
+        const int in = u.kind == 'P' ? P.F : (u.kind == 'G' ? 0 : P.B);   // input stride between sets
+        const int out = u.kind == 'G' ? P.F : P.B;
+        const int os = u.kind == 'G' ? face_of_set(u.set) : u.set;
+        for (auto& x : u.t)
+          std::printf("%c %zu %d %d %.9e\n", u.kind, p, os * out + u.idx, u.set * in + x.first, (double)x.second);
+      }
+  };
+  list(P.rtime[0], P.rtime_parts[0]);
+  list(P.rvol, P.rvol_parts);
+  list(P.rproj, P.rproj_parts);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -374,6 +568,11 @@ int main(int argc, char** argv) {
     const int O = std::atoi(argv[2]);
     if (O < 3 || O > 5) return 2;
     return list_terms(O);
+  }
+  if (argc == 3 && std::strcmp(argv[1], "--list-rows") == 0) {
+    const int O = std::atoi(argv[2]);
+    if (O < 3 || O > 5) return 2;
+    return list_rows(O);
   }
   if (argc != 2) {
     std::fprintf(stderr, "usage: gen_sparse <out.cuh> | gen_sparse --list <order>\n");

@@ -3,29 +3,35 @@
 // sparse form (one simulation, or (element, simulation) slots of fused simulations), and
 // k_neighbour_sp, the neighbour surface kernel of the same engine (below).
 //
-// Each time derivative (and the volume / face-trace step) is done in two phases separated
-// by a barrier:
-//   row phase:    thread = (part, pair), pair = (element e, quantity row r). The thread
-//                 keeps its row X_e[r][0..B) in registers and forms the products of one part
-//                 of the outputs with the nonzero operator entries as immediate operands
-//                 (sparse_ops.cuh, generated from the reference operators): Y_c[r][b] =
-//                 sum_k X[r][k] K_c[b][k] for the time kernel; Z_c[r][b] = sum_k T[r][k]
-//                 K_c[k][b] and G_i[r][f] = sum_k T[r][k] F~_i[k][f] for the volume and local
-//                 face kernels. No operator entry is read from memory and the structural zeros
-//                 of K_c and F~_i (Sec. IV-A "all sparsity") are not multiplied.
+// The products run on the rows the scheme needs and on no others. The star matrices are
+// combinations A_c = sum_d A_d dxi_c/dx_d, and A_d maps velocities to stresses and the stress
+// row sigma_d to velocities, so
+//   sum_c A_c X K_c^T  needs  K_c v_j  for the three velocities (nine velocity gradients) and
+//                             K_c tau_c with tau_c = sum_d dxi_c/dx_d sigma_d (three rows per
+//                             direction c, whose sum over c is the stress divergence),
+// 6 rows per K_c instead of 9: a third of the multiply-adds and of the staged results go. The
+// same rows carry the surface terms: dxi_c/dx is -2|S|/|det J| times the normal of the face
+// opposite to coordinate c (the fourth direction is -sum_c dxi_c/dx), so tau_c is that face's
+// scaled traction, the face's interface state (v*, scaled t*) projected through F^ adds to the
+// set of direction c, and one application of Hooke's law gives volume and surface terms together
+// (no flux rows per face).
+//
+// A derivative (and the volume / trace step, and the projection) is done in two phases
+// separated by a barrier:
+//   row phase:    lane = (row, element), elements fastest; a warp takes one part of the
+//                 generated products (immediate operands, sparse_ops.cuh) for two rows of all
+//                 16 elements, reading and writing its rows four modes at a time. No operator
+//                 entry is read from memory and the structural zeros of K_c and F~_i (Sec. IV-A
+//                 "all sparsity") are not multiplied.
 //   column phase: thread = (element e, mode b), modes fastest (fused simulations: the
-//                 simulations of an element fastest): it reads the 27 products of
-//                 its column, applies the star matrices (physical form), the
-//                 anelastic coupling and relaxation, adds the Taylor terms and writes the
-//                 next derivative's column back for the next row phase.
-// Shared-memory arrays are [mode or output][pair] with a pair stride XP = 1 mod 32, so the
-// row phase's loads and stores (consecutive pairs) and the column phase's accesses
-// (consecutive modes) fall on distinct banks.
-// The local surface kernel's interface states (closed-form Riemann solver of kernels.cuh) are
-// projected the same way (row phase with the generated F^_i products), and the column phase
-// forms the flux rows per face. A batch's DOFs arrive in shared memory by one bulk
-// asynchronous copy (TMA), issued a batch ahead. Receivers and sources are those of
-// kernels.cuh.
+//                 simulations of an element fastest): it combines the products of its mode
+//                 with dxi/dx and Hooke's law, applies the anelastic coupling and relaxation,
+//                 adds the Taylor terms and writes the next derivative's rows.
+// Staged rows are [element][row][mode] with an odd row stride and an odd element stride in
+// 16-byte units (eight lanes' 16-byte accesses fall on distinct banks), and an element stride
+// equal to the padded mode count modulo 32, so that the column phase's consecutive threads do too.
+// A batch's DOFs and element tables arrive in shared memory by bulk asynchronous copies (TMA),
+// issued a batch ahead. Receivers and sources are those of kernels.cuh.
 #pragma once
 #include "kernels.cuh"
 #include "sparse_ops.cuh"
@@ -33,75 +39,189 @@
 
 namespace ltsdev {
 
+// Shape of the predict kernel: a batch of 16 elements, so that the six rows of a set are three
+// full warps of (row, element) lanes, and NP parts of the row phases (3 NP warps). BP: padded
+// modes of a row, GP: stride of a face-state row, GS: of a face's six rows, YT: of a time-kernel
+// product's row, BBP: padded modes of top degree (column phase). Order 5: one CTA per SM (the
+// straight-line code of one phase at a time in the instruction cache); four parts, not six: a
+// part reads its rows whole, and six parts' reads bound the row phase by shared memory
+// (1,272 against 1,660 cycles a row phase at order 5).
+// What bounds it (order 5, anelastic, 16 elements, about 24,000 cycles): the row phases' staged reads
+// and multiply-adds one after the other (5,100 cycles over the four derivatives), the column
+// phases' instruction issue (5,900), the update's DOF stores. Measured on one GB300, 138,240
+// elements, one cluster: 4.7 ns per element against 6.6 ns with nine rows per K_c and 14 elements
+// per batch; with four clusters (half-step traces) 5.4 against 7.0 ns.
 template <int O>
 struct SpShape;
-// elements per CTA and parts of the row phase: NT = rup(9 NE, 32) x NPART threads, with
-// NE B <= NT (column phase), within 128 registers per thread. Order 5: one CTA of 512 threads
-// per SM (14 elements), so that the SM's warps run each phase's code together — the kernel
-// is bound by instruction fetch, and two CTAs of 7 elements in different phases fetch two
-// phases' code at once (measured: 88.5 against 72.2 M sim-element-updates/s with 4 fused
-// simulations, 88.5 against 86.7 M element-updates/s for one); orders 3 and 4: two CTAs.
 template <>
 struct SpShape<5> {
-  static constexpr int NE = 14, NPART = 4;
+  static constexpr int BP = 36, GP = 20, GS = 144, YT = 20, BBP = 16, ESM = 20, MINB = 1, NP = 4;
 };
 template <>
 struct SpShape<4> {
-  static constexpr int NE = 12, NPART = 2;
+  static constexpr int BP = 20, GP = 12, GS = 72, YT = 12, BBP = 10, ESM = 12, MINB = 2, NP = 3;
 };
 template <>
 struct SpShape<3> {
-  static constexpr int NE = 25, NPART = 1;
+  static constexpr int BP = 12, GP = 12, GS = 72, YT = 4, BBP = 6, ESM = 4, MINB = 3, NP = 1;
 };
+
+// Floats of an element's row in the sparse engine's tables (16-byte aligned rows). Predict:
+//   [0..8] dxi_c/dx_d, [9..11] -sum_c dxi_c/dx_d, lam, mu, 1/rho, [15 + 2l] lam Y^lam_l,
+//   [16 + 2l] 2 mu Y^mu_l, [23] cluster and flags (int); [24 + 12 f] of face f: normal n, then
+//   a0, a1/s, a2, s a3 of the normal and of the tangential pair, s = -2|S|/|det J|; [21] (int) two
+//   bits per face: 0 no neighbour, 1 neighbour in the same cluster, 2 finer, 3 coarser.
+// Neighbour: [0..14] as above, [16 + 12 f] the same for the neighbour side's trace (its theta is
+//   scaled by its own s_n and its own normal): n, then an0, -an1/s_n, -s an2/s_n, s an3.
+constexpr int EDS = 72, NDS = 64;
+
+// Face traces, the LTS buffers of the sparse engine: per (element, simulation) and face the six
+// rows (v, theta) in the face basis, FS floats (16-byte multiple). The neighbour kernel wants
+// X F~_j of the neighbour's buffer on its face j, and the predict kernel forms just that product
+// for its own surface term: storing the trace (O = 5: 4 x 368 bytes per element instead of
+// 1,260) leaves the neighbour kernel 368 bytes to read per face instead of 1,260, and no face
+// product. A face serves one neighbour, so it needs only the buffer that neighbour reads:
+//   same cluster:     T1 = trace of B1
+//   coarser neighbour: T1 = trace of B3 (set at even steps, added to at odd ones)
+//   finer neighbour:  T1 = trace of B2 (first half), T2 = trace of B1 - B2 (second half)
+template <int F>
+struct TraceCfg {
+  static constexpr int FS = rup(6 * F, 4), TS = 4 * FS;
+};
+
+// The direction whose stress rows are the tractions of face f.
+__host__ __device__ constexpr int set_of_face(int f) { return f < 3 ? 2 - f : 3; }
 
 template <int O, int M, bool FU = false>
 struct SpCfg {
   using C = Cfg<O, M, 1>;
+  using H = SpShape<O>;
   static constexpr int B = C::B, F = C::F, NQ = C::NQ, NA = C::NA;
-  static constexpr int NE = SpShape<O>::NE, NPART = SpShape<O>::NPART;
-  static constexpr int NPAIR = 9 * NE;                 // (element, elastic row) pairs
-  static constexpr int RT = rup(NPAIR, 32);            // threads per part
-  static constexpr int NT = RT * NPART;
-  static_assert(NE * B <= NT, "column phase needs one thread per (element, mode)");
-  static constexpr int XP = RT + 1;                    // pair stride (1 mod 32)
-  static constexpr int EDP = ED + 1;                   // staged element data stride (odd: elements
-                                                       // of one warp on distinct banks)
-  static constexpr int S_X = 0;                        // [B][XP]          row operand
-  static constexpr int S_Y = rup(S_X + B * XP, 4);     // [3 B][XP]        products Y_c / Z_c
-  static constexpr int S_G = rup(S_Y + 3 * B * XP, 4); // [4 F][XP]        face traces G_i
-  static constexpr int S_P = S_Y;                      // [4 B][XP]        projected states P_i
-  static_assert(S_P + 4 * B * XP <= S_G + 4 * F * XP, "P_i overlays Y and G");
-  static constexpr int S_W = rup(S_G + 4 * F * XP, 4); // [4 F][XP]        interface states, 6 rows
-  static constexpr int S_E = rup(S_W + 4 * F * XP, 4);
-  static constexpr int S_META = rup(S_E + NE * EDP, 4);  // [3][NE] ints: meta, element, simulation
-  // the batch's DOFs: NE elements of QS floats (one simulation), or the simulation groups
-  // that NE consecutive (element, simulation) slots touch, at most NE / G + 2 groups of
-  // NQ x B x G floats (fused, G = FUSED_GROUP)
-  static constexpr int GB = NQ * B * FUSED_GROUP;
-  static constexpr int QBUF = FU ? (NE / FUSED_GROUP + 2) * GB : NE * C::QS;
-  static constexpr int S_Q = rup(S_META + 3 * NE, 4);      // [QBUF] the batch's DOFs
-  static constexpr int S_BAR = rup(S_Q + QBUF, 4);         // mbarrier of the DOF copy (8 bytes)
-  static constexpr int TOTAL = S_BAR + 4;
+  static constexpr int NE = 16;
+  static constexpr int BP = H::BP, GP = H::GP, GS = H::GS, YT = H::YT;
+  // column phase: threads of the modes below the top degree (BA per element) first, then those
+  // of the top degree (BB, padded to BBP): the time kernel's products vanish on the latter
+  static constexpr int BA = nbasis(O - 1), BB = B - BA, BBP = H::BBP;
+  static constexpr int NTA = NE * BA, NT = rup(NTA + NE * BBP, 32);
+  static constexpr int NW = NT / 32;
+  static_assert(NE % 8 == 0, "eight lanes of a row phase share a row (NE = 14 would straddle rows: bank conflicts)");
+  static_assert(NTA % 32 == 0 && BP >= B && GP >= F && GS >= 6 * GP && BBP >= BB && 3 * H::NP <= NW, "shape");
+  static_assert(YT >= BA && (YT / 4) % 2 == 1 && (BP / 4) % 2 == 1 && (GP / 4) % 2 == 1, "row strides");
+  static constexpr bool TM = M > 0;   // part of the column state lives in tensor memory
+  // tensor-memory columns: 36 per warp of a lane quarter, a power of two in all
+  static constexpr int TMC = (NW + 3) / 4 * 36 <= 128 ? 128 : 256;
+  // element strides: ESM modulo 32, odd in 16-byte units
+  static constexpr int es(int n) { return n + (H::ESM - n % 32 + 32) % 32; }
+  static constexpr int ESX = es(15 * BP);              // v (3), tau_0, tau_1, tau_2, tau_3 (3 rows each); then
+                                                       // the projections of face 3 (6 rows)
+  static constexpr int ESY = es(18 * BP);              // products of the sets 0..2, 6 rows each
+  static constexpr int ESG = 4 * GS + 4;               // face traces, then interface states, in place
+  static constexpr int S_X = 0;
+  static constexpr int S_Y = S_X + NE * ESX;
+  static constexpr int S_G = S_Y + NE * ESY;
+  static constexpr int S_E = S_G + NE * ESG;           // [2][NE][EDS], double-buffered
+  // the batch's DOFs: NE elements of QS floats (one simulation), or the simulation groups of its
+  // NE slots (fused: groups of 4 consecutive slots, NE and the simulation count multiples of 4)
+  static constexpr int QBUF = FU ? NE * NQ * B : NE * C::QS;
+  static constexpr int S_Q = rup(S_E + 2 * NE * EDS, 4);
+  static constexpr int S_F = rup(S_Q + QBUF, 4);       // [4][B][F] F~ (half-step traces)
+  static constexpr int S_SLOT = rup(S_F + 4 * B * F, 4);   // fused: [2][2][NE] element, simulation of the slots
+  static constexpr int S_BAR = rup(S_SLOT + (FU ? 4 * NE : 0), 4);   // mbarrier of the copies (8 bytes)
+  static constexpr int TOTAL = S_BAR + 4;                             // and the tensor-memory address
 };
 
+// The part of a row phase that warp w runs (-1: none) and the third of its rows (two of the six):
+// at order 5 the warps of one scheduler (w mod 4) share a part's code.
+template <int O>
+__device__ __forceinline__ void row_job(int w, int& part, int& third) {
+  constexpr int NP = SpShape<O>::NP;
+  part = w < 3 * NP ? (O == 5 ? w % NP : w / 3) : -1;
+  third = O == 5 ? w / NP : w % 3;
+}
+
 // the generated products of order O
-template <int O, int XP>
-__device__ __forceinline__ void sp_time(int part, int variant, const float* x, float* y) {
-  if constexpr (O == 5) ltssp::sp_time_o5<XP>(part, variant, x, y);
-  if constexpr (O == 4) ltssp::sp_time_o4<XP>(part, variant, x, y);
-  if constexpr (O == 3) ltssp::sp_time_o3<XP>(part, variant, x, y);
+template <int O, int DY>
+__device__ __forceinline__ void sg_time(int variant, int part, const float* x, int dx, float* y) {
+  if constexpr (O == 5) ltssp::sg_time_o5<DY>(variant, part, x, dx, y);
+  if constexpr (O == 4) ltssp::sg_time_o4<DY>(variant, part, x, dx, y);
+  if constexpr (O == 3) ltssp::sg_time_o3<DY>(variant, part, x, dx, y);
 }
-template <int O, int XP>
-__device__ __forceinline__ void sp_vol(int part, const float* x, float* y, float* g) {
-  if constexpr (O == 5) ltssp::sp_vol_o5<XP>(part, x, y, g);
-  if constexpr (O == 4) ltssp::sp_vol_o4<XP>(part, x, y, g);
-  if constexpr (O == 3) ltssp::sp_vol_o3<XP>(part, x, y, g);
+template <int O, int DY, int DG>
+__device__ __forceinline__ void sg_vol(int part, const float* x, int dx, float* y, float* g) {
+  if constexpr (O == 5) ltssp::sg_vol_o5<DY, DG>(0, part, x, dx, y, g);
+  if constexpr (O == 4) ltssp::sg_vol_o4<DY, DG>(0, part, x, dx, y, g);
+  if constexpr (O == 3) ltssp::sg_vol_o3<DY, DG>(0, part, x, dx, y, g);
 }
-template <int O, int XP>
-__device__ __forceinline__ void sp_proj(int part, const float* x, float* y) {
-  if constexpr (O == 5) ltssp::sp_proj_o5<XP>(part, x, y);
-  if constexpr (O == 4) ltssp::sp_proj_o4<XP>(part, x, y);
-  if constexpr (O == 3) ltssp::sp_proj_o3<XP>(part, x, y);
+template <int O, int DY, int DG>
+__device__ __forceinline__ void sg_proj(int part, const float* g, float* y, float* p) {
+  if constexpr (O == 5) ltssp::sg_proj_o5<DY, DG>(0, part, g, y, p);
+  if constexpr (O == 4) ltssp::sg_proj_o4<DY, DG>(0, part, g, y, p);
+  if constexpr (O == 3) ltssp::sg_proj_o3<DY, DG>(0, part, g, y, p);
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// dxi_c/dx_d of an element, c = 3: -sum of the others (the first 12 floats of its table row)
+struct Geo {
+  float J[4][3];
+  __device__ __forceinline__ explicit Geo(const float* ed) {
+    const float4 a = ld4(ed), b = ld4(ed + 4), c = ld4(ed + 8);
+    J[0][0] = a.x, J[0][1] = a.y, J[0][2] = a.z, J[1][0] = a.w, J[1][1] = b.x, J[1][2] = b.y;
+    J[2][0] = b.z, J[2][1] = b.w, J[2][2] = c.x, J[3][0] = c.y, J[3][1] = c.z, J[3][2] = c.w;
+  }
+};
+
+// Rows of one mode for the row phase: v_j, then tau_c of the first NSET directions.
+template <int NSET, int BP>
+__device__ __forceinline__ void put_rows(float* x, const float (&q)[9], const Geo& g) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) x[j * BP] = q[6 + j];
+#pragma unroll
+  for (int c = 0; c < NSET; ++c) {
+    x[(3 + 3 * c) * BP] = g.J[c][0] * q[0] + g.J[c][1] * q[3] + g.J[c][2] * q[5];
+    x[(4 + 3 * c) * BP] = g.J[c][0] * q[3] + g.J[c][1] * q[1] + g.J[c][2] * q[4];
+    x[(5 + 3 * c) * BP] = g.J[c][0] * q[5] + g.J[c][1] * q[4] + g.J[c][2] * q[2];
+  }
+}
+
+// Hooke's law of a velocity gradient G[d][j] = d v_j / d x_d: stress rows (the elastic Jacobians'
+// velocity part) and eps = sym grad v.
+__device__ __forceinline__ void hooke(const float (&G)[3][3], float lam, float mu, float (&out)[9], float (&eps)[6]) {
+  const float ltr = lam * (G[0][0] + G[1][1] + G[2][2]), m2 = 2.f * mu;
+  const float sxy = G[0][1] + G[1][0], syz = G[1][2] + G[2][1], sxz = G[0][2] + G[2][0];
+  out[0] = fmaf(m2, G[0][0], ltr);
+  out[1] = fmaf(m2, G[1][1], ltr);
+  out[2] = fmaf(m2, G[2][2], ltr);
+  out[3] = mu * sxy;
+  out[4] = mu * syz;
+  out[5] = mu * sxz;
+  eps[0] = G[0][0];
+  eps[1] = G[1][1];
+  eps[2] = G[2][2];
+  eps[3] = 0.5f * sxy;
+  eps[4] = 0.5f * syz;
+  eps[5] = 0.5f * sxz;
+}
+
+// Upwind (Godunov) interface state of a face state g = (v, theta), theta the traction times the
+// face's s = -2|S|/|det J| (of the trace's own element), in closed form, as riemann_state of
+// kernels.cuh: fd = n, then the four coefficients of the normal and of the tangential pair, with
+// the factors of s folded in (EDS above). w = (v*, s t*).
+__device__ __forceinline__ void interface_state(const float (&g)[6], const float* fd, float (&w)[6]) {
+  const float4 f0 = ld4(fd), f1 = ld4(fd + 4), f2 = ld4(fd + 8);
+  const float nx = f0.x, ny = f0.y, nz = f0.z;
+  const float vn = g[0] * nx + g[1] * ny + g[2] * nz;
+  const float tn = g[3] * nx + g[4] * ny + g[5] * nz;
+  const float vTx = g[0] - vn * nx, vTy = g[1] - vn * ny, vTz = g[2] - vn * nz;
+  const float tTx = g[3] - tn * nx, tTy = g[4] - tn * ny, tTz = g[5] - tn * nz;
+  const float vsn = f0.w * vn + f1.x * tn;
+  const float tsn = f1.y * tn + f1.z * vn;
+  w[0] = vsn * nx + f1.w * vTx + f2.x * tTx;
+  w[1] = vsn * ny + f1.w * vTy + f2.x * tTy;
+  w[2] = vsn * nz + f1.w * vTz + f2.x * tTz;
+  w[3] = tsn * nx + f2.y * tTx + f2.z * vTx;
+  w[4] = tsn * ny + f2.y * tTy + f2.z * vTy;
+  w[5] = tsn * nz + f2.y * tTz + f2.z * vTz;
 }
 
 // Slots of a phase: one simulation (FUSED false): slot = element; fused simulations: slot =
@@ -134,79 +254,102 @@ struct Slots {
 };
 
 template <int O, int M, bool FUSED>
-__global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, (SpCfg<O, M, FUSED>::NT >= 512 ? 1 : 2))
+__global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     k_predict_sp(DevOps ops, DevState st, PhaseArgs ph) {
   using S = SpCfg<O, M, FUSED>;
   using C = typename S::C;
-  constexpr int B = S::B, F = S::F, NE = S::NE, NT = S::NT, XP = S::XP, NQ = S::NQ, NA = S::NA, EDP = S::EDP;
+  constexpr int B = S::B, F = S::F, NE = S::NE, NT = S::NT, NQ = S::NQ, NA = S::NA, BP = S::BP, YT = S::YT, GP = S::GP,
+                GS = S::GS;
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
   float* sX = smem + S::S_X;
   float* sY = smem + S::S_Y;
   float* sG = smem + S::S_G;
-  float* sP = smem + S::S_P;
-  float* sW = smem + S::S_W;
-  float* sE = smem + S::S_E;
-  int* sMeta = reinterpret_cast<int*>(smem + S::S_META);
-  int* sSlot = sMeta + NE;                    // fused: [2][NE] element, simulation of the batch's slots
   float* sQ = smem + S::S_Q;
+  float* sF = smem + S::S_F;
   uint64_t* sBar = reinterpret_cast<uint64_t*>(smem + S::S_BAR);
   const int tid = threadIdx.x;
+  if (ph.bufs & BUFS_TRACES)
+    for (int i = tid; i < 4 * B * F; i += NT) sF[i] = ops.Ft[i];
 
-  // column task (slot, mode). One simulation: modes fastest (a warp spans at most two
-  // elements, and reads a row's consecutive modes). Fused simulations: set per batch below.
-  const bool act = tid < NE * B;
-  int es = act ? tid / B : 0;
-  int b = act ? tid % B : 0;
-  // row task (part, pair): warp w takes part w mod NPART, so that the warps an SM
-  // sub-partition runs (w mod 4) all execute the same part's straight-line code and its
-  // instruction cache holds one part only
-  const int part = (tid >> 5) % S::NPART, pair = ((tid >> 5) / S::NPART) * 32 + (tid & 31);
-  const bool ract = pair < S::NPAIR;          // (element, quantity) rows of the 9 elastic rows
-  const bool pact = pair < 6 * NE;            // (element, interface-state) rows of the projection
+  // column task (slot, mode), modes fastest: the modes below the top degree of all slots (group A),
+  // then the top-degree ones. Fused simulations: set per batch below.
+  constexpr int BA = S::BA, BB = S::BB, NTA = S::NTA;
+  const bool grpA = tid < NTA;
+  constexpr int BBP = FUSED ? BB : S::BBP;
+  const int tg = grpA ? tid : tid - NTA, bg = grpA ? BA : BBP;   // task within the group, modes per slot
+  int es = FUSED ? 0 : tg / bg;
+  int b = FUSED ? 0 : (grpA ? 0 : BA) + tg % bg;
+  const bool act = grpA || (tg < NE * BBP && tg % BBP < BB);
+  // row task: row r of the sets (velocity j = r, or stress row i = r - 3) of element re
+  const int warp = tid >> 5, re = tid & 15;
   const Slots<FUSED> sl(st, ph);
   const int nbatch = (sl.n + NE - 1) / NE;
   const long long qs = FUSED ? st.qs : C::QS, bs = FUSED ? st.bs : C::BUFS;
   constexpr int RS = FUSED ? B * FUSED_GROUP : B;   // row stride of Q and the buffers
   constexpr int CS = FUSED ? FUSED_GROUP : 1;       // mode stride
-  int col = es * 9;                           // this column's pair offset
-  // A batch's DOFs arrive in shared memory by one bulk asynchronous copy (TMA) that thread 0
-  // issues for the next batch as soon as the current one has read its copy, completing on an
-  // mbarrier (one phase per batch): one simulation, the batch's contiguous elements (n x QS
-  // floats); fused simulations, the contiguous simulation groups from the batch's first slot
-  // to its last. Every wait is bounded; one that gives up sets the error word and the CTA
-  // returns.
-  constexpr int GB = S::GB;
-  auto issue_q = [&](int bt) {
+  constexpr int GB = NQ * B * FUSED_GROUP, FS = TraceCfg<F>::FS;
+  // A batch's DOFs and element tables arrive in shared memory by two bulk asynchronous copies
+  // (TMA) that thread 0 issues for the next batch as soon as the current one has read its DOFs
+  // (the tables are double-buffered), completing on an mbarrier (one phase per batch): one
+  // simulation, the batch's contiguous elements (n x QS floats); fused simulations, the
+  // contiguous simulation groups from the batch's first slot to its last. Every wait is
+  // bounded; one that gives up sets the error word and the CTA returns.
+  auto issue = [&](int bt, int buf) {
     const float* src;
     uint32_t bytes;
+    int e0, ne;
     if constexpr (!FUSED) {
-      const int e0 = ph.begin + bt * NE;
+      e0 = ph.begin + bt * NE;
+      ne = min(NE, ph.end - e0);
       src = st.Q + (size_t)e0 * C::QS;
-      bytes = (uint32_t)min(NE, ph.end - e0) * C::QS * 4;
+      bytes = (uint32_t)ne * C::QS * 4;
     } else {
-      int e0, f0, e1, f1;
+      int f0, e1, f1;
       sl.decode(bt * NE, e0, f0);
       sl.decode(min(sl.n, bt * NE + NE) - 1, e1, f1);
       const int ngr = sl.nsim / FUSED_GROUP;
-      src = st.Q + (size_t)(ph.begin + e0) * qs + (size_t)(f0 / FUSED_GROUP) * GB;
-      bytes = (uint32_t)((e1 - e0) * ngr + f1 / FUSED_GROUP - f0 / FUSED_GROUP + 1) * GB * 4;
+      ne = e1 - e0 + 1;
+      e0 += ph.begin;
+      src = st.Q + (size_t)e0 * qs + (size_t)(f0 / FUSED_GROUP) * GB;
+      bytes = (uint32_t)((e1 - (e0 - ph.begin)) * ngr + f1 / FUSED_GROUP - f0 / FUSED_GROUP + 1) * GB * 4;
     }
-    tc::bulk_load(sQ, src, bytes, sBar);
+    tc::bulk_load2(sQ, src, bytes, smem + S::S_E + buf * NE * EDS, st.sdata + (size_t)e0 * EDS, (uint32_t)ne * EDS * 4,
+                   sBar);
   };
+  // Tensor memory as per-thread storage (anelastic): the time integrals of the memory variables
+  // and the half-step integrals between the derivatives, and the update's known terms between
+  // the volume products and the update. 18 warps of 96 registers hold the rest without spills
+  // (spilling instead: 62 local-memory instructions per element, most of them missing L1).
+  uint32_t* sTm = reinterpret_cast<uint32_t*>(smem + S::S_BAR + 2);
+  uint32_t tm = 0;
   uint32_t qpar = 0;
   if (tid == 0) tc::mbar_init(sBar, 1);
+  if constexpr (S::TM) {
+    if (warp == 0) {
+      tc::tmem_alloc(sTm, S::TMC);
+      tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+  }
   __syncthreads();
-  if (tid == 0 && blockIdx.x < nbatch && !ph.suppress) issue_q(blockIdx.x);
+  if constexpr (S::TM) {
+    tc::fence_after_sync();
+    tm = *sTm + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * 36;
+  }
+  if (tid == 0 && blockIdx.x < nbatch && !ph.suppress) issue(blockIdx.x, 0);
 
   for (int batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
     const int t0 = batch * NE;
-    // element of the batch's slot k (fused: decoded below; every read of sSlot comes before
-    // the batch's second barrier, every write before its first)
+    const float* sE = smem + S::S_E + qpar * NE * EDS;
+    // fused: element, simulation of the batch's slots
+    int* sSlot = reinterpret_cast<int*>(smem + S::S_SLOT) + (FUSED ? qpar * 2 * NE : 0);
+    // element of the batch's slot k (fused: decoded below, two copies in turn, as the last tasks
+    // of a batch may still read theirs when the next one is decoded)
     auto elem_of = [&](int k) { return FUSED ? sSlot[k] : ph.begin + t0 + k; };
     if (FUSED && tid < NE) {
       int e = 0, f = 0;
-      if (t0 + tid < sl.n) sl.decode(t0 + tid, e, f);
+      sl.decode(min(t0 + tid, sl.n - 1), e, f);   // slots past the end: a staged element
       sSlot[tid] = ph.begin + e;
       sSlot[NE + tid] = f;
     }
@@ -214,22 +357,21 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, (SpCfg<O, M, FUSED>::N
     if constexpr (FUSED) __syncthreads();
     if (FUSED && act) {
       // fused column tasks ordered by (element, mode, simulation): the slots of the batch that
-      // share an element form a segment [s0, s1), and its B (s1 - s0) tasks take the modes in
+      // share an element form a segment [s0, s1), and its tasks of a group take the modes in
       // turn with the segment's simulations fastest, so that a warp's lanes read consecutive
       // floats of the simulation-blocked layout (tasks of slot m lie in segment of slot m)
-      const int m = tid / B;
+      const int m = tg / bg;
       const int nval = min(NE, sl.n - t0);
       if (m < nval) {
         const int fm = sSlot[NE + m];
         const int s0 = max(0, m - fm), s1 = min(nval, m - fm + sl.nsim);
-        const int local = tid - B * s0, nf = s1 - s0;
-        b = local / nf;
+        const int local = tg - bg * s0, nf = s1 - s0;
+        b = (grpA ? 0 : BA) + local / nf;
         es = s0 + local % nf;
       } else {
         es = m;
-        b = tid % B;
+        b = (grpA ? 0 : BA) + tg % bg;
       }
-      col = es * 9;
     }
     const int ts = t0 + es;
     const bool valid = act && ts < sl.n;
@@ -237,6 +379,12 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, (SpCfg<O, M, FUSED>::N
     const int fs = (FUSED && valid) ? sSlot[NE + es] : 0;
     const size_t qoff = (size_t)g * qs + Slots<FUSED>::sub(fs, NQ, B) + (size_t)b * CS;
     const size_t boff = (size_t)g * bs + Slots<FUSED>::sub(fs, 9, B) + (size_t)b * CS;
+    // trace buffer of slot k
+    auto trace_of = [&](int k) {
+      return (FUSED ? (size_t)sSlot[k] * st.nsim + sSlot[NE + k] : (size_t)(ph.begin + t0 + k)) * TraceCfg<F>::TS;
+    };
+    // staged table row of slot k: its element's position in the batch
+    auto ed_of = [&](int k) { return sE + (FUSED ? sSlot[k] - sSlot[0] : k) * EDS; };
     {
       // the batch's DOFs have arrived (or the wait gave up: every thread leaves)
       const bool ok = tc::mbar_wait(sBar, qpar, ph.wait);
@@ -244,455 +392,586 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, (SpCfg<O, M, FUSED>::N
       if (!__syncthreads_and(ok)) {
         if (tid == 0) {
           atomicOr(ph.err, 1);
-          tc::mbar_wait(sBar, qpar ^ 1, ph.wait);   // the copy in flight, if any, lands first
+          tc::mbar_wait(sBar, qpar ^ 1, ph.wait);   // the copies in flight, if any, land first
         }
-        return;
+        break;
       }
     }
     // this column's DOFs in the staged copy (row stride RS, as in Q)
-    size_t soff = (size_t)es * C::QS + b;
-    if constexpr (FUSED) {
-      const int ngr = sl.nsim / FUSED_GROUP;
-      const int gi = (g - sSlot[0]) * ngr + fs / FUSED_GROUP - sSlot[NE] / FUSED_GROUP;
-      soff = (size_t)gi * GB + (size_t)b * CS + fs % FUSED_GROUP;
-    }
-    float T[NQ], Th[9], Da[NA > 0 ? NA : 1];
-    float v[9];
-#pragma unroll
-    for (int r = 0; r < 9; ++r) v[r] = 0.f;
-    if (valid) {
+    int soff = es * C::QS + b;
+    if constexpr (FUSED) soff = (es / FUSED_GROUP) * GB + b * CS + es % FUSED_GROUP;
+    const float* ed = valid ? ed_of(es) : sE;
+    const int meta = valid ? __float_as_int(ed[23]) : 0;
+    const int cl = meta & 0xff;
+    const bool finer = (meta & FLAG_FINER) != 0;
+    float T[9], Th[9], Da[NA > 0 ? NA : 1];
+    float* xo = sX + es * S::ESX + b;
+    {
+      float v[9];
       const float* q = sQ + soff;
 #pragma unroll
-      for (int r = 0; r < 9; ++r) v[r] = q[r * RS];
+      for (int r = 0; r < 9; ++r) v[r] = valid ? q[r * RS] : 0.f;
 #pragma unroll
-      for (int r = 0; r < NA; ++r) Da[r] = q[(9 + r) * RS];
-    } else {
+      for (int r = 0; r < NA; ++r) Da[r] = valid ? q[(9 + r) * RS] : 0.f;
+      if (act) put_rows<3, BP>(xo, v, Geo(ed));
+      const float c0 = ph.coef[cl][0], h0 = ph.hcoef[cl][0];
 #pragma unroll
-      for (int r = 0; r < NA; ++r) Da[r] = 0.f;
+      for (int r = 0; r < 9; ++r) {
+        T[r] = c0 * v[r];
+        Th[r] = h0 * v[r];
+      }
+      if constexpr (S::TM) {
+        float ta[18];
+#pragma unroll
+        for (int r = 0; r < NA; ++r) ta[r] = c0 * Da[r];
+        tc::tmem_st18(tm, ta);
+        tc::tmem_st9(tm + 18, Th);
+        tc::tmem_wait_st();
+      }
     }
-    for (int i = tid; i < NE * ED; i += NT) {
-      const int ee = i / ED;
-      const bool in = t0 + ee < sl.n;
-      sE[ee * EDP + i % ED] = in ? st.edata[(size_t)elem_of(ee) * ED + (i % ED)] : 0.f;
-    }
-    if (tid < NE) sMeta[tid] = (t0 + tid < sl.n) ? st.meta[elem_of(tid)] : 0;
-    if (act) {
-#pragma unroll
-      for (int r = 0; r < 9; ++r) sX[b * XP + col + r] = v[r];
-    }
-    __syncthreads();
-    const float* ed = sE + es * EDP;
-    const int meta = act ? sMeta[es] : 0;
-    const int cl = meta & 0xff;
-#pragma unroll
-    for (int r = 0; r < 9; ++r) {
-      T[r] = ph.coef[cl][0] * v[r];
-      Th[r] = ph.hcoef[cl][0] * v[r];
-    }
-#pragma unroll
-    for (int r = 0; r < NA; ++r) T[9 + r] = ph.coef[cl][0] * Da[r];
+    const bool anyfiner = __any_sync(0xffffffffu, finer);
+    const bool batch_finer = __syncthreads_or(finer);
     // ---- time kernel: d^{d+1} Q from d^d Q (Cauchy-Kowalevski), Taylor sums
 #pragma unroll 1
     for (int d = 0; d < O - 1; ++d) {
       // elastic: d^d Q has degree <= O-1-d, so the product is truncated (variant d); the
       // anelastic coupling keeps every degree (variant 0)
       const int variant = (M == 0) ? d : 0;
-      if (ract) sp_time<O, XP>(part, variant, sX + pair, sY + pair);
+      {
+        int part, third;
+        row_job<O>(warp, part, third);
+        const int r = 2 * third + ((tid >> 4) & 1);
+        sg_time<O, 6 * YT>(variant, part, sX + re * S::ESX + r * BP, r < 3 ? 0 : 3 * BP, sY + re * S::ESY + r * YT);
+      }
       __syncthreads();
-      float Y[3][9];
-      // outputs b >= nbasis(O-1-variant) are identically zero and not written
-      const bool has = act && b < nbasis(O - 1 - variant);
+      const float c1 = ph.coef[cl][d + 1];
+      float out[9], eps[6];
+      // products of modes b >= nbasis(O-1-variant) are identically zero and not written (all of
+      // the top degree: whole warps)
+      const bool has = grpA && b < nbasis(O - 1 - variant);
+      if (has) {
+        const float* yp = sY + es * S::ESY + b;
+        float Y[3][6];
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int r = 0; r < 9; ++r) Y[c][r] = has ? sY[(c * B + b) * XP + col + r] : 0.f;
-      if (act) {
-        float out[9], eps[6];
-        star_apply(Y, ed, out, eps);
+          for (int r = 0; r < 6; ++r) Y[c][r] = yp[(6 * c + r) * YT];
+        const Geo geo(ed);
+        const float4 m0 = ld4(ed + 12);   // lam, mu, 1/rho, lam Y^lam_0
+        float G[3][3];
 #pragma unroll
-        for (int l = 0; l < M; ++l) coupling_add(out, Da + 6 * l, ed[12 + 2 * l], ed[13 + 2 * l]);
-        const float c1 = ph.coef[cl][d + 1], h1 = ph.hcoef[cl][d + 1];
+        for (int e = 0; e < 3; ++e)
 #pragma unroll
-        for (int r = 0; r < 9; ++r) {
-          T[r] = fmaf(c1, out[r], T[r]);
-          Th[r] = fmaf(h1, out[r], Th[r]);
-        }
+          for (int j = 0; j < 3; ++j) G[e][j] = geo.J[0][e] * Y[0][j] + geo.J[1][e] * Y[1][j] + geo.J[2][e] * Y[2][j];
+        hooke(G, m0.x, m0.y, out, eps);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) out[6 + i] = m0.z * (Y[0][3 + i] + Y[1][3 + i] + Y[2][3 + i]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 9; ++r) out[r] = 0.f;
+#pragma unroll
+        for (int r = 0; r < 6; ++r) eps[r] = 0.f;
+      }
+      if constexpr (M > 0) {
+        const float4 m0 = ld4(ed + 12), m1 = ld4(ed + 16);
+        const float ylam[3] = {m0.w, m1.y, m1.w}, ymu[3] = {m1.x, m1.z, ed[20]};
+#pragma unroll
+        for (int l = 0; l < M; ++l) coupling_add(out, Da + 6 * l, ylam[l], ymu[l]);
+        float ta[18];
+        tc::tmem_ld18(tm, ta);
 #pragma unroll
         for (int l = 0; l < M; ++l)
 #pragma unroll
           for (int r = 0; r < 6; ++r) {
             const float w = ph.omega[l] * (eps[r] - Da[6 * l + r]);
             Da[6 * l + r] = w;
-            T[9 + 6 * l + r] = fmaf(c1, w, T[9 + 6 * l + r]);
+            ta[6 * l + r] = fmaf(c1, w, ta[6 * l + r]);
           }
-        // next row operand: the next derivative, or after the last one the time integral
-        float* xo = sX + b * XP + col;
-        if (d < O - 2) {
+        tc::tmem_st18(tm, ta);
+        if (anyfiner) {
+          const float h1 = ph.hcoef[cl][d + 1];
+          tc::tmem_ld9(tm + 18, Th);
 #pragma unroll
-          for (int r = 0; r < 9; ++r) xo[r] = out[r];
-        } else {
-#pragma unroll
-          for (int r = 0; r < 9; ++r) xo[r] = T[r];
+          for (int r = 0; r < 9; ++r) Th[r] = fmaf(h1, out[r], Th[r]);
+          tc::tmem_st9(tm + 18, Th);
         }
+        tc::tmem_wait_st();
+      } else if (finer && has) {
+        const float h1 = ph.hcoef[cl][d + 1];
+#pragma unroll
+        for (int r = 0; r < 9; ++r) Th[r] = fmaf(h1, out[r], Th[r]);
+      }
+      // next row operand: the next derivative, or after the last one the time integral
+      if (act && (M > 0 || has || d == O - 2)) {
+#pragma unroll
+        for (int r = 0; r < 9; ++r) T[r] = fmaf(c1, out[r], T[r]);
+        const Geo geo(ed);
+        if (d < O - 2)
+          put_rows<3, BP>(xo, out, geo);
+        else
+          put_rows<4, BP>(xo, T, geo);
       }
       __syncthreads();
     }
-    // ---- LTS buffers (Eq. lts_buffers)
-    if (valid) {
-      float* b1 = st.B1 + boff;
-#pragma unroll
-      for (int r = 0; r < 9; ++r) b1[r * RS] = T[r];
-      if (meta & FLAG_FINER) {
-        float* b2 = st.B2 + boff;
-#pragma unroll
-        for (int r = 0; r < 9; ++r) b2[r * RS] = Th[r];
+    // ---- LTS buffers as modes (Eq. lts_buffers): the adjoint and partitioned runs read those
+    if (ph.bufs & BUFS_MODAL) {
+      if constexpr (S::TM) {
+        if (anyfiner) tc::tmem_ld9(tm + 18, Th);
       }
-      if (meta & FLAG_COARSER) {
-        float* b3 = st.B3 + boff;
-        if (ph.parity[cl] == 0) {
+      if (valid) {
+        float* b1 = st.B1 + boff;
 #pragma unroll
-          for (int r = 0; r < 9; ++r) b3[r * RS] = T[r];
-        } else {
+        for (int r = 0; r < 9; ++r) b1[r * RS] = T[r];
+        if (finer) {
+          float* b2 = st.B2 + boff;
 #pragma unroll
-          for (int r = 0; r < 9; ++r) b3[r * RS] += T[r];
+          for (int r = 0; r < 9; ++r) b2[r * RS] = Th[r];
+        }
+        if (meta & FLAG_COARSER) {
+          float* b3 = st.B3 + boff;
+          if (ph.parity[cl] == 0) {
+#pragma unroll
+            for (int r = 0; r < 9; ++r) b3[r * RS] = T[r];
+          } else {
+#pragma unroll
+            for (int r = 0; r < 9; ++r) b3[r * RS] += T[r];
+          }
         }
       }
     }
-    // ---- volume products and local face traces of T (row phase)
-    if (ract) sp_vol<O, XP>(part, sX + pair, sY + pair, sG + pair);
-    __syncthreads();
-    float acc[NQ];
+    // the update's terms that are already known: Q + E^l T^{a,l} and Q^{a,l} - omega_l T^{a,l}
+    float acc[9];
     {
-      float Z[3][9];
-      // Z_c[0] = 0: K_c[k][0] vanishes for every k (the constant mode has no derivative)
-      const bool has = act && b > 0;
+      const float* q = sQ + soff;
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+      for (int r = 0; r < 9; ++r) acc[r] = valid ? q[r * RS] : 0.f;
+      if constexpr (M > 0) {
+        float ta[18];
+        tc::tmem_ld18(tm, ta);
+        const float4 m0 = ld4(ed + 12), m1 = ld4(ed + 16);
+        const float ylam[3] = {m0.w, m1.y, m1.w}, ymu[3] = {m1.x, m1.z, ed[20]};
 #pragma unroll
-        for (int r = 0; r < 9; ++r) Z[c][r] = has ? sY[(c * B + b) * XP + col + r] : 0.f;
-      if (valid) {
-        float out[9], eps[6];
-        star_apply(Z, ed, out, eps);
-        float V[9];
-#pragma unroll
-        for (int r = 0; r < 9; ++r) V[r] = -out[r];
-#pragma unroll
-        for (int l = 0; l < M; ++l) coupling_add(V, T + 9 + 6 * l, ed[12 + 2 * l], ed[13 + 2 * l]);
-        const float* q = sQ + soff;
-#pragma unroll
-        for (int r = 0; r < 9; ++r) acc[r] = q[r * RS] + V[r];
+        for (int l = 0; l < M; ++l) coupling_add(acc, ta + 6 * l, ylam[l], ymu[l]);
 #pragma unroll
         for (int l = 0; l < M; ++l)
 #pragma unroll
           for (int r = 0; r < 6; ++r)
-            acc[9 + 6 * l + r] = q[(9 + 6 * l + r) * RS] + ph.omega[l] * (-eps[r] - T[9 + 6 * l + r]);
+            ta[6 * l + r] = fmaf(-ph.omega[l], ta[6 * l + r], valid ? q[(9 + 6 * l + r) * RS] : 0.f);
+        tc::tmem_st18(tm, ta);
+        tc::tmem_st9(tm + 27, acc);
+        tc::tmem_wait_st();
       }
     }
-    // ---- local surface kernel: interface states (v*, t*) of the face traces G_i, one task
-    // per element, face and face mode (face modes fastest), as rows of the projection
+    // ---- volume products and local face traces of T (row phase)
+    {
+      int part, third;
+      row_job<O>(warp, part, third);
+      const int r = 2 * third + ((tid >> 4) & 1);
+      sg_vol<O, 6 * BP, GS>(part, sX + re * S::ESX + r * BP, r < 3 ? 0 : 3 * BP, sY + re * S::ESY + r * BP,
+                            sG + re * S::ESG + r * GP);
+    }
+    __syncthreads();
+    // the batch's DOF copy has been read: the next batch's copies go out now
+    if (tid == 0 && batch + (int)gridDim.x < nbatch && !ph.suppress) issue(batch + gridDim.x, qpar);
+    // ---- face traces to the LTS buffers, and the local surface kernel's interface states (v*,
+    // s t*) in their place; one task per element, face and face mode (face modes fastest)
 #pragma unroll 1
     for (int t = tid; t < NE * 4 * F; t += NT) {
       const int fe = t / (4 * F), fi = (t / F) % 4, f = t % F;
-      const float* gp = sG + (fi * F + f) * XP + fe * 9;
-      float gv[9];
+      const float* ef = ed_of(fe);
+      float* gp = sG + fe * S::ESG + fi * GS + f;
+      float gv[6], w6[6];
 #pragma unroll
-      for (int r = 0; r < 9; ++r) gv[r] = gp[r];
-      float w6[6];
-      riemann_state(gv, sE + fe * EDP + 20 + 11 * fi, w6);
-      float* wp = sW + (fi * F + f) * XP + fe * 6;
+      for (int r = 0; r < 6; ++r) gv[r] = gp[r * GP];
+      if ((ph.bufs & BUFS_TRACES) && t0 + fe < sl.n) {
+        const int rel = (__float_as_int(ef[21]) >> (2 * fi)) & 3;
+        const size_t o = trace_of(fe) + fi * FS + f;
+        // added to in memory (no result read back: one addition per address and launch)
+        if (rel == 3 && ph.parity[__float_as_int(ef[23]) & 0xff] != 0) {
 #pragma unroll
-      for (int r = 0; r < 6; ++r) wp[r] = w6[r];
+          for (int r = 0; r < 6; ++r) atomicAdd(st.T1 + o + r * F, gv[r]);
+        } else if (rel != 0) {
+          float* tp = (rel == 2 ? st.T2 : st.T1) + o;
+#pragma unroll
+          for (int r = 0; r < 6; ++r) tp[r * F] = gv[r];
+        }
+      }
+      interface_state(gv, ef + 24 + 12 * fi, w6);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) gp[r * GP] = w6[r];
     }
     __syncthreads();
-    // the batch's DOF copy has been read: the next batch's copy goes out now
-    if (tid == 0 && batch + (int)gridDim.x < nbatch && !ph.suppress) issue_q(batch + gridDim.x);
-    // ---- projection P_i[r'][b] = sum_f W_i[r'][f] F^_i[f][b] (row phase, over Y and G)
-    if (pact) sp_proj<O, XP>(part, sW + pair, sP + pair);
+    // ---- projection through F^ (row phase): faces 0..2 onto the volume products of their
+    // direction, face 3 into six rows of its own (over the time integral's rows)
+    {
+      int part, third;
+      row_job<O>(warp, part, third);
+      const int r = 2 * third + ((tid >> 4) & 1);
+      sg_proj<O, 6 * BP, GS>(part, sG + re * S::ESG + r * GP, sY + re * S::ESY + r * BP, sX + re * S::ESX + r * BP);
+    }
     __syncthreads();
+    // ---- update: volume and local surface terms of all four directions at once
+    float ta[NA > 0 ? NA : 1];
+    if constexpr (S::TM) {
+      tc::tmem_ld18(tm, ta);
+      tc::tmem_ld9(tm + 27, acc);
+    }
     if (valid) {
-      constexpr int NS = (M > 0) ? 15 : 9;
-      float Sv[NS];
+      const float* yp = sY + es * S::ESY + b;
+      const Geo geo(ed);
+      const float4 m0 = ld4(ed + 12);
+      float G[3][3], dv[3];
+      {
+        float P[6];
 #pragma unroll
-      for (int r = 0; r < NS; ++r) Sv[r] = 0.f;
-      // one copy of the face code (the kernel is bound by instruction fetch)
-#pragma unroll 1
-      for (int i = 0; i < 4; ++i) {
-        const float* pp = sP + (i * B + b) * XP + es * 6;
-        float W[6];
+        for (int r = 0; r < 6; ++r) P[r] = xo[r * BP];
 #pragma unroll
-        for (int r = 0; r < 6; ++r) W[r] = pp[r];
-        flux_rows_add<NS>(W, ed + 20 + 11 * i, ed[9], ed[10], ed[11], Sv);
+        for (int e = 0; e < 3; ++e)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) G[e][j] = geo.J[3][e] * P[j];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) dv[i] = P[3 + i];
       }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float Z[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) Z[r] = yp[(6 * c + r) * BP];
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) G[e][j] = fmaf(geo.J[c][e], Z[j], G[e][j]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) dv[i] += Z[3 + i];
+      }
+      float out[9], eps[6];
+      hooke(G, m0.x, m0.y, out, eps);
       float* q = st.Q + qoff;
 #pragma unroll
-      for (int r = 0; r < 9; ++r) q[r * RS] = acc[r] + Sv[r];
-      if constexpr (M > 0) {
+      for (int r = 0; r < 6; ++r) q[r * RS] = acc[r] - out[r];
 #pragma unroll
-        for (int l = 0; l < M; ++l)
+      for (int i = 0; i < 3; ++i) q[(6 + i) * RS] = fmaf(-m0.z, dv[i], acc[6 + i]);
 #pragma unroll
-          for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = acc[9 + 6 * l + r] + ph.omega[l] * Sv[NS - 6 + r];
+      for (int l = 0; l < M; ++l)
+#pragma unroll
+        for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = fmaf(-ph.omega[l], eps[r], ta[6 * l + r]);
+    }
+    // ---- half-step traces of the faces with a finer neighbour: rows of the half-step integral over
+    // the projections (each thread its own column), then a warp per such face, lane = (velocity or
+    // stress rows, face mode). The second half's trace is the step's (stored above) minus it.
+    if ((ph.bufs & BUFS_TRACES) && batch_finer) {
+      if constexpr (S::TM) {
+        if (anyfiner) tc::tmem_ld9(tm + 18, Th);
+      }
+      if (valid && finer) put_rows<4, BP>(xo, Th, Geo(ed));
+      __syncthreads();
+      const int lane = tid & 31;
+      unsigned faces[2];   // bit per (slot, face) of the batch
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int fe = 8 * h + lane / 4;
+        faces[h] = __ballot_sync(0xffffffffu, t0 + fe < sl.n &&
+                                                  ((__float_as_int(ed_of(fe)[21]) >> (2 * (lane % 4))) & 3) == 2);
+      }
+      const int half = lane / F, f = lane % F;
+      int turn = 0;        // faces go round the warps
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h)
+#pragma unroll 1
+      for (unsigned m = faces[h]; m; m &= m - 1) {
+        const bool mine = turn == warp;
+        turn = turn + 1 == S::NW ? 0 : turn + 1;
+        if (!mine) continue;
+        const int s = 32 * h + __ffs(m) - 1, fe = s / 4, fi = s % 4;
+        if (half < 2) {
+          const float* x = sX + fe * S::ESX + (half ? 3 + 3 * set_of_face(fi) : 0) * BP;
+          const float* w = sF + fi * B * F + f;
+          float gv[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < B; k += 4) {
+            float4 xr[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) xr[r] = ld4(x + r * BP + k);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (k + j < B) {
+                const float c = w[(k + j) * F];
+#pragma unroll
+                for (int r = 0; r < 3; ++r) gv[r] = fmaf(j == 0 ? xr[r].x : (j == 1 ? xr[r].y : (j == 2 ? xr[r].z : xr[r].w)), c, gv[r]);
+              }
+          }
+          const size_t o = trace_of(fe) + fi * FS + 3 * half * F + f;
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            st.T1[o + r * F] = gv[r];
+            atomicAdd(st.T2 + o + r * F, -gv[r]);
+          }
+        }
       }
     }
+  }
+  if constexpr (S::TM) {
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tm, S::TMC);
   }
 }
 
 // ------------------------------------------------------------------ neighbour kernel
 // k_neighbour_sp: the neighbour surface kernel (Sec. III-A, with the buffer chosen by the
-// clusters' time-stepping relation, Sec. V-B), one simulation, no partition. The neighbour
-// matrices factor as F-_{j,h} = F~_j R_h (trace on the neighbour's face j, then the face-basis
-// map R_h of the orientation, block diagonal by degree), so H = X F-_{j,h} is formed as
-// (X F~_j) R_h:
-//   gather:      thread = (element, mode): the four neighbours' buffer columns (B1, B2, B3 or
-//                B1 - B2) into shared memory, rows (element, face, quantity) as pairs;
-//   trace phase: thread = (element, face, quantity): the generated sparse product X F~_j for
-//                the face j its neighbour touches (a warp computes the faces its lanes need);
+// clusters' time-stepping relation, Sec. V-B) on the face traces the predict kernel stored
+// (TraceCfg above). The neighbour matrices factor as F-_{j,h} = F~_j R_h (trace on the neighbour's
+// face j, then the face-basis map R_h of the orientation, block diagonal by degree), and the
+// trace is already there, so only R_h is left of the face product:
 //   states:      thread = (element, face, face mode): H = G R_h (degree block), closed-form
 //                interface state with the neighbour coefficients;
-//   projection:  row phase with the generated F^_i products, as in k_predict_sp;
-//   update:      thread = (element, mode): flux rows per face, Q <- Q + S^N.
-template <int O, int M, int NE_>
-struct SpnCfg {
-  using C = Cfg<O, M, 1>;
-  static constexpr int B = C::B, F = C::F, NQ = C::NQ;
-  static constexpr int NE = NE_;                        // elements per CTA (tile variant: 8 or 4)
-  static constexpr int NROW = NE * 4 * 9;               // (element, face, quantity) rows
-  static constexpr int NT = rup(NROW > NE * B ? NROW : NE * B, 32);
-  static constexpr int XN = NROW + 1;                   // row stride of gathered columns and traces
-  static constexpr int NPART = SpShape<O>::NPART;       // parts of the projection
-  static constexpr int RT6 = rup(6 * NE, 32);
-  static_assert(NPART * RT6 <= NT, "projection rows");
-  static constexpr int XP6 = RT6 + 1;                   // stride of interface states / projections
-  static constexpr int NDP = ND + 1;
-  static constexpr int S_X = 0;                                                      // [B][XN]
-  static constexpr int S_P = 0;                                                      // [4B][XP6] over X
-  static constexpr int S_G = rup((B * XN > 4 * B * XP6) ? B * XN : 4 * B * XP6, 4);  // [F][XN]
-  static constexpr int S_W = rup(S_G + F * XN, 4);                                   // [4F][XP6]
-  static constexpr int S_R = rup(S_W + 4 * F * XP6, 4);                              // [3][F][F]
-  static constexpr int S_D = rup(S_R + 3 * F * F, 4);                                // [NE][NDP]
-  static constexpr int S_I = rup(S_D + NE * NDP, 4);                                 // [NE][9] ints
-  static constexpr int S_PERM = rup(S_I + NE * 9, 4);                                // [4 NE] ints
-  static constexpr int S_SLOT = rup(S_PERM + 4 * NE, 4);                             // [2][NE] ints
-  static constexpr int S_Q = rup(S_SLOT + 2 * NE, 4);                                // [NE][QS] one simulation: DOFs
-  static constexpr int S_BAR = rup(S_Q + NE * C::QS, 4);                             // mbarrier (8 bytes)
-  static constexpr int TOTAL = S_BAR + 4;
-  static_assert(4 * NE <= 32, "one warp sorts the face slots of a batch");
+//   projection:  a warp per face (and 30 lanes): lane = (row, element), the generated F^_f
+//                product of its row;
+//   update:      thread = (element, mode): the faces' rows combined with dxi/dx and Hooke's law
+//                once (as in k_predict_sp), Q <- Q + S^N.
+// Everything a batch reads arrives by bulk asynchronous copies (TMA): a lane per face copies its
+// neighbour's trace and thread 0 the element tables while the previous batch projects and
+// updates, and the DOFs, which only the update reads, right after the previous update.
+// Measured on one GB300 (order 5, anelastic, 138,240 elements): 2.26 ns per element against 3.93 ns
+// with gathered buffers and face products in this kernel (4 x 1,260 bytes and 2,365 instructions
+// per element); bound by DRAM (9.3 KB per element: 1.4 ns at the copy rate) and by the latency of
+// its three barriers.
+template <int O>
+struct SpnShape;   // CTAs per SM, narrow and wide tile; GP: face row, BP: padded modes; ESW, ESP:
+                   // element strides (conflict-free 16-byte accesses of 5 x 6 lanes)
+template <>
+struct SpnShape<5> {
+  static constexpr int MIN1 = 3, MIN0 = 2, GP = 20, BP = 36, ESW = 484, ESP = 884;
+};
+template <>
+struct SpnShape<4> {
+  static constexpr int MIN1 = 5, MIN0 = 2, GP = 12, BP = 20, ESW = 316, ESP = 484;
+};
+template <>
+struct SpnShape<3> {
+  static constexpr int MIN1 = 7, MIN0 = 3, GP = 12, BP = 12, ESW = 316, ESP = 316;
 };
 
-template <int O, int XP>
-__device__ __forceinline__ void sp_ntrace(int j, const float* x, float* y) {
-  if constexpr (O == 5) ltssp::sp_ntrace_o5<XP>(j, x, y);
-  if constexpr (O == 4) ltssp::sp_ntrace_o4<XP>(j, x, y);
-  if constexpr (O == 3) ltssp::sp_ntrace_o3<XP>(j, x, y);
+// elements per CTA of a tile variant (fused: whole groups of simulations)
+__host__ __device__ constexpr int spn_ne(int tile, bool fused) { return fused ? (tile ? 4 : 8) : (tile ? 5 : 10); }
+
+template <int O, int M, int TILE, bool FU>
+struct SpnCfg {
+  using C = Cfg<O, M, 1>;
+  using H = SpnShape<O>;
+  static constexpr int B = C::B, F = C::F, NQ = C::NQ;
+  static constexpr int NE = spn_ne(TILE, FU);
+  static constexpr int GP = H::GP, GS = 6 * H::GP, BP = H::BP, ESW = H::ESW, ESP = H::ESP;
+  static constexpr int NL = 6 * NE, NWF = rup(NL, 32) / 32;   // projection lanes and warps per face
+  static constexpr int NT = rup(NE * B, 32) > 128 * NWF ? rup(NE * B, 32) : 128 * NWF;
+  static constexpr int MINB = TILE ? H::MIN1 : H::MIN0;
+  static_assert(ESW >= 4 * GS && ESP >= 24 * BP && 4 * NE <= 64, "strides");
+  static constexpr int FS = TraceCfg<F>::FS;
+  static constexpr int S_T = 0;                        // [NE][4][FS] the neighbours' traces
+  static constexpr int S_W = S_T + NE * 4 * FS;        // interface states
+  static constexpr int S_P = S_W + NE * ESW;           // [4][6][BP] per element: projections
+  static constexpr int S_Q = S_P + NE * ESP;           // DOFs
+  static constexpr int S_D = S_Q + rup(NE * (FU ? NQ * B : C::QS), 4);   // [2][NE][NDS] tables, double-buffered
+  static constexpr int S_R = S_D + 2 * NE * NDS;       // [3][F][F]
+  static constexpr int S_I = rup(S_R + 3 * F * F, 4);  // [2][4 NE] ints: orientation or -1, double-buffered
+  static constexpr int S_BAR = rup(S_I + 8 * NE, 4);   // two mbarriers
+  static constexpr int TOTAL = S_BAR + 4;
+};
+
+template <int O, int DY, int DG>
+__device__ __forceinline__ void sg_nproj(int face, const float* g, float* y) {
+  if constexpr (O == 5) ltssp::sg_nproj_o5<DY, DG>(0, face, g, y);
+  if constexpr (O == 4) ltssp::sg_nproj_o4<DY, DG>(0, face, g, y);
+  if constexpr (O == 3) ltssp::sg_nproj_o3<DY, DG>(0, face, g, y);
 }
 
-template <int O, int M, int NE_, bool FUSED>
-__global__ void __launch_bounds__(SpnCfg<O, M, NE_>::NT, (NE_ == 8 ? 2 : 4))
+template <int O, int M, int TILE, bool FUSED>
+__global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TILE, FUSED>::MINB)
     k_neighbour_sp(DevOps ops, DevState st, PhaseArgs ph) {
-  using S = SpnCfg<O, M, NE_>;
+  using S = SpnCfg<O, M, TILE, FUSED>;
   using C = typename S::C;
-  constexpr int B = S::B, F = S::F, NE = S::NE, NT = S::NT, XN = S::XN, XP6 = S::XP6, NQ = S::NQ, NDP = S::NDP;
+  constexpr int B = S::B, F = S::F, NE = S::NE, NT = S::NT, NQ = S::NQ, GP = S::GP, GS = S::GS, BP = S::BP, FS = S::FS;
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
-  float* sX = smem + S::S_X;
-  float* sP = smem + S::S_P;
-  float* sG = smem + S::S_G;
+  float* sT = smem + S::S_T;
   float* sW = smem + S::S_W;
-  float* sR = smem + S::S_R;
-  float* sD = smem + S::S_D;
-  int* sI = reinterpret_cast<int*>(smem + S::S_I);      // per element: nbr[4], code[4], meta
-  int* sPerm = reinterpret_cast<int*>(smem + S::S_PERM); // face slots ordered by the neighbour's face j
-  int* sSlot = reinterpret_cast<int*>(smem + S::S_SLOT); // fused: element, simulation of the batch's slots
+  float* sP = smem + S::S_P;
   float* sQ = smem + S::S_Q;
-  uint64_t* sBar = reinterpret_cast<uint64_t*>(smem + S::S_BAR);
+  float* sR = smem + S::S_R;
+  uint64_t* barT = reinterpret_cast<uint64_t*>(smem + S::S_BAR);   // traces and tables
+  uint64_t* barQ = barT + 1;                                       // DOFs
   const int tid = threadIdx.x;
   for (int i = tid; i < 3 * F * F; i += NT) sR[i] = ops.Rh[i];
 
-  const bool act = tid < NE * B;                         // column task (slot, mode), as in k_predict_sp
-  const int es = act ? (FUSED ? tid % NE : tid / B) : 0;
-  const int b = act ? (FUSED ? tid / NE : tid % B) : 0;
-
-  const int part = (tid >> 5) % S::NPART;                // projection row: as in k_predict_sp
-  const int pair6 = ((tid >> 5) / S::NPART) * 32 + (tid & 31);
-  const bool pact = pair6 < 6 * NE;
+  // column task (slot, mode): modes fastest; fused: the four simulations of a group fastest
+  const bool act = tid < NE * B;
+  const int es = act ? (FUSED ? tid / (4 * B) * 4 + tid % 4 : tid / B) : 0;
+  const int b = act ? (FUSED ? tid % (4 * B) / 4 : tid % B) : 0;
+  const int warp = tid >> 5, face = warp % 4, lane6 = warp / 4 * 32 + (tid & 31);   // projection row
+  const bool pact = warp < 4 * S::NWF && lane6 < S::NL;
+  const int pr = lane6 / NE, pe = lane6 % NE;
   const Slots<FUSED> sl(st, ph);
   const int nbatch = (sl.n + NE - 1) / NE;
-  const long long qs = FUSED ? st.qs : C::QS, bs = FUSED ? st.bs : C::BUFS;
-  constexpr int RS = FUSED ? B * FUSED_GROUP : B;   // row stride of Q and the buffers
-  constexpr int CS = FUSED ? FUSED_GROUP : 1;       // mode stride
-  // One simulation: the batch's DOFs (read by the update, the last phase) arrive by one bulk
-  // asynchronous copy that thread 0 issues at the batch's start, completing on an mbarrier;
-  // the wait before the update is bounded, as in k_predict_sp.
-  uint32_t qpar = 0;
-  if constexpr (!FUSED) {
-    if (tid == 0) tc::mbar_init(sBar, 1);
-  }
-
-  for (int batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
-    const int t0 = batch * NE;
-    // element of the batch's slot k, as in k_predict_sp
-    auto elem_of = [&](int k) { return FUSED ? sSlot[k] : ph.begin + t0 + k; };
-    if (FUSED && tid < NE) {
-      int e = 0, f = 0;
-      if (t0 + tid < sl.n) sl.decode(t0 + tid, e, f);
-      sSlot[tid] = ph.begin + e;
-      sSlot[NE + tid] = f;
-    }
-    // one simulation: no barrier here. The previous batch's update (its last reads of sD, sP
-    // and sQ) ends before the barrier below, and its last read of sI came before its states
-    // phase's barrier, so the sI writes that follow overwrite nothing still in use
-    if constexpr (FUSED) __syncthreads();
-    for (int i = tid; i < NE * 9; i += NT) {
-      const int c = i % 9;
-      int v = -1;
-      if (t0 + i / 9 < sl.n) {
-        const int gg = elem_of(i / 9);
-        v = (c < 4) ? __ldg(st.nbr + (size_t)gg * 4 + c) : (c < 8 ? __ldg(st.ncode + (size_t)gg * 4 + c - 4) : __ldg(st.meta + gg));
-      }
-      sI[i] = v;
-    }
-    __syncthreads();
+  const long long qs = FUSED ? st.qs : C::QS;
+  constexpr int RS = FUSED ? B * FUSED_GROUP : B;
+  constexpr int CS = FUSED ? FUSED_GROUP : 1;
+  constexpr int GB = NQ * B * FUSED_GROUP;
+  // first element of a batch, its simulation, and the elements the batch touches
+  auto span = [&](int bt, int& e0, int& f0, int& ne) {
     if constexpr (!FUSED) {
-      // the previous batch's update has read its copy (barrier above)
-      if (tid == 0 && !ph.suppress) {
-        const int e0 = ph.begin + t0;
-        tc::bulk_load(sQ, st.Q + (size_t)e0 * C::QS, (uint32_t)min(NE, ph.end - e0) * C::QS * 4, sBar);
-      }
+      e0 = ph.begin + bt * NE;
+      f0 = 0;
+      ne = min(NE, ph.end - e0);
+    } else {
+      int e1, f1;
+      sl.decode(bt * NE, e0, f0);
+      sl.decode(min(sl.n, bt * NE + NE) - 1, e1, f1);
+      ne = e1 - e0 + 1;
+      e0 += ph.begin;
     }
-    // neighbour coefficients, first read by the states phase (two barriers on)
-    for (int i = tid; i < NE * ND; i += NT) {
-      const int ee = i / ND;
-      sD[ee * NDP + i % ND] = (t0 + ee < sl.n) ? __ldg(st.ndata + (size_t)elem_of(ee) * ND + (i % ND)) : 0.f;
+  };
+  // thread 0: the batch's DOFs (n x QS floats, or its groups of simulations)
+  auto issue_q = [&](int bt) {
+    int e0, f0, ne;
+    span(bt, e0, f0, ne);
+    const float* src = st.Q + (size_t)e0 * qs + (FUSED ? (size_t)(f0 / FUSED_GROUP) * GB : 0);
+    const int n = min(NE, sl.n - bt * NE);
+    tc::bulk_load(sQ, src, (uint32_t)(FUSED ? n / FUSED_GROUP * GB : n * C::QS) * 4, barQ);
+  };
+  // The face slots of a batch belong to the threads of the first warps (tid < 4 NE): link() reads
+  // the neighbour and the buffer it is read from, fetch() issues the copies.
+  const float* tsrc = nullptr;
+  int torient = -1;
+  auto link = [&](int bt) {
+    tsrc = nullptr;
+    torient = -1;
+    const int t = bt * NE + tid / 4;
+    if (tid >= 4 * NE || t >= sl.n) return;
+    int e, f;
+    sl.decode(t, e, f);
+    const size_t k = (size_t)ph.begin + e;
+    const int nb = __ldg(st.nbr + 4 * k + tid % 4), code = __ldg(st.ncode + 4 * k + tid % 4);
+    if (nb < 0) return;
+    const int jh = code & 0xff, second = ((code >> 8) & 0xff) == 2 && ph.parity[__ldg(st.meta + k) & 0xff] == 1;
+    torient = jh % 3;
+    tsrc = (second ? st.T2 : st.T1) +
+           ((FUSED ? (size_t)nb * st.nsim + f : (size_t)nb) * 4 + jh / 3) * FS;
+  };
+  // the first rup(4 NE, 32) threads (whole warps)
+  auto fetch = [&](int bt, int buf) {
+    int* sI = reinterpret_cast<int*>(smem + S::S_I) + buf * 4 * NE;
+    if (tid < 4 * NE) sI[tid] = torient;
+    const unsigned m = __ballot_sync(0xffffffffu, tsrc != nullptr);
+    tc::fence_smem_to_async();
+    if ((tid & 31) == 0) {
+      uint32_t bytes = (uint32_t)__popc(m) * FS * 4;
+      int e0, f0, ne;
+      span(bt, e0, f0, ne);
+      if (tid == 0) bytes += (uint32_t)ne * NDS * 4;
+      tc::mbar_expect(barT, bytes);
+      if (tid == 0) tc::bulk_copy(smem + S::S_D + buf * NE * NDS, st.sndata + (size_t)e0 * NDS, (uint32_t)ne * NDS * 4, barT);
     }
-    // face slots (element, face) sorted by the neighbour's face j (faces without one last), so
-    // that the rows of a warp mostly ask for one face in the trace phase
-    if (tid < 32) {
-      const int fe = tid / 4, fi = tid % 4;
-      int key = 5;                                      // lanes past the batch's face slots
-      if (tid < 4 * NE) key = (t0 + fe < sl.n && sI[fe * 9 + fi] >= 0) ? (sI[fe * 9 + 4 + fi] & 0xff) / 3 : 4;
-      const unsigned lt = (1u << tid) - 1u;
-      int base = 0, rank = 0;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const unsigned m = __ballot_sync(0xffffffffu, key == k);
-        if (key == k) rank = base + __popc(m & lt);
-        base += __popc(m);
-      }
-      if (tid < 4 * NE) sPerm[rank] = tid;
-    }
-    const int ts = t0 + es;
-    const bool valid = act && ts < sl.n;
-    const int g = valid ? elem_of(es) : ph.begin;
-    const int fs = (FUSED && valid) ? sSlot[NE + es] : 0;
-    const size_t bsub = Slots<FUSED>::sub(fs, 9, B);    // this slot's simulation in the buffers
-    // ---- gather the neighbours' time-integrated DOFs by cluster relation (Sec. V-B)
-    if (act) {
-      const int* ie = sI + es * 9;
-      const int cl = ie[8] & 0xff;
-      const int par = valid ? ph.parity[cl] : 0;
-      float xv[4][9];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int nb = valid ? ie[i] : -1;
-        const int rel = (ie[4 + i] >> 8) & 0xff;
-        const float* src1 = (rel == 1) ? st.B3 : ((rel == 2 && par == 0) ? st.B2 : st.B1);
-        const bool sub = (rel == 2 && par == 1);
-        const size_t off = (size_t)(nb < 0 ? 0 : nb) * bs + bsub + (size_t)b * CS;
-#pragma unroll
-        for (int r = 0; r < 9; ++r) xv[i][r] = (nb < 0) ? 0.f : __ldg(src1 + off + r * RS);
-        if (sub) {
-#pragma unroll
-          for (int r = 0; r < 9; ++r) xv[i][r] -= __ldg(st.B2 + off + r * RS);
-        }
-      }
-      float* xo = sX + b * XN + es * 36;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int r = 0; r < 9; ++r) xo[i * 9 + r] = xv[i][r];
-    }
-    __syncthreads();
-    // ---- traces on the neighbour's face j (every thread calls: warp-uniform face branches)
-    {
-      int j = -1, row = 0;
-      if (tid < S::NROW) {
-        const int slot = sPerm[tid / 9], fe = slot / 4, fi = slot % 4;
-        row = slot * 9 + tid % 9;
-        if (t0 + fe < sl.n && sI[fe * 9 + fi] >= 0) j = (sI[fe * 9 + 4 + fi] & 0xff) / 3;
-      }
-      sp_ntrace<O, XN>(j, sX + row, sG + row);
-    }
-    __syncthreads();
-    // ---- H = G R_h per face mode (degree block), interface states with the neighbour
-    // coefficients; faces without a neighbour contribute nothing
+    __syncwarp();
+    if (tsrc) tc::bulk_copy(sT + tid * FS, tsrc, FS * 4, barT);
+  };
+  constexpr int NFT = rup(4 * NE, 32);   // fetching threads; one mbarrier arrival per warp
+  if (tid == 0) {
+    tc::mbar_init(barT, NFT / 32);
+    tc::mbar_init(barQ, 1);
+  }
+  link(blockIdx.x);
+  __syncthreads();
+  if (!ph.suppress && blockIdx.x < nbatch) {
+    if (tid < NFT) fetch(blockIdx.x, 0);
+    if (tid == 0) issue_q(blockIdx.x);
+  }
+  __syncthreads();   // the orientations written by fetch
+  uint32_t par = 0;
+  bool done = false;
+  for (int batch = blockIdx.x; batch < nbatch && !done; batch += gridDim.x, par ^= 1) {
+    const int t0 = batch * NE, next = batch + gridDim.x;
+    const int* sI = reinterpret_cast<const int*>(smem + S::S_I) + par * 4 * NE;
+    const float* sD = smem + S::S_D + par * NE * NDS;
+    int e0, f0, ne;
+    span(batch, e0, f0, ne);
+    // element position in the batch of slot k
+    auto pos_of = [&](int k) { return FUSED ? (f0 + k) / sl.nsim : k; };
+    if (next < nbatch) link(next);
+    // ---- the traces and tables have arrived (or the wait gave up). H = G R_h per face mode
+    // (degree block), interface states with the neighbour coefficients; faces without a
+    // neighbour contribute nothing
+    bool ok = tc::mbar_wait(barT, par, ph.wait);
 #pragma unroll 1
     for (int t = tid; t < NE * 4 * F; t += NT) {
-      const int fe = t / (4 * F), fi = (t / F) % 4, f = t % F;
+      const int fs = t / F, fe = fs / 4, fi = fs % 4, f = t % F;
       float w6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (t0 + fe < sl.n && sI[fe * 9 + fi] >= 0) {
-        const int h = (sI[fe * 9 + 4 + fi] & 0xff) % 3;
-        const int pf = face_degree(f), f0 = nface(pf), f1 = nface(pf + 1);
-        const float* gp = sG + (fe * 4 + fi) * 9;
+      const int h = (t0 + fe < sl.n) ? sI[fs] : -1;
+      if (ok && h >= 0) {
+        const int pf = face_degree(f), q0 = nface(pf), q1 = nface(pf + 1);
+        const float* gp = sT + fs * FS;
         const float* R = sR + h * F * F + f;
-        float hv[9];
-#pragma unroll
-        for (int r = 0; r < 9; ++r) hv[r] = 0.f;
-        for (int q = f0; q < f1; ++q) {
+        float hv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int q = q0; q < q1; ++q) {
           const float w = R[q * F];
 #pragma unroll
-          for (int r = 0; r < 9; ++r) hv[r] = fmaf(gp[q * XN + r], w, hv[r]);
+          for (int r = 0; r < 6; ++r) hv[r] = fmaf(gp[r * F + q], w, hv[r]);
         }
-        riemann_state(hv, sD + fe * NDP + 4 + 11 * fi, w6);
+        interface_state(hv, sD + pos_of(fe) * NDS + 16 + 12 * fi, w6);
       }
-      float* wp = sW + (fi * F + f) * XP6 + fe * 6;
+      float* wp = sW + fe * S::ESW + fi * GS + f;
 #pragma unroll
-      for (int r = 0; r < 6; ++r) wp[r] = w6[r];
+      for (int r = 0; r < 6; ++r) wp[r * GP] = w6[r];
     }
     __syncthreads();
-    // ---- projection P_i[r'][b] = sum_f W_i[r'][f] F^_i[f][b] (row phase, over the gathers)
-    if (pact) sp_proj<O, XP6>(part, sW + pair6, sP + pair6);
-    // one simulation: the barrier of the DOF wait below orders the projections and the update
-    if constexpr (FUSED) __syncthreads();
-    if constexpr (!FUSED) {
-      // the batch's DOFs have arrived (or the wait gave up: every thread leaves)
-      const bool ok = tc::mbar_wait(sBar, qpar, ph.wait);
-      qpar ^= 1;
-      if (!__syncthreads_and(ok)) {
-        if (tid == 0) {
-          atomicOr(ph.err, 1);
-          tc::mbar_wait(sBar, qpar ^ 1, ph.wait);   // the copy in flight, if any, lands first
-        }
-        return;
+    // the batch's traces have been read: the next batch's copies go out now
+    if (next < nbatch && !ph.suppress && tid < NFT) fetch(next, par ^ 1);
+    // ---- projection of each face's states through F^_f
+    if (pact) sg_nproj<O, 6 * BP, GS>(face, sW + pe * S::ESW + pr * GP, sP + pe * S::ESP + pr * BP);
+    // ---- the batch's DOFs have arrived (or a wait gave up: every thread leaves)
+    ok = tc::mbar_wait(barQ, par, ph.wait) && ok;
+    if (!__syncthreads_and(ok)) {
+      if (tid == 0) {
+        atomicOr(ph.err, 1);
+        tc::mbar_wait(barQ, par, ph.wait);         // the copies in flight, if any, land first
+        if (next < nbatch) tc::mbar_wait(barT, par ^ 1, ph.wait);
       }
+      done = true;
+      continue;
     }
-    if (valid) {
-      constexpr int NS = (M > 0) ? 15 : 9;
-      float* q = st.Q + (size_t)g * qs + Slots<FUSED>::sub(fs, NQ, B) + (size_t)b * CS;
-      const float* qr = FUSED ? q : sQ + es * C::QS + b;
-      float qv[NQ];
+    if (act && t0 + es < sl.n) {
+      const float* nd = sD + pos_of(es) * NDS;
+      const Geo geo(nd);
+      const float4 m0 = ld4(nd + 12);   // lam, mu, 1/rho
+      const float* pp = sP + es * S::ESP + b;
+      float G[3][3], dv[3];
 #pragma unroll
-      for (int r = 0; r < NQ; ++r) qv[r] = qr[r * RS];
-      float Sv[NS];
-#pragma unroll
-      for (int r = 0; r < NS; ++r) Sv[r] = 0.f;
-      const float* nd = sD + es * NDP;
-      // one copy of the face code (the kernel is bound by instruction fetch)
-#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
-        const float* pp = sP + (i * B + b) * XP6 + es * 6;
-        float W[6];
+        const int c = set_of_face(i);
+        float P[6];
 #pragma unroll
-        for (int r = 0; r < 6; ++r) W[r] = pp[r];
-        flux_rows_add<NS>(W, nd + 4 + 11 * i, nd[0], nd[1], nd[2], Sv);
+        for (int r = 0; r < 6; ++r) P[r] = pp[(6 * i + r) * BP];
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) G[e][j] = i == 0 ? geo.J[c][e] * P[j] : fmaf(geo.J[c][e], P[j], G[e][j]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) dv[j] = i == 0 ? P[3 + j] : dv[j] + P[3 + j];
       }
+      float out[9], eps[6];
+      hooke(G, m0.x, m0.y, out, eps);
+      const int g = e0 + pos_of(es), fsim = FUSED ? (f0 + es) % sl.nsim : 0;
+      float* q = st.Q + (size_t)g * qs + Slots<FUSED>::sub(fsim, NQ, B) + (size_t)b * CS;
+      const float* qr = sQ + (FUSED ? es / FUSED_GROUP * GB + b * CS + es % FUSED_GROUP : es * C::QS + b);
 #pragma unroll
-      for (int r = 0; r < 9; ++r) q[r * RS] = qv[r] + Sv[r];
-      if constexpr (M > 0) {
+      for (int r = 0; r < 6; ++r) q[r * RS] = qr[r * RS] - out[r];
 #pragma unroll
-        for (int l = 0; l < M; ++l)
+      for (int j = 0; j < 3; ++j) q[(6 + j) * RS] = fmaf(-m0.z, dv[j], qr[(6 + j) * RS]);
 #pragma unroll
-          for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = qv[9 + 6 * l + r] + ph.omega[l] * Sv[NS - 6 + r];
-      }
+      for (int l = 0; l < M; ++l)
+#pragma unroll
+        for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = fmaf(-ph.omega[l], eps[r], qr[(9 + 6 * l + r) * RS]);
     }
+    __syncthreads();
+    if (tid == 0 && next < nbatch && !ph.suppress) issue_q(next);
   }
 }
 

@@ -12,6 +12,7 @@ namespace ltsdev {
 
 struct Launchers {
   int B, F, NQ, QS, BUFS, NE, NT, NEN, NTN;
+  int TS;                                    // floats of an element's face traces (one simulation)
   int FG;                                    // simulations per CTA in fused mode (1: single)
   size_t smem_predict, smem_neighbour;
   int blocks_predict, blocks_neighbour;      // resident CTAs per SM (filled by init)
@@ -29,8 +30,8 @@ struct Launchers {
   void (*predict_sp)(const DevOps&, const DevState&, const PhaseArgs&, int grid, cudaStream_t);
   size_t smem_predict_sp;
   int blocks_predict_sp, NE_SP, NT_SP;
-  // neighbour kernel of the same engine (face traces and orientation maps; no partition), in
-  // two tile variants: 8 elements per CTA (two CTAs per SM) or 4 (four CTAs per SM)
+  // neighbour kernel of the same engine (on the stored face traces; no partition), in two tile
+  // variants: 10 slots per CTA (fused 8) or 5 (4)
   void (*neighbour_sp[2])(const DevOps&, const DevState&, const PhaseArgs&, int grid, cudaStream_t);
   size_t smem_neighbour_sp[2];
   int blocks_neighbour_sp[2], NEN_SP[2], NTN_SP[2];
@@ -93,15 +94,19 @@ struct Impl {
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->blocks_predict_sp, k_predict_sp<O, M, FU>,
                                                         SpCfg<O, M, FU>::NT, L->smem_predict_sp);
       if (e != cudaSuccess) return e;
-      e = smem_attrs(k_neighbour_sp<O, M, 8, FU>, L->smem_neighbour_sp[0], true);
+      // as for k_predict_tc: the query answers one CTA for a kernel that allocates tensor memory;
+      // the shape's CTAs fit registers, shared memory and tensor memory (1 KB reserved per CTA)
+      if (SpCfg<O, M, FU>::TM && SpShape<O>::MINB * (L->smem_predict_sp + 1024) <= 228 * 1024)
+        L->blocks_predict_sp = SpShape<O>::MINB;
+      e = smem_attrs(k_neighbour_sp<O, M, 0, FU>, L->smem_neighbour_sp[0], true);
       if (e != cudaSuccess) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->blocks_neighbour_sp[0], k_neighbour_sp<O, M, 8, FU>,
-                                                        SpnCfg<O, M, 8>::NT, L->smem_neighbour_sp[0]);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->blocks_neighbour_sp[0], k_neighbour_sp<O, M, 0, FU>,
+                                                        SpnCfg<O, M, 0, FU>::NT, L->smem_neighbour_sp[0]);
       if (e != cudaSuccess) return e;
-      e = smem_attrs(k_neighbour_sp<O, M, 4, FU>, L->smem_neighbour_sp[1], true);
+      e = smem_attrs(k_neighbour_sp<O, M, 1, FU>, L->smem_neighbour_sp[1], true);
       if (e != cudaSuccess) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->blocks_neighbour_sp[1], k_neighbour_sp<O, M, 4, FU>,
-                                                        SpnCfg<O, M, 4>::NT, L->smem_neighbour_sp[1]);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->blocks_neighbour_sp[1], k_neighbour_sp<O, M, 1, FU>,
+                                                        SpnCfg<O, M, 1, FU>::NT, L->smem_neighbour_sp[1]);
       if (e != cudaSuccess) return e;
     }
     if constexpr (M == 0) {
@@ -123,10 +128,10 @@ struct Impl {
     using S = SpCfg<O, M, (FG > 1)>;
     k_predict_sp<O, M, (FG > 1)><<<grid, S::NT, S::TOTAL * sizeof(float), st>>>(o, s, p);
   }
-  template <int NE>
+  template <int TILE>
   static void neighbour_sp(const DevOps& o, const DevState& s, const PhaseArgs& p, int grid, cudaStream_t st) {
-    k_neighbour_sp<O, M, NE, (FG > 1)>
-        <<<grid, SpnCfg<O, M, NE>::NT, SpnCfg<O, M, NE>::TOTAL * sizeof(float), st>>>(o, s, p);
+    using S = SpnCfg<O, M, TILE, (FG > 1)>;
+    k_neighbour_sp<O, M, TILE, (FG > 1)><<<grid, S::NT, S::TOTAL * sizeof(float), st>>>(o, s, p);
   }
   static void predict_tc(const DevOps& o, const DevState& s, const PhaseArgs& p, int grid, int passes, int* err,
                          long long wait_cycles, int suppress_commit, cudaStream_t st) {
@@ -210,14 +215,17 @@ struct Impl {
       L.smem_predict_sp = SpCfg<O, M, (FG > 1)>::TOTAL * sizeof(float);
       L.NE_SP = SpCfg<O, M, (FG > 1)>::NE;
       L.NT_SP = SpCfg<O, M, (FG > 1)>::NT;
-      L.neighbour_sp[0] = &neighbour_sp<8>;
-      L.neighbour_sp[1] = &neighbour_sp<4>;
-      L.smem_neighbour_sp[0] = SpnCfg<O, M, 8>::TOTAL * sizeof(float);
-      L.smem_neighbour_sp[1] = SpnCfg<O, M, 4>::TOTAL * sizeof(float);
-      L.NEN_SP[0] = 8;
-      L.NEN_SP[1] = 4;
-      L.NTN_SP[0] = SpnCfg<O, M, 8>::NT;
-      L.NTN_SP[1] = SpnCfg<O, M, 4>::NT;
+      using S0 = SpnCfg<O, M, 0, (FG > 1)>;
+      using S1 = SpnCfg<O, M, 1, (FG > 1)>;
+      L.neighbour_sp[0] = &neighbour_sp<0>;
+      L.neighbour_sp[1] = &neighbour_sp<1>;
+      L.smem_neighbour_sp[0] = S0::TOTAL * sizeof(float);
+      L.smem_neighbour_sp[1] = S1::TOTAL * sizeof(float);
+      L.NEN_SP[0] = S0::NE;
+      L.NEN_SP[1] = S1::NE;
+      L.NTN_SP[0] = S0::NT;
+      L.NTN_SP[1] = S1::NT;
+      L.TS = TraceCfg<C::F>::TS;
     }
     L.neighbour = &neighbour;
     L.receivers = &receivers;

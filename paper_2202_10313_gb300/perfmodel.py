@@ -108,32 +108,31 @@ def sparse_terms(order):
 
 
 def flops_predict_sparse(o, m):
-    """Flops of k_predict_sp per element: the generated sparse products (time kernel, volume,
-    face traces and face projection: nonzero operator entries only, Sec. IV-A "all
-    sparsity"), the star / relaxation / Taylor arithmetic of the column phase, the
-    interface states and flux rows, and the update."""
+    """Flops of k_predict_sp per element: the generated products on the six rows of each
+    direction (three velocities, three stress rows dxi_c/dx . sigma; nonzero operator entries
+    only, Sec. IV-A "all sparsity") for the derivatives, the volume term, the face traces and
+    the projection; per derivative and for the update one combination with dxi/dx and Hooke's
+    law, the stress rows, relaxation and Taylor sums (anelastic: the top-degree modes have no
+    products; elastic: derivative d has degree o - 1 - d); the interface states."""
     B, F, NQ = nbasis(o), nface(o), 9 + 6 * m
     t = sparse_terms(o)
-    time = sum(2 * 9 * t["time"][d if m == 0 else 0] for d in range(o - 1))
-    star = 2 * 54 + 20
-    ck_epi = star + m * 24 + m * 12 + 2 * (NQ + 9)
-    vol_epi = star + m * 24 + m * 12 + NQ
-    rows = 30 + (18 if m else 0)
-    return (time + (o - 1) * B * ck_epi + 2 * 9 * t["vol"] + B * vol_epi + 2 * 9 * t["face"] + 4 * F * 50
-            + 2 * 6 * t["face"] + B * 4 * rows + B * (NQ + 2 * 6 * m))
+    time = sum(2 * 6 * t["time"][d if m == 0 else 0] for d in range(o - 1))
+    star, rows = 45 + 20 + 9, 45                  # gradient, Hooke, divergence; stress rows
+    col = sum(nbasis(o - 1 - (d if m == 0 else 0)) * star for d in range(o - 1))
+    relax = m * (12 + 18 + 12)                    # coupling, relaxation, Taylor sums of 6 rows
+    act = sum((B if m else nbasis(o - 1 - d)) * (rows + 18 + relax) for d in range(o - 1))
+    final = B * (star + 18 + m * (12 + 24) + 9)
+    return (time + col + act + 2 * 6 * t["vol"] + 2 * 2 * 6 * t["face"] + 4 * F * 50 + B * (rows + 15) + final)
 
 
 def flops_neighbour_sparse(o, m):
-    """Flops of k_neighbour_sp per element: the traces X F~_j of the four neighbours' buffers on
-    their faces j (nonzero entries; each face of the reference element equally likely, so the
-    four faces together cost the nonzeros of all four F~), the orientation maps R_h (degree
-    blocks), the interface states, the generated F^ projection, flux rows and update."""
+    """Flops of k_neighbour_sp per element: the orientation maps R_h (degree blocks) on the six
+    rows of the four stored face traces, the interface states, the generated F^ projection of six
+    rows per face, one combination with dxi/dx and Hooke's law, and the update."""
     B, F, NQ = nbasis(o), nface(o), 9 + 6 * m
     t = sparse_terms(o)
     rh = sum((p + 1) ** 2 for p in range(o))          # terms of one R_h per face row
-    rows = 30 + (18 if m else 0)
-    return (2 * 9 * t["face"] + 2 * 9 * 4 * rh + 4 * F * 50 + 2 * 6 * t["face"] + B * 4 * rows
-            + B * (NQ + 2 * 6 * m))
+    return 2 * 6 * 4 * rh + 4 * F * 50 + 2 * 6 * t["face"] + B * (72 + 20 + 15 + NQ + 6 * m)
 
 
 def essential_flops(order, m):

@@ -69,3 +69,42 @@ def test_generated_terms_are_the_oracle_operators_nonzeros(order):
     assert sum(1 for t in terms if t[0] == "t") == nk
     assert sum(1 for t in terms if t[0] == "v") == nk
     assert sum(1 for t in terms if t[0] == "k") == nk
+
+
+@pytest.mark.parametrize("order", [3, 4, 5])
+def test_row_form_terms_are_the_oracle_operators_nonzeros(order):
+    """The row-form products of the forward kernels (gen_sparse --list-rows): per direction c the
+    rows K_c (time) and K_c^T (volume), per face F~_i (traces) and F~_i^T (projection)."""
+    build.build()
+    exe = os.path.join(build.OUT_DIR, "gen_sparse")
+    out = subprocess.run([exe, "--list-rows", str(order)], capture_output=True, text=True, check=True).stdout
+    ob = Basis(order)
+    B, F = len(ob.K[0]), ob.Ft[0].shape[1]
+    kmax = max(np.abs(k).max() for k in ob.K)
+    fmax = max(np.abs(f).max() for f in ob.Ft)
+    block = lambda ms: np.concatenate([np.pad(m, ((0, 0), (i * m.shape[1], (len(ms) - 1 - i) * m.shape[1])))
+                                       for i, m in enumerate(ms)])
+    want = {"T": block([ob.K[c] for c in range(3)]), "V": block([ob.K[c].T for c in range(3)]),
+            "P": block([ob.Ft[i] for i in range(4)])}
+    # traces: the input mode is listed without its set
+    g = np.zeros((4 * F, 4 * B))
+    for i in range(4):
+        g[i * F:(i + 1) * F, :B] = ob.Ft[i].T
+    got = {k: np.zeros_like(v) for k, v in want.items()}
+    got["G"], want["G"] = np.zeros_like(g), g
+    for line in out.splitlines():
+        kind, _, o, k, val = line.split()
+        o, k = int(o), int(k)
+        if kind == "P":
+            assert k // F == o // B
+        assert got[kind][o, k] == 0.0
+        got[kind][o, k] = float(val)
+    for kind in want:
+        scale = kmax if kind in "TV" else fmax
+        w = want[kind]
+        if kind == "T":      # outputs of the top degree vanish and are not written
+            nb1 = (order - 1) * order * (order + 1) // 6
+            for c in range(3):
+                assert np.abs(w[c * B + nb1:(c + 1) * B]).max() <= 1e-10 * kmax
+        assert np.abs(got[kind] - w).max() <= 1e-6 * scale, kind
+        assert np.all((np.abs(w) <= 1e-10 * scale) | (got[kind] != 0.0)), kind
