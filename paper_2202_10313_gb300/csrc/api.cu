@@ -718,6 +718,25 @@ PhaseArgs phase_args(const lts_solver* h, const Phase& ph) {
     }
   }
   for (int l = 0; l < 3; ++l) pa.omega[l] = l < (int)h->omega.size() ? (float)h->omega[l] : 0.f;
+  for (int m = 0; m < (int)h->omega.size() && m < 3; ++m) {
+    const double om = h->omega[m];
+    double p[6] = {1.0};
+    for (int d = 0; d < 5; ++d) {
+      p[d + 1] = -om * p[d];
+      pa.rp[m][d] = (float)p[d];
+      pa.rg[m][d] = (float)(om / p[d + 1]);
+    }
+    for (int l = 0; l < h->nc; ++l) {
+      double c = 1.0, tail[6] = {0.0}, cp[5];
+      for (int d = 0; d < h->order; ++d) {
+        c *= h->delta * std::ldexp(1.0, l) / (d + 1);
+        cp[d] = c * p[d];
+      }
+      for (int d = h->order - 1; d >= 0; --d) tail[d] = tail[d + 1] + cp[d];   // sum over d' >= d
+      pa.ra[l][m] = (float)tail[0];
+      for (int d = 0; d + 1 < h->order; ++d) pa.rh[l][m][d] = (float)(om / p[d + 1] * tail[d + 1]);
+    }
+  }
   pa.err = h->d_err;
   pa.wait = h->wait_cycles;
   pa.suppress = h->suppress_commit;

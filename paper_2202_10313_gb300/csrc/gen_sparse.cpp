@@ -39,7 +39,7 @@
 //   sg_nproj_o{O}(face, g, y): y[face DY + b] = F^_face of g[face DG + m] (neighbour kernel)
 // (x, y: the row of set 0; dx: the distance between a thread's rows of consecutive sets, 0 for
 // the velocities, which all sets share; DY, DG template parameters). Outputs are split into parts
-// of equal multiply-add count.
+// by set (partition_sets).
 // and for the reverse predict pass of the discrete adjoint (k_adj_pred_sp):
 //   sp_trace_o{O}(part, x, g): G_i[f] = sum_k x[k] F~_i[k][f] alone (the traces of sp_vol).
 //   sp_tproj_o{O}(part, x, y): y[b] = sum_i sum_f x[i F + f] F~_i[b][f] (the transposed face
@@ -95,17 +95,40 @@ struct RowOut {
 // The face opposite barycentric coordinate c: xi_c = 0 for c < 3 (faces 2, 1, 0), face 3 for c = 3.
 int face_of_set(int c) { return c < 3 ? 2 - c : 3; }
 
-// Consecutive runs of the outputs with multiply-add shares as the weights ask.
-Parts partition_weighted(const std::vector<RowOut>& outs, const std::vector<double>& weights) {
-  double total = 0.0, wsum = 0.0;
+// One part per set (a part reads each row it needs whole, so a part of two sets reads twice as
+// much shared memory), the outputs of set `cut` in two halves of nearly equal multiply-add count
+// at a multiple of four outputs (cut < 0: none).
+Parts partition_sets(const std::vector<RowOut>& outs, int cut) {
+  Parts parts;
+  for (size_t i = 0; i < outs.size();) {
+    size_t e = i, total = 0, acc = 0;
+    for (; e < outs.size() && outs[e].set == outs[i].set; ++e) total += outs[e].t.size();
+    parts.emplace_back();
+    bool split = outs[i].set != cut;
+    for (size_t o = i; o < e; ++o) {
+      size_t four = 0;
+      for (size_t q = o; q < std::min(e, o + 4); ++q) four += outs[q].t.size();
+      if (!split && outs[o].idx % 4 == 0 && acc + four / 2 > total / 2) {
+        parts.emplace_back();
+        split = true;
+      }
+      parts.back().push_back((int)o);
+      acc += outs[o].t.size();
+    }
+    i = e;
+  }
+  return parts;
+}
+
+// Consecutive runs of the outputs with equal multiply-add shares.
+Parts partition_runs(const std::vector<RowOut>& outs, int n) {
+  double total = 0.0, acc = 0.0;
   for (const RowOut& u : outs) total += u.t.size();
-  for (double w : weights) wsum += w;
-  Parts parts(weights.size());
-  size_t p = 0;
-  double acc = 0.0, upto = weights[0] / wsum * total;
+  Parts parts(n);
+  int p = 0;
   for (size_t o = 0; o < outs.size(); ++o) {
     const double w = (double)outs[o].t.size();
-    while (p + 1 < parts.size() && acc + 0.5 * w > upto) upto += weights[++p] / wsum * total;
+    while (p + 1 < n && acc + 0.5 * w > total * (p + 1) / n) ++p;
     parts[p].push_back((int)o);
     acc += w;
   }
@@ -157,7 +180,6 @@ struct Products {
 
   template <typename NzK, typename NzF>
   void build_rows(const lts::RefOps& ops, const NzK& nzk, const NzF& nzf) {
-    const std::vector<double> wt(O == 5 ? 4 : (O == 4 ? 3 : 1), 1.0), wv = wt, wp = wt;
     for (int v = 0; v <= O - 2; ++v) {
       const int kend = nb(O - v), bend = nb(O - 1 - v);
       std::vector<RowOut> outs;
@@ -168,7 +190,8 @@ struct Products {
             if (nzk(ops.K[c][b * B + k])) u.t.push_back({k, (float)ops.K[c][b * B + k]});
           outs.push_back(u);
         }
-      rtime_parts.push_back(partition_weighted(outs, wt));
+      // order 5: K_2 (287 of 647 terms) in two parts, so that 12 warps share the work evenly
+      rtime_parts.push_back(O == 3 ? partition_runs(outs, 1) : partition_sets(outs, O == 5 ? 2 : -1));
       rtime.push_back(outs);
     }
     for (int q = 0; q < 4; ++q) {
@@ -188,7 +211,7 @@ struct Products {
         rvol.push_back(u);
       }
     }
-    rvol_parts = partition_weighted(rvol, wv);
+    rvol_parts = O == 3 ? partition_runs(rvol, 1) : partition_sets(rvol, -1);
     for (int f = 0; f < 4; ++f)
       for (int b = 0; b < B; ++b) {
         RowOut u{'P', f, b, B, {}};
@@ -196,7 +219,8 @@ struct Products {
           if (nzf(ops.Ft[f][b * F + m])) u.t.push_back({m, (float)ops.Ft[f][b * F + m]});
         rproj.push_back(u);
       }
-    rproj_parts = partition_weighted(rproj, wp);
+    // by face; orders 4 and 3 have warps for three parts and for one
+    rproj_parts = O == 5 ? partition_sets(rproj, -1) : partition_runs(rproj, O == 4 ? 3 : 1);
   }
 
   void build(int order, int np) {

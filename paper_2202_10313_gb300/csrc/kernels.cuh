@@ -143,6 +143,9 @@ struct PhaseArgs {
   float hcoef[MAXC][6];        // (dt_l/2)^(d+1)/(d+1)!
   int parity[MAXC];            // step index parity of each cluster in this phase
   float omega[3];
+  // memory variables in closed form (sparse engine): d^d theta_l = (-omega_l)^d E_d with E_0 = theta_l,
+  // E_{d+1} = E_d + rg[l][d] eps_d, and the time integral ra[cluster][l] theta_l + sum_d rh[..][d] eps_d
+  float rp[3][5], rg[3][5], ra[MAXC][3], rh[MAXC][3][5];
   // bounded waits of the asynchronous copies (k_predict_sp): the device error word a kernel
   // sets when a wait gives up, the bound in SM cycles, and the failure-path test switch
   // (nothing is copied, so the waits run out)

@@ -40,12 +40,10 @@
 namespace ltsdev {
 
 // Shape of the predict kernel: a batch of 16 elements, so that the six rows of a set are three
-// full warps of (row, element) lanes, and NP parts of the row phases (3 NP warps). BP: padded
-// modes of a row, GP: stride of a face-state row, GS: of a face's six rows, YT: of a time-kernel
-// product's row, BBP: padded modes of top degree (column phase). Order 5: one CTA per SM (the
-// straight-line code of one phase at a time in the instruction cache); four parts, not six: a
-// part reads its rows whole, and six parts' reads bound the row phase by shared memory
-// (1,272 against 1,660 cycles a row phase at order 5).
+// full warps of (row, element) lanes. BP: padded modes of a row, GP: stride of a face-state row, GS:
+// of a face's six rows, YT: of a time-kernel product's row, BBP: padded modes of top degree (column
+// phase). Order 5: one CTA per SM (the straight-line code of one phase at a time in the
+// instruction cache).
 // What bounds it (order 5, anelastic, 16 elements, about 24,000 cycles): the row phases' staged reads
 // and multiply-adds one after the other (5,100 cycles over the four derivatives), the column
 // phases' instruction issue (5,900), the update's DOF stores. Measured on one GB300, 138,240
@@ -55,15 +53,15 @@ template <int O>
 struct SpShape;
 template <>
 struct SpShape<5> {
-  static constexpr int BP = 36, GP = 20, GS = 144, YT = 20, BBP = 16, ESM = 20, MINB = 1, NP = 4;
+  static constexpr int BP = 36, GP = 20, GS = 144, YT = 20, BBP = 16, ESM = 20, MINB = 1;
 };
 template <>
 struct SpShape<4> {
-  static constexpr int BP = 20, GP = 12, GS = 72, YT = 12, BBP = 10, ESM = 12, MINB = 2, NP = 3;
+  static constexpr int BP = 20, GP = 12, GS = 72, YT = 12, BBP = 10, ESM = 12, MINB = 2;
 };
 template <>
 struct SpShape<3> {
-  static constexpr int BP = 12, GP = 12, GS = 72, YT = 4, BBP = 6, ESM = 4, MINB = 3, NP = 1;
+  static constexpr int BP = 12, GP = 12, GS = 72, YT = 4, BBP = 6, ESM = 4, MINB = 3;
 };
 
 // Floats of an element's row in the sparse engine's tables (16-byte aligned rows). Predict:
@@ -105,7 +103,7 @@ struct SpCfg {
   static constexpr int NTA = NE * BA, NT = rup(NTA + NE * BBP, 32);
   static constexpr int NW = NT / 32;
   static_assert(NE % 8 == 0, "eight lanes of a row phase share a row (NE = 14 would straddle rows: bank conflicts)");
-  static_assert(NTA % 32 == 0 && BP >= B && GP >= F && GS >= 6 * GP && BBP >= BB && 3 * H::NP <= NW, "shape");
+  static_assert(NTA % 32 == 0 && BP >= B && GP >= F && GS >= 6 * GP && BBP >= BB, "shape");
   static_assert(YT >= BA && (YT / 4) % 2 == 1 && (BP / 4) % 2 == 1 && (GP / 4) % 2 == 1, "row strides");
   static constexpr bool TM = M > 0;   // part of the column state lives in tensor memory
   // tensor-memory columns: 36 per warp of a lane quarter, a power of two in all
@@ -119,10 +117,14 @@ struct SpCfg {
   static constexpr int S_X = 0;
   static constexpr int S_Y = S_X + NE * ESX;
   static constexpr int S_G = S_Y + NE * ESY;
-  static constexpr int S_E = S_G + NE * ESG;           // [2][NE][EDS], double-buffered
+  static constexpr int QBUF_ = FU ? NE * NQ * B : NE * C::QS;
+  // order 5: the updated DOFs leave through shared memory by one bulk copy (over the face states,
+  // which the next batch writes late); orders 3 and 4 have no room beside their other CTAs
+  static constexpr bool STAGE = O == 5;
+  static constexpr int S_E = S_G + rup(STAGE && QBUF_ > NE * ESG ? QBUF_ : NE * ESG, 4);   // [2][NE][EDS], double-buffered
   // the batch's DOFs: NE elements of QS floats (one simulation), or the simulation groups of its
   // NE slots (fused: groups of 4 consecutive slots, NE and the simulation count multiples of 4)
-  static constexpr int QBUF = FU ? NE * NQ * B : NE * C::QS;
+  static constexpr int QBUF = QBUF_;
   static constexpr int S_Q = rup(S_E + 2 * NE * EDS, 4);
   static constexpr int S_F = rup(S_Q + QBUF, 4);       // [4][B][F] F~ (half-step traces)
   static constexpr int S_SLOT = rup(S_F + 4 * B * F, 4);   // fused: [2][2][NE] element, simulation of the slots
@@ -130,14 +132,38 @@ struct SpCfg {
   static constexpr int TOTAL = S_BAR + 4;                             // and the tensor-memory address
 };
 
-// The part of a row phase that warp w runs (-1: none) and the third of its rows (two of the six):
-// at order 5 the warps of one scheduler (w mod 4) share a part's code.
-template <int O>
-__device__ __forceinline__ void row_job(int w, int& part, int& third) {
-  constexpr int NP = SpShape<O>::NP;
-  part = w < 3 * NP ? (O == 5 ? w % NP : w / 3) : -1;
-  third = O == 5 ? w / NP : w % 3;
+// Jobs of the row phases: (part, third of its rows: two of the six), job j for warp j mod NW. Four
+// bits each, part * 3 + third. Order 5: the 12 jobs of warps w, w + 4, w + 8 (one scheduler's) add
+// up to nearly equal multiply-add counts: time kernel parts K_0 (108), K_1 (252), K_2 (144, 143);
+// volume and traces: direction 3 (309), 0 (471), 1 (357), 2 (390); projection: the faces (103, 105,
+// 363, 309).
+template <int N>
+constexpr uint64_t job_table(const int (&c)[N]) {
+  uint64_t t = 0;
+  for (int j = 0; j < N; ++j) t |= (uint64_t)c[j] << (4 * j);
+  return t;
 }
+template <int O>
+struct SpJobs;
+template <>
+struct SpJobs<5> {
+  static constexpr int NT = 12, NV = 12, NP = 16;   // 15: none
+  static constexpr uint64_t T = job_table({3, 4, 5, 9, 6, 7, 8, 10, 0, 1, 2, 11});
+  static constexpr uint64_t V = job_table({3, 4, 5, 10, 6, 7, 9, 11, 0, 1, 2, 8});
+  static constexpr uint64_t P = job_table({6, 7, 8, 11, 9, 10, 0, 2, 15, 15, 1, 4, 15, 15, 3, 5});
+};
+template <>
+struct SpJobs<4> {   // ten warps: two of them take the light jobs of the volume phase in pairs
+  static constexpr int NT = 9, NV = 12, NP = 9;
+  static constexpr uint64_t T = job_table({6, 7, 8, 3, 4, 5, 0, 1, 2});
+  static constexpr uint64_t V = job_table({0, 2, 3, 4, 5, 9, 10, 11, 7, 8, 1, 6});
+  static constexpr uint64_t P = job_table({0, 1, 2, 3, 4, 5, 6, 7, 8});
+};
+template <>
+struct SpJobs<3> {   // one part (five warps: several jobs each measured slower)
+  static constexpr int NT = 3, NV = 3, NP = 3;
+  static constexpr uint64_t T = job_table({0, 1, 2}), V = T, P = T;
+};
 
 // the generated products of order O
 template <int O, int DY>
@@ -258,6 +284,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     k_predict_sp(DevOps ops, DevState st, PhaseArgs ph) {
   using S = SpCfg<O, M, FUSED>;
   using C = typename S::C;
+  using J = SpJobs<O>;
   constexpr int B = S::B, F = S::F, NE = S::NE, NT = S::NT, NQ = S::NQ, NA = S::NA, BP = S::BP, YT = S::YT, GP = S::GP,
                 GS = S::GS;
   extern __shared__ float4 smem4[];
@@ -295,31 +322,42 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
   // simulation, the batch's contiguous elements (n x QS floats); fused simulations, the
   // contiguous simulation groups from the batch's first slot to its last. Every wait is
   // bounded; one that gives up sets the error word and the CTA returns.
-  auto issue = [&](int bt, int buf) {
-    const float* src;
-    uint32_t bytes;
-    int e0, ne;
+  // A batch's first element, its elements, and its DOFs in Q (offset and bytes).
+  auto span = [&](int bt, int& e0, int& ne, size_t& off, uint32_t& bytes) {
     if constexpr (!FUSED) {
       e0 = ph.begin + bt * NE;
       ne = min(NE, ph.end - e0);
-      src = st.Q + (size_t)e0 * C::QS;
+      off = (size_t)e0 * C::QS;
       bytes = (uint32_t)ne * C::QS * 4;
     } else {
       int f0, e1, f1;
       sl.decode(bt * NE, e0, f0);
       sl.decode(min(sl.n, bt * NE + NE) - 1, e1, f1);
-      const int ngr = sl.nsim / FUSED_GROUP;
       ne = e1 - e0 + 1;
       e0 += ph.begin;
-      src = st.Q + (size_t)e0 * qs + (size_t)(f0 / FUSED_GROUP) * GB;
-      bytes = (uint32_t)((e1 - (e0 - ph.begin)) * ngr + f1 / FUSED_GROUP - f0 / FUSED_GROUP + 1) * GB * 4;
+      off = (size_t)e0 * qs + (size_t)(f0 / FUSED_GROUP) * GB;
+      bytes = (uint32_t)(min(NE, sl.n - bt * NE) / FUSED_GROUP) * GB * 4;
     }
-    tc::bulk_load2(sQ, src, bytes, smem + S::S_E + buf * NE * EDS, st.sdata + (size_t)e0 * EDS, (uint32_t)ne * EDS * 4,
-                   sBar);
   };
-  // Tensor memory as per-thread storage (anelastic): the time integrals of the memory variables
-  // and the half-step integrals between the derivatives, and the update's known terms between
-  // the volume products and the update. 18 warps of 96 registers hold the rest without spills
+  auto issue = [&](int bt, int buf) {
+    int e0, ne;
+    size_t off;
+    uint32_t bytes;
+    span(bt, e0, ne, off, bytes);
+    tc::bulk_load2(sQ, st.Q + off, bytes, smem + S::S_E + buf * NE * EDS, st.sdata + (size_t)e0 * EDS,
+                   (uint32_t)ne * EDS * 4, sBar);
+  };
+  // The updated DOFs of batch bt, staged in sG, leave by one bulk copy.
+  auto write_back = [&](int bt) {
+    int e0, ne;
+    size_t off;
+    uint32_t bytes;
+    span(bt, e0, ne, off, bytes);
+    tc::bulk_store(st.Q + off, sG, bytes);
+  };
+  // Tensor memory as per-thread storage (anelastic): the time integrals and the half-step integrals
+  // between the derivatives, and the update's known terms between the volume products and the
+  // update. 18 warps of 96 registers hold the rest without spills
   // (spilling instead: 62 local-memory instructions per element, most of them missing L1).
   uint32_t* sTm = reinterpret_cast<uint32_t*>(smem + S::S_BAR + 2);
   uint32_t tm = 0;
@@ -339,6 +377,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
   }
   if (tid == 0 && blockIdx.x < nbatch && !ph.suppress) issue(blockIdx.x, 0);
 
+  int last = -1;   // the batch whose updated DOFs are staged
   for (int batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
     const int t0 = batch * NE;
     const float* sE = smem + S::S_E + qpar * NE * EDS;
@@ -375,10 +414,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     }
     const int ts = t0 + es;
     const bool valid = act && ts < sl.n;
-    const int g = valid ? elem_of(es) : ph.begin;
-    const int fs = (FUSED && valid) ? sSlot[NE + es] : 0;
-    const size_t qoff = (size_t)g * qs + Slots<FUSED>::sub(fs, NQ, B) + (size_t)b * CS;
-    const size_t boff = (size_t)g * bs + Slots<FUSED>::sub(fs, 9, B) + (size_t)b * CS;
+    // (offsets into Q and the modal buffers are computed where they are needed: registers)
     // trace buffer of slot k
     auto trace_of = [&](int k) {
       return (FUSED ? (size_t)sSlot[k] * st.nsim + sSlot[NE + k] : (size_t)(ph.begin + t0 + k)) * TraceCfg<F>::TS;
@@ -397,6 +433,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
         break;
       }
     }
+    if (S::STAGE && tid == 0 && batch != (int)blockIdx.x) write_back(batch - gridDim.x);
     // this column's DOFs in the staged copy (row stride RS, as in Q)
     int soff = es * C::QS + b;
     if constexpr (FUSED) soff = (es / FUSED_GROUP) * GB + b * CS + es % FUSED_GROUP;
@@ -404,6 +441,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     const int meta = valid ? __float_as_int(ed[23]) : 0;
     const int cl = meta & 0xff;
     const bool finer = (meta & FLAG_FINER) != 0;
+    const bool anyfiner = __any_sync(0xffffffffu, finer);
     float T[9], Th[9], Da[NA > 0 ? NA : 1];
     float* xo = sX + es * S::ESX + b;
     {
@@ -423,13 +461,13 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
       if constexpr (S::TM) {
         float ta[18];
 #pragma unroll
-        for (int r = 0; r < NA; ++r) ta[r] = c0 * Da[r];
+        for (int r = 0; r < NA; ++r) ta[r] = ph.ra[cl][r / 6] * Da[r];
         tc::tmem_st18(tm, ta);
-        tc::tmem_st9(tm + 18, Th);
+        tc::tmem_st9(tm + 18, T);
+        if (anyfiner) tc::tmem_st9(tm + 27, Th);
         tc::tmem_wait_st();
       }
     }
-    const bool anyfiner = __any_sync(0xffffffffu, finer);
     const bool batch_finer = __syncthreads_or(finer);
     // ---- time kernel: d^{d+1} Q from d^d Q (Cauchy-Kowalevski), Taylor sums
 #pragma unroll 1
@@ -437,17 +475,16 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
       // elastic: d^d Q has degree <= O-1-d, so the product is truncated (variant d); the
       // anelastic coupling keeps every degree (variant 0)
       const int variant = (M == 0) ? d : 0;
-      {
-        int part, third;
-        row_job<O>(warp, part, third);
-        const int r = 2 * third + ((tid >> 4) & 1);
+#pragma unroll 1
+      for (int j = warp; j < J::NT; j += S::NW) {
+        const int job = (int)(J::T >> (4 * j)) & 15, part = job / 3, r = 2 * (job % 3) + ((tid >> 4) & 1);
         sg_time<O, 6 * YT>(variant, part, sX + re * S::ESX + r * BP, r < 3 ? 0 : 3 * BP, sY + re * S::ESY + r * YT);
       }
       __syncthreads();
       const float c1 = ph.coef[cl][d + 1];
       float out[9], eps[6];
       // products of modes b >= nbasis(O-1-variant) are identically zero and not written (all of
-      // the top degree: whole warps)
+      // the top degree: whole warps, whose memory variables follow in closed form)
       const bool has = grpA && b < nbasis(O - 1 - variant);
       if (has) {
         const float* yp = sY + es * S::ESY + b;
@@ -469,32 +506,37 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
       } else {
 #pragma unroll
         for (int r = 0; r < 9; ++r) out[r] = 0.f;
-#pragma unroll
-        for (int r = 0; r < 6; ++r) eps[r] = 0.f;
       }
       if constexpr (M > 0) {
         const float4 m0 = ld4(ed + 12), m1 = ld4(ed + 16);
         const float ylam[3] = {m0.w, m1.y, m1.w}, ymu[3] = {m1.x, m1.z, ed[20]};
 #pragma unroll
-        for (int l = 0; l < M; ++l) coupling_add(out, Da + 6 * l, ylam[l], ymu[l]);
-        float ta[18];
-        tc::tmem_ld18(tm, ta);
+        for (int l = 0; l < M; ++l) coupling_add(out, Da + 6 * l, ylam[l] * ph.rp[l][d], ymu[l] * ph.rp[l][d]);
+        if (grpA) {
+          float ta[18];
+          tc::tmem_ld18(tm, ta);
 #pragma unroll
-        for (int l = 0; l < M; ++l)
+          for (int l = 0; l < M; ++l) {
+            const float h = ph.rh[cl][l][d], g = ph.rg[l][d];
 #pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            const float w = ph.omega[l] * (eps[r] - Da[6 * l + r]);
-            Da[6 * l + r] = w;
-            ta[6 * l + r] = fmaf(c1, w, ta[6 * l + r]);
+            for (int r = 0; r < 6; ++r) {
+              ta[6 * l + r] = fmaf(h, eps[r], ta[6 * l + r]);
+              Da[6 * l + r] = fmaf(g, eps[r], Da[6 * l + r]);
+            }
           }
-        tc::tmem_st18(tm, ta);
+          tc::tmem_st18(tm, ta);
+        }
         if (anyfiner) {
           const float h1 = ph.hcoef[cl][d + 1];
-          tc::tmem_ld9(tm + 18, Th);
+          tc::tmem_ld9(tm + 27, Th);
 #pragma unroll
           for (int r = 0; r < 9; ++r) Th[r] = fmaf(h1, out[r], Th[r]);
-          tc::tmem_st9(tm + 18, Th);
+          tc::tmem_st9(tm + 27, Th);
         }
+        tc::tmem_ld9(tm + 18, T);
+#pragma unroll
+        for (int r = 0; r < 9; ++r) T[r] = fmaf(c1, out[r], T[r]);
+        tc::tmem_st9(tm + 18, T);
         tc::tmem_wait_st();
       } else if (finer && has) {
         const float h1 = ph.hcoef[cl][d + 1];
@@ -503,22 +545,28 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
       }
       // next row operand: the next derivative, or after the last one the time integral
       if (act && (M > 0 || has || d == O - 2)) {
+        if constexpr (!S::TM) {
 #pragma unroll
-        for (int r = 0; r < 9; ++r) T[r] = fmaf(c1, out[r], T[r]);
+          for (int r = 0; r < 9; ++r) T[r] = fmaf(c1, out[r], T[r]);
+        }
         const Geo geo(ed);
         if (d < O - 2)
           put_rows<3, BP>(xo, out, geo);
         else
           put_rows<4, BP>(xo, T, geo);
       }
+      // the previous batch's DOFs have left the face states' memory
+      if (S::STAGE && tid == 0 && d == O - 2) tc::bulk_store_read_wait();
       __syncthreads();
     }
     // ---- LTS buffers as modes (Eq. lts_buffers): the adjoint and partitioned runs read those
     if (ph.bufs & BUFS_MODAL) {
       if constexpr (S::TM) {
-        if (anyfiner) tc::tmem_ld9(tm + 18, Th);
+        tc::tmem_ld9(tm + 18, T);
+        if (anyfiner) tc::tmem_ld9(tm + 27, Th);
       }
       if (valid) {
+        const size_t boff = (size_t)elem_of(es) * bs + Slots<FUSED>::sub(FUSED ? sSlot[NE + es] : 0, 9, B) + (size_t)b * CS;
         float* b1 = st.B1 + boff;
 #pragma unroll
         for (int r = 0; r < 9; ++r) b1[r * RS] = T[r];
@@ -558,15 +606,14 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
           for (int r = 0; r < 6; ++r)
             ta[6 * l + r] = fmaf(-ph.omega[l], ta[6 * l + r], valid ? q[(9 + 6 * l + r) * RS] : 0.f);
         tc::tmem_st18(tm, ta);
-        tc::tmem_st9(tm + 27, acc);
+        tc::tmem_st9(tm + 18, acc);
         tc::tmem_wait_st();
       }
     }
     // ---- volume products and local face traces of T (row phase)
-    {
-      int part, third;
-      row_job<O>(warp, part, third);
-      const int r = 2 * third + ((tid >> 4) & 1);
+#pragma unroll 1
+    for (int j = warp; j < J::NV; j += S::NW) {
+      const int job = (int)(J::V >> (4 * j)) & 15, part = job / 3, r = 2 * (job % 3) + ((tid >> 4) & 1);
       sg_vol<O, 6 * BP, GS>(part, sX + re * S::ESX + r * BP, r < 3 ? 0 : 3 * BP, sY + re * S::ESY + r * BP,
                             sG + re * S::ESG + r * GP);
     }
@@ -603,10 +650,9 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     __syncthreads();
     // ---- projection through F^ (row phase): faces 0..2 onto the volume products of their
     // direction, face 3 into six rows of its own (over the time integral's rows)
-    {
-      int part, third;
-      row_job<O>(warp, part, third);
-      const int r = 2 * third + ((tid >> 4) & 1);
+#pragma unroll 1
+    for (int j = warp; j < J::NP; j += S::NW) {
+      const int job = (int)(J::P >> (4 * j)) & 15, part = job / 3, r = 2 * (job % 3) + ((tid >> 4) & 1);
       sg_proj<O, 6 * BP, GS>(part, sG + re * S::ESG + r * GP, sY + re * S::ESY + r * BP, sX + re * S::ESX + r * BP);
     }
     __syncthreads();
@@ -614,7 +660,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     float ta[NA > 0 ? NA : 1];
     if constexpr (S::TM) {
       tc::tmem_ld18(tm, ta);
-      tc::tmem_ld9(tm + 27, acc);
+      tc::tmem_ld9(tm + 18, acc);
     }
     if (valid) {
       const float* yp = sY + es * S::ESY + b;
@@ -646,7 +692,8 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
       }
       float out[9], eps[6];
       hooke(G, m0.x, m0.y, out, eps);
-      float* q = st.Q + qoff;
+      float* q = S::STAGE ? sG + soff
+                          : st.Q + (size_t)elem_of(es) * qs + Slots<FUSED>::sub(FUSED ? sSlot[NE + es] : 0, NQ, B) + (size_t)b * CS;
 #pragma unroll
       for (int r = 0; r < 6; ++r) q[r * RS] = acc[r] - out[r];
 #pragma unroll
@@ -655,13 +702,16 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
       for (int l = 0; l < M; ++l)
 #pragma unroll
         for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = fmaf(-ph.omega[l], eps[r], ta[6 * l + r]);
+      if (S::STAGE && !FUSED && b < C::QS - NQ * B) sG[es * C::QS + NQ * B + b] = 0.f;   // padding
     }
+    if constexpr (S::STAGE) tc::fence_smem_to_async();
+    last = batch;
     // ---- half-step traces of the faces with a finer neighbour: rows of the half-step integral over
     // the projections (each thread its own column), then a warp per such face, lane = (velocity or
     // stress rows, face mode). The second half's trace is the step's (stored above) minus it.
     if ((ph.bufs & BUFS_TRACES) && batch_finer) {
       if constexpr (S::TM) {
-        if (anyfiner) tc::tmem_ld9(tm + 18, Th);
+        if (anyfiner) tc::tmem_ld9(tm + 27, Th);
       }
       if (valid && finer) put_rows<4, BP>(xo, Th, Geo(ed));
       __syncthreads();
@@ -708,6 +758,13 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
           }
         }
       }
+    }
+  }
+  if constexpr (S::STAGE) {
+    __syncthreads();
+    if (tid == 0) {
+      if (last >= 0 && last + (int)gridDim.x >= nbatch) write_back(last);
+      tc::bulk_store_wait();
     }
   }
   if constexpr (S::TM) {

@@ -109,6 +109,16 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                "l"(src), "r"(bytes), "r"(smem_u32(mbar))
                : "memory");
 }
+// From shared to global memory (the writers of src have fenced and met at a barrier): one bulk group;
+// its source may be overwritten after bulk_store_read_wait, its result is complete after
+// bulk_store_wait (both by the issuing thread).
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_store_read_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // The same in steps, for copies that several threads issue: one arrival with the bytes announced,
 // and a copy (the issuing thread has ordered the destination's earlier accesses itself).
 __device__ __forceinline__ void mbar_expect(uint64_t* mbar, uint32_t bytes) {
