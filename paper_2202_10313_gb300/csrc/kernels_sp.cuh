@@ -375,6 +375,8 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     tc::fence_after_sync();
     tm = *sTm + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * 36;
   }
+  wait_for_previous_kernel();
+  let_next_kernel_launch();
   if (tid == 0 && blockIdx.x < nbatch && !ph.suppress) issue(blockIdx.x, 0);
 
   int last = -1;   // the batch whose updated DOFs are staged
@@ -937,6 +939,8 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
   }
   link(blockIdx.x);
   __syncthreads();
+  wait_for_previous_kernel();
+  let_next_kernel_launch();
   if (!ph.suppress && blockIdx.x < nbatch) {
     if (tid < NFT) fetch(blockIdx.x, 0);
     if (tid == 0) issue_q(blockIdx.x);

@@ -57,6 +57,23 @@ struct Launchers {
                  int nblocks, cudaStream_t);
 };
 
+// Launch that may start while the kernel before it in the stream still runs (the kernel calls
+// wait_for_previous_kernel before it touches the state).
+template <typename... P, typename... A>
+void launch_dependent(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <int O, int M, int FG>
 struct Impl {
   using C = Cfg<O, M, FG>;
@@ -126,12 +143,12 @@ struct Impl {
   }
   static void predict_sp(const DevOps& o, const DevState& s, const PhaseArgs& p, int grid, cudaStream_t st) {
     using S = SpCfg<O, M, (FG > 1)>;
-    k_predict_sp<O, M, (FG > 1)><<<grid, S::NT, S::TOTAL * sizeof(float), st>>>(o, s, p);
+    launch_dependent(k_predict_sp<O, M, (FG > 1)>, grid, S::NT, S::TOTAL * sizeof(float), st, o, s, p);
   }
   template <int TILE>
   static void neighbour_sp(const DevOps& o, const DevState& s, const PhaseArgs& p, int grid, cudaStream_t st) {
     using S = SpnCfg<O, M, TILE, (FG > 1)>;
-    k_neighbour_sp<O, M, TILE, (FG > 1)><<<grid, S::NT, S::TOTAL * sizeof(float), st>>>(o, s, p);
+    launch_dependent(k_neighbour_sp<O, M, TILE, (FG > 1)>, grid, S::NT, S::TOTAL * sizeof(float), st, o, s, p);
   }
   static void predict_tc(const DevOps& o, const DevState& s, const PhaseArgs& p, int grid, int passes, int* err,
                          long long wait_cycles, int suppress_commit, cudaStream_t st) {
@@ -141,10 +158,11 @@ struct Impl {
   }
   static void receivers(const DevOps& o, const float* Q, long long qs, int nsim, int fg, const float* ed,
                         const float* phi, const RecvItem* it, float* out, const float* om, int n, cudaStream_t st) {
-    k_receivers<O, M><<<n, rup(C::B, 32), 0, st>>>(o, Q, qs, nsim, fg, ed, phi, it, out, om[0], om[1], om[2]);
+    launch_dependent(k_receivers<O, M>, n, RecvCfg<O>::NT, 0, st, o, Q, qs, nsim, fg, ed, phi, it, out, om[0], om[1],
+                     om[2]);
   }
   static void sources(float* Q, long long qs, int fg, const float* phi, const SrcItem* it, int n, cudaStream_t st) {
-    k_sources<O, M><<<1, 128, 0, st>>>(Q, qs, fg, phi, it, n);
+    launch_dependent(k_sources<O, M>, 1, rup(6 * C::B, 32), 0, st, Q, qs, fg, phi, it, n);
   }
   static void pack(const DevOps& o, const DevState& s, const PhaseArgs& p, const int* se, const int* sc,
                    const int* rc, int n, float* msg, cudaStream_t st) {
