@@ -238,7 +238,7 @@ void face_orientation_maps(const lts::RefOps& ops, std::vector<float>& out) {
 }
 
 struct Layout {
-  size_t Q, B1, B2, B3, edata, ndata, sdata, sndata, nbr, ncode, meta, emat, partial, err, K, Ft, Fh, Fb, Rh, rphi, sphi, cut, msg,
+  size_t Q, B1, B2, B3, edata, ndata, sdata, sndata, nlink, nbr, ncode, meta, emat, partial, err, K, Ft, Fh, Fb, Rh, rphi, sphi, cut, msg,
       total;
 };
 
@@ -272,6 +272,7 @@ Layout layout_of(const lts_solver* h, int64_t K) {
   L.ndata = take(sizeof(float) * K * ltsdev::ND);
   L.sdata = take(sizeof(float) * K * ltsdev::EDS);
   L.sndata = take(sizeof(float) * K * ltsdev::NDS);
+  L.nlink = take(sizeof(int2) * K * 4);
   L.nbr = take(sizeof(int) * K * 4);
   L.ncode = take(sizeof(int) * K * 4);
   L.meta = take(sizeof(int) * K);
@@ -357,6 +358,7 @@ void setup_device(lts_solver* h) {
   std::vector<float> edata(K * ltsdev::ED, 0.f), ndata(K * ltsdev::ND, 0.f), sdata(K * ltsdev::EDS, 0.f),
       sndata(K * ltsdev::NDS, 0.f);
   std::vector<int> nbr(4 * K, -1), ncode(4 * K, 0), meta(K, 0);
+  std::vector<int2> nlink(4 * K, make_int2(-1, 0));
   std::vector<double> emat(4 * K);
   const lts::Mesh& M = h->mesh;
   for (int64_t nk = 0; nk < K; ++nk) {
@@ -426,6 +428,8 @@ void setup_device(lts_solver* h) {
         const int rel = dc == 0 ? 0 : (dc < 0 ? 1 : 2);
         ncode[4 * nk + f] = (M.nbr_face[4 * k + f] * 3 + M.nbr_orient[4 * k + f]) | (rel << 8);
         rels |= (dc == 0 ? 1 : (dc < 0 ? 2 : 3)) << (2 * f);
+        nlink[4 * nk + f] = make_int2(4 * (int)h->iperm[nb] + M.nbr_face[4 * k + f],
+                                      M.nbr_orient[4 * k + f] | (rel == 2 ? 4 : 0) | h->cluster[k] << 8);
         if (dc < 0) flags |= ltsdev::FLAG_FINER;
         if (dc > 0) flags |= ltsdev::FLAG_COARSER;
       }
@@ -505,6 +509,7 @@ void setup_device(lts_solver* h) {
   h->dst.ndata = reinterpret_cast<float*>(base + Lo.ndata);
   h->dst.sdata = reinterpret_cast<float*>(base + Lo.sdata);
   h->dst.sndata = reinterpret_cast<float*>(base + Lo.sndata);
+  h->dst.nlink = reinterpret_cast<int2*>(base + Lo.nlink);
   h->dst.T1 = h->dst.B1;
   h->dst.T2 = h->dst.T1 + K * (int64_t)X.TS * h->nsim;
   h->dst.nbr = reinterpret_cast<int*>(base + Lo.nbr);
@@ -536,6 +541,7 @@ void setup_device(lts_solver* h) {
   up(h->dst.ndata, ndata.data(), sizeof(float) * ndata.size());
   up(h->dst.sdata, sdata.data(), sizeof(float) * sdata.size());
   up(h->dst.sndata, sndata.data(), sizeof(float) * sndata.size());
+  up(h->dst.nlink, nlink.data(), sizeof(int2) * nlink.size());
   up(h->dst.nbr, nbr.data(), sizeof(int) * nbr.size());
   up(h->dst.ncode, ncode.data(), sizeof(int) * ncode.size());
   up(h->dst.meta, meta.data(), sizeof(int) * meta.size());

@@ -36,7 +36,8 @@
 //       trace of set c on its face f(c), g[f DG + m] = sum_k x[c dx + k] F~_f[k][m]
 //   sg_proj_o{O}(part, g, y, p): F^_f of the face states g[f DG + m], added to y[c(f) DY + b]
 //       for c < 3, written to p[b] for face 3
-//   sg_nproj_o{O}(face, g, y): y[face DY + b] = F^_face of g[face DG + m] (neighbour kernel)
+//   sg_nproj_o{O}(part, g, y): y[f DY + b] = F^_f of g[f DG + m] for the faces f (neighbour
+//       kernel; six equal parts at order 5, else four)
 // (x, y: the row of set 0; dx: the distance between a thread's rows of consecutive sets, 0 for
 // the velocities, which all sets share; DY, DG template parameters). Outputs are split into parts
 // by set (partition_sets).
@@ -513,10 +514,8 @@ void emit_rows(FILE* f, int O, const Products& P) {
                     "const float* __restrict__ g, float* __restrict__ y, float* __restrict__ p", "g, y, p",
                     {P.rproj_parts}, {P.rproj});
   std::snprintf(nm, sizeof nm, "sg_nproj_o%d", O);
-  Parts faces(4);
-  for (size_t o = 0; o < P.rproj.size(); ++o) faces[P.rproj[o].set].push_back((int)o);
   emit_row_dispatch(f, nm, "int DY, int DG", "DY, DG", "const float* __restrict__ g, float* __restrict__ y", "g, y",
-                    {faces}, {P.rproj}, true);
+                    {partition_runs(P.rproj, O == 5 ? 6 : 4)}, {P.rproj}, true);
 }
 
 void emit_order(FILE* f, int O, int nparts) {

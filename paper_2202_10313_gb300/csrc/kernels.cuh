@@ -127,6 +127,8 @@ struct DevState {
   float* T2;
   const float* sdata;    // [K][EDS]
   const float* sndata;   // [K][NDS]
+  // [K][4]: 4 * neighbour + its face, or -1; orientation | 4 if the neighbour is coarser | cluster << 8
+  const int2* nlink;
   const int* nbr;        // [K][4] neighbour (internal index) or -1
   const int* ncode;      // [K][4] (j*3+h) | (relation << 8): 0 same, 1 neighbour finer, 2 neighbour coarser
   const int* meta;       // [K] cluster | FLAG_*

@@ -783,17 +783,19 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
 // trace is already there, so only R_h is left of the face product:
 //   states:      thread = (element, face, face mode): H = G R_h (degree block), closed-form
 //                interface state with the neighbour coefficients;
-//   projection:  a warp per face (and 30 lanes): lane = (row, element), the generated F^_f
-//                product of its row;
+//   projection:  a warp per part of the generated F^ products (parts of equal multiply-add
+//                count): 30 lanes = (row, element);
 //   update:      thread = (element, mode): the faces' rows combined with dxi/dx and Hooke's law
 //                once (as in k_predict_sp), Q <- Q + S^N.
 // Everything a batch reads arrives by bulk asynchronous copies (TMA): a lane per face copies its
 // neighbour's trace and thread 0 the element tables while the previous batch projects and
 // updates, and the DOFs, which only the update reads, right after the previous update.
-// Measured on one GB300 (order 5, anelastic, 138,240 elements): 2.26 ns per element against 3.93 ns
-// with gathered buffers and face products in this kernel (4 x 1,260 bytes and 2,365 instructions
-// per element); bound by DRAM (9.3 KB per element: 1.4 ns at the copy rate) and by the latency of
-// its three barriers.
+// Measured on one GB300 (order 5, anelastic, 138,240 elements): 2.00 ns per element (1.49 elastic)
+// against 3.93 ns (3.43) with gathered buffers and face products in this kernel (4 x 1,260 bytes
+// and 2,365 instructions per element). Bound by instruction issue and latency between its three
+// barriers (42 % issue; DRAM 9.3 KB per element: 1.4 ns at the copy rate). Warps of two kinds that
+// hand batches over through double buffers (no CTA barrier, two CTAs per SM instead of three)
+// took 2.53 ns, and L2 prefetches one to four batches ahead 2.29-2.31 against 2.27 ns.
 template <int O>
 struct SpnShape;   // CTAs per SM, narrow and wide tile; GP: face row, BP: padded modes; ESW, ESP:
                    // element strides (conflict-free 16-byte accesses of 5 x 6 lanes)
@@ -820,8 +822,9 @@ struct SpnCfg {
   static constexpr int B = C::B, F = C::F, NQ = C::NQ;
   static constexpr int NE = spn_ne(TILE, FU);
   static constexpr int GP = H::GP, GS = 6 * H::GP, BP = H::BP, ESW = H::ESW, ESP = H::ESP;
-  static constexpr int NL = 6 * NE, NWF = rup(NL, 32) / 32;   // projection lanes and warps per face
-  static constexpr int NT = rup(NE * B, 32) > 128 * NWF ? rup(NE * B, 32) : 128 * NWF;
+  static constexpr int NPP = O == 5 ? 6 : 4;                  // equal parts of the projection
+  static constexpr int NL = 6 * NE, NWF = rup(NL, 32) / 32;   // its lanes, and warps per part
+  static constexpr int NT = rup(NE * B, 32) > 32 * NPP * NWF ? rup(NE * B, 32) : 32 * NPP * NWF;
   static constexpr int MINB = TILE ? H::MIN1 : H::MIN0;
   static_assert(ESW >= 4 * GS && ESP >= 24 * BP && 4 * NE <= 64, "strides");
   static constexpr int FS = TraceCfg<F>::FS;
@@ -837,10 +840,10 @@ struct SpnCfg {
 };
 
 template <int O, int DY, int DG>
-__device__ __forceinline__ void sg_nproj(int face, const float* g, float* y) {
-  if constexpr (O == 5) ltssp::sg_nproj_o5<DY, DG>(0, face, g, y);
-  if constexpr (O == 4) ltssp::sg_nproj_o4<DY, DG>(0, face, g, y);
-  if constexpr (O == 3) ltssp::sg_nproj_o3<DY, DG>(0, face, g, y);
+__device__ __forceinline__ void sg_nproj(int part, const float* g, float* y) {
+  if constexpr (O == 5) ltssp::sg_nproj_o5<DY, DG>(0, part, g, y);
+  if constexpr (O == 4) ltssp::sg_nproj_o4<DY, DG>(0, part, g, y);
+  if constexpr (O == 3) ltssp::sg_nproj_o3<DY, DG>(0, part, g, y);
 }
 
 template <int O, int M, int TILE, bool FUSED>
@@ -865,8 +868,8 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
   const bool act = tid < NE * B;
   const int es = act ? (FUSED ? tid / (4 * B) * 4 + tid % 4 : tid / B) : 0;
   const int b = act ? (FUSED ? tid % (4 * B) / 4 : tid % B) : 0;
-  const int warp = tid >> 5, face = warp % 4, lane6 = warp / 4 * 32 + (tid & 31);   // projection row
-  const bool pact = warp < 4 * S::NWF && lane6 < S::NL;
+  const int warp = tid >> 5, part = warp % S::NPP, lane6 = warp / S::NPP * 32 + (tid & 31);   // projection row
+  const bool pact = warp < S::NPP * S::NWF && lane6 < S::NL;
   const int pr = lane6 / NE, pe = lane6 % NE;
   const Slots<FUSED> sl(st, ph);
   const int nbatch = (sl.n + NE - 1) / NE;
@@ -896,53 +899,50 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
     const int n = min(NE, sl.n - bt * NE);
     tc::bulk_load(sQ, src, (uint32_t)(FUSED ? n / FUSED_GROUP * GB : n * C::QS) * 4, barQ);
   };
-  // The face slots of a batch belong to the threads of the first warps (tid < 4 NE): link() reads
-  // the neighbour and the buffer it is read from, fetch() issues the copies.
-  const float* tsrc = nullptr;
-  int torient = -1;
+  // The face slots of a batch belong to the threads of the first warps (tid < 4 NE): link() reads,
+  // two batches ahead, what names the neighbour's trace (one 8-byte load: with neighbour, code
+  // and cluster apart, two dependent loads from memory held the first warp 3,100 of 11,000 cycles
+  // a batch), fetch() issues the copies.
   auto link = [&](int bt) {
-    tsrc = nullptr;
-    torient = -1;
     const int t = bt * NE + tid / 4;
-    if (tid >= 4 * NE || t >= sl.n) return;
+    if (tid >= 4 * NE || t >= sl.n) return make_int2(-1, 0);
     int e, f;
     sl.decode(t, e, f);
-    const size_t k = (size_t)ph.begin + e;
-    const int nb = __ldg(st.nbr + 4 * k + tid % 4), code = __ldg(st.ncode + 4 * k + tid % 4);
-    if (nb < 0) return;
-    const int jh = code & 0xff, second = ((code >> 8) & 0xff) == 2 && ph.parity[__ldg(st.meta + k) & 0xff] == 1;
-    torient = jh % 3;
-    tsrc = (second ? st.T2 : st.T1) +
-           ((FUSED ? (size_t)nb * st.nsim + f : (size_t)nb) * 4 + jh / 3) * FS;
+    return __ldg(st.nlink + 4 * ((size_t)ph.begin + e) + tid % 4);
   };
   // the first rup(4 NE, 32) threads (whole warps)
-  auto fetch = [&](int bt, int buf) {
+  auto fetch = [&](int bt, int buf, int2 l) {
     int* sI = reinterpret_cast<int*>(smem + S::S_I) + buf * 4 * NE;
-    if (tid < 4 * NE) sI[tid] = torient;
-    const unsigned m = __ballot_sync(0xffffffffu, tsrc != nullptr);
+    if (tid < 4 * NE) sI[tid] = l.x < 0 ? -1 : l.y & 3;
+    const unsigned m = __ballot_sync(0xffffffffu, l.x >= 0);
     tc::fence_smem_to_async();
+    int e0, f0, ne;
+    span(bt, e0, f0, ne);
     if ((tid & 31) == 0) {
       uint32_t bytes = (uint32_t)__popc(m) * FS * 4;
-      int e0, f0, ne;
-      span(bt, e0, f0, ne);
       if (tid == 0) bytes += (uint32_t)ne * NDS * 4;
       tc::mbar_expect(barT, bytes);
       if (tid == 0) tc::bulk_copy(smem + S::S_D + buf * NE * NDS, st.sndata + (size_t)e0 * NDS, (uint32_t)ne * NDS * 4, barT);
     }
     __syncwarp();
-    if (tsrc) tc::bulk_copy(sT + tid * FS, tsrc, FS * 4, barT);
+    if (l.x >= 0) {
+      const bool second = (l.y & 4) && ph.parity[l.y >> 8] == 1;
+      const size_t face = FUSED ? ((size_t)(l.x >> 2) * st.nsim + (f0 + tid / 4) % sl.nsim) * 4 + (l.x & 3) : (size_t)l.x;
+      tc::bulk_copy(sT + tid * FS, (second ? st.T2 : st.T1) + face * FS, FS * 4, barT);
+    }
   };
   constexpr int NFT = rup(4 * NE, 32);   // fetching threads; one mbarrier arrival per warp
   if (tid == 0) {
     tc::mbar_init(barT, NFT / 32);
     tc::mbar_init(barQ, 1);
   }
-  link(blockIdx.x);
+  const int2 first = link(blockIdx.x);
+  int2 ahead = link(blockIdx.x + gridDim.x);   // of the next batch
   __syncthreads();
   wait_for_previous_kernel();
   let_next_kernel_launch();
   if (!ph.suppress && blockIdx.x < nbatch) {
-    if (tid < NFT) fetch(blockIdx.x, 0);
+    if (tid < NFT) fetch(blockIdx.x, 0, first);
     if (tid == 0) issue_q(blockIdx.x);
   }
   __syncthreads();   // the orientations written by fetch
@@ -956,7 +956,8 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
     span(batch, e0, f0, ne);
     // element position in the batch of slot k
     auto pos_of = [&](int k) { return FUSED ? (f0 + k) / sl.nsim : k; };
-    if (next < nbatch) link(next);
+    const int2 links = ahead;
+    ahead = link(next + gridDim.x);
     // ---- the traces and tables have arrived (or the wait gave up). H = G R_h per face mode
     // (degree block), interface states with the neighbour coefficients; faces without a
     // neighbour contribute nothing
@@ -967,15 +968,17 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
       float w6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const int h = (t0 + fe < sl.n) ? sI[fs] : -1;
       if (ok && h >= 0) {
-        const int pf = face_degree(f), q0 = nface(pf), q1 = nface(pf + 1);
-        const float* gp = sT + fs * FS;
-        const float* R = sR + h * F * F + f;
+        const int pf = face_degree(f), q0 = nface(pf);
+        const float* gp = sT + fs * FS + q0;
+        const float* R = sR + h * F * F + q0 * F + f;
         float hv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int q = q0; q < q1; ++q) {
-          const float w = R[q * F];
 #pragma unroll
-          for (int r = 0; r < 6; ++r) hv[r] = fmaf(gp[r * F + q], w, hv[r]);
-        }
+        for (int j = 0; j < O; ++j)
+          if (j <= pf) {
+            const float w = R[j * F];
+#pragma unroll
+            for (int r = 0; r < 6; ++r) hv[r] = fmaf(gp[r * F + j], w, hv[r]);
+          }
         interface_state(hv, sD + pos_of(fe) * NDS + 16 + 12 * fi, w6);
       }
       float* wp = sW + fe * S::ESW + fi * GS + f;
@@ -984,9 +987,9 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
     }
     __syncthreads();
     // the batch's traces have been read: the next batch's copies go out now
-    if (next < nbatch && !ph.suppress && tid < NFT) fetch(next, par ^ 1);
-    // ---- projection of each face's states through F^_f
-    if (pact) sg_nproj<O, 6 * BP, GS>(face, sW + pe * S::ESW + pr * GP, sP + pe * S::ESP + pr * BP);
+    if (next < nbatch && !ph.suppress && tid < NFT) fetch(next, par ^ 1, links);
+    // ---- projection of the faces' states through F^_f
+    if (pact) sg_nproj<O, 6 * BP, GS>(part, sW + pe * S::ESW + pr * GP, sP + pe * S::ESP + pr * BP);
     // ---- the batch's DOFs have arrived (or a wait gave up: every thread leaves)
     ok = tc::mbar_wait(barQ, par, ph.wait) && ok;
     if (!__syncthreads_and(ok)) {
