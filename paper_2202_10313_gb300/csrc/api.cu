@@ -6,10 +6,12 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <functional>
 #include <new>
 #include <numeric>
 #include <string>
+#include <system_error>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -136,6 +138,8 @@ struct lts_solver {
   DevState dst{};
   double* d_emat = nullptr;
   double* d_partial = nullptr;
+  int* d_iperm = nullptr;                   // internal index of each element
+  size_t scratch_bytes = 0;                 // of the LTS buffers, free between macro steps
   int* d_err = nullptr;                     // set by a kernel whose bounded wait gave up
   float* d_recv_phi = nullptr;
   float* d_src_phi = nullptr;
@@ -238,7 +242,7 @@ void face_orientation_maps(const lts::RefOps& ops, std::vector<float>& out) {
 }
 
 struct Layout {
-  size_t Q, B1, B2, B3, edata, ndata, sdata, sndata, nlink, nbr, ncode, meta, emat, partial, err, K, Ft, Fh, Fb, Rh, rphi, sphi, cut, msg,
+  size_t Q, B1, B2, B3, edata, ndata, sdata, sndata, nlink, iperm, nbr, ncode, meta, emat, partial, err, K, Ft, Fh, Fb, Rh, rphi, sphi, cut, msg,
       total;
 };
 
@@ -266,13 +270,16 @@ Layout layout_of(const lts_solver* h, int64_t K) {
   L.B1 = take(sizeof(float) * K * bs);
   L.B2 = take(sizeof(float) * K * bs);
   L.B3 = take(sizeof(float) * K * bs);
-  const size_t traces = sizeof(float) * 2 * K * (size_t)X.TS * h->nsim;
+  // (and at least the FP64 DOFs of one element, which are staged there)
+  const size_t traces = std::max(sizeof(float) * 2 * K * (size_t)X.TS * h->nsim,
+                                 sizeof(double) * X.NQ * X.B * (size_t)h->nsim);
   if (off < L.B1 + traces) take(L.B1 + traces - off);
   L.edata = take(sizeof(float) * K * ltsdev::ED);
   L.ndata = take(sizeof(float) * K * ltsdev::ND);
   L.sdata = take(sizeof(float) * K * ltsdev::EDS);
   L.sndata = take(sizeof(float) * K * ltsdev::NDS);
   L.nlink = take(sizeof(int2) * K * 4);
+  L.iperm = take(sizeof(int) * K);
   L.nbr = take(sizeof(int) * K * 4);
   L.ncode = take(sizeof(int) * K * 4);
   L.meta = take(sizeof(int) * K);
@@ -340,6 +347,33 @@ void free_device(lts_solver* h) {
   h->ready = false;
 }
 
+// fn(begin, end) over [0, n) in equal runs on the host's cores (small n: on this one).
+template <typename Fn>
+void host_parallel(int64_t n, int64_t grain, const Fn& fn) {
+  const int64_t cores = std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), 16);
+  const int64_t nt = std::max<int64_t>(1, std::min(cores, n / grain));
+  if (nt == 1) return fn(0, n);
+  std::vector<std::thread> pool;
+  std::exception_ptr failed[16];
+  auto part = [&](int64_t t) {
+    try {
+      fn(n * t / nt, n * (t + 1) / nt);
+    } catch (...) {
+      failed[t] = std::current_exception();
+    }
+  };
+  int64_t started = 1;
+  try {
+    for (; started < nt; ++started) pool.emplace_back(part, started);
+  } catch (const std::system_error&) {   // no more threads: the rest runs here
+  }
+  part(0);
+  for (int64_t t = started; t < nt; ++t) part(t);
+  for (std::thread& t : pool) t.join();
+  for (int64_t t = 0; t < nt; ++t)
+    if (failed[t]) std::rethrow_exception(failed[t]);
+}
+
 void setup_device(lts_solver* h) {
   const int64_t K = h->mesh.K;
   const Launchers& X = h->L;
@@ -361,7 +395,8 @@ void setup_device(lts_solver* h) {
   std::vector<int2> nlink(4 * K, make_int2(-1, 0));
   std::vector<double> emat(4 * K);
   const lts::Mesh& M = h->mesh;
-  for (int64_t nk = 0; nk < K; ++nk) {
+  host_parallel(K, 4096, [&](int64_t begin, int64_t end) {
+  for (int64_t nk = begin; nk < end; ++nk) {
     const int64_t k = h->perm[nk];
     float* ed = &edata[nk * ltsdev::ED];
     float* nd = &ndata[nk * ltsdev::ND];
@@ -438,6 +473,7 @@ void setup_device(lts_solver* h) {
     std::memcpy(sd + 23, &flags, sizeof(int));
     std::memcpy(sd + 21, &rels, sizeof(int));
   }
+  });
   // ---- operators (float)
   const int B = X.B, F = X.F;
   std::vector<float> hK(3 * B * B), hFt(4 * B * F), hFh(4 * F * B), hFb(12 * B * F);
@@ -510,6 +546,8 @@ void setup_device(lts_solver* h) {
   h->dst.sdata = reinterpret_cast<float*>(base + Lo.sdata);
   h->dst.sndata = reinterpret_cast<float*>(base + Lo.sndata);
   h->dst.nlink = reinterpret_cast<int2*>(base + Lo.nlink);
+  h->d_iperm = reinterpret_cast<int*>(base + Lo.iperm);
+  h->scratch_bytes = Lo.edata - Lo.B1;
   h->dst.T1 = h->dst.B1;
   h->dst.T2 = h->dst.T1 + K * (int64_t)X.TS * h->nsim;
   h->dst.nbr = reinterpret_cast<int*>(base + Lo.nbr);
@@ -542,6 +580,8 @@ void setup_device(lts_solver* h) {
   up(h->dst.sdata, sdata.data(), sizeof(float) * sdata.size());
   up(h->dst.sndata, sndata.data(), sizeof(float) * sndata.size());
   up(h->dst.nlink, nlink.data(), sizeof(int2) * nlink.size());
+  const std::vector<int> iperm32(h->iperm.begin(), h->iperm.end());
+  up(h->d_iperm, iperm32.data(), sizeof(int) * iperm32.size());
   up(h->dst.nbr, nbr.data(), sizeof(int) * nbr.size());
   up(h->dst.ncode, ncode.data(), sizeof(int) * ncode.size());
   up(h->dst.meta, meta.data(), sizeof(int) * meta.size());
@@ -1648,6 +1688,53 @@ int lts_quadrature_points(lts_t* h, int64_t* n_per_elem, double* xyz_out) {
 
 // Host DOF arrays are simulation-major, [F][n][N^q][B] (F = 1: [n][N^q][B]); on the device
 // an element's row holds simulation groups of G = FG: [F/G][N^q][B][G].
+// DOFs between the caller's layout ([sim][element][q][b], FP64) and the device's: `n` elements from
+// `first` on in the caller's order, staged as [sim][n][q][b]; `to_device` fills Q from the staging
+// area, else the staging area from Q.
+static __global__ void k_convert_dofs(float* Q, double* stage, const int* iperm, int64_t first, int64_t n, int nq, int B, int G,
+                               int nsim, int64_t qs, bool to_device) {
+  const int64_t per = (int64_t)nq * B, total = per * n * nsim;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t e = i / per % n;
+    const int f = (int)(i / (per * n)), rb = (int)(i % per);
+    float* q = Q + iperm[first + e] * qs + (int64_t)(f / G) * per * G + (int64_t)rb * G + f % G;
+    if (to_device)
+      *q = (float)stage[i];
+    else
+      stage[i] = *q;
+  }
+}
+
+// Between macro steps the LTS buffers hold nothing that is read again: they stage the FP64 values,
+// so that one copy per block and simulation and a kernel do what a host loop over every value did.
+static void convert_dofs(lts_t* h, double* dofs, bool to_device) {
+  const int64_t K = h->mesh.K, per = (int64_t)h->L.NQ * h->L.B;
+  double* stage = reinterpret_cast<double*>(h->dst.B1);
+  const int64_t block = std::max<int64_t>(1, std::min<int64_t>(K, (int64_t)(h->scratch_bytes / (sizeof(double) * per * h->nsim))));
+  if (h->scratch_bytes < sizeof(double) * per * h->nsim) fail(LTS_ERR_STATE, "no room to stage the DOFs");
+  for (int64_t k0 = 0; k0 < K; k0 += block) {
+    const int64_t n = std::min(block, K - k0);
+    auto copy = [&](int f) {
+      double* host = dofs + ((int64_t)f * K + k0) * per;
+      double* dev = stage + (int64_t)f * n * per;
+      const size_t bytes = sizeof(double) * n * per;
+      if (to_device)
+        ck(cudaMemcpy(dev, host, bytes, cudaMemcpyHostToDevice), "upload DOFs");
+      else
+        ck(cudaMemcpy(host, dev, bytes, cudaMemcpyDeviceToHost), "download DOFs");
+    };
+    if (to_device)
+      for (int f = 0; f < h->nsim; ++f) copy(f);
+    const int64_t blocks = std::min<int64_t>((n * per * h->nsim + 255) / 256, 16 * (int64_t)h->num_sms);
+    k_convert_dofs<<<(unsigned)blocks, 256>>>(h->dst.Q, stage, h->d_iperm, k0, n, h->L.NQ, h->L.B, h->L.FG, h->nsim,
+                                              h->dst.qs, to_device);
+    ck(cudaGetLastError(), "DOF conversion");
+    if (!to_device)
+      for (int f = 0; f < h->nsim; ++f) copy(f);
+  }
+  if (to_device) ck(cudaDeviceSynchronize(), "synchronize");
+}
+
 static int64_t row_index(const lts_t* h, int r, int b, int f) {
   const int B = h->L.B, NQ = h->L.NQ, G = h->L.FG;
   return (int64_t)(f / G) * NQ * B * G + ((int64_t)r * B + b) * G + f % G;
@@ -1668,11 +1755,9 @@ static void unpack_row(const lts_t* h, const float* row, int64_t n, int64_t i, d
 }
 
 static void upload_dofs(lts_t* h, const double* dofs) {
-  const int64_t K = h->mesh.K, qs = h->dst.qs;
-  std::vector<float> q((size_t)K * qs, 0.f);
-  for (int64_t k = 0; k < K; ++k) pack_row(h, dofs, K, k, &q[h->iperm[k] * qs]);
   ck(cudaSetDevice(h->device), "cudaSetDevice");
-  ck(cudaMemcpy(h->dst.Q, q.data(), q.size() * sizeof(float), cudaMemcpyHostToDevice), "upload Q");
+  ck(cudaDeviceSynchronize(), "synchronize");
+  convert_dofs(h, const_cast<double*>(dofs), true);
 }
 
 int lts_project_initial(lts_t* h, const double* values) {
@@ -1711,13 +1796,10 @@ int lts_get_dofs(lts_t* h, double* dofs) {
   return run(h, [&] {
     if (!h->ready) fail(LTS_ERR_STATE, "clusters not set up");
     if (!dofs) fail(LTS_ERR_ARG, "null dofs");
-    const int64_t K = h->mesh.K, qs = h->dst.qs;
-    std::vector<float> q((size_t)K * qs);
     ck(cudaSetDevice(h->device), "cudaSetDevice");
     ck(cudaDeviceSynchronize(), "synchronize");
-    ck(cudaMemcpy(q.data(), h->dst.Q, q.size() * sizeof(float), cudaMemcpyDeviceToHost), "download Q");
     check_device_error(h);
-    for (int64_t k = 0; k < K; ++k) unpack_row(h, &q[h->iperm[k] * qs], K, k, dofs);
+    convert_dofs(h, dofs, false);
   });
 }
 
