@@ -897,6 +897,17 @@ int64_t macro_msg_bytes(const lts_solver* h, const MacroPlan& mp) {
   return b;
 }
 
+// A macro step's work items; stream-ordered after the previous macro step.
+void upload_items(lts_solver* h, const MacroPlan& mp, cudaStream_t stream) {
+  if (!mp.ritems.empty())
+    ck(cudaMemcpyAsync(h->d_ritems, mp.ritems.data(), mp.ritems.size() * sizeof(RecvItem), cudaMemcpyHostToDevice, stream),
+       "upload receiver items");
+  if (!mp.sitems.empty())
+    ck(cudaMemcpyAsync(h->d_sitems, mp.sitems.data(), mp.sitems.size() * sizeof(SrcItem), cudaMemcpyHostToDevice, stream),
+       "upload source items");
+  h->h2d_bytes += (int64_t)(mp.ritems.size() * sizeof(RecvItem) + mp.sitems.size() * sizeof(SrcItem));
+}
+
 void advance_steps(lts_solver* h, int64_t n_finest, cudaStream_t stream) {
   if (!h->ready) fail(LTS_ERR_STATE, "clusters not set up");
   struct Range {
@@ -918,16 +929,7 @@ void advance_steps(lts_solver* h, int64_t n_finest, cudaStream_t stream) {
   h->seis_used = seis_need;
   for (int64_t m = 0; m < nmac; ++m) {
     const MacroPlan& mp = plans[m];
-    // this macro step's work items; stream-ordered after the previous macro step
-    if (!mp.ritems.empty())
-      ck(cudaMemcpyAsync(h->d_ritems, mp.ritems.data(), mp.ritems.size() * sizeof(RecvItem), cudaMemcpyHostToDevice,
-                         stream),
-         "upload receiver items");
-    if (!mp.sitems.empty())
-      ck(cudaMemcpyAsync(h->d_sitems, mp.sitems.data(), mp.sitems.size() * sizeof(SrcItem), cudaMemcpyHostToDevice,
-                         stream),
-         "upload source items");
-    h->h2d_bytes += (int64_t)(mp.ritems.size() * sizeof(RecvItem) + mp.sitems.size() * sizeof(SrcItem));
+    upload_items(h, mp, stream);
     h->msg_bytes += macro_msg_bytes(h, mp);
     if (!h->use_graphs || h->profiling) {
       h->launches += enqueue_macro(h, mp, stream);
@@ -1056,35 +1058,54 @@ struct GradGeom {
   long long K;
 };
 
-__device__ lts::Dual grad_face_dot(const GradGeom& g, long long k, int face, int param) {
+// Derivatives of one face's contraction (own and neighbour state operators with their
+// correlations) with respect to the element's rho, lam, mu and the neighbour's: out[4 k + face][6].
+// One thread per (element, face). The correlations enter as twelve sums each (face_flux_forms), so
+// that the six derivatives cost six evaluations of the coefficients' closed forms; contracting
+// column by column for each took 6.5 of 7.5 ms (47,040 elements), bound by the FP64 rate.
+__global__ void k_grad_faces(GradGeom g, double* out) {
   using lts::Dual;
-  auto mat = [&](long long e, int base, Dual* m) {
-    m[0] = Dual(g.rho[e], param == base ? 1.0 : 0.0);
-    m[1] = Dual(g.lam[e], param == base + 1 ? 1.0 : 0.0);
-    m[2] = Dual(g.mu[e], param == base + 2 ? 1.0 : 0.0);
-  };
-  Dual own[3], oth[3];
-  mat(k, 0, own);
-  const Dual rinv = Dual(1.0) / own[0];
-  const int bc = g.bc[4 * k + face];
-  const long long nb = g.nbr[4 * k + face];
-  if (nb >= 0)
-    mat(nb, 3, oth);
-  else
-    for (int q = 0; q < 3; ++q) oth[q] = own[q];
-  const Dual zp = lts::sqrt_t((own[1] + Dual(2.0) * own[2]) * own[0]), zs = lts::sqrt_t(own[2] * own[0]);
-  const Dual zpo = nb >= 0 ? lts::sqrt_t((oth[1] + Dual(2.0) * oth[2]) * oth[0]) : zp;
-  const Dual zso = nb >= 0 ? lts::sqrt_t(oth[2] * oth[0]) : zs;
-  const Dual scale(-2.0 * g.area[4 * k + face] / g.detJ[k]);
-  Dual cl[8], cn[8];
-  lts::face_coefficients_t<Dual>(bc, zp, zs, zpo, zso, scale, cl, cn);
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 4 * g.K) return;
+  const long long k = t / 4;
+  const int face = (int)(t % 4);
   const double* Wk = g.W + (size_t)g.iperm[k] * ltsdev::AM_SIZE;
   const double* n = g.normal + 12 * k + 3 * face;
-  return lts::face_flux_dot<Dual>(n, cl, own[1], own[2], rinv, Wk + ltsdev::AM_LOC + face * 81) +
-         lts::face_flux_dot<Dual>(n, cn, own[1], own[2], rinv, Wk + ltsdev::AM_NBR + face * 81);
+  const int bc = g.bc[t];
+  const long long nb = g.nbr[t];
+  double fl[12], fn[12];
+  lts::face_flux_forms(n, Wk + ltsdev::AM_LOC + face * 81, fl);
+  lts::face_flux_forms(n, Wk + ltsdev::AM_NBR + face * 81, fn);
+  const Dual scale(-2.0 * g.area[t] / g.detJ[k]);
+  for (int p = 0; p < 6; ++p) {
+    if (p >= 3 && nb < 0) {
+      out[6 * t + p] = 0.0;
+      continue;
+    }
+    auto mat = [&](long long e, int base, Dual* m) {
+      m[0] = Dual(g.rho[e], p == base ? 1.0 : 0.0);
+      m[1] = Dual(g.lam[e], p == base + 1 ? 1.0 : 0.0);
+      m[2] = Dual(g.mu[e], p == base + 2 ? 1.0 : 0.0);
+    };
+    Dual own[3], oth[3];
+    mat(k, 0, own);
+    const Dual rinv = Dual(1.0) / own[0];
+    const Dual zp = lts::sqrt_t((own[1] + Dual(2.0) * own[2]) * own[0]), zs = lts::sqrt_t(own[2] * own[0]);
+    Dual zpo = zp, zso = zs;
+    if (nb >= 0) {
+      mat(nb, 3, oth);
+      zpo = lts::sqrt_t((oth[1] + Dual(2.0) * oth[2]) * oth[0]);
+      zso = lts::sqrt_t(oth[2] * oth[0]);
+    }
+    Dual cl[8], cn[8];
+    lts::face_coefficients_t<Dual>(bc, zp, zs, zpo, zso, scale, cl, cn);
+    out[6 * t + p] = (lts::face_flux_dot<Dual>(cl, own[1], own[2], rinv, fl) +
+                      lts::face_flux_dot<Dual>(cn, own[1], own[2], rinv, fn)).d;
+  }
 }
 
-__global__ void k_grad_contract(GradGeom g, double* grad) {
+// The gradient: star matrices' part and the sums of the faces' derivatives in a fixed order.
+__global__ void k_grad_contract(GradGeom g, const double* faces, double* grad) {
   using lts::Dual;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= g.K) return;
@@ -1093,9 +1114,9 @@ __global__ void k_grad_contract(GradGeom g, double* grad) {
     const Dual rho(g.rho[e], p == 0 ? 1.0 : 0.0), lam(g.lam[e], p == 1 ? 1.0 : 0.0), mu(g.mu[e], p == 2 ? 1.0 : 0.0);
     double acc = lts::star_dot<Dual>(g.jinv + 9 * e, lam, mu, Dual(1.0) / rho, We + ltsdev::AM_STAR).d;
     for (int i = 0; i < 4; ++i) {
-      acc += grad_face_dot(g, e, i, p).d;
+      acc += faces[6 * (4 * e + i) + p];
       const long long nb = g.nbr[4 * e + i];
-      if (nb >= 0) acc += grad_face_dot(g, nb, g.nbr_face[4 * e + i], 3 + p).d;
+      if (nb >= 0) acc += faces[6 * (4 * nb + g.nbr_face[4 * e + i]) + 3 + p];
     }
     grad[3 * e + p] = acc;
   }
@@ -1190,10 +1211,13 @@ GradGeom upload_geometry(const lts_solver* h, GeoBufs& bufs, cudaStream_t stream
 
 void contract_gradient(GradGeom g, const double* d_w, double* grad, cudaStream_t stream) {
   g.W = d_w;
-  DevBuf d_grad;
+  DevBuf d_grad, d_faces;
   d_grad.alloc(sizeof(double) * 3 * g.K);
+  d_faces.alloc(sizeof(double) * 24 * g.K);
   const int threads = 128;
-  k_grad_contract<<<(unsigned)((g.K + threads - 1) / threads), threads, 0, stream>>>(g, d_grad.get<double>());
+  k_grad_faces<<<(unsigned)((4 * g.K + threads - 1) / threads), threads, 0, stream>>>(g, d_faces.get<double>());
+  k_grad_contract<<<(unsigned)((g.K + threads - 1) / threads), threads, 0, stream>>>(g, d_faces.get<double>(),
+                                                                                    d_grad.get<double>());
   ck(cudaGetLastError(), "gradient contraction");
   ck(cudaMemcpyAsync(grad, d_grad.p, sizeof(double) * 3 * g.K, cudaMemcpyDeviceToHost, stream), "download gradient");
   ck(cudaStreamSynchronize(stream), "synchronize");
@@ -1204,6 +1228,16 @@ void contract_gradient(GradGeom g, const double* d_w, double* grad, cudaStream_t
 // checkpoints every `every` macro steps, and per macro step a phase-by-phase recompute
 // that keeps Q before each predict pass and the buffers before each neighbour pass for the
 // reverse sweep (k_adj_pred / k_adj_nbr, phases in reverse order).
+// The adjoint of Q ([element][sim][9][B], internal order) as [sim][element][9][B], caller's order.
+__global__ void k_adjoint_to_caller(const float* lam, double* out, const int* iperm, int64_t K, int nsim, int nb9) {
+  const int64_t total = K * nsim * nb9;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t e = i / nb9 % K;
+    const int f = (int)(i / (nb9 * K));
+    out[i] = lam[((int64_t)iperm[e] * nsim + f) * nb9 + i % nb9];
+  }
+}
+
 void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* data, double* misfit, double* grad,
                  double* synth_out, double* dq0, cudaStream_t stream, const DevBuf& d_amat, const DevBuf& d_fwd,
                  const DevBuf& d_back, const DevBuf& d_relem, const DevBuf& d_rphi, int nrec, const AdjTables& tabs,
@@ -1249,13 +1283,84 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   float* cp = d_cp.get<float>();
   const int* relem = d_relem.get<int>();
   const float* rphi = d_rphi.get<float>();
-  // ---- forward sweep: samples at the macro boundaries, checkpoints
   const int64_t s0 = h->s_now;
   std::vector<size_t> nrec_t(nrec);
+  MacroPlan mp;
+  // Phase layout of a macro step (the same for every macro step; the step indices are
+  // relative) and the bytes each phase's reverse reads: Q of the active elements before a
+  // predict pass, B1, B2, B3 of the buffer owners before a neighbour pass. Elements are in
+  // cluster order, so both are prefixes.
+  std::vector<Phase> lay;
+  std::vector<size_t> snap_off, snap_len;
+  size_t per_macro = 0;
+  {
+    for (int r = 0; r < nrec; ++r) nrec_t[r] = h->receivers[r].t.size();
+    size_t seis_need = h->seis_used;
+    plan_macro(h, s0, seis_need, mp);
+    for (int r = 0; r < nrec; ++r) {
+      h->receivers[r].t.resize(nrec_t[r]);
+      h->receivers[r].slot.resize(nrec_t[r]);
+    }
+    for (const Phase& ph : mp.phases) {
+      Phase q = ph;
+      q.s -= s0;
+      lay.push_back(q);
+      const int64_t n = ph.kind == 1 ? h->cbeg[ph.top + 1] : h->cbeg[std::min(ph.top + 2, h->nc)];
+      const size_t len = ph.kind == 1 ? sizeof(float) * n * qs : 3 * sizeof(float) * n * bs;
+      snap_off.push_back(per_macro);
+      snap_len.push_back(len);
+      per_macro += (len + 255) / 256 * 256;
+    }
+  }
+  // The inputs of a whole segment's phases are kept when they fit in half the free device
+  // memory: one forward replay per segment, none for the last one, whose inputs the forward sweep
+  // keeps (5 of 54 ms for 47,040 elements and 64 steps in one segment). Otherwise the segment's macro-boundary states are
+  // kept and each macro step is replayed once more just before its reverse.
+  size_t free_b = 0, total_b = 0;
+  ck(cudaMemGetInfo(&free_b, &total_b), "memory info");
+  const double budget = h->adj_budget ? (double)h->adj_budget : 0.5 * (double)free_b;
+  const bool whole_segment = (double)segm * (double)per_macro <= budget;
+  DevBuf d_snap;
+  if (reverse) d_snap.alloc(whole_segment ? segm * per_macro : per_macro);
+  char* snap = d_snap.get<char>();
+  if (reverse && !whole_segment) d_mac.alloc(sizeof(float) * segm * K * qs);
+  float* mac = d_mac.get<float>();
+  // one macro step of the forward sweep (as advance_steps), its phases' inputs kept in `snap`
+  auto snapshot = [&](size_t pi, const Phase& ph, char* dst) {
+    if (ph.kind == 1) {
+      dcopy(dst, h->dst.Q, snap_len[pi]);
+    } else {
+      const size_t one = snap_len[pi] / 3;
+      dcopy(dst, h->dst.B1, one);
+      dcopy(dst + one, h->dst.B2, one);
+      dcopy(dst + 2 * one, h->dst.B3, one);
+    }
+  };
+  auto keep_macro = [&](int64_t m, char* snap_m) {
+    size_t seis_need = h->seis_used;
+    plan_macro(h, s0 + m * period, seis_need, mp);
+    ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, seis_need * 9 * h->nsim, sizeof(float));
+    ensure_capacity(reinterpret_cast<void**>(&h->d_ritems), &h->ritems_cap, mp.ritems.size(), sizeof(RecvItem));
+    ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, mp.sitems.size(), sizeof(SrcItem));
+    h->seis_used = seis_need;
+    upload_items(h, mp, stream);
+    h->msg_bytes += macro_msg_bytes(h, mp);
+    for (size_t pi = 0; pi < mp.phases.size(); ++pi) {
+      snapshot(pi, mp.phases[pi], snap_m + snap_off[pi]);
+      h->launches += enqueue_phase(h, mp.phases[pi], stream, true, d_tr.get<float>());
+    }
+    ck(cudaGetLastError(), "kernel launch");
+    h->s_now = s0 + (m + 1) * period;
+  };
+  // ---- forward sweep: samples at the macro boundaries, checkpoints
   X.adj_sample(h->dst.Q, qs, nsim, G, relem, rphi, nrec, d_syn.get<float>(), stream);
   for (int64_t m = 0; m < n_macro; ++m) {
     if (reverse && m % every == 0) dcopy(cp + (m / every) * K * qs, h->dst.Q, qbytes);
-    advance_steps(h, period, stream);
+    // the last segment's phase inputs are kept on the way when they all fit: no replay
+    if (reverse && whole_segment && m >= (ncp - 1) * every)
+      keep_macro(m, snap + (m - (ncp - 1) * every) * per_macro);
+    else
+      advance_steps(h, period, stream);
     X.adj_sample(h->dst.Q, qs, nsim, G, relem, rphi, nrec, d_syn.get<float>() + (m + 1) * ns, stream);
   }
   for (int r = 0; r < nrec; ++r) nrec_t[r] = h->receivers[r].t.size();
@@ -1301,32 +1406,6 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   aa.FbT = tabs.FbT;
   aa.qs = qs;
   aa.bufs = bs;
-  MacroPlan mp;
-  // Phase layout of a macro step (the same for every macro step; the step indices are
-  // relative) and the bytes each phase's reverse reads: Q of the active elements before a
-  // predict pass, B1, B2, B3 of the buffer owners before a neighbour pass. Elements are in
-  // cluster order, so both are prefixes.
-  std::vector<Phase> lay;
-  std::vector<size_t> snap_off, snap_len;
-  size_t per_macro = 0;
-  {
-    size_t seis_need = h->seis_used;
-    plan_macro(h, s0, seis_need, mp);
-    for (int r = 0; r < nrec; ++r) {
-      h->receivers[r].t.resize(nrec_t[r]);
-      h->receivers[r].slot.resize(nrec_t[r]);
-    }
-    for (const Phase& ph : mp.phases) {
-      Phase q = ph;
-      q.s -= s0;
-      lay.push_back(q);
-      const int64_t n = ph.kind == 1 ? h->cbeg[ph.top + 1] : h->cbeg[std::min(ph.top + 2, h->nc)];
-      const size_t len = ph.kind == 1 ? sizeof(float) * n * qs : 3 * sizeof(float) * n * bs;
-      snap_off.push_back(per_macro);
-      snap_len.push_back(len);
-      per_macro += (len + 255) / 256 * 256;
-    }
-  }
   auto phase_at = [&](size_t pi, int64_t sb0) {
     Phase q = lay[pi];
     q.s += sb0;
@@ -1401,15 +1480,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
          "upload source items");
     for (size_t pi = 0; pi < mp.phases.size(); ++pi) {
       const Phase& ph = mp.phases[pi];
-      char* dst = snap + snap_off[pi];
-      if (ph.kind == 1) {
-        dcopy(dst, h->dst.Q, snap_len[pi]);
-      } else {
-        const size_t one = snap_len[pi] / 3;
-        dcopy(dst, h->dst.B1, one);
-        dcopy(dst + one, h->dst.B2, one);
-        dcopy(dst + 2 * one, h->dst.B3, one);
-      }
+      snapshot(pi, ph, snap + snap_off[pi]);
       enqueue_phase(h, ph, stream, false, d_tr.get<float>());
     }
     for (int r = 0; r < nrec; ++r) {
@@ -1418,24 +1489,13 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
     }
     h->seis_used = seis_fwd;
   };
-  // The inputs of a whole segment's phases are kept when they fit in half the free device
-  // memory: one forward replay per segment. Otherwise the segment's macro-boundary states are
-  // kept and each macro step is replayed once more just before its reverse.
-  size_t free_b = 0, total_b = 0;
-  ck(cudaMemGetInfo(&free_b, &total_b), "memory info");
-  const double budget = h->adj_budget ? (double)h->adj_budget : 0.5 * (double)free_b;
-  const bool whole_segment = (double)segm * (double)per_macro <= budget;
-  DevBuf d_snap;
-  d_snap.alloc(whole_segment ? segm * per_macro : per_macro);
-  char* snap = d_snap.get<char>();
-  if (!whole_segment) d_mac.alloc(sizeof(float) * segm * K * qs);
-  float* mac = d_mac.get<float>();
   for (int64_t sgi = ncp - 1; sgi >= 0; --sgi) {
     const int64_t m0 = sgi * every, m1 = std::min(m0 + every, n_macro);
     dcopy(h->dst.Q, cp + sgi * K * qs, qbytes);
     h->s_now = s0 + m0 * period;
     if (whole_segment) {
-      for (int64_t m = m0; m < m1; ++m) replay_macro(m, snap + (m - m0) * per_macro);
+      if (sgi + 1 < ncp)
+        for (int64_t m = m0; m < m1; ++m) replay_macro(m, snap + (m - m0) * per_macro);
       for (int64_t m = m1 - 1; m >= m0; --m) reverse_macro(m, snap + (m - m0) * per_macro);
       continue;
     }
@@ -1458,21 +1518,18 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   if (nsrc > 0)
     ck(cudaMemcpyAsync(h->adj_src_grad.data(), d_sg.p, sizeof(double) * nsrc * 6, cudaMemcpyDeviceToHost, stream),
        "source gradient");
-  std::vector<float> lq;
-  if (dq0) {
-    lq.resize((size_t)K * nsim * NB9);
-    ck(cudaMemcpyAsync(lq.data(), d_lq.p, sizeof(float) * lq.size(), cudaMemcpyDeviceToHost, stream), "adjoint state");
+  if (dq0) {   // [sim][element (original order)][9][B] in FP64, staged in the buffer adjoints (12 bytes a value)
+    const int64_t total = (int64_t)K * nsim * NB9;
+    k_adjoint_to_caller<<<(unsigned)std::min<int64_t>((total + 255) / 256, 16 * (int64_t)h->num_sms), 256, 0, stream>>>(
+        d_lq.get<float>(), d_lb.get<double>(), h->d_iperm, K, nsim, NB9);
+    ck(cudaGetLastError(), "adjoint state");
+    ck(cudaMemcpyAsync(dq0, d_lb.p, sizeof(double) * total, cudaMemcpyDeviceToHost, stream), "adjoint state");
   }
   ck(cudaStreamSynchronize(stream), "synchronize");
   check_device_error(h);
   if (misfit) *misfit = J;
   if (synth_out)
     for (size_t q = 0; q < syn.size(); ++q) synth_out[q] = syn[q];
-  if (dq0)   // [sim][element (original order)][9][B]
-    for (int f = 0; f < nsim; ++f)
-      for (int64_t k = 0; k < K; ++k)
-        for (int q = 0; q < NB9; ++q)
-          dq0[((size_t)f * K + k) * NB9 + q] = lq[((size_t)h->iperm[k] * nsim + f) * NB9 + q];
   if (grad) contract_gradient(geo, d_w.get<double>(), grad, stream);
 }
 

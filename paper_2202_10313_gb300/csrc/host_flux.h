@@ -100,20 +100,53 @@ LTS_HD void face_flux_matrix(const double n[3], const T c[8], T lam, T mu, T rin
   }
 }
 
-// sum_{q,j} M[q][j] W[q*9 + j] of that matrix, column by column (no 9 x 9 storage).
-template <typename T>
-LTS_HD T face_flux_dot(const double n[3], const T c[8], T lam, T mu, T rinv, const double* W) {
-  T acc(0.0);
+// The contraction sum_{q,j} M[q][j] W[q*9 + j] of that matrix as a form in its coefficients: the flux
+// is linear in (lam, mu, rinv) and in w, and w in the coefficients, so twelve sums over W (of
+// the normal alone, out[12]) hold everything that does not depend on the material:
+//   lam (c0 P0 + c1 P1 + c4 P2 + c5 P3) + mu (c0 Q0 + ..) + rinv (c2 R0 + c3 R1 + c6 R2 + c7 R3).
+LTS_HD inline void face_flux_forms(const double n[3], const double* W, double out[12]) {
+  // L[k][j]: the vector whose product with w's velocity (k = 0: lam, 1: mu) or traction part
+  // (k = 2: rinv) is the contraction of column j
+  double X[3][3][3], V[3][3][3];   // [k][a][b]: sum over stress columns tau_j[a] L_j[b]; velocity columns L_{6+a}[b]
+  for (int k = 0; k < 3; ++k)
+    for (int a = 0; a < 3; ++a)
+      for (int b = 0; b < 3; ++b) X[k][a][b] = 0.0;
+  const double tau[6][3] = {{n[0], 0, 0}, {0, n[1], 0}, {0, 0, n[2]}, {n[1], n[0], 0}, {0, n[2], n[1]}, {n[2], 0, n[0]}};
   for (int j = 0; j < 9; ++j) {
-    T g[9], S[9];
-    for (int q = 0; q < 9; ++q) {
-      g[q] = T(q == j ? 1.0 : 0.0);
-      S[q] = T(0.0);
-    }
-    face_flux_apply(g, n, c, lam, mu, rinv, S);
-    for (int q = 0; q < 9; ++q) acc = acc + S[q] * W[q * 9 + j];
+    const double s0 = W[j], s1 = W[9 + j], s2 = W[18 + j], s3 = W[27 + j], s4 = W[36 + j], s5 = W[45 + j];
+    const double tr = s0 + s1 + s2;
+    const double L[3][3] = {{-n[0] * tr, -n[1] * tr, -n[2] * tr},
+                            {-(2.0 * n[0] * s0 + n[1] * s3 + n[2] * s5), -(2.0 * n[1] * s1 + n[0] * s3 + n[2] * s4),
+                             -(2.0 * n[2] * s2 + n[1] * s4 + n[0] * s5)},
+                            {-W[54 + j], -W[63 + j], -W[72 + j]}};
+    for (int k = 0; k < 3; ++k)
+      for (int b = 0; b < 3; ++b) {
+        if (j >= 6)
+          V[k][j - 6][b] = L[k][b];
+        else
+          for (int a = 0; a < 3; ++a) X[k][a][b] += tau[j][a] * L[k][b];
+      }
   }
-  return acc;
+  for (int k = 0; k < 3; ++k) {
+    double nv = 0.0, nx = 0.0;
+    for (int a = 0; a < 3; ++a)
+      for (int b = 0; b < 3; ++b) {
+        nv += n[a] * n[b] * V[k][a][b];
+        nx += n[a] * n[b] * X[k][a][b];
+      }
+    const double tv = V[k][0][0] + V[k][1][1] + V[k][2][2] - nv, tx = X[k][0][0] + X[k][1][1] + X[k][2][2] - nx;
+    double* o = out + 4 * k;
+    o[0] = k < 2 ? nv : nx;
+    o[1] = k < 2 ? nx : nv;
+    o[2] = k < 2 ? tv : tx;
+    o[3] = k < 2 ? tx : tv;
+  }
+}
+template <typename T>
+LTS_HD T face_flux_dot(const T c[8], T lam, T mu, T rinv, const double f[12]) {
+  return lam * (c[0] * f[0] + c[1] * f[1] + c[4] * f[2] + c[5] * f[3]) +
+         mu * (c[0] * f[4] + c[1] * f[5] + c[4] * f[6] + c[5] * f[7]) +
+         rinv * (c[2] * f[8] + c[3] * f[9] + c[6] * f[10] + c[7] * f[11]);
 }
 
 // Voigt index of the stress component (i, d).

@@ -175,7 +175,7 @@ struct Impl {
   }
   static void adj_source(float* lam, int nsim, const int* elem, const float* phi, const float* res, int nrec,
                          cudaStream_t st) {
-    k_adj_source<O><<<1, 64, 0, st>>>(lam, nsim, elem, phi, res, nrec);
+    k_adj_source<O><<<nsim, rup(3 * C::B, 32), 0, st>>>(lam, nsim, elem, phi, res, nrec);
   }
   static void adj_src_grad(const float* lam, int nsim, const SrcItem* items, const double* c, int n,
                            const float* phi, double* g, cudaStream_t st) {
