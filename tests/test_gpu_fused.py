@@ -165,3 +165,30 @@ def test_maximum_fused_count():
         one = s.get_dofs()
         s.close()
         assert np.sqrt(np.sum((got[f] - one) ** 2)) / np.sqrt(np.sum(one ** 2)) <= 1e-6, f
+
+
+@pytest.mark.parametrize("order,n_mech", [(3, 3), (4, 0), (4, 3), (5, 0), (5, 3)])
+def test_twelve_fused_simulations_equal_their_single_runs_bitwise(order, n_mech):
+    """Batches of the sparse engine that straddle elements (12 simulations, 16 slots) and a last
+    batch that is not full, three clusters (every buffer relation): each simulation bitwise equal
+    to its own single run, whose batches hold 16 and 5 elements (162 elements)."""
+    m = synth.permute_vertex_order(synth.graded_box(3, 3, 3, 250.0, 125.0, seed=12), seed=2)
+    mat = synth.random_layers(m, n_layers=3, seed=5)
+    K, F = m["tet"].shape[0], 12
+    assert K * F % 16 and K % 16 and K % 5
+    nq, nb = 9 + 6 * n_mech, order * (order + 1) * (order + 2) // 6
+    d0 = np.stack([synth.random_dofs(K, nq, nb, seed=30 + f) for f in range(F)])
+    q = {}
+    for sims in ([F], [1] * 3):
+        for i, n in enumerate(sims):
+            s = binding.Solver(order, n_mech, device=0, n_fused=n)
+            s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+            s.set_material(mat["rho"], mat["vp"], mat["vs"], *((mat["qp"], mat["qs"]) if n_mech else ()))
+            s.setup_clusters(3, 0.5)
+            f = [0, 5, 11][i]
+            s.set_dofs(d0 if n > 1 else d0[f])
+            s.advance_steps(8)
+            q[n, f] = s.get_dofs()
+            s.close()
+    for f in (0, 5, 11):
+        assert np.array_equal(q[F, 0][f], q[1, f]), f
