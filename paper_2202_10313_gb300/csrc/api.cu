@@ -1045,12 +1045,11 @@ void make_adj_tables(const lts_solver* h, AdjTables& T) {
   T.FbT = base + (fbt - kt);
 }
 
-// Material gradient from the correlations W (device, [internal element][AM_SIZE]): dJ/dp =
-// sum <dM/dp, W> over the element's star matrices and face operators and over the operators
-// of the neighbours' faces that look at it (they depend on this element's material through
-// the Riemann state). One thread per element (original order); the derivatives are exact,
-// by forward-mode dual numbers through the same closed forms the forward set-up evaluates
-// (host_flux.h), contracted with W without forming the 9 x 9 matrices.
+// Material gradient from the sums W (device, [internal element][WG_SIZE]): dJ/dp over the
+// element's star matrices and face operators and over the operators of the neighbours' faces
+// that look at it (they depend on this element's material through the Riemann state). The
+// derivatives are exact, by forward-mode dual numbers through the same closed forms the
+// forward set-up evaluates (host_flux.h).
 struct GradGeom {
   const double *jinv, *normal, *area, *detJ, *rho, *lam, *mu, *W;
   const int *bc, *nbr, *nbr_face;
@@ -1060,22 +1059,20 @@ struct GradGeom {
 
 // Derivatives of one face's contraction (own and neighbour state operators with their
 // correlations) with respect to the element's rho, lam, mu and the neighbour's: out[4 k + face][6].
-// One thread per (element, face). The correlations enter as twelve sums each (face_flux_forms), so
-// that the six derivatives cost six evaluations of the coefficients' closed forms; contracting
-// column by column for each took 6.5 of 7.5 ms (47,040 elements), bound by the FP64 rate.
+// One thread per (element, face). The correlations enter as ten sums each, so that the six
+// derivatives cost six evaluations of the coefficients' closed forms; contracting 9 x 9
+// correlations column by column for each took 6.5 of 7.5 ms (47,040 elements), bound by the
+// FP64 rate.
 __global__ void k_grad_faces(GradGeom g, double* out) {
   using lts::Dual;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * g.K) return;
   const long long k = t / 4;
   const int face = (int)(t % 4);
-  const double* Wk = g.W + (size_t)g.iperm[k] * ltsdev::AM_SIZE;
-  const double* n = g.normal + 12 * k + 3 * face;
+  const double* Wk = g.W + (size_t)g.iperm[k] * ltsdev::WG_SIZE;
   const int bc = g.bc[t];
   const long long nb = g.nbr[t];
-  double fl[12], fn[12];
-  lts::face_flux_forms(n, Wk + ltsdev::AM_LOC + face * 81, fl);
-  lts::face_flux_forms(n, Wk + ltsdev::AM_NBR + face * 81, fn);
+  const double *fl = Wk + ltsdev::WG_LOC + 10 * face, *fn = Wk + ltsdev::WG_NBR + 10 * face;
   const Dual scale(-2.0 * g.area[t] / g.detJ[k]);
   for (int p = 0; p < 6; ++p) {
     if (p >= 3 && nb < 0) {
@@ -1104,15 +1101,15 @@ __global__ void k_grad_faces(GradGeom g, double* out) {
   }
 }
 
-// The gradient: star matrices' part and the sums of the faces' derivatives in a fixed order.
+// The gradient: star matrices' part (linear in lam, mu and 1/rho) and the sums of the faces'
+// derivatives in a fixed order.
 __global__ void k_grad_contract(GradGeom g, const double* faces, double* grad) {
-  using lts::Dual;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= g.K) return;
-  const double* We = g.W + (size_t)g.iperm[e] * ltsdev::AM_SIZE;
+  const double* ws = g.W + (size_t)g.iperm[e] * ltsdev::WG_SIZE + ltsdev::WG_STAR;
+  const double star[3] = {-ws[2] / (g.rho[e] * g.rho[e]), ws[0], ws[1]};
   for (int p = 0; p < 3; ++p) {
-    const Dual rho(g.rho[e], p == 0 ? 1.0 : 0.0), lam(g.lam[e], p == 1 ? 1.0 : 0.0), mu(g.mu[e], p == 2 ? 1.0 : 0.0);
-    double acc = lts::star_dot<Dual>(g.jinv + 9 * e, lam, mu, Dual(1.0) / rho, We + ltsdev::AM_STAR).d;
+    double acc = star[p];
     for (int i = 0; i < 4; ++i) {
       acc += faces[6 * (4 * e + i) + p];
       const long long nb = g.nbr[4 * e + i];
@@ -1122,10 +1119,10 @@ __global__ void k_grad_contract(GradGeom g, const double* faces, double* grad) {
   }
 }
 
-// Explicit 9 x 9 operators of every element in FP32 (internal order): the star matrices S_c
-// and, per face, the flux solvers A- (interior state) and A+ (exterior state), from the
-// closed forms of the forward set-up (host_flux.h) evaluated in FP64. One thread per
-// (element, task): task 0 the star matrices, task 1 + i face i.
+// Operators of every element in FP32 (internal order): geometry and material (the star
+// matrices) and, per face, the 9 x 9 flux solvers A- (interior state) and A+ (exterior state),
+// from the closed forms of the forward set-up (host_flux.h) evaluated in FP64. One thread per
+// (element, task): task 0 the geometry, task 1 + i face i.
 __global__ void k_build_amat(GradGeom g, float* amat) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 5 * g.K) return;
@@ -1134,10 +1131,12 @@ __global__ void k_build_amat(GradGeom g, float* amat) {
   float* out = amat + (size_t)g.iperm[k] * ltsdev::AM_SIZE;
   const double rho = g.rho[k], lam = g.lam[k], mu = g.mu[k], rinv = 1.0 / rho;
   if (task == 0) {
-    double S[3][81];
-    lts::star_matrices_t<double>(g.jinv + 9 * k, lam, mu, rinv, S);
-    for (int c = 0; c < 3; ++c)
-      for (int q = 0; q < 81; ++q) out[ltsdev::AM_STAR + c * 81 + q] = (float)S[c][q];
+    out += ltsdev::AM_GEO;
+    for (int q = 0; q < 9; ++q) out[q] = (float)g.jinv[9 * k + q];
+    out[9] = (float)lam;
+    out[10] = (float)mu;
+    out[11] = (float)rinv;
+    for (int q = 0; q < 12; ++q) out[12 + q] = (float)g.normal[12 * k + q];
     return;
   }
   const int i = task - 1;
@@ -1262,7 +1261,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
     d_res.alloc(sizeof(float) * (n_macro + 1) * ns);
     d_lq.alloc(sizeof(float) * K * nsim * NB9);
     d_lb.alloc(sizeof(float) * 3 * K * nsim * NB9);
-    d_w.alloc(sizeof(double) * K * ltsdev::AM_SIZE);
+    d_w.alloc(sizeof(double) * K * ltsdev::WG_SIZE);
     d_cp.alloc(sizeof(float) * ncp * K * qs);
     d_qn.alloc(sizeof(float) * K * qs);
     // the replays write the LTS buffers as modes for the reverse sweep; the sparse engine's face
@@ -1385,7 +1384,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   // ---- reverse sweep
   ck(cudaMemsetAsync(d_lq.p, 0, sizeof(float) * K * nsim * NB9, stream), "memset");
   ck(cudaMemsetAsync(d_lb.p, 0, sizeof(float) * 3 * K * nsim * NB9, stream), "memset");
-  ck(cudaMemsetAsync(d_w.p, 0, sizeof(double) * K * ltsdev::AM_SIZE, stream), "memset");
+  ck(cudaMemsetAsync(d_w.p, 0, sizeof(double) * K * ltsdev::WG_SIZE, stream), "memset");
   ck(cudaMemsetAsync(d_sg.p, 0, sizeof(double) * std::max(nsrc, 1) * 6, stream), "memset");
   X.adj_source(d_lq.get<float>(), nsim, relem, rphi, d_res.get<float>() + n_macro * ns, nrec, stream);
   ltsdev::AdjLtsArgs aa{};

@@ -100,102 +100,14 @@ LTS_HD void face_flux_matrix(const double n[3], const T c[8], T lam, T mu, T rin
   }
 }
 
-// The contraction sum_{q,j} M[q][j] W[q*9 + j] of that matrix as a form in its coefficients: the flux
-// is linear in (lam, mu, rinv) and in w, and w in the coefficients, so twelve sums over W (of
-// the normal alone, out[12]) hold everything that does not depend on the material:
-//   lam (c0 P0 + c1 P1 + c4 P2 + c5 P3) + mu (c0 Q0 + ..) + rinv (c2 R0 + c3 R1 + c6 R2 + c7 R3).
-LTS_HD inline void face_flux_forms(const double n[3], const double* W, double out[12]) {
-  // L[k][j]: the vector whose product with w's velocity (k = 0: lam, 1: mu) or traction part
-  // (k = 2: rinv) is the contraction of column j
-  double X[3][3][3], V[3][3][3];   // [k][a][b]: sum over stress columns tau_j[a] L_j[b]; velocity columns L_{6+a}[b]
-  for (int k = 0; k < 3; ++k)
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) X[k][a][b] = 0.0;
-  const double tau[6][3] = {{n[0], 0, 0}, {0, n[1], 0}, {0, 0, n[2]}, {n[1], n[0], 0}, {0, n[2], n[1]}, {n[2], 0, n[0]}};
-  for (int j = 0; j < 9; ++j) {
-    const double s0 = W[j], s1 = W[9 + j], s2 = W[18 + j], s3 = W[27 + j], s4 = W[36 + j], s5 = W[45 + j];
-    const double tr = s0 + s1 + s2;
-    const double L[3][3] = {{-n[0] * tr, -n[1] * tr, -n[2] * tr},
-                            {-(2.0 * n[0] * s0 + n[1] * s3 + n[2] * s5), -(2.0 * n[1] * s1 + n[0] * s3 + n[2] * s4),
-                             -(2.0 * n[2] * s2 + n[1] * s4 + n[0] * s5)},
-                            {-W[54 + j], -W[63 + j], -W[72 + j]}};
-    for (int k = 0; k < 3; ++k)
-      for (int b = 0; b < 3; ++b) {
-        if (j >= 6)
-          V[k][j - 6][b] = L[k][b];
-        else
-          for (int a = 0; a < 3; ++a) X[k][a][b] += tau[j][a] * L[k][b];
-      }
-  }
-  for (int k = 0; k < 3; ++k) {
-    double nv = 0.0, nx = 0.0;
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        nv += n[a] * n[b] * V[k][a][b];
-        nx += n[a] * n[b] * X[k][a][b];
-      }
-    const double tv = V[k][0][0] + V[k][1][1] + V[k][2][2] - nv, tx = X[k][0][0] + X[k][1][1] + X[k][2][2] - nx;
-    double* o = out + 4 * k;
-    o[0] = k < 2 ? nv : nx;
-    o[1] = k < 2 ? nx : nv;
-    o[2] = k < 2 ? tv : tx;
-    o[3] = k < 2 ? tx : tv;
-  }
-}
+// The contraction sum_{q,j} M[q][j] l[q] x[j] of that matrix as a form in its coefficients: the
+// flux is linear in (lam, mu, rinv) and in (v*, t*), and those in the coefficients, so ten sums f
+// of (l, x) and the normal alone hold everything that does not depend on the material
+// (ltsdev::face_products; the tangential coefficients do not meet lam, n v*_T = 0).
 template <typename T>
-LTS_HD T face_flux_dot(const T c[8], T lam, T mu, T rinv, const double f[12]) {
-  return lam * (c[0] * f[0] + c[1] * f[1] + c[4] * f[2] + c[5] * f[3]) +
-         mu * (c[0] * f[4] + c[1] * f[5] + c[4] * f[6] + c[5] * f[7]) +
-         rinv * (c[2] * f[8] + c[3] * f[9] + c[6] * f[10] + c[7] * f[11]);
-}
-
-// Voigt index of the stress component (i, d).
-LTS_HD inline int voigt(int i, int d) {
-  return i == d ? i : ((i + d == 1) ? 3 : ((i + d == 3) ? 4 : 5));
-}
-
-// The terms of the star matrices (below), each handed to add(c, out * 9 + in, term); an
-// entry may receive several terms.
-template <typename T, typename Add>
-LTS_HD void star_terms_t(const double jinv[9], T lam, T mu, T rinv, Add&& add) {
-  for (int c = 0; c < 3; ++c) {
-    // stress rows from the velocity gradient g[d][j] = sum_c jinv[c][d] Y_c[6+j]
-    for (int d = 0; d < 3; ++d)
-      for (int j = 0; j < 3; ++j) {
-        const double w = jinv[c * 3 + d];     // dg[d][j] / dY_c[6+j]
-        const int col = 6 + j;
-        // tr = g00 + g11 + g22
-        if (d == j) {
-          for (int a = 0; a < 3; ++a) add(c, a * 9 + col, lam * w);
-          add(c, d * 9 + col, T(2.0) * mu * w);
-        } else {
-          // out[3] = mu (g01 + g10), out[4] = mu (g12 + g21), out[5] = mu (g02 + g20)
-          add(c, voigt(d, j) * 9 + col, mu * w);
-        }
-      }
-    // velocity rows: rinv * sum_d jinv[c][d] Y_c[SIG[i][d]]
-    for (int i = 0; i < 3; ++i)
-      for (int d = 0; d < 3; ++d) add(c, (6 + i) * 9 + voigt(i, d), rinv * jinv[c * 3 + d]);
-  }
-}
-
-// Star matrices S_c (row-major [out][in]) of the time kernel's map D_{d+1} = sum_c S_c Y_c,
-// Y_c = D_d K_c^T (the forward kernels' star_apply: physical velocity gradient W_d =
-// sum_c dxi_c/dx_d Y_c, Hooke's law on the stress rows, stress divergence / rho on the
-// velocity rows). jinv[c*3+d] = dxi_c/dx_d.
-template <typename T>
-LTS_HD void star_matrices_t(const double jinv[9], T lam, T mu, T rinv, T S[3][81]) {
-  for (int c = 0; c < 3; ++c)
-    for (int q = 0; q < 81; ++q) S[c][q] = T(0.0);
-  star_terms_t<T>(jinv, lam, mu, rinv, [&](int c, int q, T v) { S[c][q] = S[c][q] + v; });
-}
-
-// sum_c sum_q S_c[q] W[c*81 + q] of the star matrices.
-template <typename T>
-LTS_HD T star_dot(const double jinv[9], T lam, T mu, T rinv, const double* W) {
-  T acc(0.0);
-  star_terms_t<T>(jinv, lam, mu, rinv, [&](int c, int q, T v) { acc = acc + v * W[c * 81 + q]; });
-  return acc;
+LTS_HD T face_flux_dot(const T c[8], T lam, T mu, T rinv, const double f[10]) {
+  return lam * (c[0] * f[0] + c[1] * f[1]) + mu * (c[0] * f[2] + c[1] * f[3] + c[4] * f[4] + c[5] * f[5]) +
+         rinv * (c[2] * f[6] + c[3] * f[7] + c[6] * f[8] + c[7] * f[9]);
 }
 
 // Forward-mode dual number with one derivative component.

@@ -10,22 +10,35 @@
 //   mu = dJ/dT = -sum_c S_c^T lambda K_c^T + sum_i ((A-_i^T lambda) F^_i^T) F~_i^T
 //        + the adjoints of the buffers the step wrote,
 //   G_{O-1} = c_{O-1} mu, G_d = c_d mu + sum_c S_c^T G_{d+1} K_c,   dJ/dQ = lambda + G_0,
-// the transposed neighbour fluxes into the adjoints of the buffers they read, and the
-// per-element correlations that the material derivatives of S_c, A-_i, A+_i are contracted
-// with once the loop is done:
-//   W_c  += sum_{d<O-1} G_{d+1} (D_d K_c^T)^T - lambda (T K_c)^T,
-//   W-_i += lambda (T F~_i F^_i)^T,   W+_i += lambda_k (X F-_{j,h} F^_i)^T.
-// The matrices are explicit (FP32, built on the host from the same closed forms as the
-// forward kernels' star and flux code); CUDA cores.
+// the transposed neighbour fluxes into the adjoints of the buffers they read, and, for the
+// material derivatives, what is left of the correlations
+//   W_c  = sum_{d<O-1} G_{d+1} (D_d K_c^T)^T - lambda (T K_c)^T,
+//   W-_i = lambda (T F~_i F^_i)^T,   W+_i = lambda_k (X F-_{j,h} F^_i)^T
+// of S_c, A-_i, A+_i once they are contracted with everything that does not depend on the
+// material: the matrices are linear in (lambda_e, mu_e, 1/rho_e) (star matrices, three sums)
+// and in their products with the eight Riemann coefficients (flux solvers, ten sums a face
+// and side, face_products). Each sum is a scalar product per (face) mode, so the threads
+// that hold the columns form it: the 3 x 3 tiles of the 9 x 9 correlations cost k_adj_pred_sp
+// a pass over shared memory per derivative and 567 FP64 additions per element (204 us a launch,
+// 126 with the sums; 47,040 elements, order 4), k_adj_nbr another 324.
+// The flux solvers are explicit (FP32, from the same closed forms as the forward kernels'
+// flux code), the star matrices are applied by their physical form; CUDA cores.
 #pragma once
 #include "kernels.cuh"
 
 namespace ltsdev {
 
-constexpr int AM_STAR = 0;       // S_c, c = 0..2: [out][in]
-constexpr int AM_LOC = 243;      // A-_i, i = 0..3
-constexpr int AM_NBR = 567;      // A+_i, i = 0..3
-constexpr int AM_SIZE = 891;     // floats per element (also the size of the correlations W)
+// operators of an element (floats)
+constexpr int AM_LOC = 0;        // A-_i, i = 0..3: [out][in]
+constexpr int AM_NBR = 324;      // A+_i, i = 0..3
+constexpr int AM_GEO = 648;      // dxi_c/dx_d at 3 c + d, lambda, mu, 1/rho, the four unit normals
+constexpr int AM_NGEO = 24;
+constexpr int AM_SIZE = AM_GEO + AM_NGEO;
+// material sums of an element (doubles)
+constexpr int WG_STAR = 0;       // of lambda, mu, 1/rho
+constexpr int WG_LOC = 3;        // A-_i: ten sums a face (face_products)
+constexpr int WG_NBR = 43;       // A+_i
+constexpr int WG_SIZE = 83;
 
 // Threads per element group: one warp up to order 4, two at order 5 (every phase needs at
 // least one thread per mode column).
@@ -38,20 +51,6 @@ struct AdjNT {
 // consecutive threads on consecutive entries:
 //   KT[c][j][i] = K[c][i][j],  FtT[i][f][b] = F~_i[b][f],  FhT[i][b][f] = F^_i[f][b],
 //   FbT[jh][f][b] = F-_{jh}[b][f].
-// v[r] = sum_{j < N} src[r * LD + j] * tab[j * ts + t] for the 9 rows r: each table entry is
-// loaded once and the rows accumulate in registers.
-template <int N, int LD>
-__device__ __forceinline__ void rows9(const float* src, const float* __restrict__ tab, int ts, int t, float v[9]) {
-#pragma unroll
-  for (int r = 0; r < 9; ++r) v[r] = 0.f;
-#pragma unroll 4
-  for (int j = 0; j < N; ++j) {
-    const float w = __ldg(tab + j * ts + t);
-#pragma unroll
-    for (int r = 0; r < 9; ++r) v[r] = fmaf(src[r * LD + j], w, v[r]);
-  }
-}
-
 // Velocity at the receivers from Q^n: out[f][r][q] = sum_b Q_f[elem_r][6+q][b] phi_r[b] for
 // the nsim simulations of an (elastic) state in groups of G (simulation f of element k, row
 // q, mode b at k qs + (f / G) 9 B G + (q B + b) G + f % G; G = 1 for one simulation).
@@ -121,14 +120,14 @@ struct AdjLtsArgs {
   const int* owners;                  // neighbour reverse: the pass's buffer owners with an active
                                       // receiver (one CTA each), or null: owner = CTA index
   const int* meta;
-  double* W;                          // [K][AM_SIZE], per-pass sums in FP32 added in FP64
+  double* W;                          // [K][WG_SIZE], per-pass sums in FP32 added in FP64
   const float *KT, *FtT, *FhT, *FbT;  // transposed operator tables (see AdjTables)
   long long qs, bufs;
   int end;                            // active elements [0, end)
   // simulations of a fused run, in groups of G in the state and buffer snapshots (element k,
   // simulation f, row r, mode b at k qs + (f / G) 9 B G + (r B + b) G + f % G; one
   // simulation: nsim = G = 1); the adjoints are [element][simulation][9][B] and W sums the
-  // simulations' correlations
+  // simulations
   int nsim, G;
 };
 
@@ -146,48 +145,6 @@ __device__ __forceinline__ void stage(float* dst, const float* __restrict__ src,
     if (t + j * NT < N) dst[t + j * NT] = v[j];
 }
 
-// acc[i][j] += sum_{j' < n} X[(r0 + i) * LD + j'] * Y[(s0 + j) * LD + j'] for a 3 x 3 tile.
-template <int LD>
-__device__ __forceinline__ void tile33(const float* X, const float* Y, int r0, int s0, int n, float acc[3][3]) {
-  for (int j = 0; j < n; ++j) {
-    float x[3], y[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      x[i] = X[(r0 + i) * LD + j];
-      y[i] = Y[(s0 + i) * LD + j];
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) acc[i][q] = fmaf(x[i], y[q], acc[i][q]);
-  }
-}
-
-// acc[i][q] += sum_{j < n} X[(r0 + i) * LD + j] * Y[(s0 + q) * LD + j] for a 3 x 3 tile, four
-// j at a time (LD and n multiples of 4, X and Y 16-byte aligned; entries j >= the true length
-// are zero on one side at least).
-template <int LD>
-__device__ __forceinline__ void tile33v(const float* X, const float* Y, int r0, int s0, int n, float acc[3][3]) {
-#pragma unroll 1
-  for (int j = 0; j < n; j += 4) {
-    float4 x[3], y[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      x[i] = *reinterpret_cast<const float4*>(X + (r0 + i) * LD + j);
-      y[i] = *reinterpret_cast<const float4*>(Y + (s0 + i) * LD + j);
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        acc[i][q] = fmaf(x[i].x, y[q].x, acc[i][q]);
-        acc[i][q] = fmaf(x[i].y, y[q].y, acc[i][q]);
-        acc[i][q] = fmaf(x[i].z, y[q].z, acc[i][q]);
-        acc[i][q] = fmaf(x[i].w, y[q].w, acc[i][q]);
-      }
-  }
-}
-
 // The nine rows of a [9][LD] block, entries j .. j + 3 (16-byte aligned; the same address in
 // every lane, so each load is one broadcast).
 template <int LD>
@@ -198,61 +155,159 @@ __device__ __forceinline__ void load_cols4(const float* src, int j, float4 x[9])
 __device__ __forceinline__ float lane4(const float4& v, int u) { return u == 0 ? v.x : u == 1 ? v.y : u == 2 ? v.z : v.w; }
 
 // v[r] = sum_{j < N} src[r * LD + j] * tab[j * ts + t] for the 9 rows r, the broadcast
-// operand four entries at a time (N, LD multiples of 4; pad entries zero on one side).
-template <int N, int LD>
+// operand four entries at a time (LD = rup(N, 4), pad entries of src zero; the table is not
+// read past row NT - 1, so that it needs no pad rows).
+template <int NT, int LD>
 __device__ __forceinline__ void rows9v(const float* src, const float* tab, int ts, int t, float v[9]) {
 #pragma unroll
   for (int r = 0; r < 9; ++r) v[r] = 0.f;
 #pragma unroll 1
-  for (int j = 0; j < N; j += 4) {
+  for (int j = 0; j < LD; j += 4) {
     float4 x[9];
     load_cols4<LD>(src, j, x);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const float w = tab[(j + u) * ts + t];
+      const int ju = NT % 4 == 0 ? j + u : min(j + u, NT - 1);
+      const float w = tab[ju * ts + t];
 #pragma unroll
       for (int r = 0; r < 9; ++r) v[r] = fmaf(lane4(x[r], u), w, v[r]);
     }
   }
 }
 
-// Elastic star matrix S_c (row-major [out][in]) in compact form: it couples the six stresses
-// only to the three velocities and back, so only the 6 x 3 block S[r][6 + s] (row-major, 18
-// entries) and the 3 x 6 block S[6 + r][s] (18 entries) are kept, 36 floats per c.
-__device__ __forceinline__ int star_compact_index(int x) {
-  return x < 18 ? (x / 3) * 9 + 6 + x % 3 : (6 + (x - 18) / 6) * 9 + (x - 18) % 6;
+// Geometry and material of an element (AM_GEO) for the star matrices, 16-byte aligned.
+struct StarGeo {
+  float J[9], lam, mu, rinv;
+  __device__ __forceinline__ explicit StarGeo(const float* p) {
+    const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1],
+                 c = reinterpret_cast<const float4*>(p)[2];
+    J[0] = a.x; J[1] = a.y; J[2] = a.z; J[3] = a.w;
+    J[4] = b.x; J[5] = b.y; J[6] = b.z; J[7] = b.w;
+    J[8] = c.x; lam = c.y; mu = c.z; rinv = c.w;
+  }
+};
+// v = sum_c S_c y_c: the physical velocity gradient and stress divergence of the three
+// direction products, then Hooke's law and 1/rho (about 70 multiply-adds and three 16-byte
+// loads; the matrices' nonzero entries take 108 and 27).
+struct StarFwd {
+  float g[9], dv[3];   // g[3 d + j] = d v_j / d x_d
+  __device__ __forceinline__ StarFwd() {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = 0.f;
+    dv[0] = dv[1] = dv[2] = 0.f;
+  }
+  __device__ __forceinline__ void add(const float J[3], const float y[9]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) g[3 * d + j] = fmaf(J[d], y[6 + j], g[3 * d + j]);
+    dv[0] = fmaf(J[0], y[0], fmaf(J[1], y[3], fmaf(J[2], y[5], dv[0])));
+    dv[1] = fmaf(J[0], y[3], fmaf(J[1], y[1], fmaf(J[2], y[4], dv[1])));
+    dv[2] = fmaf(J[0], y[5], fmaf(J[1], y[4], fmaf(J[2], y[2], dv[2])));
+  }
+  __device__ __forceinline__ void get(const StarGeo& s, float v[9]) const {
+    const float l = s.lam * (g[0] + g[4] + g[8]), m2 = 2.f * s.mu;
+    v[0] = fmaf(m2, g[0], l);
+    v[1] = fmaf(m2, g[4], l);
+    v[2] = fmaf(m2, g[8], l);
+    v[3] = s.mu * (g[1] + g[3]);
+    v[4] = s.mu * (g[5] + g[7]);
+    v[5] = s.mu * (g[2] + g[6]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[6 + i] = s.rinv * dv[i];
+  }
+};
+// w = sum_c S_c^T z_c and its share in the sums of lambda, mu and 1/rho against the column x
+// (x^T sum_c (dS_c/dp)^T z_c): the parts of w before the material enters.
+struct StarRev {
+  float a[3], p[3], q[6];   // w_v = lambda a + mu p, w_sigma = q / rho
+  __device__ __forceinline__ StarRev() {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) a[i] = p[i] = q[i] = q[3 + i] = 0.f;
+  }
+  __device__ __forceinline__ void add(const float J[3], const float z[9]) {
+    const float tr = z[0] + z[1] + z[2];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) a[j] = fmaf(J[j], tr, a[j]);
+    p[0] = fmaf(J[0], 2.f * z[0], fmaf(J[1], z[3], fmaf(J[2], z[5], p[0])));
+    p[1] = fmaf(J[1], 2.f * z[1], fmaf(J[0], z[3], fmaf(J[2], z[4], p[1])));
+    p[2] = fmaf(J[2], 2.f * z[2], fmaf(J[1], z[4], fmaf(J[0], z[5], p[2])));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) q[d] = fmaf(J[d], z[6 + d], q[d]);
+    q[3] = fmaf(J[1], z[6], fmaf(J[0], z[7], q[3]));
+    q[4] = fmaf(J[2], z[7], fmaf(J[1], z[8], q[4]));
+    q[5] = fmaf(J[2], z[6], fmaf(J[0], z[8], q[5]));
+  }
+  __device__ __forceinline__ void get(const StarGeo& s, float w[9]) const {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = s.rinv * q[i];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) w[6 + j] = fmaf(s.lam, a[j], s.mu * p[j]);
+  }
+  __device__ __forceinline__ void sums(const float x[9], float sgn, float f[3]) const {
+    float l = 0.f, m = 0.f, r = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      l = fmaf(a[j], x[6 + j], l);
+      m = fmaf(p[j], x[6 + j], m);
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) r = fmaf(q[i], x[i], r);
+    f[0] = fmaf(sgn, l, f[0]);
+    f[1] = fmaf(sgn, m, f[1]);
+    f[2] = fmaf(sgn, r, f[2]);
+  }
+};
+
+// u = A^T l, A a 9 x 9 flux solver with rows padded to 12 (16-byte aligned).
+__device__ __forceinline__ void flux_transposed(const float* Am, const float l[9], float u[9]) {
+#pragma unroll
+  for (int r = 0; r < 9; ++r) u[r] = 0.f;
+#pragma unroll
+  for (int s = 0; s < 9; ++s) {
+    const float4 a0 = *reinterpret_cast<const float4*>(Am + s * 12);
+    const float4 a1 = *reinterpret_cast<const float4*>(Am + s * 12 + 4);
+    const float a8 = Am[s * 12 + 8];
+    u[0] = fmaf(a0.x, l[s], u[0]);
+    u[1] = fmaf(a0.y, l[s], u[1]);
+    u[2] = fmaf(a0.z, l[s], u[2]);
+    u[3] = fmaf(a0.w, l[s], u[3]);
+    u[4] = fmaf(a1.x, l[s], u[4]);
+    u[5] = fmaf(a1.y, l[s], u[5]);
+    u[6] = fmaf(a1.z, l[s], u[6]);
+    u[7] = fmaf(a1.w, l[s], u[7]);
+    u[8] = fmaf(a8, l[s], u[8]);
+  }
 }
-// y += S x (TR = false) or y += S^T x (TR = true), S in compact form (16-byte aligned).
-template <bool TR>
-__device__ __forceinline__ void star_acc(const float* Sc, const float x[9], float y[9]) {
-  float e[36];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const float4 v = reinterpret_cast<const float4*>(Sc)[i];
-    e[4 * i] = v.x;
-    e[4 * i + 1] = v.y;
-    e[4 * i + 2] = v.z;
-    e[4 * i + 3] = v.w;
-  }
-  if (!TR) {
-#pragma unroll
-    for (int r = 0; r < 6; ++r)
-#pragma unroll
-      for (int s = 0; s < 3; ++s) y[r] = fmaf(e[r * 3 + s], x[6 + s], y[r]);
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int s = 0; s < 6; ++s) y[6 + r] = fmaf(e[18 + r * 6 + s], x[s], y[6 + r]);
-  } else {
-#pragma unroll
-    for (int s = 0; s < 3; ++s)
-#pragma unroll
-      for (int r = 0; r < 6; ++r) y[6 + s] = fmaf(e[r * 3 + s], x[r], y[6 + s]);
-#pragma unroll
-    for (int s = 0; s < 6; ++s)
-#pragma unroll
-      for (int r = 0; r < 3; ++r) y[s] = fmaf(e[18 + r * 6 + s], x[6 + r], y[s]);
-  }
+
+// One face mode's share in the ten sums of a flux solver (face_flux_dot in host_flux.h): l the
+// adjoint's column, x the state's. The flux maps the velocity v and the traction t of x
+// through normal and tangential coefficients to a state (v*, t*), and n v*^T (lambda, mu) and
+// t* / rho to the result; against l these are products of (n.v, n.t, v_T, t_T) with the trace
+// of l's stresses, the vector (l n + diag(l) n) and l's velocities.
+__device__ __forceinline__ void face_products(const float* n, const float l[9], const float x[9], float o[10]) {
+  const float n0 = n[0], n1 = n[1], n2 = n[2];
+  const float tr = l[0] + l[1] + l[2];
+  const float a0 = fmaf(2.f * n0, l[0], fmaf(n1, l[3], n2 * l[5]));
+  const float a1 = fmaf(2.f * n1, l[1], fmaf(n0, l[3], n2 * l[4]));
+  const float a2 = fmaf(2.f * n2, l[2], fmaf(n1, l[4], n0 * l[5]));
+  const float t0 = fmaf(n0, x[0], fmaf(n1, x[3], n2 * x[5]));
+  const float t1 = fmaf(n1, x[1], fmaf(n0, x[3], n2 * x[4]));
+  const float t2 = fmaf(n2, x[2], fmaf(n1, x[4], n0 * x[5]));
+  const float vn = fmaf(n0, x[6], fmaf(n1, x[7], n2 * x[8])), tn = fmaf(n0, t0, fmaf(n1, t1, n2 * t2));
+  const float an = fmaf(n0, a0, fmaf(n1, a1, n2 * a2)), ln = fmaf(n0, l[6], fmaf(n1, l[7], n2 * l[8]));
+  const float v0 = fmaf(-vn, n0, x[6]), v1 = fmaf(-vn, n1, x[7]), v2 = fmaf(-vn, n2, x[8]);
+  const float s0 = fmaf(-tn, n0, t0), s1 = fmaf(-tn, n1, t1), s2 = fmaf(-tn, n2, t2);
+  o[0] = -tr * vn;
+  o[1] = -tr * tn;
+  o[2] = -an * vn;
+  o[3] = -an * tn;
+  o[4] = -fmaf(a0, v0, fmaf(a1, v1, a2 * v2));
+  o[5] = -fmaf(a0, s0, fmaf(a1, s1, a2 * s2));
+  o[6] = -ln * tn;
+  o[7] = -ln * vn;
+  o[8] = -fmaf(l[6], s0, fmaf(l[7], s1, l[8] * s2));
+  o[9] = -fmaf(l[6], v0, fmaf(l[7], v1, l[8] * v2));
 }
 
 // Polynomial degree of volume mode j (modes are ordered by degree).
@@ -273,9 +328,9 @@ template <int O>
 struct AdjPredCfg {
   static constexpr int B = nbasis(O), F = nface(O), NT = AdjNT<O>::value;
   static constexpr int BP = rup(B, 4), FP = rup(F, 4), NB9 = 9 * BP;
-  static constexpr int NSTAR = 3 * 36, NALOC = 4 * 9 * 12;       // compact S_c; A-_i rows padded to 12
-  static constexpr int NSCR = (3 * NB9 > 27 * 4 * FP) ? 3 * NB9 : 27 * 4 * FP;
-  static constexpr int ELEM = NSTAR + NALOC + (4 + O) * NB9 + NSCR;   // sS, sA, sL, sT, sG[2], sD[O], scratch
+  static constexpr int NGEO = AM_NGEO, NALOC = 4 * 9 * 12;       // geometry; A-_i rows padded to 12
+  static constexpr int NSCR = 19 * 4 * FP;
+  static constexpr int ELEM = NGEO + NALOC + (4 + O) * NB9 + NSCR;   // sS, sA, sL, sT, sG[2], sD[O], scratch
   static constexpr int TAB = 6 * BP * B + 8 * BP * F + 4 * FP * B;
   static constexpr int G_SMEM = (227 * 1024 / 4 - TAB) / ELEM;
   static constexpr int G_REG = 65536 / (128 * NT);
@@ -318,9 +373,9 @@ __device__ __forceinline__ void stage_pad(float* dst, const float* __restrict__ 
 // Degree structure used throughout (exact): K_c[i][j] vanishes unless deg i < deg j, so
 // D_d is a polynomial of degree O-1-d and lives on the first nbasis(O-d) modes; only those
 // modes of its adjoint G_d matter. With Z_c = G_{d+1} K_c the reverse time kernel is
-// G_d = c_d mu + c'_d mu_half + sum_c S_c^T Z_c and the star correlation of level d is
-// Z_c D_d^T; with V_c = lambda K_c^T the volume term is mu = -sum_c S_c^T V_c and its
-// correlation -V_c T^T. The contractions run over a multiple of four entries; the extra
+// G_d = c_d mu + c'_d mu_half + sum_c S_c^T Z_c and the star matrices' sums of level d are
+// Z_c's against D_d; with V_c = lambda K_c^T the volume term is mu = -sum_c S_c^T V_c and its
+// sums are -V_c's against T. The contractions run over a multiple of four entries; the extra
 // entries multiply structural zeros of K_c or zero pads, so the sums are those of the
 // unpadded loops, term for term.
 template <int O>
@@ -355,13 +410,13 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
   for (int i = threadIdx.x; i < C::G * C::ELEM; i += C::THREADS) smem[C::TAB + i] = 0.f;
   __syncthreads();
   const int g = threadIdx.x / NT, t = threadIdx.x % NT;
-  float* sS = smem + C::TAB + g * C::ELEM;   // compact S_c [3][36]
-  float* sA = sS + C::NSTAR;      // A-_i [4][9][12]: row s of face i at (i 9 + s) 12
+  float* sS = smem + C::TAB + g * C::ELEM;   // geometry and material
+  float* sA = sS + C::NGEO;       // A-_i [4][9][12]: row s of face i at (i 9 + s) 12
   float* sL = sA + C::NALOC;      // [9][BP] lambda
   float* sT = sL + NB9;
   float* sG0 = sT + NB9;          // G ping-pong [2][9][BP]
   float* sDb = sG0 + 2 * NB9;     // D_0 .. D_{O-1} [O][9][BP]
-  float* sScr = sDb + O * NB9;    // V_c, then the face products, then Z_c
+  float* sScr = sDb + O * NB9;    // transposed fluxes and face products; star sums
   for (int k = blockIdx.x * C::G + g; k < a.end; k += gridDim.x * C::G) {
     const int meta = a.meta[k];
     const int cl = meta & 0xff;
@@ -369,18 +424,11 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
     const bool even = ph.parity[cl] == 0;
     {
       const float* am = a.amat + (size_t)k * AM_SIZE;
-      for (int q = t; q < C::NSTAR; q += NT) sS[q] = __ldg(am + AM_STAR + (q / 36) * 81 + star_compact_index(q % 36));
+      for (int q = t; q < C::NGEO; q += NT) sS[q] = __ldg(am + AM_GEO + q);
       for (int q = t; q < 4 * 81; q += NT) sA[(q / 9) * 12 + q % 9] = __ldg(am + AM_LOC + q);
     }
-    double* Wk = a.W + (size_t)k * AM_SIZE;
-    // star correlations summed over the simulations, one 3 x 3 tile (c, row block, column
-    // block) per thread t < 27
-    const int tc = t / 9, trb = (t / 3) % 3, tsb = t % 3;
-    float wst[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) wst[i][q] = 0.f;
+    double* Wk = a.W + (size_t)k * WG_SIZE;
+    float wst[3] = {0.f, 0.f, 0.f};   // this column's star sums over the simulations
     for (int sim = 0; sim < a.nsim; ++sim) {
       const size_t kf = (size_t)k * a.nsim + sim;
       stage_pad<B, BP, NT>(sL, a.lq + kf * (9 * B), 1, t);
@@ -439,11 +487,12 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
                   for (int s = 0; s < 9; ++s) Y[c][s] = fmaf(lane4(x[s], u), kc, Y[c][s]);
                 }
             }
+          const StarGeo geo(sS);
+          StarFwd st;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) st.add(geo.J + 3 * c, Y[c]);
           float v[9];
-#pragma unroll
-          for (int r = 0; r < 9; ++r) v[r] = 0.f;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) star_acc<false>(sS + c * 36, Y[c], v);
+          st.get(geo, v);
 #pragma unroll
           for (int r = 0; r < 9; ++r) sDb[(d + 1) * NB9 + r * BP + t] = v[r];
         }
@@ -452,13 +501,13 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
       float mu[9], muh[9];
 #pragma unroll
       for (int r = 0; r < 9; ++r) mu[r] = muh[r] = 0.f;
-      float* sV = sScr;
       if (t < B) {
+        float T[9];
 #pragma unroll
         for (int r = 0; r < 9; ++r) {
           float v = 0.f;
           for (int d = 0; d < O; ++d) v = fmaf(ph.coef[cl][d], sDb[d * NB9 + r * BP + t], v);
-          sT[r * BP + t] = v;
+          sT[r * BP + t] = T[r] = v;
         }
         // V_c = lambda K_c^T and the volume term
         float V[3][9];
@@ -479,71 +528,39 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
               for (int s = 0; s < 9; ++s) V[c][s] = fmaf(lane4(x[s], u), kc, V[c][s]);
             }
         }
+        const StarGeo geo(sS);
+        StarRev st;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) st.add(geo.J + 3 * c, V[c]);
         float w[9];
-#pragma unroll
-        for (int r = 0; r < 9; ++r) w[r] = 0.f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          star_acc<true>(sS + c * 36, V[c], w);
-#pragma unroll
-          for (int s = 0; s < 9; ++s) sV[c * NB9 + s * BP + t] = V[c][s];
-        }
+        st.get(geo, w);
+        st.sums(T, -1.f, wst);
 #pragma unroll
         for (int r = 0; r < 9; ++r) mu[r] = -w[r];
       }
       gsync<NT>(g);
-      if (t < 27) {
-        float tv[3][3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) tv[i][q] = 0.f;
-        tile33v<BP>(sV + tc * NB9, sT, 3 * trb, 3 * tsb, BP, tv);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) wst[i][q] -= tv[i][q];
-      }
-      gsync<NT>(g);
       // local surface: LF_i = lambda F^_i^T, TF_i = T F~_i, U_i = A-_i^T LF_i, per (face, f);
       // the pad columns f >= F are written zero
-      float* sLF = sScr;              // [4][9][FP]
-      float* sTF = sScr + 36 * FP;
-      float* sU = sScr + 72 * FP;
+      float* sU = sScr;               // [4][9][FP]
+      float* sP = sScr + 36 * FP;     // [4][10][FP]
       for (int p = t; p < 4 * FP; p += NT) {
         const int i = p / FP, f = p % FP;
-        float lf[9], tf[9], u[9];
+        float u[9], o[10];
         if (f < F) {
+          float lf[9], tf[9];
           rows9v<BP, BP>(sL, tFhT + i * BP * F, F, f, lf);
           rows9v<BP, BP>(sT, tFt + i * BP * F, F, f, tf);
-#pragma unroll
-          for (int r = 0; r < 9; ++r) u[r] = 0.f;
-          const float* Am = sA + i * 108;
-#pragma unroll
-          for (int s = 0; s < 9; ++s) {
-            const float4 a0 = *reinterpret_cast<const float4*>(Am + s * 12);
-            const float4 a1 = *reinterpret_cast<const float4*>(Am + s * 12 + 4);
-            const float a8 = Am[s * 12 + 8];
-            u[0] = fmaf(a0.x, lf[s], u[0]);
-            u[1] = fmaf(a0.y, lf[s], u[1]);
-            u[2] = fmaf(a0.z, lf[s], u[2]);
-            u[3] = fmaf(a0.w, lf[s], u[3]);
-            u[4] = fmaf(a1.x, lf[s], u[4]);
-            u[5] = fmaf(a1.y, lf[s], u[5]);
-            u[6] = fmaf(a1.z, lf[s], u[6]);
-            u[7] = fmaf(a1.w, lf[s], u[7]);
-            u[8] = fmaf(a8, lf[s], u[8]);
-          }
+          flux_transposed(sA + i * 108, lf, u);
+          face_products(sS + 12 + 3 * i, lf, tf, o);
         } else {
 #pragma unroll
-          for (int r = 0; r < 9; ++r) lf[r] = tf[r] = u[r] = 0.f;
+          for (int r = 0; r < 9; ++r) u[r] = o[r] = 0.f;
+          o[9] = 0.f;
         }
 #pragma unroll
-        for (int r = 0; r < 9; ++r) {
-          sLF[(i * 9 + r) * FP + f] = lf[r];
-          sTF[(i * 9 + r) * FP + f] = tf[r];
-          sU[(i * 9 + r) * FP + f] = u[r];
-        }
+        for (int r = 0; r < 9; ++r) sU[(i * 9 + r) * FP + f] = u[r];
+#pragma unroll
+        for (int q = 0; q < 10; ++q) sP[(i * 10 + q) * FP + f] = o[q];
       }
       gsync<NT>(g);
       if (t < B)
@@ -560,18 +577,11 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
               for (int r = 0; r < 9; ++r) mu[r] = fmaf(lane4(x[r], u), w, mu[r]);
             }
           }
-      for (int p = t; p < 36; p += NT) {
-        const int i = p / 9, rb = (p / 3) % 3, sb = p % 3;
-        float acc[3][3];
+      for (int p = t; p < 40; p += NT) {
+        float acc = 0.f;
 #pragma unroll
-        for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) acc[ii][q] = 0.f;
-        tile33v<FP>(sLF + i * 9 * FP, sTF + i * 9 * FP, 3 * rb, 3 * sb, FP, acc);
-#pragma unroll
-        for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) atomicAdd(Wk + AM_LOC + i * 81 + (3 * rb + ii) * 9 + 3 * sb + q, (double)acc[ii][q]);
+        for (int f = 0; f < F; ++f) acc += sP[p * FP + f];
+        atomicAdd(Wk + WG_LOC + p, (double)acc);
       }
       // the buffers this pass wrote
       if (t < B) {
@@ -586,7 +596,6 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
       }
       gsync<NT>(g);
       // ---- reverse time kernel
-      float* sZ = sScr;
 #pragma unroll
       for (int d = O - 2; d >= 0; --d) {
         const int nk = nbasis(O - 1 - d), nout = nbasis(O - d);
@@ -615,17 +624,24 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
           float gv[9];
 #pragma unroll
           for (int r = 0; r < 9; ++r) gv[r] = ph.coef[cl][d] * mu[r] + ph.hcoef[cl][d] * muh[r];
+          // entries t >= nout of Z_c are zero and those of D_d not part of the sums
+          if (t < nout) {
+            const StarGeo geo(sS);
+            StarRev st;
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            star_acc<true>(sS + c * 36, Z[c], gv);
+            for (int c = 0; c < 3; ++c) st.add(geo.J + 3 * c, Z[c]);
+            float w[9], x[9];
+            st.get(geo, w);
 #pragma unroll
-            for (int r = 0; r < 9; ++r) sZ[c * NB9 + r * BP + t] = Z[c][r];
+            for (int r = 0; r < 9; ++r) {
+              x[r] = sDb[d * NB9 + r * BP + t];
+              gv[r] += w[r];
+            }
+            st.sums(x, 1.f, wst);
           }
 #pragma unroll
           for (int r = 0; r < 9; ++r) sG0[(d & 1) * NB9 + r * BP + t] = gv[r];
         }
-        gsync<NT>(g);
-        if (t < 27) tile33v<BP>(sZ + tc * NB9, sDb + d * NB9, 3 * trb, 3 * tsb, rup(nout, 4), wst);
         gsync<NT>(g);
       }
       if (t < B)
@@ -633,28 +649,44 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
         for (int r = 0; r < 9; ++r) a.lq[kf * (9 * B) + r * B + t] = sL[r * BP + t] + sG0[r * BP + t];
       gsync<NT>(g);   // the group's region is refilled for the next simulation or element
     }
-    if (t < 27)
+    // the star sums over the columns, in order
+    if (t < B)
 #pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) atomicAdd(Wk + AM_STAR + tc * 81 + (3 * trb + i) * 9 + 3 * tsb + q, (double)wst[i][q]);
+      for (int q = 0; q < 3; ++q) sScr[q * B + t] = wst[q];
+    gsync<NT>(g);
+    if (t < 3) {
+      double acc = 0.0;
+      for (int x = 0; x < B; ++x) acc += (double)sScr[t * B + x];
+      atomicAdd(Wk + WG_STAR + t, acc);
+    }
+    gsync<NT>(g);
   }
 }
 
 // Reverse of a neighbour pass, one CTA per buffer owner (every element): for each face
 // whose neighbour (the receiver) was active, the receiver's transposed flux goes to the
-// adjoint of the buffer it read, and the receiver's correlation with that buffer is
+// adjoint of the buffer it read, and the receiver's ten sums with that buffer are
 // accumulated. Every (receiver, face) pair is visited by exactly one owner. The four faces
 // are handled together: with LF = lambda_k F^_ip^T and XF = X F-_jh (9 x F each), the
-// transposed flux is (A+^T LF) F-_jh^T and the correlation LF XF^T.
+// transposed flux is (A+^T LF) F-_jh^T and the sums are face_products of LF and XF. Bound by
+// instruction issue (4,900 warp instructions an owner at order 4, 59 % of the issue slots, two
+// fifths of the stalls on operator-table loads), so the CTA has a thread for every (side, face,
+// face mode), then (face, face mode), (face, mode) and (row, mode): 167 us a launch against 187
+// with one warp an owner (47,040 elements, order 4, two clusters, mean of both).
 template <int O>
-__global__ void __launch_bounds__(AdjNT<O>::value) k_adj_nbr(DevOps ops, AdjLtsArgs a, PhaseArgs ph) {
-  constexpr int B = nbasis(O), F = nface(O), NB9 = 9 * B;
-  __shared__ float sA[4][81];
-  __shared__ float sLk[4][NB9], sX[4][NB9];
-  __shared__ float sLF[4][9 * F], sXF[4][9 * F], sU[4][9 * F];
+struct AdjNbrNT {
+  static constexpr int value = rup(8 * nface(O), 32);
+};
+template <int O>
+__global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjLtsArgs a, PhaseArgs ph) {
+  constexpr int B = nbasis(O), F = nface(O), BP = rup(B, 4), FP = rup(F, 4), NB9 = 9 * B;
+  __shared__ __align__(16) float sA[4][108];
+  __shared__ __align__(16) float sLk[4][9 * BP], sX[4][9 * BP];
+  __shared__ __align__(16) float sLF[4][9 * FP];   // then A+^T LF
+  __shared__ float sXF[4][9 * FP], sP9[4][FP];     // then the ten products
+  __shared__ float sN[4][3];
   __shared__ int sF[8], sBk[8];
-  const int kn = a.owners ? a.owners[blockIdx.x] : (int)blockIdx.x, t = threadIdx.x, nt = blockDim.x;
+  const int kn = a.owners ? a.owners[blockIdx.x] : (int)blockIdx.x, t = threadIdx.x;
   if (t < 8) {
     sF[t] = a.fwd[kn * 8 + t];
     sBk[t] = a.back[kn * 8 + t];
@@ -675,10 +707,21 @@ __global__ void __launch_bounds__(AdjNT<O>::value) k_adj_nbr(DevOps ops, AdjLtsA
   }
   if (modes == 0) return;   // the same for every thread of the CTA
   auto mode = [modes](int i) { return ((modes >> (3 * i)) & 7) - 1; };
-  constexpr int NT = AdjNT<O>::value, R = (NB9 + NT - 1) / NT;
+  constexpr int NT = AdjNbrNT<O>::value, R = (NB9 + NT - 1) / NT;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
-    if (mode(i) >= 0) stage<81, NT>(sA[i], a.amat + (size_t)sF[2 * i] * AM_SIZE + AM_NBR + sBk[2 * i] * 81, t);
+    if (mode(i) >= 0) {
+      const float* am = a.amat + (size_t)sF[2 * i] * AM_SIZE;
+      for (int q = t; q < 81; q += NT) sA[i][(q / 9) * 12 + q % 9] = __ldg(am + AM_NBR + sBk[2 * i] * 81 + q);
+      if (t < 3) sN[i][t] = __ldg(am + AM_GEO + 12 + 3 * sBk[2 * i] + t);
+    }
+  // pad entries of the rows: zero, never written afterwards
+  for (int q = t; q < 36; q += NT) {
+#pragma unroll
+    for (int x = B; x < BP; ++x) sLk[q / 9][(q % 9) * BP + x] = sX[q / 9][(q % 9) * BP + x] = 0.f;
+#pragma unroll
+    for (int x = F; x < FP; ++x) sLF[q / 9][(q % 9) * FP + x] = 0.f;
+  }
   for (int sim = 0; sim < a.nsim; ++sim) {
     // this simulation's block of the owner's buffers (stride G between modes)
     const size_t xo = (size_t)kn * a.bufs + (size_t)(sim / a.G) * (NB9 * a.G) + sim % a.G;
@@ -687,7 +730,7 @@ __global__ void __launch_bounds__(AdjNT<O>::value) k_adj_nbr(DevOps ops, AdjLtsA
       const int m = mode(i);
       if (m < 0) continue;
       const int k = sF[2 * i];
-      stage<NB9, NT>(sLk[i], a.lq + ((size_t)k * a.nsim + sim) * NB9, t);
+      stage_pad<B, BP, NT>(sLk[i], a.lq + ((size_t)k * a.nsim + sim) * NB9, 1, t);
       const float* b0 = (m == 1) ? a.B3s : (m == 2) ? a.B2s : a.B1s;
       float x[R], x2[R];
 #pragma unroll
@@ -700,79 +743,82 @@ __global__ void __launch_bounds__(AdjNT<O>::value) k_adj_nbr(DevOps ops, AdjLtsA
         }
       }
 #pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (t + j * NT < NB9) sX[i][t + j * NT] = x[j] - x2[j];
-    }
-    __syncthreads();
-    for (int p = t; p < 4 * F; p += nt) {
-      const int i = p / F, f = p % F;
-      if (mode(i) < 0) continue;
-      const int ip = sBk[2 * i], jh = sBk[2 * i + 1];
-      float lf[9], xf[9];
-      rows9<B, B>(sLk[i], a.FhT + ip * B * F, F, f, lf);
-      rows9<B, B>(sX[i], ops.Fb + jh * B * F, F, f, xf);
-#pragma unroll
-      for (int r = 0; r < 9; ++r) {
-        float u = 0.f;
-#pragma unroll
-        for (int s = 0; s < 9; ++s) u = fmaf(sA[i][s * 9 + r], lf[s], u);
-        sLF[i][r * F + f] = lf[r];
-        sXF[i][r * F + f] = xf[r];
-        sU[i][r * F + f] = u;
+      for (int j = 0; j < R; ++j) {
+        const int q = t + j * NT;
+        if (q < NB9) sX[i][(q / B) * BP + q % B] = x[j] - x2[j];
       }
     }
     __syncthreads();
-    if (t < B) {
-      // the faces' contributions summed per buffer, then one update of each adjoint touched
-      float y1[9], y2[9], y3[9];
+    for (int p = t; p < 8 * F; p += NT) {
+      const int i = (p / F) % 4, f = p % F;
+      if (mode(i) < 0) continue;
+      const int ip = sBk[2 * i], jh = sBk[2 * i + 1];
+      const bool state = p >= 4 * F;
+      float v[9];
+      rows9v<B, BP>(state ? sX[i] : sLk[i], state ? ops.Fb + jh * B * F : a.FhT + ip * B * F, F, f, v);
+      float* dst = state ? sXF[i] : sLF[i];
 #pragma unroll
-      for (int r = 0; r < 9; ++r) y1[r] = y2[r] = y3[r] = 0.f;
+      for (int r = 0; r < 9; ++r) dst[r * FP + f] = v[r];
+    }
+    __syncthreads();
+    for (int p = t; p < 4 * F; p += NT) {
+      const int i = p / F, f = p % F;
+      if (mode(i) < 0) continue;
+      float lf[9], xf[9], u[9], o[10];
+#pragma unroll
+      for (int r = 0; r < 9; ++r) {
+        lf[r] = sLF[i][r * FP + f];
+        xf[r] = sXF[i][r * FP + f];
+      }
+      flux_transposed(sA[i], lf, u);
+      face_products(sN[i], lf, xf, o);
+#pragma unroll
+      for (int r = 0; r < 9; ++r) {
+        sLF[i][r * FP + f] = u[r];
+        sXF[i][r * FP + f] = o[r];
+      }
+      sP9[i][f] = o[9];
+    }
+    __syncthreads();
+    // the transposed fluxes, in place of the receivers' adjoints
+    for (int p = t; p < 4 * B; p += NT) {
+      const int i = p / B, b = p % B;
+      if (mode(i) < 0) continue;
+      float y[9];
+      rows9v<F, FP>(sLF[i], a.FbT + sBk[2 * i + 1] * F * B, B, b, y);
+#pragma unroll
+      for (int r = 0; r < 9; ++r) sLk[i][r * BP + b] = y[r];
+    }
+    for (int p = t; p < 40; p += NT) {
+      const int i = p / 10, q = p % 10;
+      if (mode(i) < 0) continue;
+      float acc = 0.f;
+#pragma unroll
+      for (int f = 0; f < F; ++f) acc += q < 9 ? sXF[i][q * FP + f] : sP9[i][f];
+      atomicAdd(a.W + (size_t)sF[2 * i] * WG_SIZE + WG_NBR + sBk[2 * i] * 10 + q, (double)acc);
+    }
+    __syncthreads();
+    // the faces' contributions summed per buffer in order, then one update of each adjoint touched
+    for (int p = t; p < NB9; p += NT) {
+      float y1 = 0.f, y2 = 0.f, y3 = 0.f;
       bool u1 = false, u2 = false, u3 = false;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int m = mode(i);
         if (m < 0) continue;
-        float y[9];
-        rows9<F, F>(sU[i], a.FbT + sBk[2 * i + 1] * F * B, B, t, y);
-#pragma unroll
-        for (int r = 0; r < 9; ++r) {
-          if (m == 1) {
-            y3[r] += y[r];
-          } else if (m == 2) {
-            y2[r] += y[r];
-          } else if (m == 3) {
-            y1[r] += y[r];
-            y2[r] -= y[r];
-          } else {
-            y1[r] += y[r];
-          }
-        }
+        const float y = sLk[i][(p / B) * BP + p % B];
+        if (m == 1) y3 += y;
+        if (m == 2) y2 += y;
+        if (m == 0 || m == 3) y1 += y;
+        if (m == 3) y2 -= y;
         u1 |= (m == 0 || m == 3);
         u2 |= (m == 2 || m == 3);
         u3 |= (m == 1);
       }
-      const size_t o = ((size_t)kn * a.nsim + sim) * NB9 + t;
-#pragma unroll
-      for (int r = 0; r < 9; ++r) {
-        if (u1) atomicAdd(a.lb1 + o + r * B, y1[r]);
-        if (u2) atomicAdd(a.lb2 + o + r * B, y2[r]);
-        if (u3) atomicAdd(a.lb3 + o + r * B, y3[r]);
-      }
-    }
-    for (int p = t; p < 36; p += nt) {
-      const int i = p / 9, rb = (p / 3) % 3, sb = p % 3;
-      if (mode(i) < 0) continue;
-      float acc[3][3];
-#pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) acc[ii][q] = 0.f;
-      tile33<F>(sLF[i], sXF[i], 3 * rb, 3 * sb, F, acc);
-      double* Wk = a.W + (size_t)sF[2 * i] * AM_SIZE + AM_NBR + sBk[2 * i] * 81;
-#pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) atomicAdd(Wk + (3 * rb + ii) * 9 + 3 * sb + q, (double)acc[ii][q]);
+      const size_t o = ((size_t)kn * a.nsim + sim) * NB9 + p;
+      if (u1) atomicAdd(a.lb1 + o, y1);
+      if (u2) atomicAdd(a.lb2 + o, y2);
+      if (u3) atomicAdd(a.lb3 + o, y3);
     }
     __syncthreads();   // the staged blocks are refilled for the next simulation
   }

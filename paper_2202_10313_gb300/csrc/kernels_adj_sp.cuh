@@ -9,11 +9,12 @@
 //                 V_c = lambda K_c^T), the face traces lambda F~_i and T F~_i (F^_i = F~_i^T in
 //                 the orthonormal face basis), the summed transposed traces sum_i U_i F~_i^T
 //                 and the reverse time kernel Z_c = G_{d+1} K_c on the support of level d;
-//   column phase: thread = (element e, mode b): star matrices (S_c, S_c^T, compact), Taylor
-//                 weights, the buffer adjoints, and the next row operand;
-//   face phase:   thread = (element, face, face mode): U_i = A-_i^T (lambda F~_i);
-//   correlations: thread = (element, 3 x 3 tile): W_c and W-_i over the modes (face modes),
-//                 the batch's W_c summed in shared memory and added to the FP64 totals once.
+//   column phase: thread = (element e, mode b): star matrices (S_c, S_c^T) and this mode's
+//                 share of their three sums, Taylor weights, the buffer adjoints, and the next
+//                 row operand;
+//   face phase:   thread = (element, face, face mode): U_i = A-_i^T (lambda F~_i) and the ten
+//                 products of lambda F~_i and T F~_i, in place of T F~_i; summed over the
+//                 face modes per (element, face, product) while the time kernel starts.
 // Staging arrays are [mode or output][pair] with an odd pair stride XP, as in k_predict_sp.
 #pragma once
 #include "kernels_adj.cuh"
@@ -55,14 +56,15 @@ struct AdjSpCfg {
   static constexpr int XP = NPAIR | 1;                      // odd pair stride
   static constexpr int DROWS = adj_drow(O, O - 1);          // D_0 .. D_{O-2}
   static constexpr int WROWS = (3 * B > 8 * F) ? 3 * B : 8 * F;
+  static_assert(3 * B * NE <= WROWS * XP, "star sums of a batch fit into the row outputs");
   static constexpr int S_X = 0;                             // [B] row operand
   static constexpr int S_T = S_X + B * XP;                  // [B] T
   static constexpr int S_D = S_T + B * XP;                  // [DROWS] D_d
   static constexpr int S_W = S_D + DROWS * XP;              // [3B] Y_c, V_c, Z_c or [8F] LF_i (U_i), TF_i
-  static constexpr int S_STAR = rup(S_W + WROWS * XP, 4);   // [NE][3][36] compact S_c
-  static constexpr int S_AL = S_STAR + NE * 108;            // [NE][4][9][12] A-_i, rows padded to 12
-  static constexpr int S_WC = S_AL + NE * 432;              // [NE][243] W_c of the batch
-  static constexpr int S_META = S_WC + NE * 243;            // [NE] ints
+  static constexpr int S_GEO = rup(S_W + WROWS * XP, 4);    // [NE][AM_NGEO] geometry and material
+  static constexpr int S_AL = S_GEO + NE * AM_NGEO;         // [NE][4][9][12] A-_i, rows padded to 12
+  static constexpr int S_P9 = S_AL + NE * 432;              // [4F][NE] the tenth product
+  static constexpr int S_META = S_P9 + 4 * F * NE;          // [NE] ints
   static constexpr int TOTAL = rup(S_META + NE, 4);
 };
 
@@ -91,41 +93,6 @@ __device__ __forceinline__ void sp_time_adj(int part, int variant, const float* 
   if constexpr (O == 3) ltssp::sp_time_o3<XP>(part, variant, x, y);
 }
 
-// Star correlations of a batch: W_c[r][s] (+/-)= sum_{b0 <= b < n} X[(c B + b) XP + 9 e + r]
-// Y[(y0 + b) XP + 9 e + s], one 3 x 3 tile (element, c, row block, column block) per task,
-// accumulated into the batch's W_c in shared memory (one writer per entry).
-template <int B, int XP, int NE, int NT>
-__device__ __forceinline__ void star_corr(const float* X, const float* Y, int y0, int b0, int n, bool sub, float* sWc,
-                                          int tid) {
-  for (int j = tid; j < 27 * NE; j += NT) {
-    const int e = j / 27, c = (j / 9) % 3, rb = (j / 3) % 3, sb = j % 3;
-    float acc[3][3];
-    float* w = sWc + e * 243 + c * 81 + (3 * rb) * 9 + 3 * sb;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) acc[i][q] = sub ? 0.f : w[i * 9 + q];
-    const float* x = X + c * B * XP + 9 * e + 3 * rb;
-    const float* y = Y + y0 * XP + 9 * e + 3 * sb;
-    for (int b = b0; b < n; ++b) {
-      float xv[3], yv[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        xv[i] = x[b * XP + i];
-        yv[i] = y[b * XP + i];
-      }
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) acc[i][q] = fmaf(xv[i], yv[q], acc[i][q]);
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) w[i * 9 + q] = sub ? w[i * 9 + q] - acc[i][q] : acc[i][q];
-  }
-}
-
 template <int O>
 __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a, PhaseArgs ph) {
   using S = AdjSpCfg<O>;
@@ -136,9 +103,9 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
   float* sT = smem + S::S_T;
   float* sD = smem + S::S_D;
   float* sW = smem + S::S_W;
-  float* sStar = smem + S::S_STAR;
+  float* sGeo = smem + S::S_GEO;
   float* sAl = smem + S::S_AL;
-  float* sWc = smem + S::S_WC;
+  float* sP9 = smem + S::S_P9;
   int* sMeta = reinterpret_cast<int*>(smem + S::S_META);
   const int tid = threadIdx.x;
   // column task (element, mode), modes fastest
@@ -155,24 +122,22 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
     __syncthreads();   // the previous batch is done with shared memory
     const int k = k0 + es;
     const bool valid = act && k < a.end;
-    // the batch's star matrices (compact), A-_i (rows padded), and zero star correlations
+    // the batch's geometry, A-_i (rows padded)
     if (tid < NE) sMeta[tid] = (k0 + tid < a.end) ? a.meta[k0 + tid] : 0;
-    for (int q = tid; q < NE * 108; q += NT) {
-      const int e = q / 108, x = q % 108;
-      sStar[q] = (k0 + e < a.end)
-                     ? __ldg(a.amat + (size_t)(k0 + e) * AM_SIZE + AM_STAR + (x / 36) * 81 + star_compact_index(x % 36))
-                     : 0.f;
+    for (int q = tid; q < NE * AM_NGEO; q += NT) {
+      const int e = q / AM_NGEO, x = q % AM_NGEO;
+      sGeo[q] = (k0 + e < a.end) ? __ldg(a.amat + (size_t)(k0 + e) * AM_SIZE + AM_GEO + x) : 0.f;
     }
     for (int q = tid; q < NE * 324; q += NT) {
       const int e = q / 324, x = q % 324;
       sAl[e * 432 + (x / 9) * 12 + x % 9] = (k0 + e < a.end) ? __ldg(a.amat + (size_t)(k0 + e) * AM_SIZE + AM_LOC + x) : 0.f;
     }
-    for (int q = tid; q < NE * 243; q += NT) sWc[q] = 0.f;
+    float wst[3] = {0.f, 0.f, 0.f};   // this column's star sums over the simulations
     const int meta = valid ? a.meta[k] : 0;
     const int cl = meta & 0xff;
     // fused runs take the simulations of the batch in turn: the operator matrices are staged
-    // once, W_c sums over the simulations (in order) and W-_i receives one addition per
-    // simulation, in order
+    // once, the star sums run over the simulations and the faces' sums receive one addition
+    // per simulation, in order
     for (int sim = 0; sim < a.nsim; ++sim) {
       // this simulation's adjoints [element][simulation][9][B]
       const size_t ao = ((size_t)k * a.nsim + sim) * (9 * B) + b;
@@ -216,7 +181,7 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
           }
         }
       }
-      const float* Sk = sStar + es * 108;
+      const float* Gk = sGeo + es * AM_NGEO;
       // ---- forward time kernel: D_{d+1} = sum_c S_c D_d K_c^T (variant d: D_d on nbasis(O - d)
       // modes, D_{d+1} on nbasis(O - 1 - d))
 #pragma unroll 1
@@ -229,13 +194,16 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
 #pragma unroll
           for (int r = 0; r < 9; ++r) v[r] = 0.f;
           if (b < nout) {
+            const StarGeo geo(Gk);
+            StarFwd st;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
               float y[9];
 #pragma unroll
               for (int s = 0; s < 9; ++s) y[s] = sW[(c * B + b) * XP + col + s];
-              star_acc<false>(Sk + c * 36, y, v);
+              st.add(geo.J + 3 * c, y);
             }
+            st.get(geo, v);
           }
           const float c1 = ph.coef[cl][d + 1];
 #pragma unroll
@@ -252,7 +220,7 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
         __syncthreads();
       }
       // ---- volume: V_c = lambda K_c^T (on nbasis(O - 1) modes), mu = -sum_c S_c^T V_c,
-      // W_c -= V_c T^T
+      // its star sums
       float lam[9], mu[9], muh[9];
 #pragma unroll
       for (int r = 0; r < 9; ++r) lam[r] = 0.f;
@@ -277,18 +245,21 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
 #pragma unroll
         for (int r = 0; r < 9; ++r) w[r] = 0.f;
         if (act && b < NV) {
+          const StarGeo geo(Gk);
+          StarRev st;
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
             float v[9];
 #pragma unroll
             for (int s = 0; s < 9; ++s) v[s] = sW[(c * B + b) * XP + col + s];
-            star_acc<true>(Sk + c * 36, v, w);
+            st.add(geo.J + 3 * c, v);
           }
+          st.get(geo, w);
+          st.sums(T, -1.f, wst);
         }
 #pragma unroll
         for (int r = 0; r < 9; ++r) mu[r] = -w[r];
       }
-      star_corr<B, XP, NE, NT>(sW, sT, 0, 0, NV, true, sWc, tid);
       __syncthreads();
       // ---- local surface: LF_i = lambda F~_i and TF_i = T F~_i (row phase)
       if (ract) {
@@ -296,65 +267,25 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
         sp_trace<O, XP>(part, sT + pair, sW + 4 * F * XP + pair);
       }
       __syncthreads();
-      // W-_i += LF_i TF_i^T: one writer per entry (the simulations in turn)
-      for (int j = tid; j < 36 * NE; j += NT) {
-        const int e = j / 36, i = (j / 9) % 4, rb = (j / 3) % 3, sb = j % 3;
-        float acc[3][3];
-#pragma unroll
-        for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) acc[ii][q] = 0.f;
-        const float* x = sW + i * F * XP + 9 * e + 3 * rb;
-        const float* y = sW + (4 + i) * F * XP + 9 * e + 3 * sb;
-        for (int f = 0; f < F; ++f) {
-          float xv[3], yv[3];
-#pragma unroll
-          for (int ii = 0; ii < 3; ++ii) {
-            xv[ii] = x[f * XP + ii];
-            yv[ii] = y[f * XP + ii];
-          }
-#pragma unroll
-          for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) acc[ii][q] = fmaf(xv[ii], yv[q], acc[ii][q]);
-        }
-        if (k0 + e < a.end) {
-          double* Wk = a.W + (size_t)(k0 + e) * AM_SIZE + AM_LOC + i * 81 + (3 * rb) * 9 + 3 * sb;
-#pragma unroll
-          for (int ii = 0; ii < 3; ++ii)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) atomicAdd(Wk + ii * 9 + q, (double)acc[ii][q]);
-        }
-      }
-      __syncthreads();
-      // U_i = A-_i^T LF_i per (element, face, face mode), over LF_i
+      // per (element, face, face mode): U_i = A-_i^T LF_i over LF_i, the ten products over TF_i
       for (int j = tid; j < NE * 4 * F; j += NT) {
         const int e = j / (4 * F), i = (j / F) % 4, f = j % F;
         float* lp = sW + (i * F + f) * XP + 9 * e;
-        float lf[9], u[9];
+        float* tp = lp + 4 * F * XP;
+        float lf[9], tf[9], u[9], o[10];
 #pragma unroll
         for (int s = 0; s < 9; ++s) {
           lf[s] = lp[s];
-          u[s] = 0.f;
+          tf[s] = tp[s];
         }
-        const float* Am = sAl + e * 432 + i * 108;
+        flux_transposed(sAl + e * 432 + i * 108, lf, u);
+        face_products(sGeo + e * AM_NGEO + 12 + 3 * i, lf, tf, o);
 #pragma unroll
-        for (int s = 0; s < 9; ++s) {
-          const float4 a0 = *reinterpret_cast<const float4*>(Am + s * 12);
-          const float4 a1 = *reinterpret_cast<const float4*>(Am + s * 12 + 4);
-          const float a8 = Am[s * 12 + 8];
-          u[0] = fmaf(a0.x, lf[s], u[0]);
-          u[1] = fmaf(a0.y, lf[s], u[1]);
-          u[2] = fmaf(a0.z, lf[s], u[2]);
-          u[3] = fmaf(a0.w, lf[s], u[3]);
-          u[4] = fmaf(a1.x, lf[s], u[4]);
-          u[5] = fmaf(a1.y, lf[s], u[5]);
-          u[6] = fmaf(a1.z, lf[s], u[6]);
-          u[7] = fmaf(a1.w, lf[s], u[7]);
-          u[8] = fmaf(a8, lf[s], u[8]);
+        for (int r = 0; r < 9; ++r) {
+          lp[r] = u[r];
+          tp[r] = o[r];
         }
-#pragma unroll
-        for (int r = 0; r < 9; ++r) lp[r] = u[r];
+        sP9[(i * F + f) * NE + e] = o[9];
       }
       // the adjoints of the buffers this pass wrote: lambda_B1 (+ lambda_B3) join mu,
       // lambda_B2 is mu_half; reset here (lambda_B3 survives an accumulation)
@@ -381,9 +312,20 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
       // mu += sum_i U_i F~_i^T (row phase, into the row operand's place)
       if (ract) sp_tproj<O, XP>(part, sW + pair, sX + pair);
       __syncthreads();
+      // the faces' sums (one writer per entry, the simulations in turn); the row outputs are
+      // written again after the next barrier
+      for (int j = tid; j < 40 * NE; j += NT) {
+        const int e = j / 40, i = (j / 10) % 4, q = j % 10;
+        const float* p = q < 9 ? sW + (4 + i) * F * XP + 9 * e + q : sP9 + i * F * NE + e;
+        const int ld = q < 9 ? XP : NE;
+        float acc = 0.f;
+#pragma unroll
+        for (int f = 0; f < F; ++f) acc += p[f * ld];
+        if (k0 + e < a.end) atomicAdd(a.W + (size_t)(k0 + e) * WG_SIZE + WG_LOC + 10 * i + q, (double)acc);
+      }
       // ---- reverse time kernel: G_{O-1} = c_{O-1} mu + c'_{O-1} mu_half (over this column's
       // face sum: read and written by the same thread), then G_d = c_d mu + c'_d mu_half +
-      // sum_c S_c^T Z_c with Z_c = G_{d+1} K_c, and W_c += Z_c D_d^T
+      // sum_c S_c^T Z_c with Z_c = G_{d+1} K_c, and the star sums against D_d
       if (act) {
 #pragma unroll
         for (int r = 0; r < 9; ++r) {
@@ -405,13 +347,24 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
           for (int r = 0; r < 9; ++r) gv[r] = ph.coef[cl][d] * mu[r] + ph.hcoef[cl][d] * muh[r];
           // Z_c[0] = 0 (not written)
           if (b >= 1 && b < nout) {
+            const StarGeo geo(Gk);
+            StarRev st;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
               float z[9];
 #pragma unroll
               for (int r = 0; r < 9; ++r) z[r] = sW[(c * B + b) * XP + col + r];
-              star_acc<true>(Sk + c * 36, z, gv);
+              st.add(geo.J + 3 * c, z);
             }
+            float w[9], x[9];
+            st.get(geo, w);
+            const float* dp = sD + (adj_drow(O, d) + b) * XP + col;
+#pragma unroll
+            for (int r = 0; r < 9; ++r) {
+              gv[r] += w[r];
+              x[r] = dp[r];
+            }
+            st.sums(x, 1.f, wst);
           }
 #pragma unroll
           for (int r = 0; r < 9; ++r) {
@@ -419,7 +372,6 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
             g0[r] = gv[r];
           }
         }
-        star_corr<B, XP, NE, NT>(sW, sD, adj_drow(O, d), 1, nout, false, sWc, tid);
         __syncthreads();
       }
       if (valid) {
@@ -428,10 +380,17 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
         for (int r = 0; r < 9; ++r) lp[r * B] = lam[r] + g0[r];
       }
     }  // simulations
-    // the batch's star correlations into the FP64 totals (one addition per entry and pass)
-    for (int q = tid; q < NE * 243; q += NT) {
-      const int e = q / 243;
-      if (k0 + e < a.end) atomicAdd(a.W + (size_t)(k0 + e) * AM_SIZE + AM_STAR + q % 243, (double)sWc[q]);
+    // the batch's star sums over the columns, in order, into the FP64 totals
+    if (act)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) sW[q * (NE * B) + tid] = wst[q];
+    __syncthreads();
+    for (int q = tid; q < 3 * NE; q += NT) {
+      const int e = q / 3;
+      const float* p = sW + (q % 3) * (NE * B) + e * B;
+      double acc = 0.0;
+      for (int x = 0; x < B; ++x) acc += (double)p[x];
+      if (k0 + e < a.end) atomicAdd(a.W + (size_t)(k0 + e) * WG_SIZE + WG_STAR + q % 3, acc);
     }
   }
 }
