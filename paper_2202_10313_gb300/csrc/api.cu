@@ -1,4 +1,7 @@
 // C ABI of the solver: set-up tables, device state and the clustered-LTS schedule.
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include <algorithm>
 #include <array>
 #include <thread>
@@ -1761,6 +1764,23 @@ static __global__ void k_convert_dofs(float* Q, double* stage, const int* iperm,
   }
 }
 
+// Write to every page of [p, p + bytes) (about to be overwritten) unless all are resident: a
+// device copy into pages that the caller has not touched yet now and then takes 23 ms instead of
+// 0.7 (29 MB), faulting them in here 0.3. A look at resident pages costs a few microseconds.
+static void fault_in(void* p, size_t bytes) {
+  if (bytes == 0) return;
+  const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  char* first = (char*)((uintptr_t)p / page * page);
+  const size_t n = ((char*)p + bytes - first + page - 1) / page;
+  std::vector<unsigned char> in(n);
+  if (mincore(first, n * page, in.data()) == 0 &&
+      std::all_of(in.begin(), in.end(), [](unsigned char c) { return c & 1; }))
+    return;
+  host_parallel((int64_t)n, 64, [&](int64_t begin, int64_t end) {
+    for (int64_t i = begin; i < end; ++i) *(volatile char*)std::max(first + i * page, (char*)p) = 0;
+  });
+}
+
 // Between macro steps the LTS buffers hold nothing that is read again: they stage the FP64 values,
 // so that one copy per block and simulation and a kernel do what a host loop over every value did.
 static void convert_dofs(lts_t* h, double* dofs, bool to_device) {
@@ -1768,6 +1788,7 @@ static void convert_dofs(lts_t* h, double* dofs, bool to_device) {
   double* stage = reinterpret_cast<double*>(h->dst.B1);
   const int64_t block = std::max<int64_t>(1, std::min<int64_t>(K, (int64_t)(h->scratch_bytes / (sizeof(double) * per * h->nsim))));
   if (h->scratch_bytes < sizeof(double) * per * h->nsim) fail(LTS_ERR_STATE, "no room to stage the DOFs");
+  if (!to_device) fault_in(dofs, sizeof(double) * K * per * h->nsim);
   for (int64_t k0 = 0; k0 < K; k0 += block) {
     const int64_t n = std::min(block, K - k0);
     auto copy = [&](int f) {
