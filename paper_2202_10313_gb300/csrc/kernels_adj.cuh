@@ -669,10 +669,11 @@ __global__ void __launch_bounds__(AdjPredCfg<O>::THREADS, 1) k_adj_pred(DevOps o
 // accumulated. Every (receiver, face) pair is visited by exactly one owner. The four faces
 // are handled together: with LF = lambda_k F^_ip^T and XF = X F-_jh (9 x F each), the
 // transposed flux is (A+^T LF) F-_jh^T and the sums are face_products of LF and XF. Bound by
-// instruction issue (4,900 warp instructions an owner at order 4, 59 % of the issue slots, two
-// fifths of the stalls on operator-table loads), so the CTA has a thread for every (side, face,
-// face mode), then (face, face mode), (face, mode) and (row, mode): 167 us a launch against 187
-// with one warp an owner (47,040 elements, order 4, two clusters, mean of both).
+// instruction issue (59 % of the issue slots, two fifths of the stalls on operator-table loads), so
+// the CTA has a thread for every (side, face, face mode), then (face, face mode), (face, mode) and
+// (row, mode), and blocks of a multiple of 16 bytes (order 4) move four entries at a time: 147 us
+// a launch; 167 with single entries, 187 with one warp an owner (47,040 elements, order 4, two
+// clusters, mean of both).
 template <int O>
 struct AdjNbrNT {
   static constexpr int value = rup(8 * nface(O), 32);
@@ -708,6 +709,9 @@ __global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjL
   if (modes == 0) return;   // the same for every thread of the CTA
   auto mode = [modes](int i) { return ((modes >> (3 * i)) & 7) - 1; };
   constexpr int NT = AdjNbrNT<O>::value, R = (NB9 + NT - 1) / NT;
+  // order 4: rows without pads and blocks of a multiple of 16 bytes, moved four entries at a time
+  constexpr bool V4 = B % 4 == 0;
+  constexpr int V = V4 ? NB9 / 4 : 1;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     if (mode(i) >= 0) {
@@ -725,27 +729,46 @@ __global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjL
   for (int sim = 0; sim < a.nsim; ++sim) {
     // this simulation's block of the owner's buffers (stride G between modes)
     const size_t xo = (size_t)kn * a.bufs + (size_t)(sim / a.G) * (NB9 * a.G) + sim % a.G;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int m = mode(i);
-      if (m < 0) continue;
-      const int k = sF[2 * i];
-      stage_pad<B, BP, NT>(sLk[i], a.lq + ((size_t)k * a.nsim + sim) * NB9, 1, t);
-      const float* b0 = (m == 1) ? a.B3s : (m == 2) ? a.B2s : a.B1s;
-      float x[R], x2[R];
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const int q = t + j * NT;
-        x[j] = x2[j] = 0.f;
-        if (q < NB9) {
-          x[j] = __ldg(b0 + xo + (size_t)q * a.G);
-          if (m == 3) x2[j] = __ldg(a.B2s + xo + (size_t)q * a.G);
+    if (V4 && a.G == 1) {   // (fused simulations: G apart)
+      for (int p = t; p < 4 * V; p += NT) {
+        const int i = p / V, q = p % V, m = mode(i);
+        if (m < 0) continue;
+        const float* b0 = (m == 1) ? a.B3s : (m == 2) ? a.B2s : a.B1s;
+        const float4 l = __ldg(reinterpret_cast<const float4*>(a.lq + ((size_t)sF[2 * i] * a.nsim + sim) * NB9) + q);
+        float4 x = __ldg(reinterpret_cast<const float4*>(b0 + xo) + q);
+        if (m == 3) {
+          const float4 x2 = __ldg(reinterpret_cast<const float4*>(a.B2s + xo) + q);
+          x.x -= x2.x;
+          x.y -= x2.y;
+          x.z -= x2.z;
+          x.w -= x2.w;
         }
+        reinterpret_cast<float4*>(sLk[i])[q] = l;
+        reinterpret_cast<float4*>(sX[i])[q] = x;
       }
+    } else {
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const int q = t + j * NT;
-        if (q < NB9) sX[i][(q / B) * BP + q % B] = x[j] - x2[j];
+      for (int i = 0; i < 4; ++i) {
+        const int m = mode(i);
+        if (m < 0) continue;
+        const int k = sF[2 * i];
+        stage_pad<B, BP, NT>(sLk[i], a.lq + ((size_t)k * a.nsim + sim) * NB9, 1, t);
+        const float* b0 = (m == 1) ? a.B3s : (m == 2) ? a.B2s : a.B1s;
+        float x[R], x2[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          const int q = t + j * NT;
+          x[j] = x2[j] = 0.f;
+          if (q < NB9) {
+            x[j] = __ldg(b0 + xo + (size_t)q * a.G);
+            if (m == 3) x2[j] = __ldg(a.B2s + xo + (size_t)q * a.G);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          const int q = t + j * NT;
+          if (q < NB9) sX[i][(q / B) * BP + q % B] = x[j] - x2[j];
+        }
       }
     }
     __syncthreads();
@@ -799,26 +822,56 @@ __global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjL
     }
     __syncthreads();
     // the faces' contributions summed per buffer in order, then one update of each adjoint touched
-    for (int p = t; p < NB9; p += NT) {
-      float y1 = 0.f, y2 = 0.f, y3 = 0.f;
-      bool u1 = false, u2 = false, u3 = false;
+    if constexpr (V4) {
+      for (int p = t; p < V; p += NT) {
+        float4 y1 = make_float4(0.f, 0.f, 0.f, 0.f), y2 = y1, y3 = y1;
+        bool u1 = false, u2 = false, u3 = false;
+        auto add = [](float4& d, const float4& y, float sgn) {
+          d.x = fmaf(sgn, y.x, d.x);
+          d.y = fmaf(sgn, y.y, d.y);
+          d.z = fmaf(sgn, y.z, d.z);
+          d.w = fmaf(sgn, y.w, d.w);
+        };
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int m = mode(i);
-        if (m < 0) continue;
-        const float y = sLk[i][(p / B) * BP + p % B];
-        if (m == 1) y3 += y;
-        if (m == 2) y2 += y;
-        if (m == 0 || m == 3) y1 += y;
-        if (m == 3) y2 -= y;
-        u1 |= (m == 0 || m == 3);
-        u2 |= (m == 2 || m == 3);
-        u3 |= (m == 1);
+        for (int i = 0; i < 4; ++i) {
+          const int m = mode(i);
+          if (m < 0) continue;
+          const float4 y = reinterpret_cast<const float4*>(sLk[i])[p];
+          if (m == 1) add(y3, y, 1.f);
+          if (m == 2) add(y2, y, 1.f);
+          if (m == 0 || m == 3) add(y1, y, 1.f);
+          if (m == 3) add(y2, y, -1.f);
+          u1 |= (m == 0 || m == 3);
+          u2 |= (m == 2 || m == 3);
+          u3 |= (m == 1);
+        }
+        const size_t o = ((size_t)kn * a.nsim + sim) * V + p;
+        if (u1) atomicAdd(reinterpret_cast<float4*>(a.lb1) + o, y1);
+        if (u2) atomicAdd(reinterpret_cast<float4*>(a.lb2) + o, y2);
+        if (u3) atomicAdd(reinterpret_cast<float4*>(a.lb3) + o, y3);
       }
-      const size_t o = ((size_t)kn * a.nsim + sim) * NB9 + p;
-      if (u1) atomicAdd(a.lb1 + o, y1);
-      if (u2) atomicAdd(a.lb2 + o, y2);
-      if (u3) atomicAdd(a.lb3 + o, y3);
+    } else {
+      for (int p = t; p < NB9; p += NT) {
+        float y1 = 0.f, y2 = 0.f, y3 = 0.f;
+        bool u1 = false, u2 = false, u3 = false;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int m = mode(i);
+          if (m < 0) continue;
+          const float y = sLk[i][(p / B) * BP + p % B];
+          if (m == 1) y3 += y;
+          if (m == 2) y2 += y;
+          if (m == 0 || m == 3) y1 += y;
+          if (m == 3) y2 -= y;
+          u1 |= (m == 0 || m == 3);
+          u2 |= (m == 2 || m == 3);
+          u3 |= (m == 1);
+        }
+        const size_t o = ((size_t)kn * a.nsim + sim) * NB9 + p;
+        if (u1) atomicAdd(a.lb1 + o, y1);
+        if (u2) atomicAdd(a.lb2 + o, y2);
+        if (u3) atomicAdd(a.lb3 + o, y3);
+      }
     }
     __syncthreads();   // the staged blocks are refilled for the next simulation
   }
