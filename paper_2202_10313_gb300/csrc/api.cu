@@ -377,6 +377,23 @@ void host_parallel(int64_t n, int64_t grain, const Fn& fn) {
     if (failed[t]) std::rethrow_exception(failed[t]);
 }
 
+// Write to every page of [p, p + bytes) (about to be overwritten) unless all are resident: a
+// device copy into pages that the caller has not touched yet now and then takes 23 ms instead of
+// 0.7 (29 MB), faulting them in here 0.3. A look at resident pages costs a few microseconds.
+void fault_in(void* p, size_t bytes) {
+  if (bytes == 0) return;
+  const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  char* first = (char*)((uintptr_t)p / page * page);
+  const size_t n = ((char*)p + bytes - first + page - 1) / page;
+  std::vector<unsigned char> in(n);
+  if (mincore(first, n * page, in.data()) == 0 &&
+      std::all_of(in.begin(), in.end(), [](unsigned char c) { return c & 1; }))
+    return;
+  host_parallel((int64_t)n, 64, [&](int64_t begin, int64_t end) {
+    for (int64_t i = begin; i < end; ++i) *(volatile char*)std::max(first + i * page, (char*)p) = 0;
+  });
+}
+
 void setup_device(lts_solver* h) {
   const int64_t K = h->mesh.K;
   const Launchers& X = h->L;
@@ -1055,17 +1072,19 @@ void make_adj_tables(const lts_solver* h, AdjTables& T) {
 // forward set-up evaluates (host_flux.h).
 struct GradGeom {
   const double *jinv, *normal, *area, *detJ, *rho, *lam, *mu, *W;
-  const int *bc, *nbr, *nbr_face;
+  const int *bc, *nbr, *nbr_code;   // nbr_code: the neighbour's face * 3 + orientation
   const long long* iperm;
   long long K;
 };
 
 // Derivatives of one face's contraction (own and neighbour state operators with their
 // correlations) with respect to the element's rho, lam, mu and the neighbour's: out[4 k + face][6].
-// One thread per (element, face). The correlations enter as ten sums each, so that the six
-// derivatives cost six evaluations of the coefficients' closed forms; contracting 9 x 9
-// correlations column by column for each took 6.5 of 7.5 ms (47,040 elements), bound by the
-// FP64 rate.
+// One thread per (element, face). The correlations enter as ten sums each, and the material through
+// the four impedances and directly through lam, mu, 1/rho: the coefficients' closed forms are
+// evaluated once, the derivatives of the normal and the tangential pair by the own impedance in
+// one component and by the neighbour's in the other (each pair has its own coefficients). Bound
+// by the FP64 rate: six evaluations, one per parameter, took 1.0 ms (47,040 elements;
+// 0.15 now), contracting 9 x 9 correlations column by column for each 7.5.
 __global__ void k_grad_faces(GradGeom g, double* out) {
   using lts::Dual;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1076,31 +1095,31 @@ __global__ void k_grad_faces(GradGeom g, double* out) {
   const int bc = g.bc[t];
   const long long nb = g.nbr[t];
   const double *fl = Wk + ltsdev::WG_LOC + 10 * face, *fn = Wk + ltsdev::WG_NBR + 10 * face;
-  const Dual scale(-2.0 * g.area[t] / g.detJ[k]);
-  for (int p = 0; p < 6; ++p) {
-    if (p >= 3 && nb < 0) {
-      out[6 * t + p] = 0.0;
-      continue;
-    }
-    auto mat = [&](long long e, int base, Dual* m) {
-      m[0] = Dual(g.rho[e], p == base ? 1.0 : 0.0);
-      m[1] = Dual(g.lam[e], p == base + 1 ? 1.0 : 0.0);
-      m[2] = Dual(g.mu[e], p == base + 2 ? 1.0 : 0.0);
-    };
-    Dual own[3], oth[3];
-    mat(k, 0, own);
-    const Dual rinv = Dual(1.0) / own[0];
-    const Dual zp = lts::sqrt_t((own[1] + Dual(2.0) * own[2]) * own[0]), zs = lts::sqrt_t(own[2] * own[0]);
-    Dual zpo = zp, zso = zs;
-    if (nb >= 0) {
-      mat(nb, 3, oth);
-      zpo = lts::sqrt_t((oth[1] + Dual(2.0) * oth[2]) * oth[0]);
-      zso = lts::sqrt_t(oth[2] * oth[0]);
-    }
-    Dual cl[8], cn[8];
-    lts::face_coefficients_t<Dual>(bc, zp, zs, zpo, zso, scale, cl, cn);
-    out[6 * t + p] = (lts::face_flux_dot<Dual>(cl, own[1], own[2], rinv, fl) +
-                      lts::face_flux_dot<Dual>(cn, own[1], own[2], rinv, fn)).d;
+  const double rho = g.rho[k], lam = g.lam[k], mu = g.mu[k], rinv = 1.0 / rho;
+  const double zp = lts::sqrt_t((lam + 2.0 * mu) * rho), zs = lts::sqrt_t(mu * rho);
+  const Dual zpi(zp, 1.0), zsi(zs, 1.0);
+  Dual zpo = zpi, zso = zsi;
+  if (nb >= 0) {
+    zpo = Dual(lts::sqrt_t((g.lam[nb] + 2.0 * g.mu[nb]) * g.rho[nb]), 0.0, 1.0);
+    zso = Dual(lts::sqrt_t(g.mu[nb] * g.rho[nb]), 0.0, 1.0);
+  }
+  Dual cl[8], cn[8];
+  lts::face_coefficients_t<Dual>(bc, zpi, zsi, zpo, zso, Dual(-2.0 * g.area[t] / g.detJ[k]), cl, cn);
+  double dm[3] = {0.0, 0.0, 0.0}, dp[2] = {0.0, 0.0}, ds[2] = {0.0, 0.0};
+  lts::face_flux_gradient(cl, lam, mu, rinv, fl, dm, dp, ds);
+  lts::face_flux_gradient(cn, lam, mu, rinv, fn, dm, dp, ds);
+  // z_p^2 = (lam + 2 mu) rho, z_s^2 = mu rho
+  double* o = out + 6 * t;
+  const double hp = 0.5 * dp[0] / zp, hs = 0.5 * ds[0] / zs;
+  o[0] = hp * (lam + 2.0 * mu) + hs * mu - dm[2] * rinv * rinv;
+  o[1] = hp * rho + dm[0];
+  o[2] = (2.0 * hp + hs) * rho + dm[1];
+  o[3] = o[4] = o[5] = 0.0;
+  if (nb >= 0) {
+    const double np = 0.5 * dp[1] / zpo.v, ns = 0.5 * ds[1] / zso.v;
+    o[3] = np * (g.lam[nb] + 2.0 * g.mu[nb]) + ns * g.mu[nb];
+    o[4] = np * g.rho[nb];
+    o[5] = (2.0 * np + ns) * g.rho[nb];
   }
 }
 
@@ -1116,7 +1135,7 @@ __global__ void k_grad_contract(GradGeom g, const double* faces, double* grad) {
     for (int i = 0; i < 4; ++i) {
       acc += faces[6 * (4 * e + i) + p];
       const long long nb = g.nbr[4 * e + i];
-      if (nb >= 0) acc += faces[6 * (4 * nb + g.nbr_face[4 * e + i]) + 3 + p];
+      if (nb >= 0) acc += faces[6 * (4 * nb + g.nbr_code[4 * e + i] / 3) + 3 + p];
     }
     grad[3 * e + p] = acc;
   }
@@ -1157,6 +1176,53 @@ __global__ void k_build_amat(GradGeom g, float* amat) {
   for (int q = 0; q < 81; ++q) out[ltsdev::AM_NBR + i * 81 + q] = (float)M[q];
 }
 
+// Face links of the reverse neighbour pass (internal order), one thread per (element, face): fwd the
+// neighbour and its face * 3 + orientation (-1 without one), back the neighbour's face and this
+// element's face * 3 + orientation as the neighbour sees it. (Loops on one host core took 3 ms for
+// 47,040 elements, with the lists below.)
+__global__ void k_adj_links(GradGeom g, int* fwd, int* back) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 4 * g.K) return;
+  const long long k = t / 4, nb = g.nbr[t];
+  const int i = (int)(t % 4);
+  const size_t o = 8 * (size_t)g.iperm[k] + 2 * i;
+  int4 v = make_int4(-1, 0, 0, 0);
+  if (nb >= 0) {
+    const int code = g.nbr_code[t], ip = code / 3;
+    v = make_int4((int)g.iperm[nb], code, ip, i * 3 + g.nbr_code[4 * nb + ip] % 3);
+  }
+  fwd[o] = v.x;
+  fwd[o + 1] = v.y;
+  back[o] = v.z;
+  back[o + 1] = v.w;
+}
+
+// Per cluster level t, the buffer owners of a neighbour pass whose highest cluster is t that have
+// a receiver in clusters 0..t: own[off[t] ..], count[t] of them. Their order varies from run to
+// run; every value of the pass has one owner as its only writer, so its results do not.
+struct OwnerLevels {
+  int beg[ltsdev::MAXC + 1], off[ltsdev::MAXC], nc;
+};
+__global__ void k_adj_owners(const int* fwd, OwnerLevels lv, int* own, int* count) {
+  const int kn = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const bool in = kn < lv.beg[lv.nc];
+  int first = 0x7fffffff;   // the receiver of the finest cluster
+  if (in)
+    for (int i = 0; i < 4; ++i) {
+      const int k = fwd[8 * (size_t)kn + 2 * i];
+      if (k >= 0) first = min(first, k);
+    }
+  for (int t = 0; t < lv.nc; ++t) {
+    const bool take = in && kn < lv.beg[min(t + 2, lv.nc)] && first < lv.beg[t + 1];
+    const unsigned mask = __ballot_sync(0xffffffffu, take);
+    if (mask == 0) continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(count + t, __popc(mask));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (take) own[lv.off[t] + base + __popc(mask & ((1u << lane) - 1))] = kn;
+  }
+}
+
 // Geometry and material of every element on the device (original element order), for the
 // operator build and the gradient contraction; the buffers live as long as `bufs`.
 struct GeoBufs {
@@ -1165,12 +1231,12 @@ struct GeoBufs {
 GradGeom upload_geometry(const lts_solver* h, GeoBufs& bufs, cudaStream_t stream) {
   const lts::Mesh& M = h->mesh;
   const int64_t K = M.K;
-  std::vector<int> bc(4 * K), nbr(4 * K), nface(4 * K);
+  std::vector<int> bc(4 * K), nbr(4 * K), code(4 * K);
   std::vector<long long> iperm(K);
   for (int64_t i = 0; i < 4 * K; ++i) {
     bc[i] = M.bc[i];
     nbr[i] = (int)M.nbr[i];
-    nface[i] = M.nbr_face[i];
+    code[i] = M.nbr[i] < 0 ? 0 : M.nbr_face[i] * 3 + M.nbr_orient[i];
   }
   for (int64_t k = 0; k < K; ++k) iperm[k] = (long long)h->iperm[k];
   const size_t nd = (size_t)K * (9 + 12 + 4 + 1 + 3);
@@ -1192,7 +1258,7 @@ GradGeom upload_geometry(const lts_solver* h, GeoBufs& bufs, cudaStream_t stream
   g.mu = geo + 28 * K;
   g.bc = in;
   g.nbr = in + 4 * K;
-  g.nbr_face = in + 8 * K;
+  g.nbr_code = in + 8 * K;
   g.iperm = bufs.perm.get<long long>();
   g.K = K;
   up(const_cast<double*>(g.jinv), M.Jinv.data(), sizeof(double) * 9 * K);
@@ -1204,7 +1270,7 @@ GradGeom upload_geometry(const lts_solver* h, GeoBufs& bufs, cudaStream_t stream
   up(const_cast<double*>(g.mu), h->mu.data(), sizeof(double) * K);
   up(in, bc.data(), sizeof(int) * 4 * K);
   up(in + 4 * K, nbr.data(), sizeof(int) * 4 * K);
-  up(in + 8 * K, nface.data(), sizeof(int) * 4 * K);
+  up(in + 8 * K, code.data(), sizeof(int) * 4 * K);
   up(bufs.perm.p, iperm.data(), sizeof(long long) * K);
   // the host vectors must outlive the copies: the stream is synchronised before they go
   ck(cudaStreamSynchronize(stream), "synchronize");
@@ -1243,7 +1309,7 @@ __global__ void k_adjoint_to_caller(const float* lam, double* out, const int* ip
 void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* data, double* misfit, double* grad,
                  double* synth_out, double* dq0, cudaStream_t stream, const DevBuf& d_amat, const DevBuf& d_fwd,
                  const DevBuf& d_back, const DevBuf& d_relem, const DevBuf& d_rphi, int nrec, const AdjTables& tabs,
-                 const GradGeom& geo, const DevBuf& d_own, const std::vector<int64_t>& own_off) {
+                 const GradGeom& geo, const DevBuf& d_own, const DevBuf& d_cnt, const OwnerLevels& lv) {
   const Launchers& X = h->L;
   const int64_t K = h->mesh.K;
   const int B = X.B, NB9 = 9 * B;
@@ -1370,6 +1436,9 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   if (reverse) dcopy(d_qn.p, h->dst.Q, qbytes);
   std::vector<float> syn((size_t)(n_macro + 1) * ns);
   ck(cudaMemcpyAsync(syn.data(), d_syn.p, sizeof(float) * syn.size(), cudaMemcpyDeviceToHost, stream), "samples");
+  int owners_at[ltsdev::MAXC] = {};
+  if (reverse)
+    ck(cudaMemcpyAsync(owners_at, d_cnt.p, sizeof(int) * h->nc, cudaMemcpyDeviceToHost, stream), "owner counts");
   ck(cudaStreamSynchronize(stream), "synchronize");
   check_device_error(h);
   std::vector<float> res(syn.size());
@@ -1463,8 +1532,8 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
         aa.B2s = base + (size_t)owners * bs;
         aa.B3s = base + 2 * (size_t)owners * bs;
         aa.bufs = bs;
-        aa.owners = d_own.get<int>() + own_off[ph.top];
-        X.adj_nbr(h->dops, aa, pa, (int)(own_off[ph.top + 1] - own_off[ph.top]), stream);
+        aa.owners = d_own.get<int>() + lv.off[ph.top];
+        X.adj_nbr(h->dops, aa, pa, owners_at[ph.top], stream);
       }
     }
     X.adj_source(d_lq.get<float>(), nsim, relem, rphi, d_res.get<float>() + m * ns, nrec, stream);
@@ -1520,6 +1589,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   if (nsrc > 0)
     ck(cudaMemcpyAsync(h->adj_src_grad.data(), d_sg.p, sizeof(double) * nsrc * 6, cudaMemcpyDeviceToHost, stream),
        "source gradient");
+  if (dq0) fault_in(dq0, sizeof(double) * (size_t)K * nsim * NB9);   // while the sweep runs
   if (dq0) {   // [sim][element (original order)][9][B] in FP64, staged in the buffer adjoints (12 bytes a value)
     const int64_t total = (int64_t)K * nsim * NB9;
     k_adjoint_to_caller<<<(unsigned)std::min<int64_t>((total + 255) / 256, 16 * (int64_t)h->num_sms), 256, 0, stream>>>(
@@ -1762,23 +1832,6 @@ static __global__ void k_convert_dofs(float* Q, double* stage, const int* iperm,
     else
       stage[i] = *q;
   }
-}
-
-// Write to every page of [p, p + bytes) (about to be overwritten) unless all are resident: a
-// device copy into pages that the caller has not touched yet now and then takes 23 ms instead of
-// 0.7 (29 MB), faulting them in here 0.3. A look at resident pages costs a few microseconds.
-static void fault_in(void* p, size_t bytes) {
-  if (bytes == 0) return;
-  const size_t page = (size_t)sysconf(_SC_PAGESIZE);
-  char* first = (char*)((uintptr_t)p / page * page);
-  const size_t n = ((char*)p + bytes - first + page - 1) / page;
-  std::vector<unsigned char> in(n);
-  if (mincore(first, n * page, in.data()) == 0 &&
-      std::all_of(in.begin(), in.end(), [](unsigned char c) { return c & 1; }))
-    return;
-  host_parallel((int64_t)n, 64, [&](int64_t begin, int64_t end) {
-    for (int64_t i = begin; i < end; ++i) *(volatile char*)std::max(first + i * page, (char*)p) = 0;
-  });
 }
 
 // Between macro steps the LTS buffers hold nothing that is read again: they stage the FP64 values,
@@ -2395,71 +2448,54 @@ int lts_misfit_gradient(lts_t* h, int64_t n_steps, int64_t every, const double* 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const int64_t K = h->mesh.K;
     const int B = X.B;
-    // ---- face links (internal order)
-    std::vector<int> fwd(8 * K, -1), back(8 * K, 0);
-    for (int64_t k = 0; k < K; ++k) {
-      const int64_t nk = h->iperm[k];
-      for (int i = 0; i < 4; ++i) {
-        const int64_t nb = h->mesh.nbr[4 * k + i];
-        if (nb < 0) continue;
-        const int ip = h->mesh.nbr_face[4 * k + i];
-        fwd[8 * nk + 2 * i] = (int)h->iperm[nb];
-        fwd[8 * nk + 2 * i + 1] = ip * 3 + h->mesh.nbr_orient[4 * k + i];
-        back[8 * nk + 2 * i] = ip;
-        back[8 * nk + 2 * i + 1] = i * 3 + h->mesh.nbr_orient[4 * nb + ip];
-      }
-    }
-    // per cluster level t, the buffer owners of a neighbour pass whose highest cluster is t
-    // that have a receiver in clusters 0..t (internal order, ascending)
-    std::vector<int> own;
-    std::vector<int64_t> own_off(1, 0);
-    for (int t = 0; t < h->nc; ++t) {
-      const int64_t nown = h->cbeg[std::min(t + 2, h->nc)], nact = h->cbeg[t + 1];
-      for (int64_t kn = 0; kn < nown; ++kn)
-        for (int i = 0; i < 4; ++i) {
-          const int k = fwd[8 * kn + 2 * i];
-          if (k >= 0 && k < nact) {
-            own.push_back((int)kn);
-            break;
-          }
-        }
-      own_off.push_back((int64_t)own.size());
-    }
     std::vector<int> relem(nrec);
     std::vector<float> rphi((size_t)nrec * B);
     for (int r = 0; r < nrec; ++r) {
       relem[r] = (int)h->iperm[h->receivers[r].elem];
       for (int b = 0; b < B; ++b) rphi[(size_t)r * B + b] = (float)h->receivers[r].phi[b];
     }
-    // ---- device buffers; the explicit operators (reverse sweep only) are built on the device
-    DevBuf d_amat, d_fwd, d_back, d_relem, d_rphi, d_own;
+    // ---- device buffers; operators, face links and owner lists (reverse sweep only) are built on
+    // the device
+    DevBuf d_amat, d_fwd, d_back, d_relem, d_rphi, d_own, d_cnt;
     GeoBufs geo_bufs;
     GradGeom geo{};
+    OwnerLevels lv{};
     if (grad || dq0) {
       geo = upload_geometry(h, geo_bufs, stream);
       d_amat.alloc(sizeof(float) * K * ltsdev::AM_SIZE);
       const long long nt = 5 * K;
       k_build_amat<<<(unsigned)((nt + 127) / 128), 128, 0, stream>>>(geo, d_amat.get<float>());
       ck(cudaGetLastError(), "operator build");
+      lv.nc = h->nc;
+      int64_t owners = 0;
+      for (int t = 0; t <= h->nc; ++t) lv.beg[t] = (int)h->cbeg[t];
+      for (int t = 0; t < h->nc; ++t) {
+        lv.off[t] = (int)owners;
+        owners += h->cbeg[std::min(t + 2, h->nc)];
+      }
+      if (owners > INT32_MAX) fail(LTS_ERR_ARG, "mesh too large for the adjoint");
+      d_fwd.alloc(sizeof(int) * 8 * K);
+      d_back.alloc(sizeof(int) * 8 * K);
+      d_own.alloc(sizeof(int) * owners);
+      d_cnt.alloc(sizeof(int) * ltsdev::MAXC);
+      ck(cudaMemsetAsync(d_cnt.p, 0, sizeof(int) * ltsdev::MAXC, stream), "memset");
+      k_adj_links<<<(unsigned)((4 * K + 255) / 256), 256, 0, stream>>>(geo, d_fwd.get<int>(), d_back.get<int>());
+      k_adj_owners<<<(unsigned)((K + 255) / 256), 256, 0, stream>>>(d_fwd.get<int>(), lv, d_own.get<int>(),
+                                                                   d_cnt.get<int>());
+      ck(cudaGetLastError(), "face links");
     }
-    d_fwd.alloc(sizeof(int) * fwd.size());
-    d_back.alloc(sizeof(int) * back.size());
     d_relem.alloc(sizeof(int) * nrec);
     d_rphi.alloc(sizeof(float) * rphi.size());
     auto up = [&](void* dst, const void* src, size_t bytes) {
       ck(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream), "adjoint upload");
     };
-    up(d_fwd.p, fwd.data(), sizeof(int) * fwd.size());
-    up(d_back.p, back.data(), sizeof(int) * back.size());
-    d_own.alloc(sizeof(int) * own.size());
-    up(d_own.p, own.data(), sizeof(int) * own.size());
     up(d_relem.p, relem.data(), sizeof(int) * nrec);
     up(d_rphi.p, rphi.data(), sizeof(float) * rphi.size());
     AdjTables tabs;
     make_adj_tables(h, tabs);
     // the phase-level sweep for every cluster count (one cluster: a macro step is one step)
     adjoint_lts(h, n_steps / period, every, data, misfit, grad, synth_out, dq0, stream, d_amat, d_fwd, d_back,
-                d_relem, d_rphi, nrec, tabs, geo, d_own, own_off);
+                d_relem, d_rphi, nrec, tabs, geo, d_own, d_cnt, lv);
   });
 }
 

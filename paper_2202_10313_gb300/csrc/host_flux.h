@@ -103,36 +103,45 @@ LTS_HD void face_flux_matrix(const double n[3], const T c[8], T lam, T mu, T rin
 // The contraction sum_{q,j} M[q][j] l[q] x[j] of that matrix as a form in its coefficients: the
 // flux is linear in (lam, mu, rinv) and in (v*, t*), and those in the coefficients, so ten sums f
 // of (l, x) and the normal alone hold everything that does not depend on the material
-// (ltsdev::face_products; the tangential coefficients do not meet lam, n v*_T = 0).
+// (ltsdev::face_products; the tangential coefficients do not meet lam, n v*_T = 0):
+//   lam (c0 f0 + c1 f1) + mu (c0 f2 + c1 f3 + c4 f4 + c5 f5)
+//   + rinv (c2 f6 + c3 f7 + c6 f8 + c7 f9).
+// Its derivatives with respect to lam, mu, rinv (added to dm) and, through the coefficients, to
+// the two components of the normal pair's and the tangential pair's impedances (dp, ds).
 template <typename T>
-LTS_HD T face_flux_dot(const T c[8], T lam, T mu, T rinv, const double f[10]) {
-  return lam * (c[0] * f[0] + c[1] * f[1]) + mu * (c[0] * f[2] + c[1] * f[3] + c[4] * f[4] + c[5] * f[5]) +
-         rinv * (c[2] * f[6] + c[3] * f[7] + c[6] * f[8] + c[7] * f[9]);
+LTS_HD void face_flux_gradient(const T c[8], double lam, double mu, double rinv, const double f[10], double dm[3],
+                               double dp[2], double ds[2]) {
+  dm[0] += c[0].v * f[0] + c[1].v * f[1];
+  dm[1] += c[0].v * f[2] + c[1].v * f[3] + c[4].v * f[4] + c[5].v * f[5];
+  dm[2] += c[2].v * f[6] + c[3].v * f[7] + c[6].v * f[8] + c[7].v * f[9];
+  const double w0 = lam * f[0] + mu * f[2], w1 = lam * f[1] + mu * f[3];
+  for (int i = 0; i < 2; ++i) {
+    dp[i] += c[0].d[i] * w0 + c[1].d[i] * w1 + rinv * (c[2].d[i] * f[6] + c[3].d[i] * f[7]);
+    ds[i] += mu * (c[4].d[i] * f[4] + c[5].d[i] * f[5]) + rinv * (c[6].d[i] * f[8] + c[7].d[i] * f[9]);
+  }
 }
 
-// Forward-mode dual number with one derivative component.
+// Forward-mode dual number with two derivative components.
 struct Dual {
-  double v, d;
-  LTS_HD Dual(double x = 0.0, double dx = 0.0) : v(x), d(dx) {}
+  double v, d[2];
+  LTS_HD Dual(double x = 0.0, double d0 = 0.0, double d1 = 0.0) : v(x), d{d0, d1} {}
 };
-LTS_HD inline Dual operator+(Dual a, Dual b) { return Dual(a.v + b.v, a.d + b.d); }
-LTS_HD inline Dual operator-(Dual a, Dual b) { return Dual(a.v - b.v, a.d - b.d); }
-LTS_HD inline Dual operator-(Dual a) { return Dual(-a.v, -a.d); }
-LTS_HD inline Dual operator*(Dual a, Dual b) { return Dual(a.v * b.v, a.d * b.v + a.v * b.d); }
-LTS_HD inline Dual operator/(Dual a, Dual b) { return Dual(a.v / b.v, (a.d * b.v - a.v * b.d) / (b.v * b.v)); }
-LTS_HD inline Dual operator*(Dual a, double b) { return Dual(a.v * b, a.d * b); }
-LTS_HD inline Dual operator*(double a, Dual b) { return Dual(a * b.v, a * b.d); }
-LTS_HD inline double sqrt_d(double a) {
+LTS_HD inline Dual operator+(Dual a, Dual b) { return Dual(a.v + b.v, a.d[0] + b.d[0], a.d[1] + b.d[1]); }
+LTS_HD inline Dual operator-(Dual a, Dual b) { return Dual(a.v - b.v, a.d[0] - b.d[0], a.d[1] - b.d[1]); }
+LTS_HD inline Dual operator-(Dual a) { return Dual(-a.v, -a.d[0], -a.d[1]); }
+LTS_HD inline Dual operator*(Dual a, Dual b) {
+  return Dual(a.v * b.v, a.d[0] * b.v + a.v * b.d[0], a.d[1] * b.v + a.v * b.d[1]);
+}
+LTS_HD inline Dual operator/(Dual a, Dual b) {
+  const double r = 1.0 / b.v, q = a.v * r;
+  return Dual(q, (a.d[0] - q * b.d[0]) * r, (a.d[1] - q * b.d[1]) * r);
+}
+LTS_HD inline double sqrt_t(double a) {
 #ifdef __CUDA_ARCH__
   return ::sqrt(a);
 #else
   return std::sqrt(a);
 #endif
 }
-LTS_HD inline Dual sqrt_t(Dual a) {
-  const double s = sqrt_d(a.v);
-  return Dual(s, a.d / (2.0 * s));
-}
-LTS_HD inline double sqrt_t(double a) { return sqrt_d(a); }
 
 }  // namespace lts
