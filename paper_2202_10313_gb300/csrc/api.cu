@@ -127,6 +127,7 @@ struct lts_solver {
   double lambda = 1.0, dt_min = 0.0, delta = 0.0, speedup = 1.0;
   std::vector<int32_t> cluster;             // original order
   std::vector<int64_t> perm, iperm;         // perm[new] = old, iperm[old] = new
+  std::vector<int> meta;                    // cluster and buffer roles (internal order), as on the device
   std::vector<int64_t> cbeg;                // cluster ranges (internal order), nc+1
   int64_t s_now = 0;
   int64_t launches = 0;
@@ -605,6 +606,7 @@ void setup_device(lts_solver* h) {
   up(h->dst.nbr, nbr.data(), sizeof(int) * nbr.size());
   up(h->dst.ncode, ncode.data(), sizeof(int) * ncode.size());
   up(h->dst.meta, meta.data(), sizeof(int) * meta.size());
+  h->meta = meta;
   up(h->d_emat, emat.data(), sizeof(double) * emat.size());
   up(h->dops.K, hK.data(), sizeof(float) * hK.size());
   up(h->dops.Ft, hFt.data(), sizeof(float) * hFt.size());
@@ -1291,11 +1293,15 @@ void contract_gradient(GradGeom g, const double* d_w, double* grad, cudaStream_t
   ck(cudaStreamSynchronize(stream), "synchronize");
 }
 
+// dst[i] = src[rows[i]], rows of n4 16-byte units.
+__global__ void k_gather_rows(const float4* __restrict__ src, const int* __restrict__ rows, float4* __restrict__ dst,
+                              long long n, int n4) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n * n4; i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / n4;
+    dst[i] = src[(size_t)rows[r] * n4 + i % n4];
+  }
+}
 
-// Clustered-LTS branch of lts_misfit_gradient: samples at the macro-step boundaries, Q
-// checkpoints every `every` macro steps, and per macro step a phase-by-phase recompute
-// that keeps Q before each predict pass and the buffers before each neighbour pass for the
-// reverse sweep (k_adj_pred / k_adj_nbr, phases in reverse order).
 // The adjoint of Q ([element][sim][9][B], internal order) as [sim][element][9][B], caller's order.
 __global__ void k_adjoint_to_caller(const float* lam, double* out, const int* iperm, int64_t K, int nsim, int nb9) {
   const int64_t total = K * nsim * nb9;
@@ -1306,6 +1312,10 @@ __global__ void k_adjoint_to_caller(const float* lam, double* out, const int* ip
   }
 }
 
+// Clustered-LTS branch of lts_misfit_gradient: samples at the macro-step boundaries, Q
+// checkpoints every `every` macro steps, and per macro step a phase-by-phase recompute
+// that keeps Q before each predict pass and the buffers before each neighbour pass for the
+// reverse sweep (k_adj_pred / k_adj_nbr, phases in reverse order).
 void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* data, double* misfit, double* grad,
                  double* synth_out, double* dq0, cudaStream_t stream, const DevBuf& d_amat, const DevBuf& d_fwd,
                  const DevBuf& d_back, const DevBuf& d_relem, const DevBuf& d_rphi, int nrec, const AdjTables& tabs,
@@ -1354,10 +1364,42 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   const int64_t s0 = h->s_now;
   std::vector<size_t> nrec_t(nrec);
   MacroPlan mp;
+  // the elements with a B2 (a finer neighbour) and with a B3 (a coarser one): their list and each
+  // element's place in it, and how many lie in clusters 0..t-1
+  std::vector<int> role_rows[2], role_slot(2 * K, 0);
+  std::vector<int64_t> role_cnt[2];
+  for (int w = 0; w < 2; ++w) {
+    const int flag = w == 0 ? ltsdev::FLAG_FINER : ltsdev::FLAG_COARSER;
+    for (int64_t k = 0; k < K; ++k)
+      if (h->meta[k] & flag) {
+        role_slot[w * K + k] = (int)role_rows[w].size();
+        role_rows[w].push_back((int)k);
+      }
+    for (int t = 0; t <= h->nc; ++t)
+      role_cnt[w].push_back(std::lower_bound(role_rows[w].begin(), role_rows[w].end(), (int)h->cbeg[t]) -
+                            role_rows[w].begin());
+  }
+  DevBuf d_roles;   // the two lists, then the places
+  const int* d_rows[2] = {nullptr, nullptr};
+  if (reverse) {
+    const size_t n2 = role_rows[0].size(), n3 = role_rows[1].size();
+    d_roles.alloc(sizeof(int) * (n2 + n3 + 2 * K));
+    int* p = d_roles.get<int>();
+    d_rows[0] = p;
+    d_rows[1] = p + n2;
+    auto up = [&](int* dst, const std::vector<int>& v) {
+      if (!v.empty())
+        ck(cudaMemcpyAsync(dst, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice, stream), "buffer roles");
+    };
+    up(p, role_rows[0]);
+    up(p + n2, role_rows[1]);
+    up(p + n2 + n3, role_slot);
+  }
   // Phase layout of a macro step (the same for every macro step; the step indices are
   // relative) and the bytes each phase's reverse reads: Q of the active elements before a
-  // predict pass, B1, B2, B3 of the buffer owners before a neighbour pass. Elements are in
-  // cluster order, so both are prefixes.
+  // predict pass, B1 of the buffer owners and the B2 and B3 that there are before a neighbour pass.
+  // Elements are in cluster order, so all are prefixes. (B2 and B3 of every owner doubled what a macro
+  // step holds: copying and freeing them took 4 of 42 ms for 47,040 elements and 64 steps.)
   std::vector<Phase> lay;
   std::vector<size_t> snap_off, snap_len;
   size_t per_macro = 0;
@@ -1373,8 +1415,9 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
       Phase q = ph;
       q.s -= s0;
       lay.push_back(q);
-      const int64_t n = ph.kind == 1 ? h->cbeg[ph.top + 1] : h->cbeg[std::min(ph.top + 2, h->nc)];
-      const size_t len = ph.kind == 1 ? sizeof(float) * n * qs : 3 * sizeof(float) * n * bs;
+      const int t = std::min(ph.top + 2, h->nc);
+      const size_t len = ph.kind == 1 ? sizeof(float) * h->cbeg[ph.top + 1] * qs
+                                      : sizeof(float) * (h->cbeg[t] + role_cnt[0][t] + role_cnt[1][t]) * bs;
       snap_off.push_back(per_macro);
       snap_len.push_back(len);
       per_macro += (len + 255) / 256 * 256;
@@ -1398,10 +1441,19 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
     if (ph.kind == 1) {
       dcopy(dst, h->dst.Q, snap_len[pi]);
     } else {
-      const size_t one = snap_len[pi] / 3;
-      dcopy(dst, h->dst.B1, one);
-      dcopy(dst + one, h->dst.B2, one);
-      dcopy(dst + 2 * one, h->dst.B3, one);
+      const int t = std::min(ph.top + 2, h->nc);
+      float* d = reinterpret_cast<float*>(dst);
+      dcopy(d, h->dst.B1, sizeof(float) * h->cbeg[t] * bs);
+      d += h->cbeg[t] * bs;
+      const float* src[2] = {h->dst.B2, h->dst.B3};
+      for (int w = 0; w < 2; ++w) {
+        const int64_t n = role_cnt[w][t] * (bs / 4);
+        if (n == 0) continue;
+        k_gather_rows<<<(unsigned)std::min<int64_t>((n + 255) / 256, 16 * (int64_t)h->num_sms), 256, 0, stream>>>(
+            reinterpret_cast<const float4*>(src[w]), d_rows[w], reinterpret_cast<float4*>(d), role_cnt[w][t], (int)(bs / 4));
+        ck(cudaGetLastError(), "adjoint copy");
+        d += role_cnt[w][t] * bs;
+      }
     }
   };
   auto keep_macro = [&](int64_t m, char* snap_m) {
@@ -1477,6 +1529,8 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   aa.FbT = tabs.FbT;
   aa.qs = qs;
   aa.bufs = bs;
+  aa.slot2 = d_rows[1] + role_rows[1].size();
+  aa.slot3 = aa.slot2 + K;
   auto phase_at = [&](size_t pi, int64_t sb0) {
     Phase q = lay[pi];
     q.s += sb0;
@@ -1530,7 +1584,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
         const int owners = (int)h->cbeg[std::min(ph.top + 2, h->nc)];
         aa.B1s = base;
         aa.B2s = base + (size_t)owners * bs;
-        aa.B3s = base + 2 * (size_t)owners * bs;
+        aa.B3s = aa.B2s + (size_t)role_cnt[0][std::min(ph.top + 2, h->nc)] * bs;
         aa.bufs = bs;
         aa.owners = d_own.get<int>() + lv.off[ph.top];
         X.adj_nbr(h->dops, aa, pa, owners_at[ph.top], stream);

@@ -111,7 +111,9 @@ __global__ void k_adj_src_grad(const float* lam, int nsim, const SrcItem* items,
 // accumulation) and runs the transposed time kernel with both Taylor weights.
 struct AdjLtsArgs {
   const float* Qs;                    // Q before this predict pass (element stride qs)
-  const float *B1s, *B2s, *B3s;       // buffers before this neighbour pass (element stride bufs)
+  const float *B1s, *B2s, *B3s;       // buffers before this neighbour pass (element stride bufs): B1 of
+                                      // every owner, B2 and B3 of the elements that have one, at
+  const int *slot2, *slot3;           // their rows slot2, slot3
   float* lq;                          // [K][9B] adjoint of Q
   float *lb1, *lb2, *lb3;             // [K][9B] adjoints of B1, B2, B3
   const float* amat;
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjL
   __syncthreads();
   // buffer each active receiver read: 0 B1 (same cluster), 1 B3 (receiver coarser),
   // 2 B2 / 3 B1 - B2 (receiver finer, first / second half); -1 receiver not active
-  const int lo = a.meta[kn] & 0xff;
+  const int lo = a.meta[kn] & 0xff, s2 = a.slot2[kn], s3 = a.slot3[kn];
   // modes packed 3 bits per face as mode + 1, so that a runtime face index needs no stack
   int modes = 0;
 #pragma unroll
@@ -728,16 +730,19 @@ __global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjL
   }
   for (int sim = 0; sim < a.nsim; ++sim) {
     // this simulation's block of the owner's buffers (stride G between modes)
-    const size_t xo = (size_t)kn * a.bufs + (size_t)(sim / a.G) * (NB9 * a.G) + sim % a.G;
+    const size_t so = (size_t)(sim / a.G) * (NB9 * a.G) + sim % a.G;
+    const float* b1 = a.B1s + (size_t)kn * a.bufs + so;
+    const float* b2 = a.B2s + (size_t)s2 * a.bufs + so;
+    const float* b3 = a.B3s + (size_t)s3 * a.bufs + so;
     if (V4 && a.G == 1) {   // (fused simulations: G apart)
       for (int p = t; p < 4 * V; p += NT) {
         const int i = p / V, q = p % V, m = mode(i);
         if (m < 0) continue;
-        const float* b0 = (m == 1) ? a.B3s : (m == 2) ? a.B2s : a.B1s;
+        const float* b0 = (m == 1) ? b3 : (m == 2) ? b2 : b1;
         const float4 l = __ldg(reinterpret_cast<const float4*>(a.lq + ((size_t)sF[2 * i] * a.nsim + sim) * NB9) + q);
-        float4 x = __ldg(reinterpret_cast<const float4*>(b0 + xo) + q);
+        float4 x = __ldg(reinterpret_cast<const float4*>(b0) + q);
         if (m == 3) {
-          const float4 x2 = __ldg(reinterpret_cast<const float4*>(a.B2s + xo) + q);
+          const float4 x2 = __ldg(reinterpret_cast<const float4*>(b2) + q);
           x.x -= x2.x;
           x.y -= x2.y;
           x.z -= x2.z;
@@ -753,15 +758,15 @@ __global__ void __launch_bounds__(AdjNbrNT<O>::value) k_adj_nbr(DevOps ops, AdjL
         if (m < 0) continue;
         const int k = sF[2 * i];
         stage_pad<B, BP, NT>(sLk[i], a.lq + ((size_t)k * a.nsim + sim) * NB9, 1, t);
-        const float* b0 = (m == 1) ? a.B3s : (m == 2) ? a.B2s : a.B1s;
+        const float* b0 = (m == 1) ? b3 : (m == 2) ? b2 : b1;
         float x[R], x2[R];
 #pragma unroll
         for (int j = 0; j < R; ++j) {
           const int q = t + j * NT;
           x[j] = x2[j] = 0.f;
           if (q < NB9) {
-            x[j] = __ldg(b0 + xo + (size_t)q * a.G);
-            if (m == 3) x2[j] = __ldg(a.B2s + xo + (size_t)q * a.G);
+            x[j] = __ldg(b0 + (size_t)q * a.G);
+            if (m == 3) x2[j] = __ldg(b2 + (size_t)q * a.G);
           }
         }
 #pragma unroll
