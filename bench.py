@@ -342,8 +342,8 @@ def run_ours(args, rank, world, local_rank):
     fl = fl_block
     if engine == "sparse" and F == 1:
         fl = perfmodel.flops_predict_sparse(order, nmech) if kind == 0 else perfmodel.flops_neighbour_sparse(order, nmech)
-    by = (perfmodel.bytes_predict(order, nmech, n_fused=F) if kind == 0
-          else perfmodel.bytes_neighbour(order, nmech, n_fused=F))
+    sp = "_sparse" if engine == "sparse" and args.partition <= 1 else ""
+    by = getattr(perfmodel, ("bytes_predict" if kind == 0 else "bytes_neighbour") + sp)(order, nmech, n_fused=F)
     achieved_tf = fl * elems_per_launch / (avg_ms / 1000.0) / 1e12
     achieved_gbs = by * elems_per_launch / (avg_ms / 1000.0) / 1e9
     traffic = None

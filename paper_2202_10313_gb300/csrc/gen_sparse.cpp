@@ -1,4 +1,5 @@
-// Build-time generator of the sparse operator products of k_predict_sp (ahead-of-time
+// Build-time generator of the sparse operator products of k_predict_sp, k_neighbour_sp and
+// k_adj_pred_sp (ahead-of-time
 // specialisation, the GPU counterpart of the paper's generated sparse kernels, Sec. IV-A
 // "all sparsity" and Sec. IV-B).
 //
@@ -15,17 +16,22 @@
 // contiguous run of the outputs ordered by mode, so its outputs share most of their inputs
 // and a thread loads only the inputs its part uses.
 //
-// Emitted, per order O and part count P (O = 3, 4, 5 with P = 1, 2, 4):
+// Emitted, per order O, with one part per thread group (O = 3, 4, 5: 1, 2, 4) for the discrete
+// adjoint's reverse predict pass (k_adj_pred_sp):
 //   sp_time_o{O}(part, variant, x, y): Y_c[b] = sum_k x[k] K_c[b][k]        (time kernel,
 //       d^{d+1}Q from d^dQ; K_c[b][k] != 0 only for deg b < deg k). Variant v takes only
 //       the modes k < nbasis(O - v) and outputs b < nbasis(O - 1 - v) (the elastic time
 //       kernel's degree truncation at derivative v; v = 0 is the full product).
-//   sp_vol_o{O}(part, x, y, g): Z_c[b] = sum_k x[k] K_c[k][b] (volume kernel) and
-//       G_i[f] = sum_k x[k] F~_i[k][f] (local face traces), from the same row.
-//   sp_proj_o{O}(part, x, y): P_i[b] = sum_f x[i F + f] F^_i[f][b] (projection of one row of
-//       the four faces' interface states, F^_i = F~_i^T in the orthonormal face basis).
-//   sp_ntrace_o{O}(j, x, y): G_j[f] = sum_k x[k] F~_j[k][f] of one row of a neighbour's
-//       buffer on the face j that each thread asks for (neighbour kernel).
+//   sp_trace_o{O}(part, x, g): the face traces G_i[f] = sum_k x[k] F~_i[k][f].
+//   sp_tproj_o{O}(part, x, y): y[b] = sum_i sum_f x[i F + f] F~_i[b][f] (the transposed face
+//       traces of the four faces, summed).
+//   sp_kvol_o{O}(part, variant, x, y): Z_c[b] = sum_k x[k] K_c[k][b] for 1 <= b < nbasis(O - v)
+//       (the reverse time kernel at level v; K_c[k][b] != 0 only for deg k < deg b, so the
+//       inputs are k < nbasis(O - 1 - v)).
+// x[k * XP] is the thread's row, y[(c B + b) XP] and g[(i F + f) XP] the outputs (XP the pair
+// stride of the staging arrays, a template parameter so that every address is an immediate
+// offset). Every output the kernel reads is written (identically zero ones as 0); Z_c[0], which
+// vanishes for every c, is not.
 // The forward kernels' products come in row form (sg_*): a thread holds one row of a set,
 // contiguous in memory, and reads and writes it four modes at a time. Set c (0, 1, 2: reference
 // direction xi_c; 3: the direction of the fourth barycentric coordinate) has six rows: the
@@ -41,28 +47,17 @@
 // (x, y: the row of set 0; dx: the distance between a thread's rows of consecutive sets, 0 for
 // the velocities, which all sets share; DY, DG template parameters). Outputs are split into parts
 // by set (partition_sets).
-// and for the reverse predict pass of the discrete adjoint (k_adj_pred_sp):
-//   sp_trace_o{O}(part, x, g): G_i[f] = sum_k x[k] F~_i[k][f] alone (the traces of sp_vol).
-//   sp_tproj_o{O}(part, x, y): y[b] = sum_i sum_f x[i F + f] F~_i[b][f] (the transposed face
-//       traces of the four faces, summed).
-//   sp_kvol_o{O}(part, variant, x, y): Z_c[b] = sum_k x[k] K_c[k][b] for 1 <= b < nbasis(O - v)
-//       (the reverse time kernel at level v; K_c[k][b] != 0 only for deg k < deg b, so the
-//       inputs are k < nbasis(O - 1 - v)).
-// x[k * XP] is the thread's row, y[(c B + b) XP] (or y[(i B + b) XP]) and g[(i F + f) XP]
-// the outputs (XP the pair stride of the staging arrays, a template parameter so that
-// every address is an immediate offset). Every output the kernel reads is written
-// (identically zero ones as 0); Z_c[0], which vanishes for every c, is not.
 //
 // Usage: gen_sparse <out.cuh>      writes the header
 //        gen_sparse --list <order> lists every product term, one line each:
-//        gen_sparse --list-rows <order> lists the terms of the row-form products likewise:
-//        kind T (output c B + b, input c B + k), V (volume, the same), G (trace, output f F + m,
-//        input k) or P (output f B + b, input f F + m);
 //        "<kind> <part> <output> <input> <value>", kind t (time kernel, output c B + b, full
 //        variant), v (volume, output c B + b), g (face trace, output i F + f), p (face
 //        projection, output i B + b, input i F + f), n (neighbour face trace, output j F + f),
 //        s (summed transposed traces, output b, input i F + f) or k (reverse time kernel,
 //        output c B + b, full variant); for checks against other operators.
+//        gen_sparse --list-rows <order> lists the terms of the row-form products likewise:
+//        kind T (output c B + b, input c B + k), V (volume, the same), G (trace, output f F + m,
+//        input k) or P (output f B + b, input f F + m).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>

@@ -44,11 +44,20 @@ namespace ltsdev {
 // of a face's six rows, YT: of a time-kernel product's row, BBP: padded modes of top degree (column
 // phase). Order 5: one CTA per SM (the straight-line code of one phase at a time in the
 // instruction cache).
-// What bounds it (order 5, anelastic, 16 elements, about 24,000 cycles): the row phases' staged reads
-// and multiply-adds one after the other (5,100 cycles over the four derivatives), the column
-// phases' instruction issue (5,900), the update's DOF stores. Measured on one GB300, 138,240
-// elements, one cluster: 4.7 ns per element against 6.6 ns with nine rows per K_c and 14 elements
-// per batch; with four clusters (half-step traces) 5.4 against 7.0 ns.
+// What bounds it (order 5, anelastic; about 20,700 cycles per 16 elements): phases of 18 warps
+// between barriers, each short of the SM's limits by its own latency. Time kernel: row phases
+// 5,000 cycles over the four derivatives (staged reads, multiply-adds), column phases 6,400 (issue:
+// Hooke's law, coupling and relaxation); volume and traces 3,200, interface states 2,600,
+// projection 1,800, update 1,900. 57 % of the issue slots, 2,964 warp instructions and 764
+// shared-memory wavefronts per element; barriers are the largest stall. Measured on one GB300,
+// 138,240 elements, ns per element, with nine rows per K_c and 14-element batches (order 5) before
+// and with the row form now:
+//   order 5, 3 mechanisms: 6.61 -> 4.25 (one cluster), 6.97 -> 4.86 (four clusters: half-step
+//   traces 0.42 of it); elastic 4.55 -> 3.20; 16 simulations 6.88 -> 4.66
+//   order 4: 3.10 -> 2.15, elastic 2.24 -> 1.38; order 3: 2.27 -> 1.05, elastic 1.15 -> 0.66
+// No gain from: the next batch started without a barrier after the update (-0.7 % with one cluster,
+// +1.4 % with four), the interface states with a face per lane, 15 instead of 16 row parts, two
+// CTAs of 8 elements per SM at order 5 (4.26 -> 4.92: instruction fetch).
 template <int O>
 struct SpShape;
 template <>

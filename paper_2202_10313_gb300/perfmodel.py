@@ -6,7 +6,8 @@ the face matrices block-triangular; the kernels skip those zero blocks); a fused
 multiply-add counts 2. Bytes count every value the kernel must move to or from HBM
 once: DOFs read and written, LTS buffers written (predict) or one 9 x B buffer read
 (neighbour: each element's buffer is needed once; the other three face neighbours'
-re-reads are assumed to hit L2), and the per-element tables.
+re-reads are assumed to hit L2; the sparse engine stores one trace per face, which one
+neighbour reads), and the per-element tables.
 """
 
 
@@ -73,6 +74,23 @@ def bytes_neighbour(o, m, n_fused=1):
     """HBM bytes of k_neighbour per element and simulation."""
     B, NQ = nbasis(o), 9 + 6 * m
     return 4 * 2 * NQ * B + 4 * 9 * B + (4 * 48 + 4 * 9) / n_fused
+
+
+def _traces(o):
+    """Bytes of an element's four stored face traces (six rows per face, 16-byte multiples)."""
+    return 4 * 4 * (-(-6 * nface(o) // 4) * 4)
+
+
+def bytes_predict_sparse(o, m, n_fused=1):
+    """HBM bytes of k_predict_sp per element and simulation: DOFs read and written, four face
+    traces written, the element's row of the tables."""
+    return 4 * 2 * (9 + 6 * m) * nbasis(o) + _traces(o) + (4 * 72 + 4) / n_fused
+
+
+def bytes_neighbour_sparse(o, m, n_fused=1):
+    """HBM bytes of k_neighbour_sp per element and simulation: DOFs read and written, the traces
+    of the four neighbours' faces read, tables and face links."""
+    return 4 * 2 * (9 + 6 * m) * nbasis(o) + _traces(o) + (4 * 64 + 4 * 8) / n_fused
 
 
 def paper_flops_per_update():
