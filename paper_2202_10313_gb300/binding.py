@@ -419,7 +419,7 @@ class Solver:
         self._check(lib().lts_set_adjoint_memory(self._h, int(nbytes)))
 
     def set_wait_limit(self, cycles=2000000000, suppress_commit=False):
-        self._check(lib().lts_set_wait_limit(self._h, int(cycles), 1 if suppress_commit else 0))
+        self._check(lib().lts_set_wait_limit(self._h, int(cycles), int(suppress_commit)))
 
     def set_contraction(self, mode):
         """'fp32' (CUDA cores), 'sparse' (CUDA cores, generated sparse products), 'tf32x3'

@@ -2586,7 +2586,7 @@ int lts_set_wait_limit(lts_t* h, int64_t cycles, int suppress_commit) {
   return run(h, [&] {
     if (cycles <= 0) fail(LTS_ERR_ARG, "wait limit must be positive");
     h->wait_cycles = cycles;
-    h->suppress_commit = suppress_commit != 0;
+    h->suppress_commit = suppress_commit == ltsdev::SUPPRESS_PART ? ltsdev::SUPPRESS_PART : suppress_commit != 0;
   });
 }
 

@@ -135,6 +135,10 @@ struct DevState {
   const float* msg;      // [cut faces][nsim][9][F] face-local messages of a partitioned run (else unused)
 };
 
+// Failure-path test: no copy is issued, or the neighbour kernel announces its traces and tables
+// without copying them (its DOFs are copied).
+constexpr int SUPPRESS_ALL = 1, SUPPRESS_PART = 2;
+
 // LTS buffers a predict pass of the sparse engine writes: face traces and / or modes
 constexpr int BUFS_TRACES = 1, BUFS_MODAL = 2;
 
@@ -148,9 +152,9 @@ struct PhaseArgs {
   // memory variables in closed form (sparse engine): d^d theta_l = (-omega_l)^d E_d with E_0 = theta_l,
   // E_{d+1} = E_d + rg[l][d] eps_d, and the time integral ra[cluster][l] theta_l + sum_d rh[..][d] eps_d
   float rp[3][5], rg[3][5], ra[MAXC][3], rh[MAXC][3][5];
-  // bounded waits of the asynchronous copies (k_predict_sp): the device error word a kernel
-  // sets when a wait gives up, the bound in SM cycles, and the failure-path test switch
-  // (nothing is copied, so the waits run out)
+  // bounded waits of the asynchronous copies (sparse engine): the device error word a kernel
+  // sets when a wait gives up, the bound in SM cycles, and the failure-path test switch (nonzero:
+  // the waits run out; SUPPRESS_ALL, SUPPRESS_PART)
   int* err;
   long long wait;
   int suppress;

@@ -931,10 +931,10 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
       uint32_t bytes = (uint32_t)__popc(m) * FS * 4;
       if (tid == 0) bytes += (uint32_t)ne * NDS * 4;
       tc::mbar_expect(barT, bytes);
-      if (tid == 0) tc::bulk_copy(smem + S::S_D + buf * NE * NDS, st.sndata + (size_t)e0 * NDS, (uint32_t)ne * NDS * 4, barT);
+      if (tid == 0 && !ph.suppress) tc::bulk_copy(smem + S::S_D + buf * NE * NDS, st.sndata + (size_t)e0 * NDS, (uint32_t)ne * NDS * 4, barT);
     }
     __syncwarp();
-    if (l.x >= 0) {
+    if (l.x >= 0 && !ph.suppress) {
       const bool second = (l.y & 4) && ph.parity[l.y >> 8] == 1;
       const size_t face = FUSED ? ((size_t)(l.x >> 2) * st.nsim + (f0 + tid / 4) % sl.nsim) * 4 + (l.x & 3) : (size_t)l.x;
       tc::bulk_copy(sT + tid * FS, (second ? st.T2 : st.T1) + face * FS, FS * 4, barT);
@@ -950,14 +950,13 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
   __syncthreads();
   wait_for_previous_kernel();
   let_next_kernel_launch();
-  if (!ph.suppress && blockIdx.x < nbatch) {
+  if (ph.suppress != SUPPRESS_ALL && blockIdx.x < nbatch) {
     if (tid < NFT) fetch(blockIdx.x, 0, first);
     if (tid == 0) issue_q(blockIdx.x);
   }
   __syncthreads();   // the orientations written by fetch
   uint32_t par = 0;
-  bool done = false;
-  for (int batch = blockIdx.x; batch < nbatch && !done; batch += gridDim.x, par ^= 1) {
+  for (int batch = blockIdx.x; batch < nbatch; batch += gridDim.x, par ^= 1) {
     const int t0 = batch * NE, next = batch + gridDim.x;
     const int* sI = reinterpret_cast<const int*>(smem + S::S_I) + par * 4 * NE;
     const float* sD = smem + S::S_D + par * NE * NDS;
@@ -994,21 +993,29 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
 #pragma unroll
       for (int r = 0; r < 6; ++r) wp[r * GP] = w6[r];
     }
-    __syncthreads();
+    // a wait that gave up: the phase is still open (its copies may land yet), so nothing more may
+    // arrive on its mbarrier or be copied into its memory, and every thread leaves
+    if (!__syncthreads_and(ok)) {
+      if (tid == 0) {
+        atomicOr(ph.err, 1);
+        tc::mbar_wait(barT, par, ph.wait);         // the copies in flight, if any, land first
+        tc::mbar_wait(barQ, par, ph.wait);
+      }
+      break;
+    }
     // the batch's traces have been read: the next batch's copies go out now
-    if (next < nbatch && !ph.suppress && tid < NFT) fetch(next, par ^ 1, links);
+    if (next < nbatch && tid < NFT) fetch(next, par ^ 1, links);
     // ---- projection of the faces' states through F^_f
     if (pact) sg_nproj<O, 6 * BP, GS>(part, sW + pe * S::ESW + pr * GP, sP + pe * S::ESP + pr * BP);
-    // ---- the batch's DOFs have arrived (or a wait gave up: every thread leaves)
-    ok = tc::mbar_wait(barQ, par, ph.wait) && ok;
+    // ---- the batch's DOFs have arrived (or the wait gave up: every thread leaves)
+    ok = tc::mbar_wait(barQ, par, ph.wait);
     if (!__syncthreads_and(ok)) {
       if (tid == 0) {
         atomicOr(ph.err, 1);
         tc::mbar_wait(barQ, par, ph.wait);         // the copies in flight, if any, land first
         if (next < nbatch) tc::mbar_wait(barT, par ^ 1, ph.wait);
       }
-      done = true;
-      continue;
+      break;
     }
     if (act && t0 + es < sl.n) {
       const float* nd = sD + pos_of(es) * NDS;
@@ -1044,7 +1051,7 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
         for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = fmaf(-ph.omega[l], eps[r], qr[(9 + 6 * l + r) * RS]);
     }
     __syncthreads();
-    if (tid == 0 && next < nbatch && !ph.suppress) issue_q(next);
+    if (tid == 0 && next < nbatch) issue_q(next);
   }
 }
 

@@ -242,3 +242,37 @@ def test_dof_copy_wait_runs_out_and_handle_recovers():
     ora.run_gts(ora.time_step_gts(0.5), 2)
     err = rel_l2_groups(gpu.get_dofs(), ora.Q, 9)
     assert err["all"] <= TOL, err
+
+
+@pytest.mark.parametrize("order,n_mech,fused,tile", [(3, 0, 1, 1), (4, 3, 1, 0), (5, 3, 1, 1), (5, 0, 4, 0)])
+def test_trace_copy_wait_runs_out_on_an_open_phase(order, n_mech, fused, tile):
+    """Failure path of the neighbour kernel's trace copies: announced but never issued, while the
+    DOFs are copied, over more batches than resident CTAs hold at once. The wait runs out on a phase
+    that is still open: nothing more may arrive on it, the copies in flight land, the call reports
+    LTS_ERR_TIMEOUT, and the same handle then gives bitwise what a handle that never timed out gives."""
+    from paper_2202_10313_gb300 import binding
+    m = synth.permute_vertex_order(synth.graded_box(18, 17, 5, 200.0, 100.0, seed=7), seed=3)
+    mat = synth.random_layers(m, n_layers=2, seed=3)
+    K = m["tet"].shape[0]
+    d0 = synth.random_dofs(K, 9 + 6 * n_mech, order * (order + 1) * (order + 2) // 6, seed=12)
+    d0 = d0 if fused == 1 else np.stack([d0 * (f + 1) for f in range(fused)])
+    got = []
+    for fails in (True, False):
+        s = binding.Solver(order, n_mech, device=0, n_fused=fused)
+        s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+        s.set_material(mat["rho"], mat["vp"], mat["vs"], *((mat["qp"], mat["qs"]) if n_mech else ()))
+        s.set_tile(tile)
+        s.setup_clusters(2, 0.5)
+        s.set_dofs(d0)
+        if fails:
+            s.set_wait_limit(200000, suppress_commit=2)
+            s.advance_steps(2)
+            with pytest.raises(binding.LtsError) as ei:
+                s.get_dofs()
+            assert ei.value.code == binding.LTS_ERR_TIMEOUT
+            s.set_wait_limit()
+            s.set_dofs(d0)
+        s.advance_steps(4)
+        got.append(s.get_dofs())
+        s.close()
+    assert np.array_equal(got[0], got[1])
