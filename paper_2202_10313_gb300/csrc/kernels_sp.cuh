@@ -115,8 +115,8 @@ struct SpCfg {
   static_assert(NTA % 32 == 0 && BP >= B && GP >= F && GS >= 6 * GP && BBP >= BB, "shape");
   static_assert(YT >= BA && (YT / 4) % 2 == 1 && (BP / 4) % 2 == 1 && (GP / 4) % 2 == 1, "row strides");
   static constexpr bool TM = M > 0;   // part of the column state lives in tensor memory
-  // tensor-memory columns: 36 per warp of a lane quarter, a power of two in all
-  static constexpr int TMC = (NW + 3) / 4 * 36 <= 128 ? 128 : 256;
+  // tensor-memory columns: TMW per warp of a lane quarter, a power of two in all
+  static constexpr int TMW = 54, TMC = (NW + 3) / 4 * TMW <= 128 ? 128 : (NW + 3) / 4 * TMW <= 256 ? 256 : 512;
   // element strides: ESM modulo 32, odd in 16-byte units
   static constexpr int es(int n) { return n + (H::ESM - n % 32 + 32) % 32; }
   static constexpr int ESX = es(15 * BP);              // v (3), tau_0, tau_1, tau_2, tau_3 (3 rows each); then
@@ -365,8 +365,8 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     tc::bulk_store(st.Q + off, sG, bytes);
   };
   // Tensor memory as per-thread storage (anelastic): the time integrals and the half-step integrals
-  // between the derivatives, and the update's known terms between the volume products and the
-  // update. 18 warps of 96 registers hold the rest without spills
+  // between the derivatives, and the update's known terms and the memory variables between the
+  // volume products and the update. 18 warps of 96 registers hold the rest without spills
   // (spilling instead: 62 local-memory instructions per element, most of them missing L1).
   uint32_t* sTm = reinterpret_cast<uint32_t*>(smem + S::S_BAR + 2);
   uint32_t tm = 0;
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
   __syncthreads();
   if constexpr (S::TM) {
     tc::fence_after_sync();
-    tm = *sTm + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * 36;
+    tm = *sTm + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * S::TMW;
   }
   wait_for_previous_kernel();
   let_next_kernel_launch();
@@ -598,25 +598,30 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
         }
       }
     }
-    // the update's terms that are already known: Q + E^l T^{a,l} and Q^{a,l} - omega_l T^{a,l}
+    // the update's terms that are already known: Q + E^l T^{a,l}, and Q^{a,l}, kept apart from
+    // T^{a,l} until the strain rate is known: what is added to a row of Q first costs it a rounding
+    // (order 5, 34,560 elements, 4 steps against 64 bits: stress 1.26e-7 -> 1.05e-7 with the
+    // mechanisms summed first, memory variables 1.13e-7 -> 1.07e-7 with one rounding; no slower)
     float acc[9];
     {
       const float* q = sQ + soff;
+      if constexpr (M == 0) {
 #pragma unroll
-      for (int r = 0; r < 9; ++r) acc[r] = valid ? q[r * RS] : 0.f;
-      if constexpr (M > 0) {
+        for (int r = 0; r < 9; ++r) acc[r] = valid ? q[r * RS] : 0.f;
+      } else {
         float ta[18];
         tc::tmem_ld18(tm, ta);
         const float4 m0 = ld4(ed + 12), m1 = ld4(ed + 16);
         const float ylam[3] = {m0.w, m1.y, m1.w}, ymu[3] = {m1.x, m1.z, ed[20]};
 #pragma unroll
+        for (int r = 0; r < 9; ++r) acc[r] = 0.f;
+#pragma unroll
         for (int l = 0; l < M; ++l) coupling_add(acc, ta + 6 * l, ylam[l], ymu[l]);
 #pragma unroll
-        for (int l = 0; l < M; ++l)
+        for (int r = 0; r < 9; ++r) acc[r] += valid ? q[r * RS] : 0.f;
 #pragma unroll
-          for (int r = 0; r < 6; ++r)
-            ta[6 * l + r] = fmaf(-ph.omega[l], ta[6 * l + r], valid ? q[(9 + 6 * l + r) * RS] : 0.f);
-        tc::tmem_st18(tm, ta);
+        for (int r = 0; r < NA; ++r) ta[r] = valid ? q[(9 + r) * RS] : 0.f;
+        tc::tmem_st18(tm + 36, ta);
         tc::tmem_st9(tm + 18, acc);
         tc::tmem_wait_st();
       }
@@ -668,11 +673,10 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     }
     __syncthreads();
     // ---- update: volume and local surface terms of all four directions at once
-    float ta[NA > 0 ? NA : 1];
-    if constexpr (S::TM) {
-      tc::tmem_ld18(tm, ta);
-      tc::tmem_ld9(tm + 18, acc);
-    }
+    if constexpr (S::TM) tc::tmem_ld9(tm + 18, acc);
+    float* q = S::STAGE ? sG + soff
+                        : st.Q + (size_t)(valid ? elem_of(es) : 0) * qs + Slots<FUSED>::sub(FUSED ? sSlot[NE + es] : 0, NQ, B) + (size_t)b * CS;
+    float out[9], eps[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (valid) {
       const float* yp = sY + es * S::ESY + b;
       const Geo geo(ed);
@@ -701,19 +705,24 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
 #pragma unroll
         for (int i = 0; i < 3; ++i) dv[i] += Z[3 + i];
       }
-      float out[9], eps[6];
       hooke(G, m0.x, m0.y, out, eps);
-      float* q = S::STAGE ? sG + soff
-                          : st.Q + (size_t)elem_of(es) * qs + Slots<FUSED>::sub(FUSED ? sSlot[NE + es] : 0, NQ, B) + (size_t)b * CS;
 #pragma unroll
       for (int r = 0; r < 6; ++r) q[r * RS] = acc[r] - out[r];
 #pragma unroll
       for (int i = 0; i < 3; ++i) q[(6 + i) * RS] = fmaf(-m0.z, dv[i], acc[6 + i]);
-#pragma unroll
-      for (int l = 0; l < M; ++l)
-#pragma unroll
-        for (int r = 0; r < 6; ++r) q[(9 + 6 * l + r) * RS] = fmaf(-ph.omega[l], eps[r], ta[6 * l + r]);
       if (S::STAGE && !FUSED && b < C::QS - NQ * B) sG[es * C::QS + NQ * B + b] = 0.f;   // padding
+    }
+    if constexpr (S::TM) {
+      float ta[18], qa[18];
+      tc::tmem_ld18(tm, ta);
+      tc::tmem_ld18(tm + 36, qa);
+      if (valid) {
+#pragma unroll
+        for (int l = 0; l < M; ++l)
+#pragma unroll
+          for (int r = 0; r < 6; ++r)
+            q[(9 + 6 * l + r) * RS] = fmaf(-ph.omega[l], ta[6 * l + r] + eps[r], qa[6 * l + r]);
+      }
     }
     if constexpr (S::STAGE) tc::fence_smem_to_async();
     last = batch;
