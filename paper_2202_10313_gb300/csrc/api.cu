@@ -1131,7 +1131,8 @@ __global__ void k_grad_contract(GradGeom g, const double* faces, double* grad) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= g.K) return;
   const double* ws = g.W + (size_t)g.iperm[e] * ltsdev::WG_SIZE + ltsdev::WG_STAR;
-  const double star[3] = {-ws[2] / (g.rho[e] * g.rho[e]), ws[0], ws[1]};
+  // the sums carry the factors of the star matrices' entries (StarGeo)
+  const double star[3] = {-ws[2] / g.rho[e], g.lam[e] != 0.0 ? ws[0] / g.lam[e] : ws[0], ws[1] / g.mu[e]};
   for (int p = 0; p < 3; ++p) {
     double acc = star[p];
     for (int i = 0; i < 4; ++i) {
@@ -1156,11 +1157,14 @@ __global__ void k_build_amat(GradGeom g, float* amat) {
   const double rho = g.rho[k], lam = g.lam[k], mu = g.mu[k], rinv = 1.0 / rho;
   if (task == 0) {
     out += ltsdev::AM_GEO;
-    for (int q = 0; q < 9; ++q) out[q] = (float)g.jinv[9 * k + q];
-    out[9] = (float)lam;
-    out[10] = (float)mu;
-    out[11] = (float)rinv;
-    for (int q = 0; q < 12; ++q) out[12 + q] = (float)g.normal[12 * k + q];
+    for (int q = 0; q < 9; ++q) {
+      const double j = g.jinv[9 * k + q];
+      out[q] = (float)(mu * j);
+      out[9 + q] = (float)(lam != 0.0 ? lam * j : j);
+      out[18 + q] = (float)(rinv * j);
+    }
+    out[27] = lam != 0.0 ? 1.f : 0.f;
+    for (int q = 0; q < 12; ++q) out[ltsdev::AM_NRM + q] = (float)g.normal[12 * k + q];
     return;
   }
   const int i = task - 1;

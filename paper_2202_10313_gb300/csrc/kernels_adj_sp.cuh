@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
               float y[9];
 #pragma unroll
               for (int s = 0; s < 9; ++s) y[s] = sW[(c * B + b) * XP + col + s];
-              st.add(geo.J + 3 * c, y);
+              st.add(geo, c, y);
             }
             st.get(geo, v);
           }
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
             float v[9];
 #pragma unroll
             for (int s = 0; s < 9; ++s) v[s] = sW[(c * B + b) * XP + col + s];
-            st.add(geo.J + 3 * c, v);
+            st.add(geo, c, v);
           }
           st.get(geo, w);
           st.sums(T, -1.f, wst);
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
           tf[s] = tp[s];
         }
         flux_transposed(sAl + e * 432 + i * 108, lf, u);
-        face_products(sGeo + e * AM_NGEO + 12 + 3 * i, lf, tf, o);
+        face_products(sGeo + e * AM_NGEO + AM_NRM + 3 * i, lf, tf, o);
 #pragma unroll
         for (int r = 0; r < 9; ++r) {
           lp[r] = u[r];
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(AdjSpCfg<O>::NT, 2) k_adj_pred_sp(AdjLtsArgs a
               float z[9];
 #pragma unroll
               for (int r = 0; r < 9; ++r) z[r] = sW[(c * B + b) * XP + col + r];
-              st.add(geo.J + 3 * c, z);
+              st.add(geo, c, z);
             }
             float w[9], x[9];
             st.get(geo, w);

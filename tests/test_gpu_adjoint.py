@@ -485,3 +485,38 @@ def test_moment_tensor_gradient_against_central_differences(clustered):
                 t.close()
             fd = (vals[0] - vals[1]) / (2 * h)
             assert abs(fd - g[i, r]) <= 2e-3 * np.abs(g).max(), (i, r, fd, g[i, r])
+
+
+def _badly_rounded(lo, hi, fn, n=4000):
+    """The value x in [lo, hi) (of n) whose fn(x) gains most by rounding to FP32."""
+    x = lo + (hi - lo) * np.arange(n) / n
+    y = fn(x)
+    return float(x[np.argmax(np.float32(y).astype(float) / y)])
+
+
+@pytest.mark.parametrize("engine", ["sparse", "fp32"])
+@pytest.mark.parametrize("order", [3, 4])
+def test_adjoint_error_does_not_depend_on_how_the_material_rounds(order, engine):
+    """dJ/dQ0 against the FP64 oracle in two homogeneous models: one whose 1/rho, lambda and mu are
+    FP32 numbers, one in which each of them is rounded up by nearly half a unit. The reverse sweep's
+    operators hold the material only in entries that are rounded once, each by itself, so the errors
+    agree (15 %: two sets of some 5,000 roundings a step over 24 steps); with the three factors held
+    apart each scales an element's whole matrix by up to 6e-8 in every step. The observed data are
+    large against the samples: the forward sweep's own rounding does not show."""
+    m, _, q0, rec, src = _case(order)
+    K, n = m["tet"].shape[0], 24
+    models = [(2048.0, 2.0 ** 34, 2.0 ** 34)]
+    models.append((_badly_rounded(2100.0, 2200.0, lambda x: 1.0 / x), _badly_rounded(1.75e10, 1.8e10, lambda x: x),
+                   _badly_rounded(1.75e10, 1.8e10, lambda x: x)))
+    data = 1e4 * np.random.default_rng(3).normal(size=(n + 1, 3, 3))
+    err = []
+    for values in models:
+        rho, lam, mu = (np.full(K, v) for v in values)
+        om = Mesh(m["xyz"], m["tet"], m["face_bc"])
+        dt = Oracle(order, 0, om, rho, np.sqrt((lam + 2 * mu) / rho), np.sqrt(mu / rho)).time_step_gts(0.5)
+        (_, _, want, _), _ = _oracle(order, m, rho, lam, mu, q0, rec, src, data, dt, n)
+        s = _gpu(order, m, rho, lam, mu, q0, rec, src, dt, engine)
+        _, _, _, dq0 = s.misfit_gradient(n, data, every=n, want_dq0=True)
+        s.close()
+        err.append(_rel(dq0, want))
+    assert err[1] <= 1.15 * err[0], err
