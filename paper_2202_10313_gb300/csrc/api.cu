@@ -645,13 +645,19 @@ void require_material(lts_solver* h) {
   if (!h->has_mat) fail(LTS_ERR_STATE, "no material");
 }
 
-void ensure_capacity(void** ptr, size_t* cap, size_t need, size_t elem) {
+// Grows a buffer that kernels already queued on `stream` may still read or write (a copy on the legacy
+// default stream is not ordered after a non-blocking stream): the copy follows them, and the old
+// memory goes once it has completed.
+void ensure_capacity(void** ptr, size_t* cap, size_t need, size_t elem, cudaStream_t stream) {
   if (need <= *cap) return;
   size_t nc = std::max(need, *cap * 2 + 16);
   void* p = nullptr;
   ck(cudaMalloc(&p, nc * elem), "cudaMalloc scratch");
   if (*ptr) {
-    ck(cudaMemcpy(p, *ptr, *cap * elem, cudaMemcpyDeviceToDevice), "grow copy");
+    cudaError_t e = cudaMemcpyAsync(p, *ptr, *cap * elem, cudaMemcpyDeviceToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) cudaFree(p);
+    ck(e, "grow copy");
     cudaFree(*ptr);
   }
   *ptr = p;
@@ -945,9 +951,9 @@ void advance_steps(lts_solver* h, int64_t n_finest, cudaStream_t stream) {
   std::vector<MacroPlan> plans(nmac);
   size_t seis_need = h->seis_used;
   for (int64_t m = 0; m < nmac; ++m) plan_macro(h, s0 + m * period, seis_need, plans[m]);
-  ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, seis_need * 9 * h->nsim, sizeof(float));
-  ensure_capacity(reinterpret_cast<void**>(&h->d_ritems), &h->ritems_cap, plans[0].ritems.size(), sizeof(RecvItem));
-  ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, plans[0].sitems.size(), sizeof(SrcItem));
+  ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, seis_need * 9 * h->nsim, sizeof(float), stream);
+  ensure_capacity(reinterpret_cast<void**>(&h->d_ritems), &h->ritems_cap, plans[0].ritems.size(), sizeof(RecvItem), stream);
+  ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, plans[0].sitems.size(), sizeof(SrcItem), stream);
   h->seis_used = seis_need;
   for (int64_t m = 0; m < nmac; ++m) {
     const MacroPlan& mp = plans[m];
@@ -1463,9 +1469,9 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   auto keep_macro = [&](int64_t m, char* snap_m) {
     size_t seis_need = h->seis_used;
     plan_macro(h, s0 + m * period, seis_need, mp);
-    ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, seis_need * 9 * h->nsim, sizeof(float));
-    ensure_capacity(reinterpret_cast<void**>(&h->d_ritems), &h->ritems_cap, mp.ritems.size(), sizeof(RecvItem));
-    ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, mp.sitems.size(), sizeof(SrcItem));
+    ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, seis_need * 9 * h->nsim, sizeof(float), stream);
+    ensure_capacity(reinterpret_cast<void**>(&h->d_ritems), &h->ritems_cap, mp.ritems.size(), sizeof(RecvItem), stream);
+    ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, mp.sitems.size(), sizeof(SrcItem), stream);
     h->seis_used = seis_need;
     upload_items(h, mp, stream);
     h->msg_bytes += macro_msg_bytes(h, mp);
@@ -1602,7 +1608,7 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
     h->s_now = sb0;
     size_t seis_need = h->seis_used;
     plan_macro(h, sb0, seis_need, mp);
-    ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, mp.sitems.size(), sizeof(SrcItem));
+    ensure_capacity(reinterpret_cast<void**>(&h->d_sitems), &h->sitems_cap, mp.sitems.size(), sizeof(SrcItem), stream);
     if (!mp.sitems.empty())
       ck(cudaMemcpyAsync(h->d_sitems, mp.sitems.data(), mp.sitems.size() * sizeof(SrcItem), cudaMemcpyHostToDevice,
                          stream),
@@ -2208,7 +2214,7 @@ int lts_checkpoint_load(lts_t* h, const char* path) {
     ck(cudaDeviceSynchronize(), "synchronize");
     ck(cudaMemcpy(h->dst.Q, q.data(), q.size() * sizeof(float), cudaMemcpyHostToDevice), "upload Q");
     const size_t nsamp = seis.size() / (9 * h->nsim);
-    ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, nsamp * 9 * h->nsim, sizeof(float));
+    ensure_capacity(reinterpret_cast<void**>(&h->d_seis), &h->seis_cap, nsamp * 9 * h->nsim, sizeof(float), nullptr);
     if (!seis.empty())
       ck(cudaMemcpy(h->d_seis, seis.data(), seis.size() * sizeof(float), cudaMemcpyHostToDevice), "upload samples");
     int64_t slot = 0;

@@ -73,3 +73,31 @@ def test_energy_sentinel_flags_non_finite_state():
     with pytest.raises(binding.LtsError) as ei:
         g.energy()
     assert ei.value.code == binding.LTS_ERR_NONFINITE
+
+
+@pytest.mark.parametrize("fused,graphs", [(1, True), (1, False), (4, True)])
+def test_samples_survive_the_growth_of_their_buffer_on_a_side_stream(fused, graphs):
+    """Many asynchronous calls on a non-blocking stream without a synchronisation: the sample buffer
+    grows while receiver kernels of earlier calls are still queued. Every sample equals that of one
+    call over the same steps, which sizes the buffer once."""
+    torch = pytest.importorskip("torch")
+    m = synth.permute_vertex_order(synth.graded_box(24, 24, 8, 250.0, 125.0, seed=4), seed=2)
+    mat = synth.random_layers(m, n_layers=3, seed=5)
+    K, calls = m["tet"].shape[0], 24
+    d0 = synth.random_dofs(K, 9, 20, seed=12)
+    out = []
+    for n in (calls, 1):
+        s = binding.Solver(4, 0, device=0, n_fused=fused)
+        s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+        s.set_material(mat["rho"], mat["vp"], mat["vs"])
+        s.set_graphs(graphs)
+        ids = [s.add_receiver(np.array([1500.0 + 700.0 * i, 2000.0, -100.0]), 2e-4) for i in range(4)]
+        s.setup_clusters(2, 0.5)
+        s.set_dofs(d0 if fused == 1 else np.stack([d0 * (f + 1) for f in range(fused)]))
+        stream = torch.cuda.Stream()
+        for _ in range(n):
+            s.advance_steps(2 * calls // n, stream=stream)
+        out.append([s.seismogram(i, f) for i in ids for f in range(fused)])
+        s.close()
+    for (ta, va), (tb, vb) in zip(*out):
+        assert len(ta) > calls and np.array_equal(ta, tb) and np.array_equal(va, vb)
