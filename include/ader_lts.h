@@ -337,8 +337,9 @@ int lts_set_graphs(lts_t* h, int enable);
  * timeout, lets its copies in flight land (again within the bound), releases its tensor memory
  * and returns; the next synchronising call returns LTS_ERR_TIMEOUT (and clears the report) while
  * the handle stays usable. The DOFs are then undefined. suppress_commit = 2: the same, but the
- * sparse neighbour kernel copies its DOFs and announces its traces and tables without copying
- * them (a wait that runs out on an open phase). Errors: LTS_ERR_ARG for cycles <= 0. */
+ * sparse predict kernel copies the first batch of each CTA, and the sparse neighbour kernel
+ * copies its DOFs and announces its traces and tables without copying them (a wait that runs out
+ * after a finished batch, and one on an open phase). Errors: LTS_ERR_ARG for cycles <= 0. */
 int lts_set_wait_limit(lts_t* h, int64_t cycles, int suppress_commit);
 
 /* Autotuner over launch configurations: contraction engine (FP32 CUDA cores, sparse

@@ -135,8 +135,8 @@ struct DevState {
   const float* msg;      // [cut faces][nsim][9][F] face-local messages of a partitioned run (else unused)
 };
 
-// Failure-path test: no copy is issued, or the neighbour kernel announces its traces and tables
-// without copying them (its DOFs are copied).
+// Failure-path test: no copy is issued, or only those of the first batch of a predict CTA, and the
+// neighbour kernel announces its traces and tables without copying them (its DOFs are copied).
 constexpr int SUPPRESS_ALL = 1, SUPPRESS_PART = 2;
 
 // LTS buffers a predict pass of the sparse engine writes: face traces and / or modes

@@ -306,3 +306,34 @@ def test_anelastic_update_rounds_no_more_than_the_dense_engine(order):
         gpu.close()
     for k in ("stress", "velocity", "memory"):
         assert err["sparse"][k] <= 1.1 * err["fp32"][k], err
+
+
+@pytest.mark.parametrize("order,n_mech,fused", [(5, 3, 1), (5, 0, 4), (4, 3, 1)])
+def test_predict_wait_that_runs_out_keeps_the_finished_batches(order, n_mech, fused):
+    """A predict CTA whose second batch never arrives has finished its first one: its traces are in
+    the LTS buffers, so its DOFs must be too (order 5 writes them back a batch later). One cluster, a
+    CTA per SM and order in the caller's numbering: exactly the first 16 slots of every CTA change."""
+    import torch
+    from paper_2202_10313_gb300 import binding
+    m = synth.permute_vertex_order(synth.graded_box(12, 10, 8, 200.0, 100.0, seed=7), seed=3)
+    mat = synth.random_layers(m, n_layers=2, seed=3)
+    K = m["tet"].shape[0]
+    d0 = synth.random_dofs(K, 9 + 6 * n_mech, order * (order + 1) * (order + 2) // 6, seed=12)
+    d0 = d0 if fused == 1 else np.stack([d0 * (f + 1) for f in range(fused)])
+    s = binding.Solver(order, n_mech, device=0, n_fused=fused)
+    s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+    s.set_material(mat["rho"], mat["vp"], mat["vs"], *((mat["qp"], mat["qs"]) if n_mech else ()))
+    s.setup_clusters(1, 0.5)
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count * s.launch_config()["ctas_per_sm"][0]
+    assert 16 * ctas < K * fused
+    s.set_dofs(d0)
+    before = s.get_dofs()
+    s.set_wait_limit(200000, suppress_commit=2)
+    s.advance_steps(1)
+    with pytest.raises(binding.LtsError) as ei:
+        s.get_dofs()
+    assert ei.value.code == binding.LTS_ERR_TIMEOUT
+    changed = np.any(s.get_dofs() != before, axis=(-1, -2))
+    s.close()
+    want = np.arange(K * fused) < 16 * ctas
+    assert np.array_equal(changed if fused == 1 else changed.T.ravel(), want), (changed.sum(), want.sum())
