@@ -2308,9 +2308,10 @@ int lts_autotune(lts_t* h, int allow_tf32, void* cuda_stream, int* chosen, doubl
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const Launchers& X = h->L;
     const int64_t K = h->mesh.K;
-    const size_t qbytes = sizeof(float) * K * h->dst.qs, bbytes = sizeof(float) * K * h->dst.bs;
+    // the DOFs and the LTS buffers, modes or face traces (which are more than the modes at order 3)
+    const size_t sz[2] = {sizeof(float) * K * h->dst.qs, h->scratch_bytes};
     void* snap = nullptr;
-    if (cudaMalloc(&snap, qbytes + 3 * bbytes) != cudaSuccess) {
+    if (cudaMalloc(&snap, sz[0] + sz[1]) != cudaSuccess) {
       cudaGetLastError();
       fail(LTS_ERR_OOM, "no device memory for the autotune snapshot");
     }
@@ -2319,11 +2320,10 @@ int lts_autotune(lts_t* h, int allow_tf32, void* cuda_stream, int* chosen, doubl
       ~Free() { cudaFree(p); }
     } free_snap{snap};
     char* sp = static_cast<char*>(snap);
-    float* dev[4] = {h->dst.Q, h->dst.B1, h->dst.B2, h->dst.B3};
-    const size_t sz[4] = {qbytes, bbytes, bbytes, bbytes};
+    float* dev[2] = {h->dst.Q, h->dst.B1};
     auto copy_state = [&](bool save) {
       size_t off = 0;
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < 2; ++i) {
         ck(cudaMemcpyAsync(save ? static_cast<void*>(sp + off) : static_cast<void*>(dev[i]),
                            save ? static_cast<const void*>(dev[i]) : static_cast<const void*>(sp + off), sz[i],
                            cudaMemcpyDeviceToDevice, stream),

@@ -337,3 +337,33 @@ def test_predict_wait_that_runs_out_keeps_the_finished_batches(order, n_mech, fu
     s.close()
     want = np.arange(K * fused) < 16 * ctas
     assert np.array_equal(changed if fused == 1 else changed.T.ravel(), want), (changed.sum(), want.sum())
+
+
+@pytest.mark.parametrize("order,n_mech,fused", [(3, 0, 1), (3, 3, 4), (5, 3, 1)])
+def test_autotune_restores_the_traces(order, n_mech, fused):
+    """lts_autotune restores the DOFs and the LTS buffers exactly: the caller's block holds the same
+    bytes afterwards, at order 3 too, where the face traces take more room than the modal buffers."""
+    import torch
+    from paper_2202_10313_gb300 import binding
+    m = synth.permute_vertex_order(synth.graded_box(5, 4, 3, 200.0, 100.0, seed=7), seed=3)
+    mat = synth.random_layers(m, n_layers=2, seed=3)
+    K, nq, nb, nf = m["tet"].shape[0], 9 + 6 * n_mech, order * (order + 1) * (order + 2) // 6, order * (order + 1) // 2
+    s = binding.Solver(order, n_mech, device=0, n_fused=fused)
+    s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+    s.set_material(mat["rho"], mat["vp"], mat["vs"], *((mat["qp"], mat["qs"]) if n_mech else ()))
+    s.use_torch_memory(2)
+    s.setup_clusters(2, 0.5)
+    d0 = synth.random_dofs(K, nq, nb, seed=12)
+    s.set_dofs(d0 if fused == 1 else np.stack([d0 * (f + 1) for f in range(fused)]))
+    s.advance_steps(4)
+    torch.cuda.synchronize()
+    rows = lambda n: (n + 3) // 4 * 4 if fused == 1 else n * fused
+    up = lambda n: (n + 255) // 256 * 256
+    buffers = max(3 * up(4 * K * rows(9 * nb)), 4 * 2 * K * 4 * ((6 * nf + 3) // 4 * 4) * fused)
+    off = (-s._mem.data_ptr()) % 256
+    state = s._mem[off:off + up(4 * K * rows(nq * nb)) + buffers]
+    want = state.clone()
+    s.autotune()
+    torch.cuda.synchronize()
+    assert torch.equal(state, want)
+    s.close()
