@@ -9,12 +9,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <exception>
 #include <functional>
 #include <new>
 #include <numeric>
 #include <string>
-#include <system_error>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -22,6 +20,7 @@
 #include "../../include/ader_lts.h"
 #include "host.h"
 #include "host_flux.h"
+#include "host_parallel.h"
 #include "host_partition.h"
 #include "launch.h"
 
@@ -351,33 +350,6 @@ void free_device(lts_solver* h) {
   h->ready = false;
 }
 
-// fn(begin, end) over [0, n) in equal runs on the host's cores (small n: on this one).
-template <typename Fn>
-void host_parallel(int64_t n, int64_t grain, const Fn& fn) {
-  const int64_t cores = std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), 16);
-  const int64_t nt = std::max<int64_t>(1, std::min(cores, n / grain));
-  if (nt == 1) return fn(0, n);
-  std::vector<std::thread> pool;
-  std::exception_ptr failed[16];
-  auto part = [&](int64_t t) {
-    try {
-      fn(n * t / nt, n * (t + 1) / nt);
-    } catch (...) {
-      failed[t] = std::current_exception();
-    }
-  };
-  int64_t started = 1;
-  try {
-    for (; started < nt; ++started) pool.emplace_back(part, started);
-  } catch (const std::system_error&) {   // no more threads: the rest runs here
-  }
-  part(0);
-  for (int64_t t = started; t < nt; ++t) part(t);
-  for (std::thread& t : pool) t.join();
-  for (int64_t t = 0; t < nt; ++t)
-    if (failed[t]) std::rethrow_exception(failed[t]);
-}
-
 // Write to every page of [p, p + bytes) (about to be overwritten) unless all are resident: a
 // device copy into pages that the caller has not touched yet now and then takes 23 ms instead of
 // 0.7 (29 MB), faulting them in here 0.3. A look at resident pages costs a few microseconds.
@@ -390,7 +362,7 @@ void fault_in(void* p, size_t bytes) {
   if (mincore(first, n * page, in.data()) == 0 &&
       std::all_of(in.begin(), in.end(), [](unsigned char c) { return c & 1; }))
     return;
-  host_parallel((int64_t)n, 64, [&](int64_t begin, int64_t end) {
+  lts::host_parallel((int64_t)n, 64, [&](int64_t begin, int64_t end) {
     for (int64_t i = begin; i < end; ++i) *(volatile char*)std::max(first + i * page, (char*)p) = 0;
   });
 }
@@ -416,7 +388,7 @@ void setup_device(lts_solver* h) {
   std::vector<int2> nlink(4 * K, make_int2(-1, 0));
   std::vector<double> emat(4 * K);
   const lts::Mesh& M = h->mesh;
-  host_parallel(K, 4096, [&](int64_t begin, int64_t end) {
+  lts::host_parallel(K, 4096, [&](int64_t begin, int64_t end) {
   for (int64_t nk = begin; nk < end; ++nk) {
     const int64_t k = h->perm[nk];
     float* ed = &edata[nk * ltsdev::ED];
