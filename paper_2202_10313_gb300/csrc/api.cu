@@ -756,6 +756,17 @@ void plan_macro(lts_solver* h, int64_t s_begin, size_t& seis_need, MacroPlan& mp
 }
 
 // Kernel arguments of one phase (Taylor coefficients per cluster, element range, step parities).
+// The sparse predict kernel keeps a memory variable's derivatives as (-omega)^d E_d (PhaseArgs),
+// d <= 3, so E_d holds strain rates times (rate / omega)^(d - 1) of the mesh's fastest rate. That and
+// the powers of omega stay far inside FP32 in every seismic band (rate / omega = 1e4..1e7). Beyond
+// these bounds, (1e14)^2 with 1e10 to spare for the strain rates themselves, the handle takes the
+// dense kernels, whose recursion has no such factors.
+bool closed_form_in_range(const lts_solver* h) {
+  for (double om : h->omega)
+    if (!(om >= 1e-12 && om <= 1e12 && 10.0 / h->dt_min <= 1e14 * om)) return false;
+  return true;
+}
+
 PhaseArgs phase_args(const lts_solver* h, const Phase& ph) {
   PhaseArgs pa{};
   for (int l = 0; l < h->nc; ++l) {
@@ -807,7 +818,7 @@ PhaseArgs phase_args(const lts_solver* h, const Phase& ph) {
 int enqueue_phase(lts_solver* h, const Phase& ph, cudaStream_t stream, bool with_receivers = true,
                   float* adjoint_traces = nullptr) {
   const Launchers& X = h->L;
-  const bool use_sp = h->contraction == LTS_CONTRACT_SPARSE;
+  const bool use_sp = h->contraction == LTS_CONTRACT_SPARSE && closed_form_in_range(h);
   const bool use_tc = h->contraction == LTS_CONTRACT_TF32X3 || h->contraction == LTS_CONTRACT_TF32;
   const int passes = h->contraction == LTS_CONTRACT_TF32X3 ? 3 : 1;
   const int maxp = std::max(1, use_tc ? X.blocks_predict_tc : (use_sp ? X.blocks_predict_sp : X.blocks_predict));

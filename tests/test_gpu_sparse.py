@@ -367,3 +367,28 @@ def test_autotune_restores_the_traces(order, n_mech, fused):
     torch.cuda.synchronize()
     assert torch.equal(state, want)
     s.close()
+
+
+@pytest.mark.parametrize("order,fused,f_min", [(5, 1, 1e-20), (4, 4, 1e-39), (5, 1, 1e-9), (3, 1, 1e-4)])
+def test_relaxation_frequencies_far_below_the_mesh_rate(order, fused, f_min):
+    """Relaxation frequencies so low against the mesh that powers of their ratio leave FP32: finite,
+    and as close to the oracle as in any other band (at the two higher frequencies here the sparse
+    kernel itself runs)."""
+    from paper_2202_10313_gb300 import binding
+    m = synth.permute_vertex_order(synth.graded_box(4, 3, 3, 200.0, 100.0, seed=7), seed=3)
+    mat = synth.random_layers(m, n_layers=2, seed=3)
+    K, nb = m["tet"].shape[0], order * (order + 1) * (order + 2) // 6
+    _, ora, _ = make_pair(order, 3, m, mat, f_min, 5.0)
+    d0 = synth.random_dofs(K, 27, nb, seed=12)
+    s = binding.Solver(order, 3, device=0, n_fused=fused)
+    s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+    s.set_material(mat["rho"], mat["vp"], mat["vs"], mat["qp"], mat["qs"], f_min, 5.0)
+    s.setup_clusters(2, 0.5)
+    s.set_dofs(d0 if fused == 1 else np.stack([d0 * (f + 1) for f in range(fused)]))
+    s.advance_steps(4)
+    ora.setup_clusters(2, 0.5)
+    ora.Q = d0.copy()
+    ora.run_lts(4)
+    got = s.get_dofs()
+    s.close()
+    check_parity(got if fused == 1 else got[0], ora.Q, 27, TOL)
