@@ -81,7 +81,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct GraphKey {
   const void *seis, *ritems, *sitems, *block;
-  int contraction, ctas_p, ctas_n, suppress, parts, tile;
+  int contraction, ctas_p, ctas_n, suppress, parts, tile, modal;
   long long wait;
   size_t n_r, n_s;
 };
@@ -98,6 +98,7 @@ struct lts_solver {
   int contraction = LTS_CONTRACT_FP32;
   int ctas_predict = 0, ctas_neighbour = 0;  // resident CTAs per SM the grids are sized for (0: occupancy)
   int tile = 1;                              // tile variant of the sparse engine's neighbour kernel
+  bool modal_buffers = false;                // sparse engine: LTS buffers as modes only (other neighbour kernel)
   long long wait_cycles = ltsdev::TC_WAIT_CYCLES;   // bound of the tensor-core completion waits
   int suppress_commit = 0;                          // failure-path test: waits run out
   // emulated partitioned run (Sec. V-C): cut faces receive face-local messages
@@ -824,7 +825,7 @@ int enqueue_phase(lts_solver* h, const Phase& ph, cudaStream_t stream, bool with
   const int maxp = std::max(1, use_tc ? X.blocks_predict_tc : (use_sp ? X.blocks_predict_sp : X.blocks_predict));
   // the sparse engine's neighbour kernel reads every neighbour from local buffers: partitioned
   // runs (face-local messages) keep the gather-and-product neighbour kernel
-  const bool use_nsp = use_sp && X.neighbour_sp[0] && h->n_parts <= 1;
+  const bool use_nsp = use_sp && X.neighbour_sp[0] && h->n_parts <= 1 && !h->modal_buffers;
   const int tv = h->tile & 1;
   const int maxn = std::max(1, use_nsp ? X.blocks_neighbour_sp[tv] : X.blocks_neighbour);
   const int grid_cap_p = h->num_sms * (h->ctas_predict > 0 ? std::min(h->ctas_predict, maxp) : maxp);
@@ -962,6 +963,7 @@ void advance_steps(lts_solver* h, int64_t n_finest, cudaStream_t stream) {
     key.ctas_p = h->ctas_predict;
     key.ctas_n = h->ctas_neighbour;
     key.tile = h->tile;
+    key.modal = h->modal_buffers;
     key.wait = h->wait_cycles;
     key.suppress = h->suppress_commit;
     key.parts = h->n_parts;
@@ -1008,12 +1010,14 @@ struct DevBuf {
   T* get() const {
     return static_cast<T*>(p);
   }
+  bool try_alloc(size_t bytes) {
+    if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) == cudaSuccess) return true;
+    p = nullptr;
+    cudaGetLastError();
+    return false;
+  }
   void alloc(size_t bytes) {
-    if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) {
-      p = nullptr;
-      cudaGetLastError();
-      fail(LTS_ERR_OOM, "device allocation for the adjoint failed");
-    }
+    if (!try_alloc(bytes)) fail(LTS_ERR_OOM, "device allocation for the adjoint failed");
   }
 };
 
@@ -1340,11 +1344,12 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
     d_w.alloc(sizeof(double) * K * ltsdev::WG_SIZE);
     d_cp.alloc(sizeof(float) * ncp * K * qs);
     d_qn.alloc(sizeof(float) * K * qs);
-    // the replays write the LTS buffers as modes for the reverse sweep; the sparse engine's face
-    // traces, which usually share their memory, get their own
-    if (h->contraction == LTS_CONTRACT_SPARSE && h->n_parts <= 1)
-      d_tr.alloc(sizeof(float) * 2 * K * (size_t)X.TS * nsim);
   }
+  // the replays write the LTS buffers as modes for the reverse sweep; the sparse engine's face traces,
+  // which usually share their memory, get their own
+  const size_t trace_bytes = reverse && h->contraction == LTS_CONTRACT_SPARSE && h->n_parts <= 1
+                                 ? sizeof(float) * 2 * K * (size_t)X.TS * nsim
+                                 : 0;
   // moment-tensor gradient: [source][6] and one pass's source items with their scales
   const int nsrc = (int)h->sources.size();
   DevBuf d_sg, d_sgi, d_sgc;
@@ -1426,13 +1431,20 @@ void adjoint_lts(lts_solver* h, int64_t n_macro, int64_t every, const double* da
   // kept and each macro step is replayed once more just before its reverse.
   size_t free_b = 0, total_b = 0;
   ck(cudaMemGetInfo(&free_b, &total_b), "memory info");
-  const double budget = h->adj_budget ? (double)h->adj_budget : 0.5 * (double)free_b;
+  const double budget = h->adj_budget ? (double)h->adj_budget : 0.5 * ((double)free_b - (double)trace_bytes);
   const bool whole_segment = (double)segm * (double)per_macro <= budget;
   DevBuf d_snap;
   if (reverse) d_snap.alloc(whole_segment ? segm * per_macro : per_macro);
   char* snap = d_snap.get<char>();
   if (reverse && !whole_segment) d_mac.alloc(sizeof(float) * segm * K * qs);
   float* mac = d_mac.get<float>();
+  // last, and for speed alone: without room for the traces this call's steps use the modal buffers
+  // and the neighbour kernel that reads them (2,944 bytes per element and simulation at order 5)
+  struct Modal {
+    bool& flag;
+    ~Modal() { flag = false; }
+  } modal{h->modal_buffers};
+  if (trace_bytes > 0) h->modal_buffers = !d_tr.try_alloc(trace_bytes);
   // one macro step of the forward sweep (as advance_steps), its phases' inputs kept in `snap`
   auto snapshot = [&](size_t pi, const Phase& ph, char* dst) {
     if (ph.kind == 1) {

@@ -520,3 +520,44 @@ def test_adjoint_error_does_not_depend_on_how_the_material_rounds(order, engine)
         s.close()
         err.append(_rel(dq0, want))
     assert err[1] <= 1.15 * err[0], err
+
+
+def test_fused_adjoint_without_room_for_the_face_traces():
+    """64 simulations with the device memory all but full: enough for the adjoint's states and phase
+    inputs, not for the sparse engine's face traces beside them. The gradient is the one of the call
+    with all the memory, to the rounding of two neighbour kernels."""
+    import torch
+    order, F = 4, 64
+    m = synth.permute_vertex_order(synth.graded_box(12, 8, 6, 200.0, 100.0, seed=6), seed=5)
+    K = m["tet"].shape[0]
+    mat = synth.random_layers(m, n_layers=2, seed=3)
+    q0 = synth.random_dofs(K, 9, 20, seed=4)
+    out = []
+    for full in (False, True):
+        s = binding.Solver(order, 0, device=0, n_fused=F)
+        s.set_mesh(m["xyz"], m["tet"], m["face_bc"])
+        s.set_material(mat["rho"], mat["vp"], mat["vs"])
+        s.add_receiver(m["xyz"].mean(axis=0), 1e-3)
+        s.setup_clusters(1, 0.5)
+        s.set_adjoint_memory(1)                    # one macro step's phase inputs at a time
+        s.set_dofs(np.stack([q0 * (1 + 0.1 * f) for f in range(F)]))
+        s.advance_steps(2)
+        torch.cuda.synchronize()
+        # floats per element and simulation: adjoints 4 x 180, two checkpoints, the end state, a
+        # macro-boundary state and the phase inputs (Q, B1) 6 x 180; the traces 2 x 240. (The room left
+        # would do for all three buffers among the inputs instead of the traces.)
+        unit, rest, traces = 4 * K * F, 10 * 180, 480
+        if full:
+            torch.cuda.empty_cache()
+            room = unit * (rest + traces - 100) + (48 << 20)
+            hog = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        J, g, _, dq0 = s.misfit_gradient(2, np.zeros((3, F, 1, 3)), every=1, want_dq0=True)
+        if full:
+            del hog
+            torch.cuda.empty_cache()
+        s.close()
+        out.append((J, g, dq0))
+    (Ja, ga, da), (Jb, gb, db) = out
+    assert abs(Ja / Jb - 1) <= 1e-5 and _rel(da, db) <= 1e-5
+    for p in range(3):
+        assert _rel(ga[:, p], gb[:, p]) <= 1e-4
