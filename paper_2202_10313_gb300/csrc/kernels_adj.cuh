@@ -133,20 +133,6 @@ struct AdjLtsArgs {
   int nsim, G;
 };
 
-// dst[q] = src[q] for q < N by a CTA of NT threads: every load is issued before the first
-// store, so the element's copies are in flight together.
-template <int N, int NT>
-__device__ __forceinline__ void stage(float* dst, const float* __restrict__ src, int t) {
-  constexpr int R = (N + NT - 1) / NT;
-  float v[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j)
-    if (t + j * NT < N) v[j] = __ldg(src + t + j * NT);
-#pragma unroll
-  for (int j = 0; j < R; ++j)
-    if (t + j * NT < N) dst[t + j * NT] = v[j];
-}
-
 // The nine rows of a [9][LD] block, entries j .. j + 3 (16-byte aligned; the same address in
 // every lane, so each load is one broadcast).
 template <int LD>
