@@ -58,6 +58,11 @@
 //        gen_sparse --list-rows <order> lists the terms of the row-form products likewise:
 //        kind T (output c B + b, input c B + k), V (volume, the same), G (trace, output f F + m,
 //        input k) or P (output f B + b, input f F + m).
+//        gen_sparse --list-parts <order> lists what the other two leave out: every variant of the
+//        row-form time products and the neighbour kernel's partition of the projections, a line
+//        "O kind variant part output" for each output that a part writes, then its terms,
+//        "kind variant part output input value" (kind T or N, output and input as for T and P).
+// (The kinds v, p and n of --list have no function of their own: the forward kernels use the row form.)
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -495,6 +500,9 @@ void emit_row_dispatch(FILE* f, const char* name, const char* tmpl, const char* 
   std::fprintf(f, "}\n");
 }
 
+// The neighbour kernel's parts of the projections: one per warp, of equal multiply-add count.
+Parts nproj_parts(const Products& P) { return partition_runs(P.rproj, P.O == 5 ? 6 : 4); }
+
 void emit_rows(FILE* f, int O, const Products& P) {
   char nm[64];
   std::snprintf(nm, sizeof nm, "sg_time_o%d", O);
@@ -510,7 +518,7 @@ void emit_rows(FILE* f, int O, const Products& P) {
                     {P.rproj_parts}, {P.rproj});
   std::snprintf(nm, sizeof nm, "sg_nproj_o%d", O);
   emit_row_dispatch(f, nm, "int DY, int DG", "DY, DG", "const float* __restrict__ g, float* __restrict__ y", "g, y",
-                    {partition_runs(P.rproj, O == 5 ? 6 : 4)}, {P.rproj}, true);
+                    {nproj_parts(P)}, {P.rproj}, true);
 }
 
 void emit_order(FILE* f, int O, int nparts) {
@@ -519,8 +527,6 @@ void emit_order(FILE* f, int O, int nparts) {
   std::fprintf(f, "// ---- order %d (B = %d, F = %d), %d parts\n", O, P.B, P.F, nparts);
   std::fprintf(f, "// multiply-adds per row: time kernel %zu (full variant), volume %zu, face traces %zu\n",
                P.time_terms, P.vol_terms, P.face_terms);
-  std::fprintf(f, "constexpr int kSpTimeTerms_o%d = %zu, kSpVolTerms_o%d = %zu, kSpFaceTerms_o%d = %zu;\n", O,
-               P.time_terms, O, P.vol_terms, O, P.face_terms);
   char nm[64];
   std::snprintf(nm, sizeof nm, "sp_time_o%d", O);
   emit_dispatch(f, nm, "const float* __restrict__ x, float* __restrict__ y", "x, y", P.time_parts, P.time, true);
@@ -579,6 +585,24 @@ int list_rows(int O) {
   return 0;
 }
 
+int list_parts(int O) {
+  Products P;
+  P.build(O, parts_of(O));
+  auto list = [&](char kind, size_t variant, const std::vector<RowOut>& outs, const Parts& parts, int in) {
+    for (size_t p = 0; p < parts.size(); ++p)
+      for (int o : parts[p]) {
+        const RowOut& u = outs[o];
+        std::printf("O %c %zu %zu %d\n", kind, variant, p, u.set * P.B + u.idx);
+        for (auto& x : u.t)
+          std::printf("%c %zu %zu %d %d %.9e\n", kind, variant, p, u.set * P.B + u.idx, u.set * in + x.first,
+                      (double)x.second);
+      }
+  };
+  for (size_t v = 0; v < P.rtime.size(); ++v) list('T', v, P.rtime[v], P.rtime_parts[v], P.B);
+  list('N', 0, P.rproj, nproj_parts(P), P.F);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -592,8 +616,13 @@ int main(int argc, char** argv) {
     if (O < 3 || O > 5) return 2;
     return list_rows(O);
   }
+  if (argc == 3 && std::strcmp(argv[1], "--list-parts") == 0) {
+    const int O = std::atoi(argv[2]);
+    if (O < 3 || O > 5) return 2;
+    return list_parts(O);
+  }
   if (argc != 2) {
-    std::fprintf(stderr, "usage: gen_sparse <out.cuh> | gen_sparse --list <order>\n");
+    std::fprintf(stderr, "usage: gen_sparse <out.cuh> | gen_sparse --list|--list-rows|--list-parts <order>\n");
     return 2;
   }
   FILE* f = std::fopen(argv[1], "w");

@@ -108,3 +108,40 @@ def test_row_form_terms_are_the_oracle_operators_nonzeros(order):
                 assert np.abs(w[c * B + nb1:(c + 1) * B]).max() <= 1e-10 * kmax
         assert np.abs(got[kind] - w).max() <= 1e-6 * scale, kind
         assert np.all((np.abs(w) <= 1e-10 * scale) | (got[kind] != 0.0)), kind
+
+
+@pytest.mark.parametrize("order", [3, 4, 5])
+def test_row_form_parts_write_every_output_once(order):
+    """Every variant of the row-form time products (modes k < nbasis(order - v) in, modes
+    b < nbasis(order - 1 - v) out, the elastic kernel's truncation) and the neighbour kernel's parts of
+    the projections (gen_sparse --list-parts): each output written by one part, with the oracle's
+    entries."""
+    build.build()
+    exe = os.path.join(build.OUT_DIR, "gen_sparse")
+    lines = subprocess.run([exe, "--list-parts", str(order)], capture_output=True, text=True, check=True).stdout.split("\n")
+    ob = Basis(order)
+    B, F = len(ob.K[0]), ob.Ft[0].shape[1]
+    n = lambda o: o * (o + 1) * (o + 2) // 6
+    want = {}
+    for v in range(order - 1):
+        w = np.zeros((3 * B, 3 * B))
+        for c in range(3):
+            w[c * B:c * B + n(order - 1 - v), c * B:c * B + n(order - v)] = ob.K[c][:n(order - 1 - v), :n(order - v)]
+        want["T", v] = (w, {c * B + b for c in range(3) for b in range(n(order - 1 - v))})
+    w = np.zeros((4 * B, 4 * F))
+    for f in range(4):
+        w[f * B:(f + 1) * B, f * F:(f + 1) * F] = ob.Ft[f]
+    want["N", 0] = (w, set(range(4 * B)))
+    got = {k: np.zeros_like(v[0]) for k, v in want.items()}
+    written = {k: [] for k in want}
+    for t in (x.split() for x in lines if x):
+        if t[0] == "O":
+            written[t[1], int(t[2])].append(int(t[4]))
+        else:
+            assert got[t[0], int(t[1])][int(t[3]), int(t[4])] == 0.0
+            got[t[0], int(t[1])][int(t[3]), int(t[4])] = float(t[5])
+    for k, (w, outs) in want.items():
+        assert len(written[k]) == len(outs) and set(written[k]) == outs, k
+        scale = max(np.abs(m).max() for m in (ob.K if k[0] == "T" else ob.Ft))
+        assert np.abs(got[k] - w).max() <= 1e-6 * scale, k
+        assert np.all((np.abs(w) <= 1e-10 * scale) | (got[k] != 0.0)), k
