@@ -22,7 +22,11 @@
 // a pass over shared memory per derivative and 567 FP64 additions per element (204 us a launch,
 // 126 with the sums; 47,040 elements, order 4), k_adj_nbr another 324.
 // The flux solvers are explicit (FP32, from the same closed forms as the forward kernels'
-// flux code), the star matrices are applied by their physical form; CUDA cores.
+// flux code), the star matrices are applied by their physical form (StarGeo); CUDA cores. The sums
+// are FP32 within a pass, with the normals and the star entries rounded to FP32, and FP64 over the
+// passes (the correlations were contracted with FP64 geometry once, at the end): against the FP64
+// gradient of 32 seeded cases each (1,008 elements, 12 steps) the errors are those of the correlations
+// times 1.03, 0.98, 0.97 (dJ/dlambda, orders 3, 4, 5), 1.06, 1.04, 0.97 (mu) and 0.81, 0.92, 0.80 (rho).
 #pragma once
 #include "kernels.cuh"
 
@@ -283,7 +287,7 @@ __device__ __forceinline__ void flux_transposed(const float* Am, const float l[9
   }
 }
 
-// One face mode's share in the ten sums of a flux solver (face_flux_dot in host_flux.h): l the
+// One face mode's share in the ten sums of a flux solver (face_flux_gradient in host_flux.h): l the
 // adjoint's column, x the state's. The flux maps the velocity v and the traction t of x
 // through normal and tangential coefficients to a state (v*, t*), and n v*^T (lambda, mu) and
 // t* / rho to the result; against l these are products of (n.v, n.t, v_T, t_T) with the trace

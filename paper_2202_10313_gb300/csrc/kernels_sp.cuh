@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
   let_next_kernel_launch();
   if (tid == 0 && blockIdx.x < nbatch && ph.suppress != SUPPRESS_ALL) issue(blockIdx.x, 0);
 
-  int last = -1;   // the batch whose updated DOFs are staged, not yet written back
+  int last = -1;   // the batch whose updated DOFs are staged (written back once the next has arrived)
   for (int batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
     const int t0 = batch * NE;
     const float* sE = smem + S::S_E + qpar * NE * EDS;
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
         break;
       }
     }
-    if (S::STAGE && tid == 0 && last >= 0) write_back(last);
+    if (S::STAGE && tid == 0 && batch != (int)blockIdx.x) write_back(batch - gridDim.x);
     // this column's DOFs in the staged copy (row stride RS, as in Q)
     int soff = es * C::QS + b;
     if constexpr (FUSED) soff = (es / FUSED_GROUP) * GB + b * CS + es % FUSED_GROUP;
