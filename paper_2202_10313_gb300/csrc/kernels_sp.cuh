@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
   }
   wait_for_previous_kernel();
   let_next_kernel_launch();
-  if (tid == 0 && blockIdx.x < nbatch && ph.suppress != SUPPRESS_ALL) issue(blockIdx.x, 0);
+  if (tid == 0 && blockIdx.x < nbatch && !(ph.suppress & SUPPRESS_ALL)) issue(blockIdx.x, 0);
 
   int last = -1;   // the batch whose updated DOFs are staged (written back once the next has arrived)
   for (int batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
@@ -440,6 +440,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
         if (tid == 0) {
           atomicOr(ph.err, 1);
           tc::mbar_wait(sBar, qpar ^ 1, ph.wait);   // the copies in flight, if any, land first
+          if (S::STAGE && last >= 0) write_back(last);   // the batch before is finished: its traces are out
         }
         break;
       }
@@ -674,8 +675,11 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
     __syncthreads();
     // ---- update: volume and local surface terms of all four directions at once
     if constexpr (S::TM) tc::tmem_ld9(tm + 18, acc);
-    float* q = S::STAGE ? sG + soff
-                        : st.Q + (size_t)(valid ? elem_of(es) : 0) * qs + Slots<FUSED>::sub(FUSED ? sSlot[NE + es] : 0, NQ, B) + (size_t)b * CS;
+    // this column of Q (anelastic: also for the memory variables, past the branch)
+    auto column = [&](int e) {
+      return S::STAGE ? sG + soff : st.Q + (size_t)e * qs + Slots<FUSED>::sub(FUSED ? sSlot[NE + es] : 0, NQ, B) + (size_t)b * CS;
+    };
+    float* q = S::TM ? column(valid ? elem_of(es) : 0) : nullptr;
     float out[9], eps[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (valid) {
       const float* yp = sY + es * S::ESY + b;
@@ -706,6 +710,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
         for (int i = 0; i < 3; ++i) dv[i] += Z[3 + i];
       }
       hooke(G, m0.x, m0.y, out, eps);
+      if constexpr (!S::TM) q = column(elem_of(es));
 #pragma unroll
       for (int r = 0; r < 6; ++r) q[r * RS] = acc[r] - out[r];
 #pragma unroll
@@ -783,7 +788,7 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
   if constexpr (S::STAGE) {
     __syncthreads();
     if (tid == 0) {
-      if (last >= 0) write_back(last);   // the CTA's last batch, or the one before a wait that gave up
+      if (last >= 0 && last + (int)gridDim.x >= nbatch) write_back(last);
       tc::bulk_store_wait();
     }
   }
@@ -959,7 +964,7 @@ __global__ void __launch_bounds__(SpnCfg<O, M, TILE, FUSED>::NT, SpnCfg<O, M, TI
   __syncthreads();
   wait_for_previous_kernel();
   let_next_kernel_launch();
-  if (ph.suppress != SUPPRESS_ALL && blockIdx.x < nbatch) {
+  if (!(ph.suppress & SUPPRESS_ALL) && blockIdx.x < nbatch) {
     if (tid < NFT) fetch(blockIdx.x, 0, first);
     if (tid == 0) issue_q(blockIdx.x);
   }
