@@ -204,7 +204,8 @@ int lts_transfer_bytes(lts_t* h, int64_t* h2d, int64_t* d2h);
  * in a neighbour kernel that reads the traces X F~_j which the predict kernel stores as its LTS
  * buffers and forms X F-_{j,h} as (X F~_j) R_h (R_h the face-basis map of the
  * orientation); with fused simulations it runs (element, simulation) slots, and a
- * partitioned run keeps the other engines' neighbour kernel. The adjoint's reverse predict
+ * partitioned run keeps the other engines' neighbour kernel, and relaxation frequencies below
+ * 1e-12 rad/s or 1e14 times below the mesh's rates the dense kernels (FP32 range). The adjoint's reverse predict
  * pass (lts_misfit_gradient) uses the same generated products (their transposed forms);
  * every other engine takes its dense-block kernel. The tensor-core engines' surface products run on CUDA cores. Takes effect at the next lts_advance. Errors: LTS_ERR_ARG for an unknown mode or a
  * mode the handle's shape has no kernel for (tensor cores: order 3 with one simulation).
@@ -244,7 +245,8 @@ int lts_cut_faces(lts_t* h, const int32_t* part, int64_t cap, int64_t* faces, in
  * its neighbour contribution from a face-local message instead of the neighbour's buffer —
  * before each neighbour pass a pack kernel computes, on the sending side, H = X F-_{j,h}
  * for the cut faces whose receivers are active, and the receiver's neighbour kernel reads
- * it. The arithmetic is the one of the unpartitioned run, in the same order. Fused runs
+ * it. The arithmetic is the one of the unpartitioned run, in the same order (sparse engine: that of
+ * the other engines' neighbour kernel, equal to rounding). Fused runs
  * send one message per simulation. If clusters are set up, re-creates the device state
  * (time 0, DOFs zero). n_parts <= 1 (part may be NULL) switches it off. Errors: LTS_ERR_ARG, LTS_ERR_STATE. */
 int lts_set_partition(lts_t* h, int n_parts, const int32_t* part);
@@ -292,7 +294,9 @@ int lts_set_finest_dt(lts_t* h, double dt);
  * fits the adjoint memory budget (lts_set_adjoint_memory; default half the free device
  * memory) the segment is replayed once; otherwise its macro-boundary states are kept and
  * each macro step is replayed once more just before its reverse, keeping one macro step's
- * phase inputs. Both orders give bitwise the same results.
+ * phase inputs. Both orders give bitwise the same results. The sparse engine's face traces take
+ * memory beside these, if there is any left; else the call's steps use the modal buffers (equal to
+ * rounding).
  * With grad and dq0 both NULL only the forward sweep and the misfit run.
  * Errors: LTS_ERR_ARG, LTS_ERR_STATE, LTS_ERR_OOM, LTS_ERR_CUDA. */
 int lts_misfit_gradient(lts_t* h, int64_t n_steps, int64_t every, const double* data, double* misfit,

@@ -20,13 +20,16 @@
 // and side, face_products). Each sum is a scalar product per (face) mode, so the threads
 // that hold the columns form it: the 3 x 3 tiles of the 9 x 9 correlations cost k_adj_pred_sp
 // a pass over shared memory per derivative and 567 FP64 additions per element (204 us a launch,
-// 126 with the sums; 47,040 elements, order 4), k_adj_nbr another 324.
+// 126 with the sums; 3 % more with the star matrices' entries as StarGeo holds them; 47,040
+// elements, order 4), k_adj_nbr another 324.
 // The flux solvers are explicit (FP32, from the same closed forms as the forward kernels'
 // flux code), the star matrices are applied by their physical form (StarGeo); CUDA cores. The sums
 // are FP32 within a pass, with the normals and the star entries rounded to FP32, and FP64 over the
 // passes (the correlations were contracted with FP64 geometry once, at the end): against the FP64
-// gradient of 32 seeded cases each (1,008 elements, 12 steps) the errors are those of the correlations
-// times 1.03, 0.98, 0.97 (dJ/dlambda, orders 3, 4, 5), 1.06, 1.04, 0.97 (mu) and 0.81, 0.92, 0.80 (rho).
+// gradient of 48 to 64 seeded cases each (1,008 elements, 12 steps) the errors are those of the
+// correlations times 1.05, 0.98, 1.00 (dJ/dlambda, orders 3, 4, 5), 1.03, 0.99, 0.98 (mu) and 0.91, 0.87,
+// 0.79 (rho), with a standard error of 2 to 4 %; with the normals as two FP32 numbers each 1.01 instead
+// of 1.05, and the gradient of 47,040 elements 6 % slower: not kept.
 #pragma once
 #include "kernels.cuh"
 

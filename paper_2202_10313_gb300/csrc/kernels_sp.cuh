@@ -52,12 +52,12 @@ namespace ltsdev {
 // shared-memory wavefronts per element; barriers are the largest stall. Measured on one GB300,
 // 138,240 elements, ns per element, with nine rows per K_c and 14-element batches (order 5) before
 // and with the row form now:
-//   order 5, 3 mechanisms: 6.61 -> 4.25 (one cluster), 6.97 -> 4.86 (four clusters: half-step
-//   traces 0.42 of it); elastic 4.55 -> 3.20; 16 simulations 6.88 -> 4.66
-//   order 4: 3.10 -> 2.15, elastic 2.24 -> 1.38; order 3: 2.27 -> 1.05, elastic 1.15 -> 0.66
+//   order 5, 3 mechanisms: 6.59 -> 4.19 (one cluster), 6.95 -> 4.82 (four clusters: half-step
+//   traces 0.42 of it); elastic 4.52 -> 3.19; 16 simulations 6.85 -> 4.62
+//   order 4: 3.09 -> 2.14, elastic 2.24 -> 1.37; order 3: 2.27 -> 1.03, elastic 1.13 -> 0.66
 // No gain from: the next batch started without a barrier after the update (-0.7 % with one cluster,
 // +1.4 % with four), the interface states with a face per lane, 15 instead of 16 row parts, two
-// CTAs of 8 elements per SM at order 5 (4.26 -> 4.92: instruction fetch).
+// CTAs of 8 elements per SM at order 5 (4.26 -> 4.92 when measured: instruction fetch).
 template <int O>
 struct SpShape;
 template <>
@@ -813,10 +813,10 @@ __global__ void __launch_bounds__(SpCfg<O, M, FUSED>::NT, SpShape<O>::MINB)
 // Everything a batch reads arrives by bulk asynchronous copies (TMA): a lane per face copies its
 // neighbour's trace and thread 0 the element tables while the previous batch projects and
 // updates, and the DOFs, which only the update reads, right after the previous update.
-// Measured on one GB300 (order 5, anelastic, 138,240 elements): 2.00 ns per element (1.49 elastic)
+// Measured on one GB300 (order 5, anelastic, 138,240 elements): 1.99 ns per element (1.49 elastic)
 // against 3.93 ns (3.43) with gathered buffers and face products in this kernel (4 x 1,260 bytes
 // and 2,365 instructions per element). Bound by instruction issue and latency between its three
-// barriers (42 % issue; DRAM 9.3 KB per element: 1.4 ns at the copy rate). Warps of two kinds that
+// barriers (41 % issue; DRAM 9.3 KB per element: 1.4 ns at the copy rate). Warps of two kinds that
 // hand batches over through double buffers (no CTA barrier, two CTAs per SM instead of three)
 // took 2.53 ns, and L2 prefetches one to four batches ahead 2.29-2.31 against 2.27 ns.
 template <int O>
